@@ -221,6 +221,68 @@ def run(state):
             "dinv_sqrt": csr.dinv_sqrt, "rdeg": csr.rdeg, "row_order": csr.row_order}
 
 
+# ---------------------------------------------------------------- the same results in 64 bits
+
+def _csr64(c, seed):
+    """(row pointers, sources, destinations) of the entries in (destination, source) order, as torch makes them."""
+    make = _rmat_graph if c["graph"] == "rmat" else _power_graph
+    src, dst = make(c["n"], c["e"], seed, torch.int64)
+    if "s" in c["flags"]:
+        loop = src == dst
+        src, dst = torch.cat([src, dst[~loop]]), torch.cat([dst, src[~loop]])
+    if "l" in c["flags"]:
+        keep, own = src != dst, torch.arange(c["n"], device="cuda")
+        src, dst = torch.cat([src[keep], own]), torch.cat([dst[keep], own])
+    keys = dst * c["n"] + src
+    keys = torch.unique(keys) if "d" in c["flags"] else keys.sort().values
+    dst = keys // c["n"]
+    row_ptr = torch.searchsorted(dst, torch.arange(c["n"] + 1, device="cuda"))
+    return row_ptr, keys % c["n"], dst
+
+
+def _attention64(c, col, row, s_src, s_dst):
+    """Edge softmax of LeakyReLU(s_src[source] + s_dst[destination]), slope 0.2, one head after the other."""
+    alpha = torch.empty((col.numel(), s_src.shape[1]), dtype=torch.float64, device="cuda")
+    for h in range(s_src.shape[1]):
+        logit = torch.nn.functional.leaky_relu(s_src[col, h] + s_dst[row, h], 0.2)
+        top = torch.full((c["n"],), -math.inf, dtype=torch.float64, device="cuda").scatter_reduce_(0, row, logit, "amax")
+        value = (logit - top[row]).exp_()
+        alpha[:, h] = value / torch.zeros(c["n"], dtype=torch.float64, device="cuda").index_add_(0, row, value)[row]
+    return alpha
+
+
+def _sum64(row_ptr, col, weight, x):
+    """Rows' weighted sums of x, 64 columns at a time."""
+    a = torch.sparse_csr_tensor(row_ptr, col, weight, size=(row_ptr.numel() - 1, x.shape[0]))
+    return torch.cat([a @ part.contiguous() for part in x.split(64, dim=1)], dim=1)
+
+
+def exact(case, seed):
+    c = case
+    if c["kind"] not in ("softmax", "build"):
+        x = _matrix(c["n"], c["f_in"] or c["f"], c["ld"], c["dtype"], seed, 2)[:, :c["f_in"] or c["f"]].double()
+    if c["f_in"]:
+        w_t = _matrix(c["f"], c["f_in"], c["ld"], c["dtype"], seed, 4, c["f_in"] ** -0.5)[:, :c["f_in"]].double()
+        z = x @ w_t.T
+        if c["kind"] == "combine":
+            return z
+        x = z.to(torch.bfloat16).double() if c["dtype"] == "bf16" else z      # a layer keeps z in the features' type
+    row_ptr, col, row = _csr64(c, seed)
+    deg = (row_ptr[1:] - row_ptr[:-1]).double()
+    dinv, rdeg = (torch.where(deg > 0, deg.clamp_min(1) ** p, 0.0) for p in (-0.5, -1.0))
+    if c["kind"] == "build":
+        return {"row_ptr": None, "col_idx": None, "perm": None, "edge_weight": dinv[col] * dinv[row], "dinv_sqrt": dinv,
+                "rdeg": rdeg, "row_order": None}
+    if c["kind"] == "softmax":
+        return _attention64(c, col, row, *(_matrix(c["n"], c["heads"], c["heads"], "f32", seed, k).double() for k in (2, 3)))
+    if c["model"] == "gat":
+        a_src, a_dst = (_matrix(c["heads"], c["dim"], c["dim"], "f32", seed, k, 0.1).double() for k in (5, 6))
+        heads = x.reshape(c["n"], c["heads"], c["dim"])
+        alpha = _attention64(c, col, row, (heads * a_src).sum(2), (heads * a_dst).sum(2))
+        return torch.cat([_sum64(row_ptr, col, alpha[:, h].contiguous(), heads[:, h]) for h in range(c["heads"])], dim=1)
+    return _sum64(row_ptr, col, dinv[col] * dinv[row] if c["model"] == "gcn" else rdeg[row], x)
+
+
 # ---------------------------------------------------------------- floors and tolerances
 
 def work(case):
