@@ -21,7 +21,8 @@ struct BuildCounts {
     int32_t max_degree;
     int32_t n_segments;      // hub segments
     int32_t bin_count[kNumBins];
-    int32_t pad[6];
+    int32_t sort_failed;     // a sweep of the sort gave up waiting: nothing after it is meaningful
+    int32_t pad[5];
 };
 
 }  // namespace gnnfd

@@ -1,10 +1,11 @@
-// Device CSR-by-destination builder: key generation, stable LSD radix sort of (dst, src) keys,
-// duplicate removal, row pointers, degree normalisers, GCN edge weights and the launch schedule
-// (degree bins, hub segments).  Integer work throughout; the only host synchronisation is the
+// Device CSR-by-destination builder: digit histograms of the (dst, src) keys, stable LSD radix sort with one
+// sweep per digit, duplicate removal, row pointers, degree normalisers, GCN edge weights and the launch
+// schedule (degree bins, hub segments).  Integer work throughout; the only host synchronisation is the
 // final read of the counters.
 #include <cstddef>
 #include <cstring>
 #include <new>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -15,17 +16,7 @@ using u64 = unsigned long long;
 constexpr int kThreads = 256;
 constexpr int kMaxDigitBits = 9;
 constexpr int kRadix = 1 << kMaxDigitBits;           // histogram bins (a pass may use fewer)
-constexpr int kSortTile = 4096;                      // keys per block of a sort pass
-#ifndef GNNFD_SCATTER_THREADS
-#define GNNFD_SCATTER_THREADS 256
-#endif
-constexpr int kHistItems = kSortTile / kThreads;     // keys per thread of the histogram kernel
-constexpr int kScatterThreads = GNNFD_SCATTER_THREADS;
-constexpr int kSortItems = kSortTile / kScatterThreads;   // keys per thread of the scatter kernel
-constexpr int kSortWarps = kScatterThreads / 32;
-constexpr int kWarpItems = 32 * kSortItems;
-constexpr int kOwnDigits = kRadix / kScatterThreads; // digit values a scatter thread looks after
-static_assert(kRadix % kScatterThreads == 0 && kOwnDigits >= 1, "a scatter block must cover the digit values evenly");
+constexpr int kSmCount = 148;
 
 static inline unsigned blocks_for(size_t count, int per_block)
 {
@@ -38,123 +29,168 @@ static inline unsigned blocks_for(size_t count, int per_block)
 // Candidate i < e: input edge i.  e <= i < 2e (symmetrise): reverse of edge i - e.  Then one
 // self-loop per vertex (value -1).  key = (dst << src_bits) | src; dropped candidates get the
 // destination n, above every valid key, so the sort moves them behind the kept ones.  When key and
-// value fit one 64-bit word together (vals == nullptr) the word is key << val_bits | (value + 1) and
-// every later kernel reads the key as word >> val_bits.
-constexpr int kKeyItems = 4;                          // candidates per thread of make_keys / entries per thread of finalize_entries
+// value fit one 64-bit word together (val_bits > 0) the word is key << val_bits | (value + 1) and
+// every later kernel reads the key as word >> val_bits.  Candidates are never written out as such: the
+// histogram kernel and the first sweep both form them from the edge list.
+struct Candidates {
+    const void* src;
+    const void* dst;
+    int64_t n, e, m;
+    uint32_t flags;
+    int src_bits;
+};
+
+__device__ __forceinline__ u64 edge_key(const Candidates& c, int64_t s64, int64_t d64, bool reverse, bool* kept, bool* bad)
+{
+    *bad = s64 < 0 || s64 >= c.n || d64 < 0 || d64 >= c.n;
+    *kept = !*bad && !((reverse || (c.flags & GNNFD_CSR_ADD_SELF_LOOPS)) && s64 == d64);
+    return *kept ? ((u64)d64 << c.src_bits) | (u64)s64 : (u64)c.n << c.src_bits;
+}
+
+// key and value of candidate i < m
+template <typename IdT>
+__device__ __forceinline__ u64 candidate_key(const Candidates& c, int64_t i, int32_t* val, bool* kept, bool* bad)
+{
+    const IdT* src = static_cast<const IdT*>(c.src);
+    const IdT* dst = static_cast<const IdT*>(c.dst);
+    *val = (int32_t)i;
+    if (i < c.e) return edge_key(c, (int64_t)__ldcs(src + i), (int64_t)__ldcs(dst + i), false, kept, bad);
+    const int64_t n_rev = (c.flags & GNNFD_CSR_SYMMETRIZE) ? c.e : 0;
+    if (i < c.e + n_rev) {
+        const u64 key = edge_key(c, (int64_t)__ldcs(dst + i - c.e), (int64_t)__ldcs(src + i - c.e), true, kept, bad);
+        *bad = false;                                  // counted once, by the edge itself
+        return key;
+    }
+    const u64 v = (u64)(i - c.e - n_rev);
+    *val = -1;
+    *kept = true;
+    *bad = false;
+    return (v << c.src_bits) | v;
+}
+
+// Digit counts of every pass, the number of kept candidates and of bad ids, in one read of the edge list.  The
+// grid is a few blocks per SM that walk the list, so that the counters are flushed with few global atomics.
+constexpr int kHistItems = 8;                        // candidates per thread and step
+constexpr int kHistTile = kThreads * kHistItems;
 
 template <typename IdT>
 __global__ void __launch_bounds__(kThreads)
-make_keys(const IdT* __restrict__ src, const IdT* __restrict__ dst, int64_t n, int64_t e, int64_t m, uint32_t flags,
-          int src_bits, int val_bits, u64* __restrict__ keys, int32_t* __restrict__ vals,
-          BuildCounts* __restrict__ counts)
+edge_histograms(const __grid_constant__ Candidates c, int first_bit, int digit_bits, int passes, int32_t* __restrict__ hist,
+                BuildCounts* __restrict__ counts)
 {
-    const int64_t base = (int64_t)blockIdx.x * (kThreads * kKeyItems) + threadIdx.x;
-    const u64 invalid = (u64)n << src_bits;
-    const int64_t n_rev = (flags & GNNFD_CSR_SYMMETRIZE) ? e : 0;
-    int kept = 0, bads = 0;
-    auto emit = [&](int64_t i, int64_t sv, int64_t dv, int32_t val, bool keep) {
-        const u64 key = keep ? (((u64)dv << src_bits) | (u64)sv) : invalid;
-        if (vals) {
-            __stcs(keys + i, key);
-            __stcs(vals + i, val);
-        } else {
-            __stcs(keys + i, (key << val_bits) | (u64)(uint32_t)(val + 1));   // value travels in the low bits
-        }
-        kept += keep ? 1 : 0;
+    extern __shared__ int32_t hist_smem[];           // [passes][kRadix]
+    for (int i = threadIdx.x; i < passes * kRadix; i += kThreads) hist_smem[i] = 0;
+    __syncthreads();
+    const unsigned mask = (1u << digit_bits) - 1u;
+    int n_kept = 0, n_bad = 0;
+    auto count = [&](u64 key) {
+        key >>= first_bit;
+        for (int p = 0; p < passes; ++p, key >>= digit_bits) atomicAdd(&hist_smem[p * kRadix + ((unsigned)key & mask)], 1);
     };
-    if ((int64_t)(blockIdx.x + 1) * (kThreads * kKeyItems) <= e) {
-        // the block lies inside the plain input edges: all loads are issued before the first store
-        IdT sv[kKeyItems], dv[kKeyItems];
+    const IdT* src = static_cast<const IdT*>(c.src);
+    const IdT* dst = static_cast<const IdT*>(c.dst);
+    for (int64_t base = (int64_t)blockIdx.x * kHistTile; base < c.m; base += (int64_t)gridDim.x * kHistTile) {
+        if (base + kHistTile <= c.e) {
+            // inside the plain input edges: all loads are issued before the first shared-memory atomic
+            IdT sv[kHistItems], dv[kHistItems];
 #pragma unroll
-        for (int j = 0; j < kKeyItems; ++j) {
-            sv[j] = __ldcs(src + base + j * kThreads);
-            dv[j] = __ldcs(dst + base + j * kThreads);
-        }
+            for (int j = 0; j < kHistItems; ++j) {
+                sv[j] = __ldcs(src + base + j * kThreads + threadIdx.x);
+                dv[j] = __ldcs(dst + base + j * kThreads + threadIdx.x);
+            }
 #pragma unroll
-        for (int j = 0; j < kKeyItems; ++j) {
-            const int64_t s64 = (int64_t)sv[j], d64 = (int64_t)dv[j];
-            const bool bad = s64 < 0 || s64 >= n || d64 < 0 || d64 >= n;
-            bads += bad ? 1 : 0;
-            emit(base + j * kThreads, s64, d64, (int32_t)(base + j * kThreads),
-                 !bad && !((flags & GNNFD_CSR_ADD_SELF_LOOPS) && s64 == d64));
-        }
-    } else {
-        for (int j = 0; j < kKeyItems; ++j) {
-            const int64_t i = base + j * kThreads;
-            if (i >= m) break;
-            if (i < e) {
-                const int64_t s64 = (int64_t)src[i], d64 = (int64_t)dst[i];
-                const bool bad = s64 < 0 || s64 >= n || d64 < 0 || d64 >= n;
-                bads += bad ? 1 : 0;
-                emit(i, s64, d64, (int32_t)i, !bad && !((flags & GNNFD_CSR_ADD_SELF_LOOPS) && s64 == d64));
-            } else if (i < e + n_rev) {
-                const int64_t s64 = (int64_t)dst[i - e], d64 = (int64_t)src[i - e];
-                emit(i, s64, d64, (int32_t)i, !(s64 < 0 || s64 >= n || d64 < 0 || d64 >= n) && s64 != d64);
-            } else {
-                emit(i, i - e - n_rev, i - e - n_rev, -1, true);
+            for (int j = 0; j < kHistItems; ++j) {
+                bool kept, bad;
+                const u64 key = edge_key(c, (int64_t)sv[j], (int64_t)dv[j], false, &kept, &bad);
+                n_kept += kept;
+                n_bad += bad;
+                count(key);
+            }
+        } else {
+#pragma unroll 2
+            for (int j = 0; j < kHistItems; ++j) {
+                const int64_t i = base + j * kThreads + threadIdx.x;
+                if (i >= c.m) break;
+                int32_t val;
+                bool kept, bad;
+                const u64 key = candidate_key<IdT>(c, i, &val, &kept, &bad);
+                n_kept += kept;
+                n_bad += bad;
+                count(key);
             }
         }
     }
-    // one atomic per block and counter: all blocks add to the same two words
-    __shared__ int warp_kept[kThreads / 32], warp_bads[kThreads / 32];
-    const int kept_warp = __reduce_add_sync(0xffffffffu, kept), bads_warp = __reduce_add_sync(0xffffffffu, bads);
+    __syncthreads();
+    for (int i = threadIdx.x; i < passes * kRadix; i += kThreads)
+        if (hist_smem[i]) atomicAdd(hist + i, hist_smem[i]);
+    n_kept = __reduce_add_sync(0xffffffffu, n_kept);
+    n_bad = __reduce_add_sync(0xffffffffu, n_bad);
     if ((threadIdx.x & 31) == 0) {
-        warp_kept[threadIdx.x >> 5] = kept_warp;
-        warp_bads[threadIdx.x >> 5] = bads_warp;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int kept_all = 0, bads_all = 0;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) { kept_all += warp_kept[w]; bads_all += warp_bads[w]; }
-        if (kept_all) atomicAdd(&counts->n_valid, kept_all);
-        if (bads_all) atomicAdd(&counts->bad_index, bads_all);
+        if (n_kept) atomicAdd(&counts->n_valid, n_kept);
+        if (n_bad) atomicAdd(&counts->bad_index, n_bad);
     }
 }
 
-// ------------------------------------------------------------------ radix sort (one digit of up to 9 bits per pass)
+// ------------------------------------------------------------------ radix sort (one digit of up to 9 bits per sweep)
+//
+// A sweep reads every key once and writes it once to its place in the order of the digit.  A block takes a tile
+// of keys, ranks them, publishes how many keys of each digit value it holds, and finds out how many the tiles
+// before it hold by walking back over their published counts until it meets one that already knows its own sum
+// (a chained scan with look-back).  Against the former histogram + three-kernel scan + scatter per digit
+// this drops one read of the keys and four launches.
+//
+// The walk waits for other blocks, but only for tiles with a smaller number, and tile numbers are drawn from a
+// counter by blocks that are already running: tile 0 never waits, and every tile publishes its own counts before it
+// waits, so some waiting block can always go on.  The wait is limited all the same: a block that polls one
+// word kMaxPolls times marks the build as failed and leaves, the others follow, and the host returns
+// GNNFD_CUDA_ERROR.
 
-__global__ void __launch_bounds__(kThreads)
-radix_histogram(const u64* __restrict__ keys, int64_t m, int shift, int mask, int64_t n_tiles, int32_t* __restrict__ hist)
+// A published word: 0 nothing yet; count + 1: the tile's own count; kSumBit | sum: keys of this digit value in all tiles
+// up to and including this one, plus the keys of smaller digit values (so the sum is a position).
+constexpr uint32_t kSumBit = 0x80000000u;
+constexpr int kMaxPolls = 1 << 20;                   // at up to 1 us a poll
+constexpr int kWalk = 4;                             // earlier tiles read together
+
+__device__ __forceinline__ uint32_t load_published(const uint32_t* p)
 {
-    __shared__ int32_t h[kRadix];
-    h[threadIdx.x] = 0;
-    h[threadIdx.x + kThreads] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    if (base + kSortTile <= m) {
-        // full tile: 16-byte loads, all of them issued before the first shared-memory atomic
-        const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(keys + base);
-        ulonglong2 v[kHistItems / 2];
-#pragma unroll
-        for (int i = 0; i < kHistItems / 2; ++i) v[i] = __ldcs(k2 + i * kThreads + threadIdx.x);
-#pragma unroll
-        for (int i = 0; i < kHistItems / 2; ++i) {
-            atomicAdd(&h[(int)(v[i].x >> shift) & mask], 1);
-            atomicAdd(&h[(int)(v[i].y >> shift) & mask], 1);
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < kHistItems; ++i) {
-            const int64_t idx = base + i * kThreads + threadIdx.x;
-            if (idx < m) atomicAdd(&h[(int)(keys[idx] >> shift) & mask], 1);
-        }
-    }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
-    hist[(int64_t)(threadIdx.x + kThreads) * n_tiles + blockIdx.x] = h[threadIdx.x + kThreads];
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void publish(uint32_t* p, uint32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
 }
 
-struct ScatterSmem {
-    u64 keys[kSortTile];
-    int32_t warp_count[kSortWarps][kRadix];
-    int32_t digit_base[kRadix];     // first slot of each digit inside the sorted tile
-    int32_t to_global[kRadix];      // global position of tile slot i holding digit d: to_global[d] + i
-    int32_t scan[kSortWarps];
-    int32_t vals[kSortTile];        // last: not allocated when the values travel inside the keys
-};
+// position of the tile's first key of one digit value: `column` points at the digit's word of tile 0, words of
+// consecutive tiles are kRadix apart.  false: gave up.
+__device__ __forceinline__ bool look_back(const uint32_t* column, int64_t tile, const int32_t* failed, uint32_t* before)
+{
+    uint32_t sum = 0;
+    int polls = 0;
+    for (int64_t t = tile - 1; t >= 0;) {
+        uint32_t w[kWalk];
+#pragma unroll
+        for (int i = 0; i < kWalk; ++i) w[i] = t - i >= 0 ? load_published(column + (t - i) * kRadix) : 0u;
+        int used = 0;
+#pragma unroll
+        for (int i = 0; i < kWalk; ++i) {
+            if (used == i && w[i] != 0u) {
+                if (w[i] & kSumBit) { *before = sum + (w[i] & ~kSumBit); return true; }
+                sum += w[i] - 1u;
+                ++used;
+            }
+        }
+        t -= used;
+        if (used == 0 && (++polls & 255) == 0 && (polls >= kMaxPolls || load_published(reinterpret_cast<const uint32_t*>(failed)) != 0u))
+            return false;
+    }
+    *before = sum;
+    return true;
+}
 
-// exclusive scan of one value per thread over a scatter block; *total receives the block sum
+// exclusive scan of one value per thread over a block of up to 1024 threads; *total receives the block sum.
+// smem[32] must not be in use by a scan that another thread may still be reading.
 __device__ __forceinline__ int32_t block_scan(int32_t v, int32_t* total, int32_t* smem)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -164,123 +200,311 @@ __device__ __forceinline__ int32_t block_scan(int32_t v, int32_t* total, int32_t
         const int32_t t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
     }
-    __syncthreads();
     if (lane == 31) smem[warp] = inc;
     __syncthreads();
-    int32_t off = 0, all = 0;
-#pragma unroll
-    for (int w = 0; w < kSortWarps; ++w) {
-        const int32_t s = smem[w];
-        if (w < warp) off += s;
-        all += s;
-    }
-    *total = all;
-    return off + inc - v;
+    const int32_t sums = lane < (int)(blockDim.x >> 5) ? smem[lane] : 0;       // every warp adds up the warps before it
+    *total = __reduce_add_sync(0xffffffffu, sums);
+    return __reduce_add_sync(0xffffffffu, lane < warp ? sums : 0) + inc - v;
 }
 
-// Lanes of the warp that hold the same digit value (among the valid ones): one ballot per digit bit.
-// The match instruction gives the same mask, but measured on this part it occupies its pipe for about
-// 56 cycles per warp, against about 21 ALU cycles for the nine ballots and their masking.  The two run
-// on different pipes, so the scatter uses the match instruction for GNNFD_SCATTER_MATCH_ROUNDS of a
-// warp's 16 rounds and ballots for the rest (config 4, per build: all match 3.59 ms, all ballots 3.09,
-// 3 / 5 / 7 rounds of match 3.02 / 2.86 / 2.99).
-__device__ __forceinline__ unsigned lanes_with_equal_digit(int digit, bool valid)
+enum Source { kWords, kEdges32, kEdges64, kRows };    // where a sweep takes its keys from
+
+struct SweepArgs {
+    Candidates cand;               // kEdges*: the edge list (first sweep)
+    const u64* keys_in;            // kWords
+    const int32_t* vals_in;        // kWords, values apart from the keys
+    const int32_t* row_ptr;        // kRows: the keys are the rows' degree classes
+    u64* keys_out;
+    int32_t* vals_out;             // values apart from the keys; kRows: the row ids
+    int64_t m;
+    int n_tiles;
+    int shift, mask, val_bits;
+    const int32_t* digit_count;    // [kRadix] keys per digit value
+    int32_t* ticket;               // next tile number
+    uint32_t* published;           // [tiles][kRadix], all 0
+    uint32_t* published_next;      // set to 0 for the next sweep (may be null)
+    BuildCounts* counts;
+};
+
+// Degree class of a row: exact degree up to 8, then quarter octaves of (deg - 1) up to the hub
+// threshold, then one class for hub rows.  Classes are monotone in the degree, so each of the five
+// launch bins (<= 8, <= 32, <= 128, <= hub threshold, hub) is a contiguous range of classes.
+constexpr int kHubClass = 41;
+__device__ __forceinline__ int degree_class(int32_t deg)
 {
-    unsigned peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-    for (int b = 0; b < kMaxDigitBits; ++b) {
-        const bool bit = (digit >> b) & 1;
-        const unsigned with_bit = __ballot_sync(0xffffffffu, bit);
-        peers &= bit ? with_bit : ~with_bit;
-    }
-    return valid ? peers : 0u;
+    if (deg <= kBinDeg0) return deg;
+    if (deg > kBinDeg3) return kHubClass;
+    const int t = deg - 1;
+    const int o = 31 - __clz(t);                       // 3 .. 10
+    return 9 + (o - 3) * 4 + ((t >> (o - 2)) & 3);
+}
+__device__ __forceinline__ int degree_bin(int32_t deg)
+{
+    return deg <= kBinDeg0 ? 0 : deg <= kBinDeg1 ? 1 : deg <= kBinDeg2 ? 2 : deg <= kBinDeg3 ? 3 : 4;
 }
 
-// Stable scatter of one tile.  A warp owns kWarpItems consecutive keys and walks them 32 at a time: keys
-// with equal digits inside a round are ranked by lane (ballots over the digit's bits), across rounds by a per-warp running
-// count, across warps by a prefix over the per-warp counts.  The tile is then laid out sorted by
-// digit in shared memory and written out run by run, so that consecutive threads store to
-// consecutive addresses; the run of digit d starts at the scanned histogram entry of (d, tile).
-#ifndef GNNFD_SCATTER_MATCH_ROUNDS
-#define GNNFD_SCATTER_MATCH_ROUNDS 5
-#endif
-#ifndef GNNFD_SCATTER_MIN_BLOCKS
-#define GNNFD_SCATTER_MIN_BLOCKS 3
-#endif
-template <bool HAS_VALS>
-__global__ void __launch_bounds__(kScatterThreads, GNNFD_SCATTER_MIN_BLOCKS)
-radix_scatter(const u64* __restrict__ keys_in, const int32_t* __restrict__ vals_in, u64* __restrict__ keys_out,
-              int32_t* __restrict__ vals_out, int64_t m, int shift, int mask, int64_t n_tiles,
-              const int32_t* __restrict__ tile_offset)
+// Block shapes of a sweep.  Large inputs: 512 threads x 16 keys, two blocks per SM.  Inputs of fewer than 4 such tiles
+// per SM: 256 threads x 8 keys, so that more SMs take part.
+struct LargeTile { static constexpr int kThreads = 512, kItems = 16, kMinBlocks = 2; };
+struct SmallTile { static constexpr int kThreads = 256, kItems = 8, kMinBlocks = 4; };
+template <typename Shape> constexpr int tile_keys() { return Shape::kThreads * Shape::kItems; }
+static bool use_large_tile(int64_t m) { return m >= (int64_t)4 * kSmCount * tile_keys<LargeTile>(); }
+static int64_t sweep_tiles(int64_t m)
 {
+    const int keys = use_large_tile(m) ? tile_keys<LargeTile>() : tile_keys<SmallTile>();
+    return m > 0 ? (m + keys - 1) / keys : 1;
+}
+
+template <typename Shape>
+struct SweepSmem {
+    u64 keys[tile_keys<Shape>()];
+    union {
+        int32_t warp_count[Shape::kThreads / 32][kRadix];      // keys of a warp per digit value, then their first slot
+        int32_t vals[tile_keys<Shape>()];                      // while writing out
+    };
+    int32_t to_global[kRadix];      // global position of tile slot i holding digit value d: to_global[d] + i
+    int32_t scan[32];
+    int32_t tile[2];
+};
+
+// Ranking: a warp owns 32 * kItems consecutive keys and walks them 32 at a time, with a running count per digit value.
+// Rounds are ranked in one of two ways, which load different pipes.  (1) The match instruction gives the lanes
+// with the same digit, and the first of them adds their number to the count; the instruction holds its pipe
+// for about 56 cycles.  (2) Every lane reads its digit's count and then adds one to it atomically.  A lane whose
+// addition found the count as it was read comes first; any other shares its digit with a lane of this round, and
+// the order in which the hardware served them says nothing, so those digits (about one per round for random
+// keys) are ranked by lane, one ballot each.  Across rounds the running count ranks, across warps a prefix over the
+// per-warp counts.  The tile is then laid out sorted by digit in shared memory and written out run by run, so
+// that consecutive threads store to consecutive addresses.
+//
+// Blocks stay and draw one tile after the other; the next tile's keys are requested as soon as this tile's have
+// moved to shared memory, so that they arrive while the block walks back and writes out.
+//
+// Bound by the shared-memory pipe and by latency, not by HBM: 116 M words of 8 bytes on 233 k vertices take 0.74 ms per
+// sweep (2.5 TB/s; the former histogram, scans and scatter took 0.96), of which the counters (at 20 M words) give
+// the pipe for shared and global accesses 55 % and the issue slots 45 %.  Measured per four sweeps: of every four
+// rounds 0 / 1 / 2 / 3 / 4 with the match instruction 3.02 / 3.03 / 3.28 / 3.70 / 4.18 ms (with values of their own,
+// 122 M keys, five sweeps: 6.63 / 6.24 / 6.36 / 6.65 / 7.60); 2 / 4 / 8 / 16 earlier tiles read together in the walk 3.11 /
+// 2.97 / 3.03 / 3.49 ms; 512 x 8 keys with three blocks per SM 3.69, 256 x 16 with four 3.79 ms.
+constexpr int kRankRounds = 4;      // rounds whose counts are in flight together
+constexpr int kMatchRounds = 1;     // how many of them use the match instruction
+
+template <typename Shape, int SOURCE, bool HAS_VALS>
+__global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_sweep(const __grid_constant__ SweepArgs a)
+{
+    constexpr int kBlock = Shape::kThreads, kItems = Shape::kItems, kWarps = kBlock / 32, kTile = kBlock * kItems;
+    constexpr int kOwn = kRadix / kBlock;            // digit values a thread looks after
+    static_assert(kRadix % kBlock == 0 && kTile <= kWarps * kRadix, "digit values per thread; values fit the counts' place");
+    static_assert(kItems % kRankRounds == 0 && kTile <= 1 << 16, "rounds; 16-bit slots");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ScatterSmem& sm = *reinterpret_cast<ScatterSmem*>(smem_raw);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kScatterThreads) (&sm.warp_count[0][0])[i] = 0;
-    __syncthreads();
+    SweepSmem<Shape>& sm = *reinterpret_cast<SweepSmem<Shape>*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int in_tile = warp * (32 * kItems) + lane;       // key r of this thread: in_tile + r * 32 within its tile
+    u64 key[kItems];
 
-    const int64_t tile_base = (int64_t)blockIdx.x * kSortTile;
-    const int64_t warp_base = tile_base + (int64_t)warp * kWarpItems;
-    u64 key[kSortItems];
+    auto load_keys = [&](int64_t base) {
+        const int64_t first = base + in_tile;
+        if constexpr (SOURCE == kWords) {
+            if (base + kTile <= a.m) {
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t idx = warp_base + r * 32 + lane;
-        key[r] = idx < m ? __ldcs(keys_in + idx) : 0ull;
-    }
-    int32_t rank[kSortItems];
+                for (int r = 0; r < kItems; ++r) key[r] = __ldcs(a.keys_in + first + r * 32);
+            } else {
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const bool valid = warp_base + r * 32 + lane < m;
-        const int digit = (int)(key[r] >> shift) & mask;
-        // some rounds use the match instruction, the others ballots: the two run on different pipes
-        const unsigned peers = r < GNNFD_SCATTER_MATCH_ROUNDS ? __match_any_sync(0xffffffffu, valid ? digit : kRadix)
-                                                              : lanes_with_equal_digit(digit, valid);
-        const int leader = __ffs(peers) - 1;
-        // the leader of each digit bumps the warp's running count; a warp's shared-memory atomics on one
-        // address complete in program order, so the rounds need no barrier between them
-        int32_t before = 0;
-        if (lane == leader && valid) before = atomicAdd(&sm.warp_count[warp][digit], __popc(peers));
-        before = __shfl_sync(0xffffffffu, before, leader);
-        rank[r] = before + __popc(peers & ((1u << lane) - 1u));
-    }
+                for (int r = 0; r < kItems; ++r) key[r] = first + r * 32 < a.m ? __ldcs(a.keys_in + first + r * 32) : 0ull;
+            }
+        } else if constexpr (SOURCE == kRows) {
+#pragma unroll
+            for (int r = 0; r < kItems; ++r) {
+                const int64_t v = first + r * 32;
+                key[r] = v < a.m ? ((u64)degree_class(a.row_ptr[v + 1] - a.row_ptr[v]) << 32) | (u64)v : 0ull;
+            }
+        } else {
+            using IdT = typename std::conditional<SOURCE == kEdges32, int32_t, long long>::type;
+            auto word = [&](u64 k, int32_t val) { return HAS_VALS ? k : (k << a.val_bits) | (u64)(uint32_t)(val + 1); };
+            bool kept, bad;
+            if (base + kTile <= a.cand.e) {          // inside the plain input edges: straight-line loads
+#pragma unroll
+                for (int r = 0; r < kItems; ++r) {
+                    const int64_t sv = (int64_t)__ldcs(static_cast<const IdT*>(a.cand.src) + first + r * 32);
+                    const int64_t dv = (int64_t)__ldcs(static_cast<const IdT*>(a.cand.dst) + first + r * 32);
+                    key[r] = word(edge_key(a.cand, sv, dv, false, &kept, &bad), (int32_t)(first + r * 32));
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < kItems; ++r) {
+                    int32_t val;
+                    key[r] = 0ull;
+                    if (first + r * 32 < a.m) {
+                        const u64 k = candidate_key<IdT>(a.cand, first + r * 32, &val, &kept, &bad);
+                        key[r] = word(k, val);
+                    }
+                }
+            }
+        }
+    };
+    auto clear_counts = [&]() {
+        for (int i = tid; i < kWarps * kRadix / 4; i += kBlock) reinterpret_cast<int4*>(&sm.warp_count[0][0])[i] = make_int4(0, 0, 0, 0);
+    };
+
+    if (tid == 0) sm.tile[0] = atomicAdd(a.ticket, 1);
+    clear_counts();
     __syncthreads();
-    {
-        // per-warp counts -> exclusive prefix over warps; thread t owns digit values t, t + blockDim, ...
-        int32_t carry = 0;
+    int tile = sm.tile[0];
+    if (tile >= a.n_tiles) return;
+    load_keys((int64_t)tile * kTile);
+
+    for (int turn = 1;; turn ^= 1) {
+        if (tid == 0) sm.tile[turn] = atomicAdd(a.ticket, 1);
+        const int64_t tile_base = (int64_t)tile * kTile;
+        const int count = (int)min((int64_t)kTile, a.m - tile_base);
+        uint32_t* const published = a.published + (int64_t)tile * kRadix;
+        if (a.published_next)
+            for (int i = tid; i < kRadix / 4; i += kBlock)
+                reinterpret_cast<uint4*>(a.published_next + (int64_t)tile * kRadix)[i] = make_uint4(0u, 0u, 0u, 0u);
+
+        uint32_t rank[kItems / 2];                   // two 16-bit numbers per register
+        int32_t* const warp_count = sm.warp_count[warp];
 #pragma unroll
-        for (int q = 0; q < kOwnDigits; ++q) {
-            const int d = threadIdx.x + q * kScatterThreads;
-            int32_t run = 0;
+        for (int r0 = 0; r0 < kItems; r0 += kRankRounds) {
+            int digit[kRankRounds];
+            int32_t before[kRankRounds], mine[kRankRounds];
 #pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) {
-                const int32_t c = sm.warp_count[w][d];
-                sm.warp_count[w][d] = run;
+            for (int g = 0; g < kRankRounds; ++g) {
+                const bool valid = in_tile + (r0 + g) * 32 < count;
+                digit[g] = valid ? (int)(key[r0 + g] >> a.shift) & a.mask : -1;
+                if (g < kMatchRounds) {
+                    const unsigned same = __match_any_sync(0xffffffffu, digit[g]);
+                    mine[g] = 0;
+                    if (valid && lane == __ffs(same) - 1) mine[g] = atomicAdd(warp_count + digit[g], __popc(same));
+                    before[g] = (int32_t)same;
+                } else {
+                    before[g] = valid ? *(volatile int32_t*)(warp_count + digit[g]) : 0;
+                    __syncwarp();
+                    mine[g] = valid ? atomicAdd(warp_count + digit[g], 1) : 0;
+                }
+                __syncwarp();
+            }
+#pragma unroll
+            for (int g = 0; g < kRankRounds; ++g) {
+                const unsigned lower = (1u << lane) - 1u;
+                if (g < kMatchRounds) {
+                    const unsigned same = (unsigned)before[g];
+                    mine[g] = __shfl_sync(0xffffffffu, mine[g], __ffs(same) - 1) + __popc(same & lower);
+                } else {
+                    unsigned shared = __ballot_sync(0xffffffffu, mine[g] != before[g]);
+                    while (shared) {
+                        const int d = __shfl_sync(0xffffffffu, digit[g], __ffs(shared) - 1);
+                        const unsigned same = __ballot_sync(0xffffffffu, digit[g] == d);
+                        if (digit[g] == d) mine[g] = before[g] + __popc(same & lower);
+                        shared &= ~same;
+                    }
+                }
+                const int r = r0 + g;
+                rank[r / 2] = r & 1 ? rank[r / 2] | ((uint32_t)mine[g] << 16) : (uint32_t)mine[g];
+            }
+        }
+        __syncthreads();
+        const int next = sm.tile[turn];
+        // the tile's totals are published at once; the walk back over the earlier tiles comes after the keys
+        // have moved to their slots
+        int32_t total[kOwn], base[kOwn], carry = 0;
+#pragma unroll
+        for (int q = 0; q < kOwn; ++q) {
+            total[q] = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) total[q] += sm.warp_count[w][tid + q * kBlock];
+            if (tile > 0) publish(published + tid + q * kBlock, (uint32_t)total[q] + 1u);
+        }
+#pragma unroll
+        for (int q = 0; q < kOwn; ++q) {
+            int32_t sum;
+            if (q) __syncthreads();
+            base[q] = block_scan(total[q], &sum, sm.scan) + carry;
+            carry += sum;
+            int32_t run = base[q];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const int32_t c = sm.warp_count[w][tid + q * kBlock];
+                sm.warp_count[w][tid + q * kBlock] = run;
                 run += c;
             }
-            int32_t total;
-            const int32_t base = block_scan(run, &total, sm.scan) + carry;
-            carry += total;
-            sm.digit_base[d] = base;
-            sm.to_global[d] = tile_offset[(int64_t)d * n_tiles + blockIdx.x] - base;
         }
-    }
-    __syncthreads();
+        if (tile == 0) {                             // the only tile that starts from the digit counts of the whole input
+            int32_t smaller = 0;
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        if (warp_base + r * 32 + lane < m) {
-            const int digit = (int)(key[r] >> shift) & mask;
-            const int slot = sm.digit_base[digit] + sm.warp_count[warp][digit] + rank[r];
-            sm.keys[slot] = key[r];
-            if (HAS_VALS) sm.vals[slot] = __ldcs(vals_in + warp_base + r * 32 + lane);
+            for (int q = 0; q < kOwn; ++q) {
+                int32_t sum;
+                __syncthreads();
+                const int32_t start = block_scan(a.digit_count[tid + q * kBlock], &sum, sm.scan) + smaller;
+                smaller += sum;
+                publish(published + tid + q * kBlock, kSumBit | (uint32_t)(start + total[q]));
+                sm.to_global[tid + q * kBlock] = start - base[q];
+            }
         }
-    }
-    __syncthreads();
-    const int count = (int)min((int64_t)kSortTile, m - tile_base);
-    for (int i = threadIdx.x; i < count; i += kScatterThreads) {
-        const u64 k = sm.keys[i];
-        const int64_t pos = (int64_t)sm.to_global[(int)(k >> shift) & mask] + i;
-        keys_out[pos] = k;
-        if (HAS_VALS) vals_out[pos] = sm.vals[i];
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kItems; ++r) {
+            if (in_tile + r * 32 < count) {
+                const uint32_t ahead = (uint32_t)warp_count[(int)(key[r] >> a.shift) & a.mask];
+                rank[r / 2] += r & 1 ? ahead << 16 : ahead;              // now the key's slot
+                sm.keys[rank[r / 2] >> (r & 1 ? 16 : 0) & 0xffffu] = key[r];
+            }
+        }
+        int32_t val[HAS_VALS ? kItems : 1];
+        if constexpr (HAS_VALS) {
+#pragma unroll
+            for (int r = 0; r < kItems; ++r) {
+                const int64_t i = tile_base + in_tile + r * 32;
+                if constexpr (SOURCE == kWords) {
+                    val[r] = in_tile + r * 32 < count ? __ldcs(a.vals_in + i) : 0;
+                } else {
+                    const int64_t edges = a.cand.e + ((a.cand.flags & GNNFD_CSR_SYMMETRIZE) ? a.cand.e : 0);
+                    val[r] = i < edges ? (int32_t)i : -1;
+                }
+            }
+        } else if (next < a.n_tiles) {
+            load_keys((int64_t)next * kTile);
+        }
+        bool ok = true;
+        if (tile > 0) {
+#pragma unroll
+            for (int q = 0; q < kOwn; ++q) {
+                const int d = tid + q * kBlock;
+                uint32_t before = 0;
+                if (look_back(a.published + d, tile, &a.counts->sort_failed, &before))
+                    publish(published + d, kSumBit | (before + (uint32_t)total[q]));
+                else
+                    ok = false;
+                sm.to_global[d] = (int32_t)before - base[q];
+            }
+        }
+        if (__syncthreads_or(!ok)) {
+            if (tid == 0) atomicExch(&a.counts->sort_failed, 1);
+            return;
+        }
+        if constexpr (HAS_VALS) {                    // the values take the place of the counts, which nobody reads any more
+#pragma unroll
+            for (int r = 0; r < kItems; ++r)
+                if (in_tile + r * 32 < count) sm.vals[rank[r / 2] >> (r & 1 ? 16 : 0) & 0xffffu] = val[r];
+            if (next < a.n_tiles) load_keys((int64_t)next * kTile);
+            __syncthreads();
+        }
+#pragma unroll 4
+        for (int i = tid; i < count; i += kBlock) {
+            const u64 k = sm.keys[i];
+            const int64_t pos = (int64_t)sm.to_global[(int)(k >> a.shift) & a.mask] + i;
+            if constexpr (SOURCE == kRows) {
+                a.vals_out[pos] = (int32_t)(uint32_t)k;
+            } else {
+                a.keys_out[pos] = k;
+                if constexpr (HAS_VALS) a.vals_out[pos] = sm.vals[i];
+            }
+        }
+        if (next >= a.n_tiles) return;
+        if constexpr (HAS_VALS) __syncthreads();
+        clear_counts();
+        tile = next;
+        __syncthreads();
     }
 }
 
@@ -388,74 +612,51 @@ compact_unique(const u64* __restrict__ keys, const int32_t* __restrict__ vals, c
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) counts->nnz = tile_first[blockIdx.x] + total;
 }
 
-// row_ptr[v] = number of kept keys with dst < v (binary search in the sorted keys).  Without
-// duplicate removal every kept candidate is an entry, which thread 0 records.
+// row_ptr[v] = number of kept keys with dst < v (binary search in the sorted keys), then the degree normalisers
+// (rounded once from fp64), the bin sizes and the counts of the degree classes.  A block looks after kThreads - 1
+// rows, whose pointers and the one behind them its threads search.  Without duplicate removal every kept candidate
+// is an entry, which thread 0 records.
+constexpr int kRowsPerBlock = kThreads - 1;
+constexpr int kClasses = kHubClass + 1;
+
 __global__ void __launch_bounds__(kThreads)
-row_pointers(const u64* __restrict__ keys, BuildCounts* __restrict__ counts, int64_t n, int src_bits, int val_bits,
-             int dedup, int32_t* __restrict__ row_ptr)
+rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts, int64_t n, int src_bits, int val_bits,
+                 int dedup, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
+                 int32_t* __restrict__ class_count)
 {
-    const int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    __shared__ int32_t ptr[kThreads], class_smem[kClasses], bin_smem[kNumBins], max_smem;
+    if (counts->sort_failed) return;
+    if (threadIdx.x < kClasses) class_smem[threadIdx.x] = 0;
+    if (threadIdx.x < kNumBins) bin_smem[threadIdx.x] = 0;
+    if (threadIdx.x == 0) max_smem = 0;
+    const int64_t v = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.x;
     const int32_t nnz = dedup ? counts->nnz : counts->n_valid;
     if (v == 0 && !dedup) counts->nnz = nnz;
-    if (v > n) return;
+    int32_t lo = 0, hi = v <= n ? nnz : 0;
     const u64 target = (u64)v << src_bits;
-    int32_t lo = 0, hi = nnz;
     while (lo < hi) {
         const int32_t mid = lo + ((hi - lo) >> 1);
         if ((keys[mid] >> val_bits) < target) lo = mid + 1; else hi = mid;
     }
-    row_ptr[v] = lo;
-}
-
-// Degree class of a row: exact degree up to 8, then quarter octaves of (deg - 1) up to the hub
-// threshold, then one class for hub rows.  Classes are monotone in the degree, so each of the five
-// launch bins (<= 8, <= 32, <= 128, <= hub threshold, hub) is a contiguous range of classes.
-constexpr int kHubClass = 41;
-__device__ __forceinline__ int degree_class(int32_t deg)
-{
-    if (deg <= kBinDeg0) return deg;
-    if (deg > kBinDeg3) return kHubClass;
-    const int t = deg - 1;
-    const int o = 31 - __clz(t);                       // 3 .. 10
-    return 9 + (o - 3) * 4 + ((t >> (o - 2)) & 3);
-}
-__device__ __forceinline__ int degree_bin(int32_t deg)
-{
-    return deg <= kBinDeg0 ? 0 : deg <= kBinDeg1 ? 1 : deg <= kBinDeg2 ? 2 : deg <= kBinDeg3 ? 3 : 4;
-}
-
-// degree normalisers (rounded once from fp64), the bin sizes, and the (class, row) sort keys
-__global__ void __launch_bounds__(kThreads)
-degrees_and_classes(const int32_t* __restrict__ row_ptr, int64_t n, float* __restrict__ dinv, float* __restrict__ rdeg,
-                    u64* __restrict__ class_keys, int32_t* __restrict__ class_vals, BuildCounts* __restrict__ counts)
-{
-    const int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    int32_t deg = 0;
-    int bin = -1;
-    if (v < n) {
-        deg = row_ptr[v + 1] - row_ptr[v];
+    ptr[threadIdx.x] = lo;
+    __syncthreads();
+    if (threadIdx.x < kRowsPerBlock && v <= n) row_ptr[v] = lo;      // v == n belongs to the block after the last full one
+    if (threadIdx.x < kRowsPerBlock && v < n) {
+        const int32_t deg = ptr[threadIdx.x + 1] - lo;
         dinv[v] = deg > 0 ? (float)(1.0 / sqrt((double)deg)) : 0.f;
         rdeg[v] = deg > 0 ? (float)(1.0 / (double)deg) : 0.f;
-        bin = degree_bin(deg);
-        class_keys[v] = ((u64)degree_class(deg) << 32) | (u64)v;
-        class_vals[v] = (int32_t)v;
+        atomicAdd(&class_smem[degree_class(deg)], 1);
+        atomicAdd(&bin_smem[degree_bin(deg)], 1);
+        atomicMax(&max_smem, deg);
     }
-#pragma unroll
-    for (int b = 0; b < kNumBins; ++b) {
-        const int c = __syncthreads_count(bin == b);
-        if (threadIdx.x == 0 && c) atomicAdd(&counts->bin_count[b], c);
-    }
-    // block maximum, then one atomic per block (every block updates the same word)
-    __shared__ int32_t warp_max[kThreads / 32];
-    deg = __reduce_max_sync(0xffffffffu, deg);
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = deg;
     __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int w = 1; w < kThreads / 32; ++w) deg = max(deg, warp_max[w]);
-        if (deg > 0) atomicMax(&counts->max_degree, deg);
-    }
+    // few global atomics: all blocks add to the same words
+    if (threadIdx.x < kClasses && class_smem[threadIdx.x]) atomicAdd(class_count + threadIdx.x, class_smem[threadIdx.x]);
+    if (threadIdx.x < kNumBins && bin_smem[threadIdx.x]) atomicAdd(&counts->bin_count[threadIdx.x], bin_smem[threadIdx.x]);
+    if (threadIdx.x == 0 && max_smem) atomicMax(&counts->max_degree, max_smem);
 }
+
+constexpr int kKeyItems = 4;                          // entries per thread of finalize_entries
 
 // col_idx, the GCN weight and (unless the duplicate removal already wrote it) perm of every slot
 __global__ void __launch_bounds__(kThreads)
@@ -464,7 +665,7 @@ finalize_entries(const u64* __restrict__ keys, const int32_t* __restrict__ vals,
                  int32_t* __restrict__ col_idx, float* __restrict__ edge_w, int32_t* __restrict__ perm, int64_t m)
 {
     const int64_t base = (int64_t)blockIdx.x * (kThreads * kKeyItems) + threadIdx.x;
-    const int64_t nnz = counts->nnz;
+    const int64_t nnz = counts->sort_failed ? 0 : counts->nnz;
     u64 word[kKeyItems];
 #pragma unroll
     for (int j = 0; j < kKeyItems; ++j) {
@@ -506,6 +707,45 @@ __device__ __forceinline__ int32_t lower_bound_col(const int32_t* __restrict__ c
     return lo;
 }
 
+// segments of hub row v per source range (stored `pitch` apart) and altogether
+__device__ __forceinline__ int32_t count_row_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+                                                      int32_t v, int32_t* range_count, int64_t pitch, int32_t n_ranges,
+                                                      int64_t range_rows)
+{
+    int32_t pos = row_ptr[v], total = 0;
+    const int32_t e = row_ptr[v + 1];
+    for (int32_t r = 0; r < n_ranges; ++r) {
+        const int32_t nxt = r == n_ranges - 1 ? e : lower_bound_col(col_idx, pos, e, (int64_t)(r + 1) * range_rows);
+        const int32_t c = (nxt - pos + kHubSegment - 1) / kHubSegment;
+        range_count[r * pitch] = c;
+        total += c;
+        pos = nxt;
+    }
+    return total;
+}
+
+// the segments themselves: `slot` is the row's first slot, range_first (`pitch` apart) its first schedule position per range
+__device__ __forceinline__ void fill_row_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+                                                  int32_t v, int32_t slot, const int32_t* range_first, int64_t pitch,
+                                                  int32_t n_ranges, int64_t range_rows, int32_t* __restrict__ seg_row,
+                                                  int32_t* __restrict__ seg_begin, int32_t* __restrict__ seg_end,
+                                                  int32_t* __restrict__ seg_slot)
+{
+    int32_t pos = row_ptr[v];
+    const int32_t e = row_ptr[v + 1];
+    for (int32_t r = 0; r < n_ranges; ++r) {
+        const int32_t nxt = r == n_ranges - 1 ? e : lower_bound_col(col_idx, pos, e, (int64_t)(r + 1) * range_rows);
+        int32_t p = range_first[r * pitch];
+        for (int32_t x0 = pos; x0 < nxt; x0 += kHubSegment, ++p, ++slot) {
+            seg_row[p] = v;
+            seg_begin[p] = x0;
+            seg_end[p] = min(x0 + kHubSegment, nxt);
+            seg_slot[p] = slot;
+        }
+        pos = nxt;
+    }
+}
+
 // per hub row and source range: the number of segments (range-major: count[r * hub_cap + i]) and per hub row
 // the total; entries past the last hub row are 0 so that the scans yield the totals
 __global__ void __launch_bounds__(kThreads)
@@ -515,19 +755,10 @@ hub_segment_counts(const int32_t* __restrict__ row_ptr, const int32_t* __restric
 {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i > hub_cap) return;
-    const int32_t n_hub = counts->bin_count[4];
+    const int32_t n_hub = counts->sort_failed ? 0 : counts->bin_count[4];
     int32_t total = 0;
     if (i < n_hub) {
-        const int32_t v = row_order[n - n_hub + i];
-        int32_t pos = row_ptr[v];
-        const int32_t e = row_ptr[v + 1];
-        for (int32_t r = 0; r < n_ranges; ++r) {
-            const int32_t nxt = r == n_ranges - 1 ? e : lower_bound_col(col_idx, pos, e, (int64_t)(r + 1) * range_rows);
-            const int32_t c = (nxt - pos + kHubSegment - 1) / kHubSegment;
-            range_count[(int64_t)r * hub_cap + i] = c;
-            total += c;
-            pos = nxt;
-        }
+        total = count_row_segments(row_ptr, col_idx, row_order[n - n_hub + i], range_count + i, hub_cap, n_ranges, range_rows);
     } else if (i < hub_cap) {
         for (int32_t r = 0; r < n_ranges; ++r) range_count[(int64_t)r * hub_cap + i] = 0;
     }
@@ -545,32 +776,59 @@ fill_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ c
               int32_t* __restrict__ seg_slot)
 {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    const int32_t n_hub = counts->bin_count[4];
+    const int32_t n_hub = counts->sort_failed ? 0 : counts->bin_count[4];
     if (i == 0) counts->n_segments = hub_seg_ptr[n_hub];
     if (i >= hub_cap || i >= n_hub) return;
-    const int32_t v = row_order[n - n_hub + i];
-    int32_t pos = row_ptr[v];
-    const int32_t e = row_ptr[v + 1];
-    int32_t slot = hub_seg_ptr[i];
-    for (int32_t r = 0; r < n_ranges; ++r) {
-        const int32_t nxt = r == n_ranges - 1 ? e : lower_bound_col(col_idx, pos, e, (int64_t)(r + 1) * range_rows);
-        int32_t p = range_first[(int64_t)r * hub_cap + i];
-        for (int32_t x0 = pos; x0 < nxt; x0 += kHubSegment, ++p, ++slot) {
-            seg_row[p] = v;
-            seg_begin[p] = x0;
-            seg_end[p] = min(x0 + kHubSegment, nxt);
-            seg_slot[p] = slot;
+    fill_row_segments(row_ptr, col_idx, row_order[n - n_hub + i], hub_seg_ptr[i], range_first + i, hub_cap, n_ranges, range_rows,
+                      seg_row, seg_begin, seg_end, seg_slot);
+}
+
+// The three steps above in one block, for graphs that can have few hub rows (hub_cap * n_ranges up to kFewHubPieces):
+// counts, both scans and the fill without a launch in between.
+constexpr int kFewHubPieces = 8192;
+constexpr int kHubThreads = 1024;
+
+__global__ void __launch_bounds__(kHubThreads)
+hub_segments_few(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ row_order,
+                 int64_t n, BuildCounts* __restrict__ counts, int32_t n_ranges, int64_t range_rows, int32_t* range_count,
+                 int32_t* hub_seg_ptr, int32_t* __restrict__ seg_row, int32_t* __restrict__ seg_begin,
+                 int32_t* __restrict__ seg_end, int32_t* __restrict__ seg_slot)
+{
+    __shared__ int32_t smem[32];
+    const int32_t n_hub = counts->sort_failed ? 0 : counts->bin_count[4];
+    for (int32_t i = threadIdx.x; i < n_hub; i += kHubThreads)
+        hub_seg_ptr[i] = count_row_segments(row_ptr, col_idx, row_order[n - n_hub + i], range_count + i, n_hub, n_ranges, range_rows);
+    __syncthreads();
+    auto scan_in_place = [&](int32_t* p, int32_t count) {
+        int32_t carry = 0;
+        for (int32_t base = 0; base < count; base += kHubThreads) {
+            const int32_t i = base + threadIdx.x;
+            const int32_t mine = i < count ? p[i] : 0;
+            int32_t sum;
+            const int32_t before = block_scan(mine, &sum, smem) + carry;
+            if (i < count) p[i] = before;
+            carry += sum;
+            __syncthreads();
         }
-        pos = nxt;
+        return carry;
+    };
+    const int32_t total = scan_in_place(hub_seg_ptr, n_hub);
+    scan_in_place(range_count, n_hub * n_ranges);
+    if (threadIdx.x == 0) {
+        hub_seg_ptr[n_hub] = total;
+        counts->n_segments = total;
     }
+    for (int32_t i = threadIdx.x; i < n_hub; i += kHubThreads)
+        fill_row_segments(row_ptr, col_idx, row_order[n - n_hub + i], hub_seg_ptr[i], range_count + i, n_hub, n_ranges, range_rows,
+                          seg_row, seg_begin, seg_end, seg_slot);
 }
 
 // ------------------------------------------------------------------ host side
 
 struct BuildLayout {
     int64_t m;             // candidate edges
-    int64_t n_tiles;       // sort tiles of the edge sort
-    int64_t row_tiles;     // sort tiles of the row (degree class) sort
+    int64_t n_tiles;       // tiles of an edge sweep
+    int64_t row_tiles;     // tiles of the row (degree class) sweep
     int64_t hub_cap;       // upper bound on hub rows
     int64_t seg_cap;       // upper bound on hub segments
     int src_bits, key_bits, passes, digit_bits;
@@ -594,9 +852,8 @@ static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L)
     if (flags & GNNFD_CSR_ADD_SELF_LOOPS) m += n;
     if (m > limit) return GNNFD_TOO_LARGE;
     L->m = m;
-    L->n_tiles = (m + kSortTile - 1) / kSortTile;
-    if (L->n_tiles == 0) L->n_tiles = 1;
-    L->row_tiles = (n + kSortTile - 1) / kSortTile;
+    L->n_tiles = sweep_tiles(m);
+    L->row_tiles = sweep_tiles(n);
     L->hub_cap = m / (GNNFD_HUB_DEGREE + 1) + 1;
     // source ranges of GNNFD_HUB_RANGE_ROWS vertices, at most 64 of them (narrower ranges would keep a band of x
     // resident in L2, but on the RMAT workload the extra, shorter segments cost more than the saved traffic: 32
@@ -657,33 +914,58 @@ static void carve_persistent(Carver& c, int64_t n, const BuildLayout& L, Persist
 
 struct ScratchPtrs {
     u64 *keys_a, *keys_b;
-    int32_t *vals_a, *vals_b, *hist, *flags, *scan_temp;
+    int32_t *vals_a, *vals_b, *flags, *scan_temp;
+    // zeroed together before the first kernel: digit counts (a row per edge sweep, then the degree classes), tile
+    // counters (likewise), the words the row sweep's and the first edge sweep's tiles publish
+    int32_t *digit_count, *ticket;
+    uint32_t *row_published, *published, *published_alt;
+    size_t zero_bytes;
 };
 
-static size_t flag_ints(int64_t n, const BuildLayout& L)
+static size_t flag_ints(const BuildLayout& L)
 {
-    // one count per tile of the duplicate removal, a 64-bit dump for the row sort's keys (2 ints per row),
-    // hub segment counts (per source range and hub row, then per hub row)
-    size_t a = (size_t)L.m / kUniqueTile + 2, b = 2 * (size_t)n + 2, c = (size_t)L.hub_cap * (L.n_ranges + 1) + 4;
-    size_t r = a > b ? a : b;
-    return (r > c ? r : c) + 1;
+    // one count per tile of the duplicate removal; hub segment counts (per source range and hub row, then per hub row)
+    size_t a = (size_t)L.m / kUniqueTile + 2, c = (size_t)L.hub_cap * (L.n_ranges + 1) + 4;
+    return (a > c ? a : c) + 1;
 }
 
-static void carve_scratch(Carver& c, int64_t n, const BuildLayout& L, ScratchPtrs* p)
+static void carve_scratch(Carver& c, const BuildLayout& L, ScratchPtrs* p)
 {
-    const size_t cap = (size_t)(L.m > n ? L.m : n);      // the row sort reuses the edge sort's buffers
+    const size_t cap = (size_t)(L.m > 0 ? L.m : 1);
     p->keys_a = c.take<u64>(cap);
     p->keys_b = c.take<u64>(cap);
-    // when the values travel inside the key words only the row sort needs value buffers
-    const size_t val_cap = L.val_bits > 0 ? (size_t)n : cap;
+    const size_t val_cap = L.val_bits > 0 ? 1 : cap;      // no value buffers when the values travel inside the key words
     p->vals_a = c.take<int32_t>(val_cap);
     p->vals_b = c.take<int32_t>(val_cap);
-    const size_t hist_ints = (size_t)kRadix * (size_t)(L.n_tiles > L.row_tiles ? L.n_tiles : L.row_tiles);
-    p->hist = c.take<int32_t>(hist_ints);
-    const size_t fl = flag_ints(n, L);
+    const size_t zero_begin = c.off;
+    p->digit_count = c.take<int32_t>((size_t)(L.passes + 1) * kRadix);
+    p->ticket = c.take<int32_t>((size_t)L.passes + 1);
+    p->row_published = c.take<uint32_t>((size_t)kRadix * L.row_tiles);
+    p->published = c.take<uint32_t>((size_t)kRadix * L.n_tiles);
+    p->zero_bytes = c.off - zero_begin;
+    p->published_alt = c.take<uint32_t>((size_t)kRadix * L.n_tiles);
+    const size_t fl = flag_ints(L);
     p->flags = c.take<int32_t>(fl);
-    const size_t biggest = hist_ints > fl ? hist_ints : fl;
-    p->scan_temp = c.take<int32_t>(scan_temp_ints(biggest));
+    p->scan_temp = c.take<int32_t>(scan_temp_ints(fl));
+}
+
+template <typename Shape, int SOURCE, bool HAS_VALS>
+static int launch_sweep_shape(const char* name, const SweepArgs& a, cudaStream_t s)
+{
+    const auto kernel = radix_sweep<Shape, SOURCE, HAS_VALS>;
+    const int blocks = a.n_tiles < Shape::kMinBlocks * kSmCount ? a.n_tiles : Shape::kMinBlocks * kSmCount;
+    const int smem = (int)sizeof(SweepSmem<Shape>);
+    GNNFD_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    GNNFD_LAUNCH(name, s, kernel, (unsigned)blocks, Shape::kThreads, smem, a);
+    return GNNFD_OK;
+}
+
+template <int SOURCE, bool HAS_VALS>
+static int launch_sweep(const char* name, SweepArgs& a, cudaStream_t s)
+{
+    a.n_tiles = (int)sweep_tiles(a.m);
+    return use_large_tile(a.m) ? launch_sweep_shape<LargeTile, SOURCE, HAS_VALS>(name, a, s)
+                               : launch_sweep_shape<SmallTile, SOURCE, HAS_VALS>(name, a, s);
 }
 
 }  // namespace gnnfd
@@ -705,7 +987,7 @@ int gnnfd_csr_workspace_bytes(int64_t n, int64_t e, uint32_t flags, size_t* pers
     if (scratch_bytes) {
         Carver c(nullptr, ~size_t(0));
         ScratchPtrs s;
-        carve_scratch(c, n, L, &s);
+        carve_scratch(c, L, &s);
         *scratch_bytes = c.off;
     }
     return GNNFD_OK;
@@ -729,7 +1011,7 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     PersistentPtrs P;
     ScratchPtrs S;
     carve_persistent(pc, n, L, &P);
-    carve_scratch(sc, n, L, &S);
+    carve_scratch(sc, L, &S);
     if (!pc.ok || !sc.ok) return GNNFD_WORKSPACE_TOO_SMALL;
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -746,36 +1028,42 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     const bool dedup = (flags & GNNFD_CSR_DEDUP) != 0;
     const int vb = L.val_bits;
     const bool packed = vb > 0;                     // values ride in the low bits of the keys
-    const size_t scatter_smem = packed ? offsetof(ScatterSmem, vals) : sizeof(ScatterSmem);
-    GNNFD_CUDA_CHECK(cudaFuncSetAttribute(radix_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sizeof(ScatterSmem)));
-    GNNFD_CUDA_CHECK(cudaFuncSetAttribute(radix_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)offsetof(ScatterSmem, vals)));
+    GNNFD_CUDA_CHECK(cudaMemsetAsync(S.digit_count, 0, S.zero_bytes, s));
+    SweepArgs sw{};
+    sw.cand = Candidates{d_src, d_dst, n, e, m, flags, L.src_bits};
+    sw.m = m;
+    sw.val_bits = vb;
+    sw.counts = P.counts;
     if (m > 0) {
-        int32_t* key_vals = packed ? nullptr : vals;
+        const unsigned walkers = blocks_for(m, kHistTile) < 6u * kSmCount ? blocks_for(m, kHistTile) : 6u * kSmCount;
+        const size_t hist_bytes = (size_t)L.passes * kRadix * sizeof(int32_t);
         if (itype == GNNFD_I32)
-            GNNFD_LAUNCH("make_keys", s, make_keys<int32_t>, blocks_for(m, kThreads * kKeyItems), kThreads, 0,
-                         static_cast<const int32_t*>(d_src), static_cast<const int32_t*>(d_dst), n, e, m, flags, L.src_bits,
-                         vb, keys, key_vals, P.counts);
+            GNNFD_LAUNCH("edge_histograms", s, edge_histograms<int32_t>, walkers, kThreads, hist_bytes, sw.cand, L.first_bit,
+                         L.digit_bits, L.passes, S.digit_count, P.counts);
         else
-            GNNFD_LAUNCH("make_keys", s, make_keys<long long>, blocks_for(m, kThreads * kKeyItems), kThreads, 0,
-                         static_cast<const long long*>(d_src), static_cast<const long long*>(d_dst), n, e, m, flags,
-                         L.src_bits, vb, keys, key_vals, P.counts);
-        const int mask = (1 << L.digit_bits) - 1;
+            GNNFD_LAUNCH("edge_histograms", s, edge_histograms<long long>, walkers, kThreads, hist_bytes, sw.cand, L.first_bit,
+                         L.digit_bits, L.passes, S.digit_count, P.counts);
+        sw.mask = (1 << L.digit_bits) - 1;
+        uint32_t* published = S.published;
+        uint32_t* published_alt = S.published_alt;
         for (int pass = 0; pass < L.passes; ++pass) {
-            const int shift = L.first_bit + pass * L.digit_bits + vb;
-            GNNFD_LAUNCH("radix_histogram", s, radix_histogram, (unsigned)L.n_tiles, kThreads, 0, keys, m, shift, mask,
-                         L.n_tiles, S.hist);
-            rc = exclusive_scan_i32(S.hist, S.hist, (size_t)kRadix * (size_t)L.n_tiles, S.scan_temp, s);
-            if (rc) return rc;
-            if (packed)
-                GNNFD_LAUNCH("radix_scatter", s, radix_scatter<false>, (unsigned)L.n_tiles, kScatterThreads, scatter_smem, keys,
-                             (const int32_t*)nullptr, keys_alt, (int32_t*)nullptr, m, shift, mask, L.n_tiles, S.hist);
+            sw.shift = L.first_bit + pass * L.digit_bits + vb;
+            sw.digit_count = S.digit_count + (size_t)pass * kRadix;
+            sw.ticket = S.ticket + pass;
+            sw.published = published;
+            sw.published_next = pass + 1 < L.passes ? published_alt : nullptr;
+            sw.keys_in = keys; sw.keys_out = keys_alt;
+            sw.vals_in = vals; sw.vals_out = vals_alt;
+            if (pass > 0)
+                rc = packed ? launch_sweep<kWords, false>("radix_sweep", sw, s) : launch_sweep<kWords, true>("radix_sweep", sw, s);
+            else if (itype == GNNFD_I32)
+                rc = packed ? launch_sweep<kEdges32, false>("radix_sweep", sw, s) : launch_sweep<kEdges32, true>("radix_sweep", sw, s);
             else
-                GNNFD_LAUNCH("radix_scatter", s, radix_scatter<true>, (unsigned)L.n_tiles, kScatterThreads, scatter_smem, keys,
-                             (const int32_t*)vals, keys_alt, vals_alt, m, shift, mask, L.n_tiles, S.hist);
+                rc = packed ? launch_sweep<kEdges64, false>("radix_sweep", sw, s) : launch_sweep<kEdges64, true>("radix_sweep", sw, s);
+            if (rc) return rc;
             u64* tk = keys; keys = keys_alt; keys_alt = tk;
             int32_t* tv = vals; vals = vals_alt; vals_alt = tv;
+            uint32_t* tp = published; published = published_alt; published_alt = tp;
         }
         if (dedup) {
             const unsigned unique_tiles = blocks_for(m, kUniqueTile);
@@ -789,41 +1077,51 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
             u64* tk = keys; keys = keys_alt; keys_alt = tk;
         }
     }
-    GNNFD_LAUNCH("row_pointers", s, row_pointers, blocks_for((size_t)n + 1, kThreads), kThreads, 0, keys, P.counts, n,
-                 L.src_bits, vb, dedup ? 1 : 0, P.row_ptr);
-    // keys_alt / vals_alt are free from here on: they take the (degree class, row) pairs
-    GNNFD_LAUNCH("degrees_and_classes", s, degrees_and_classes, blocks_for((size_t)n, kThreads), kThreads, 0, P.row_ptr, n,
-                 P.dinv, P.rdeg, keys_alt, vals_alt, P.counts);
+    int32_t* class_count = S.digit_count + (size_t)L.passes * kRadix;
+    GNNFD_LAUNCH("rows_and_degrees", s, rows_and_degrees, blocks_for((size_t)n + 1, kRowsPerBlock), kThreads, 0, keys, P.counts, n,
+                 L.src_bits, vb, dedup ? 1 : 0, P.row_ptr, P.dinv, P.rdeg, class_count);
     if (m > 0)
         GNNFD_LAUNCH("finalize_entries", s, finalize_entries, blocks_for(m, kThreads * kKeyItems), kThreads, 0, keys,
                      packed ? (const int32_t*)nullptr : (const int32_t*)vals, dedup ? 0 : 1, P.counts, L.src_bits, vb,
                      P.dinv, P.col_idx, P.edge_w, P.perm, m);
-    // row_order = rows sorted by degree class, ascending row id inside a class: one stable radix pass
-    {
-        GNNFD_LAUNCH("radix_histogram", s, radix_histogram, (unsigned)L.row_tiles, kThreads, 0, keys_alt, n, 32, kRadix - 1,
-                     L.row_tiles, S.hist);
-        rc = exclusive_scan_i32(S.hist, S.hist, (size_t)kRadix * (size_t)L.row_tiles, S.scan_temp, s);
-        if (rc) return rc;
-        GNNFD_LAUNCH("radix_scatter", s, radix_scatter<true>, (unsigned)L.row_tiles, kScatterThreads, sizeof(ScatterSmem), keys_alt,
-                     vals_alt, reinterpret_cast<u64*>(S.flags), P.row_order, n, 32, kRadix - 1, L.row_tiles, S.hist);
-    }
-    // the flag buffer is free again: segment counts per (source range, hub row), then per hub row
+    // row_order = rows sorted by degree class, ascending row id inside a class: one sweep over the rows
+    sw.row_ptr = P.row_ptr;
+    sw.vals_out = P.row_order;
+    sw.m = n;
+    sw.shift = 32;
+    sw.mask = kRadix - 1;
+    sw.digit_count = class_count;
+    sw.ticket = S.ticket + L.passes;
+    sw.published = S.row_published;
+    sw.published_next = nullptr;
+    rc = launch_sweep<kRows, false>("radix_sweep_rows", sw, s);
+    if (rc) return rc;
+    // segment counts per (source range, hub row), then per hub row
     int32_t* range_count = S.flags;
-    int32_t* seg_count = S.flags + (size_t)L.hub_cap * L.n_ranges + 1;
-    GNNFD_LAUNCH("hub_segment_counts", s, hub_segment_counts, blocks_for((size_t)L.hub_cap + 1, kThreads), kThreads, 0,
-                 P.row_ptr, P.col_idx, P.row_order, n, P.counts, L.hub_cap, L.n_ranges, L.range_rows, range_count, seg_count);
-    rc = exclusive_scan_i32(seg_count, P.hub_seg_ptr, (size_t)L.hub_cap + 1, S.scan_temp, s);
-    if (rc) return rc;
-    rc = exclusive_scan_i32(range_count, range_count, (size_t)L.hub_cap * L.n_ranges + 1, S.scan_temp, s);
-    if (rc) return rc;
-    GNNFD_LAUNCH("fill_segments", s, fill_segments, blocks_for((size_t)L.hub_cap, kThreads), kThreads, 0, P.row_ptr, P.col_idx,
-                 P.row_order, n, P.counts, P.hub_seg_ptr, range_count, L.hub_cap, L.n_ranges, L.range_rows, P.seg_row,
-                 P.seg_begin, P.seg_end, P.seg_slot);
+    if (L.hub_cap * L.n_ranges <= kFewHubPieces) {
+        GNNFD_LAUNCH("hub_segments_few", s, hub_segments_few, 1, kHubThreads, 0, P.row_ptr, P.col_idx, P.row_order, n, P.counts,
+                     L.n_ranges, L.range_rows, range_count, P.hub_seg_ptr, P.seg_row, P.seg_begin, P.seg_end, P.seg_slot);
+    } else {
+        int32_t* seg_count = S.flags + (size_t)L.hub_cap * L.n_ranges + 1;
+        GNNFD_LAUNCH("hub_segment_counts", s, hub_segment_counts, blocks_for((size_t)L.hub_cap + 1, kThreads), kThreads, 0,
+                     P.row_ptr, P.col_idx, P.row_order, n, P.counts, L.hub_cap, L.n_ranges, L.range_rows, range_count, seg_count);
+        rc = exclusive_scan_i32(seg_count, P.hub_seg_ptr, (size_t)L.hub_cap + 1, S.scan_temp, s);
+        if (rc) return rc;
+        rc = exclusive_scan_i32(range_count, range_count, (size_t)L.hub_cap * L.n_ranges + 1, S.scan_temp, s);
+        if (rc) return rc;
+        GNNFD_LAUNCH("fill_segments", s, fill_segments, blocks_for((size_t)L.hub_cap, kThreads), kThreads, 0, P.row_ptr, P.col_idx,
+                     P.row_order, n, P.counts, P.hub_seg_ptr, range_count, L.hub_cap, L.n_ranges, L.range_rows, P.seg_row,
+                     P.seg_begin, P.seg_end, P.seg_slot);
+    }
     GNNFD_CUDA_CHECK(cudaGetLastError());
     GNNFD_CUDA_CHECK(cudaMemcpyAsync(&host_counts, P.counts, sizeof(BuildCounts), cudaMemcpyDeviceToHost, s));
     GNNFD_CUDA_CHECK(cudaStreamSynchronize(s));
 
     if (host_counts.bad_index > 0) return GNNFD_BAD_INDEX;
+    if (host_counts.sort_failed) {
+        set_cuda_error(cudaErrorLaunchTimeout);
+        return GNNFD_CUDA_ERROR;
+    }
 
     gnnfd_csr_t* h = new (std::nothrow) gnnfd_csr_t;
     if (!h) return GNNFD_INVALID_ARG;

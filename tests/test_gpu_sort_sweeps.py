@@ -1,0 +1,90 @@
+"""The sort behind the CSR build at the edges of its tiles and block shapes, against numpy's stable sort: tile sizes 2048 and
+8192 (the larger from 4 * 148 * 8192 candidates on), key and value in one word or apart, digits that are all equal."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SL, DD, SY, LIGHT = 1, 2, 4, 8
+LARGE = 4 * 148 * 8192
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2104_03058_b200 as lib
+    lib.lib()
+    return lib
+
+
+def reference(n, src, dst, flags):
+    """row_ptr, col, perm by a stable sort (or by destination only for the light build)"""
+    e = len(src)
+    s, d, p = src.astype(np.int64), dst.astype(np.int64), np.arange(e)
+    if flags & SY:
+        rev = s != d
+        s, d, p = np.concatenate([s, d[rev]]), np.concatenate([d, s[rev]]), np.concatenate([p, e + p[rev]])
+    if flags & SL:
+        keep = s != d
+        own = np.arange(n)
+        s, d, p = np.concatenate([s[keep], own]), np.concatenate([d[keep], own]), np.concatenate([p[keep], np.full(n, -1)])
+    order = np.argsort(d if flags & LIGHT else d * n + s, kind="stable")
+    s, d, p = s[order], d[order], p[order]
+    if flags & DD:
+        first = np.ones(len(s), bool)
+        first[1:] = (s[1:] != s[:-1]) | (d[1:] != d[:-1])
+        s, d, p = s[first], d[first], p[first]
+    return np.searchsorted(d, np.arange(n + 1)), s, p
+
+
+def check(g, n, src, dst, flags):
+    csr = g.build_csr(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), flags)
+    row_ptr, col, perm = reference(n, src, dst, flags)
+    assert csr.nnz == len(col)
+    np.testing.assert_array_equal(csr.row_ptr.cpu().numpy(), row_ptr)
+    np.testing.assert_array_equal(csr.col_idx.cpu().numpy(), col)
+    np.testing.assert_array_equal(csr.perm.cpu().numpy(), perm)
+    deg = np.diff(row_ptr)
+    assert csr.max_degree == deg.max()
+    assert csr.bin_count == [int(((deg > lo) & (deg <= hi)).sum()) for lo, hi in
+                             ((-1, 8), (8, 32), (32, 128), (128, 2048), (2048, 1 << 31))]
+    order = csr.row_order.cpu().numpy()
+    assert np.array_equal(np.sort(order), np.arange(n))
+    c = deg[order].astype(np.int64)
+    o = np.int64(np.log2(np.maximum(c - 1, 8)))                     # classes: exact degree to 8, quarter octaves, hub rows
+    cls = np.where(c <= 8, c, np.where(c > 2048, 41, 9 + (o - 3) * 4 + ((c - 1) >> (o - 2) & 3)))
+    assert ((cls[1:] > cls[:-1]) | ((cls[1:] == cls[:-1]) & (order[1:] > order[:-1]))).all()
+
+
+@pytest.mark.parametrize("m", [1, 31, 2047, 2048, 2049, 4097, 148 * 4 * 2048 + 5, LARGE - 1, LARGE, LARGE + 8191])
+@pytest.mark.parametrize("ids", [np.int32, np.int64])
+def test_tile_edges(g, m, ids):
+    rng = np.random.default_rng(m)
+    n = 1000 if m < 100_000 else 70_001
+    check(g, n, rng.integers(0, n, m).astype(ids), rng.integers(0, n, m).astype(ids), 0)
+
+
+@pytest.mark.parametrize("flags", [SL, SY, SL | SY | DD, DD, LIGHT | SL | SY])
+def test_candidates_that_are_no_plain_edges_fill_tiles(g, flags):
+    rng = np.random.default_rng(flags)
+    n, e = 30_000, LARGE // 2 + 777                                 # reverses and loops begin inside a tile
+    check(g, n, rng.integers(0, n, e).astype(np.int32), rng.integers(0, n, e).astype(np.int32), flags)
+
+
+@pytest.mark.parametrize("m", [300_000, LARGE + 1])
+@pytest.mark.parametrize("flags", [0, DD, SL, LIGHT])
+def test_key_and_value_apart(g, m, flags):
+    n = (1 << 22) + 3                                               # 23 + 23 key bits and at least 19 value bits: two words
+    rng = np.random.default_rng(m + flags)
+    check(g, n, rng.integers(0, n, m).astype(np.int32), rng.integers(n - 5000, n, m).astype(np.int32), flags)
+
+
+@pytest.mark.parametrize("m", [10_000, LARGE + 100])
+@pytest.mark.parametrize("kind", ["one pair", "one destination", "pairs in turn", "sorted"])
+def test_equal_and_ordered_digits(g, m, kind):
+    n = 5000
+    rng = np.random.default_rng(7)
+    i = np.arange(m)
+    src, dst = {"one pair": (np.full(m, 4999), np.full(m, 17)), "one destination": (rng.integers(0, n, m), np.full(m, 3)),
+                "pairs in turn": (i // 2 % n, i // 3 % n), "sorted": (i * n // m, i * n // m)}[kind]
+    check(g, n, src.astype(np.int32), dst.astype(np.int32), 0)
