@@ -145,8 +145,14 @@ void gnnfd_csr_destroy(gnnfd_csr_t* csr);
  * of gnnfd_aggregate_workspace_bytes(csr, f) bytes (holds the per-segment partial sums of hub rows;
  * 0 bytes when the graph has no hub row, NULL is then accepted).  The call only enqueues work.
  * 16-byte-aligned pointers with ldx*sizeof(x) and chunk offsets multiples of 16 bytes take the
- * 128-bit load path; anything else is still correct through narrower loads. */
+ * 128-bit load path; anything else is still correct through narrower loads.  Where the features are not aligned
+ * like that, a scratch buffer of gnnfd_aggregate_best_workspace_bytes(csr, d_x, ldx, xdt, f, chunk_width) bytes lets
+ * the call gather from an aligned copy of them wherever that is faster (the same sums in another order);
+ * elsewhere that size equals gnnfd_aggregate_workspace_bytes. */
 int gnnfd_aggregate_workspace_bytes(const gnnfd_csr_t* csr, int32_t f, size_t* scratch_bytes);
+
+int gnnfd_aggregate_best_workspace_bytes(const gnnfd_csr_t* csr, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f,
+                                         int32_t chunk_width, size_t* scratch_bytes);
 
 int gnnfd_aggregate_gcn(const gnnfd_csr_t* csr, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt,
                         void* d_out, int64_t ldo, gnnfd_dtype_t odt, int32_t f, int32_t chunk_width,
@@ -185,7 +191,7 @@ int gnnfd_tune_chunk_width(const gnnfd_csr_t* csr, int model, const void* d_x, i
  * leave the timing off where allocation is not allowed.
  *
  * Same arguments and same results (bit for bit: it runs the same kernels on the same data) as
- * gnnfd_aggregate_gcn, minus the scratch pair.
+ * gnnfd_aggregate_gcn with gnnfd_aggregate_workspace_bytes of scratch, minus the scratch pair.
  * Limits and rules:
  *   - returns GNNFD_STATIC_SCRATCH_EXCEEDED when gnnfd_aggregate_workspace_bytes(csr, f) is larger
  *     than GNNFD_STATIC_SCRATCH_BYTES (hub segments x f rounded up to 4, x 4 bytes); nothing is launched;

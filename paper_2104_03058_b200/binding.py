@@ -52,6 +52,7 @@ def lib() -> ctypes.CDLL:
         L.gnnfd_csr_destroy.argtypes = [vp]
         L.gnnfd_csr_destroy.restype = None
         L.gnnfd_aggregate_workspace_bytes.argtypes = [vp, i32, pp(sz)]
+        L.gnnfd_aggregate_best_workspace_bytes.argtypes = [vp, vp, i64, i32, i32, i32, pp(sz)]
         agg = [vp, vp, i64, i32, vp, i64, i32, i32, i32, vp, sz, vp]
         L.gnnfd_aggregate_gcn.argtypes = agg
         L.gnnfd_aggregate_sage.argtypes = agg
@@ -274,6 +275,16 @@ def aggregate_workspace_bytes(csr: Csr, f: int) -> int:
     return s.value
 
 
+def aggregate_best_workspace_bytes(csr: Csr, x: torch.Tensor, f: int | None = None, chunk_width: int | None = None) -> int:
+    """Scratch with which an aggregation of these features is fastest (at least aggregate_workspace_bytes)."""
+    f = x.shape[1] if f is None else f
+    xp, ldx = _matrix(x, f, "x")
+    s = ctypes.c_size_t()
+    _check(lib().gnnfd_aggregate_best_workspace_bytes(csr.handle, xp, ldx, _dtype_code(x), f, f if chunk_width is None else chunk_width,
+                                                      ctypes.byref(s)), "gnnfd_aggregate_best_workspace_bytes")
+    return s.value
+
+
 def _aggregate(fn, name, csr: Csr, x, f, chunk_width, out, out_dtype, scratch, stream):
     f = x.shape[1] if f is None else f
     chunk_width = f if chunk_width is None else chunk_width
@@ -282,9 +293,10 @@ def _aggregate(fn, name, csr: Csr, x, f, chunk_width, out, out_dtype, scratch, s
     xp, ldx = _matrix(x, f, "x")
     op, ldo = _matrix(out, f, "out")
     _check_aggregate_operands(csr, x, out, f)
-    need = aggregate_workspace_bytes(csr, f)
-    if scratch is None and need:
-        scratch = _alloc_bytes(need, x.device, stream)
+    if scratch is None:
+        need = aggregate_best_workspace_bytes(csr, x, f, chunk_width)
+        if need:
+            scratch = _alloc_bytes(need, x.device, stream)
     _same_device(csr.device, scratch=scratch)
     sp = ctypes.c_void_p(scratch.data_ptr()) if scratch is not None else None
     sn = scratch.numel() * scratch.element_size() if scratch is not None else 0
@@ -393,9 +405,10 @@ def tune_chunk_width(csr: Csr, x: torch.Tensor, model: str = "gcn", f: int | Non
     xp, ldx = _matrix(x, f, "x")
     op, ldo = _matrix(out, f, "out")
     _check_aggregate_operands(csr, x, out, f)
-    need = aggregate_workspace_bytes(csr, f)
-    if scratch is None and need:
-        scratch = _alloc_bytes(need, x.device, stream)
+    if scratch is None:
+        need = max([aggregate_best_workspace_bytes(csr, x, f, w) for w in candidates if w > 0], default=0)
+        if need:
+            scratch = _alloc_bytes(need, x.device, stream)
     _same_device(csr.device, scratch=scratch)
     sp = ctypes.c_void_p(scratch.data_ptr()) if scratch is not None else None
     sn = scratch.numel() * scratch.element_size() if scratch is not None else 0

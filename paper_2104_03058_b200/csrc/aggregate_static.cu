@@ -48,7 +48,8 @@ extern "C" int gnnfd_aggregate_gcn_static(const gnnfd_csr_t* csr, const void* d_
     void* scratch = nullptr;
     rc = static_scratch_address(&scratch);
     if (rc) return rc;
+    // Only the partial sums' share is handed over: a call without hub rows touches nothing of the array.
     // Every partial sum that the reduction reads is written by the gather kernel of the same call, so
     // nothing in the array has to be cleared between calls.
-    return gnnfd_aggregate_gcn(csr, d_x, ldx, xdt, d_out, ldo, odt, f, chunk_width, scratch, kStaticScratchBytes, stream);
+    return gnnfd_aggregate_gcn(csr, d_x, ldx, xdt, d_out, ldo, odt, f, chunk_width, scratch, need, stream);
 }

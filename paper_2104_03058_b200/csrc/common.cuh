@@ -11,6 +11,7 @@ namespace gnnfd {
 
 constexpr int kNumBins = 5;                 // four degree classes + hub rows
 constexpr int kBinDeg0 = 8, kBinDeg1 = 32, kBinDeg2 = 128, kBinDeg3 = GNNFD_HUB_DEGREE;   // upper degree of each class
+constexpr int kOctaves = 4;                 // octaves of the degree in the fourth class
 constexpr int kHubSegment = GNNFD_HUB_SEGMENT;
 
 // Device-side counters filled during the build and copied to the host once.
@@ -22,7 +23,8 @@ struct BuildCounts {
     int32_t n_segments;      // hub segments
     int32_t bin_count[kNumBins];
     int32_t sort_failed;     // a sweep of the sort gave up waiting: nothing after it is meaningful
-    int32_t pad[5];
+    int32_t octave_count[kOctaves]; // rows of the fourth bin by octave of the degree: 129..256, ..512, ..1024, ..2048
+    int32_t pad[1];
 };
 
 }  // namespace gnnfd
@@ -32,6 +34,7 @@ struct gnnfd_csr {
     int32_t max_degree;
     int64_t bin_count[gnnfd::kNumBins];
     int64_t bin_start[gnnfd::kNumBins];
+    int64_t octave_count[gnnfd::kOctaves];       // the fourth bin (129 .. 2048 entries) by octave of the degree, ascending
     int64_t n_segments;
     const int32_t* row_ptr;
     const int32_t* col_idx;

@@ -624,10 +624,11 @@ rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts,
                  int dedup, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
                  int32_t* __restrict__ class_count)
 {
-    __shared__ int32_t ptr[kThreads], class_smem[kClasses], bin_smem[kNumBins], max_smem;
+    __shared__ int32_t ptr[kThreads], class_smem[kClasses], bin_smem[kNumBins], octave_smem[kOctaves], max_smem;
     if (counts->sort_failed) return;
     if (threadIdx.x < kClasses) class_smem[threadIdx.x] = 0;
     if (threadIdx.x < kNumBins) bin_smem[threadIdx.x] = 0;
+    if (threadIdx.x < kOctaves) octave_smem[threadIdx.x] = 0;
     if (threadIdx.x == 0) max_smem = 0;
     const int64_t v = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.x;
     const int32_t nnz = dedup ? counts->nnz : counts->n_valid;
@@ -647,12 +648,14 @@ rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts,
         rdeg[v] = deg > 0 ? (float)(1.0 / (double)deg) : 0.f;
         atomicAdd(&class_smem[degree_class(deg)], 1);
         atomicAdd(&bin_smem[degree_bin(deg)], 1);
+        if (degree_bin(deg) == 3) atomicAdd(&octave_smem[31 - __clz((deg - 1) / kBinDeg2)], 1);
         atomicMax(&max_smem, deg);
     }
     __syncthreads();
     // few global atomics: all blocks add to the same words
     if (threadIdx.x < kClasses && class_smem[threadIdx.x]) atomicAdd(class_count + threadIdx.x, class_smem[threadIdx.x]);
     if (threadIdx.x < kNumBins && bin_smem[threadIdx.x]) atomicAdd(&counts->bin_count[threadIdx.x], bin_smem[threadIdx.x]);
+    if (threadIdx.x < kOctaves && octave_smem[threadIdx.x]) atomicAdd(&counts->octave_count[threadIdx.x], octave_smem[threadIdx.x]);
     if (threadIdx.x == 0 && max_smem) atomicMax(&counts->max_degree, max_smem);
 }
 
@@ -1134,6 +1137,7 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
         h->bin_start[b] = start;
         start += host_counts.bin_count[b];
     }
+    for (int o = 0; o < kOctaves; ++o) h->octave_count[o] = host_counts.octave_count[o];
     h->n_segments = host_counts.n_segments;
     h->row_ptr = P.row_ptr;
     h->col_idx = P.col_idx;

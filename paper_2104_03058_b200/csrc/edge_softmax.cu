@@ -180,7 +180,7 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
             e = a.seg_end[slot];
             part = a.seg_slot[slot];
         } else {
-            row = a.row_order[rg.item_begin + slot];
+            row = a.row_order[rg.item_last - slot];
             b = a.row_ptr[row];
             e = a.row_ptr[row + 1];
         }
@@ -355,7 +355,7 @@ static size_t softmax_scratch_bytes(const gnnfd_csr_t* csr, int32_t heads)
 template <int HB, int LPS>
 static int launch_softmax(const gnnfd_csr_t* csr, SoftmaxArgs& a, cudaStream_t s)
 {
-    const int64_t blocks = plan_ranges(csr, LPS, a.range, &a.n_ranges);
+    const int64_t blocks = plan_ranges(csr, LPS, 1, 0, a.range, &a.n_ranges);
     if (blocks > 0x7fffffffll) return GNNFD_TOO_LARGE;
     if (blocks == 0) return GNNFD_OK;
     if (csr->n_segments > 0) {

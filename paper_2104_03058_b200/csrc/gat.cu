@@ -125,7 +125,7 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
             b = a.seg_begin[slot];
             e = a.seg_end[slot];
         } else {
-            row = a.row_order[rg.item_begin + slot];
+            row = a.row_order[rg.item_last - slot];
             b = a.row_ptr[row];
             e = a.row_ptr[row + 1];
         }
@@ -502,7 +502,7 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
     a.wide_ok = vec && vpl == 2 && ((uintptr_t)d_z % 32 == 0) && ((ldz * zsize) % 32 == 0) &&
                 (n_chunks == 1 || (cw * zsize) % 32 == 0);
 
-    const int64_t blocks = plan_ranges(csr, lpr, a.range, &a.n_ranges);
+    const int64_t blocks = plan_ranges(csr, lpr, 1, 0, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;
     if (grid_x > 0x7fffffffll) return GNNFD_TOO_LARGE;

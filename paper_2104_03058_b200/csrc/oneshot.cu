@@ -45,9 +45,11 @@ static int oneshot(bool weighted, int64_t n, int64_t e, const void* d_src, const
     rc = gnnfd_build_csr(n, e, d_src, d_dst, itype, oneshot_flags(flags), base, L.persistent, base + L.persistent,
                          L.build_scratch, stream, &csr);
     if (rc) return rc;
-    void* agg = base + L.persistent + L.build_scratch;
-    rc = weighted ? gnnfd_aggregate_gcn(csr, d_x, ldx, xdt, d_out, ldo, odt, f, chunk_width, agg, L.aggregate, stream)
-                  : gnnfd_aggregate_sage(csr, d_x, ldx, xdt, d_out, ldo, odt, f, chunk_width, agg, L.aggregate, stream);
+    // the build is done with its scratch (same stream), so the aggregation gets that as well: room for an aligned copy of x
+    void* agg = base + L.persistent;
+    const size_t agg_bytes = L.build_scratch + L.aggregate;
+    rc = weighted ? gnnfd_aggregate_gcn(csr, d_x, ldx, xdt, d_out, ldo, odt, f, chunk_width, agg, agg_bytes, stream)
+                  : gnnfd_aggregate_sage(csr, d_x, ldx, xdt, d_out, ldo, odt, f, chunk_width, agg, agg_bytes, stream);
     gnnfd_csr_destroy(csr);       // the enqueued kernels hold device pointers only
     return rc;
 }

@@ -10,15 +10,16 @@ namespace gnnfd {
 #define GNNFD_GATHER_BLOCK 256
 #endif
 constexpr int kBlock = GNNFD_GATHER_BLOCK;      // threads per block of the gather kernels
-constexpr int kMaxRanges = 5;
+constexpr int kMaxRanges = kNumBins - 1 + kOctaves;     // hub segments, the octaves of the fourth class, three classes
 constexpr int kMaxGridY = 65535;               // chunks one launch of a gather kernel covers (grid y)
 
 struct Range {
     int32_t first_block;   // first block (within one column tile of one sweep) of this range
-    int32_t item_begin;    // offset into row_order (rows) or 0 (hub segments)
+    int32_t item_last;     // rows: place of the last one in row_order, from where the range goes down (longest first)
     int32_t item_count;
     int32_t ep_log2;       // log2 of the edge-parallel groups per row
     int32_t hub;           // 1: items are hub segments writing partial results
+    int32_t warps_log2;    // log2 of the warps that share an item (more than one only where a row has all lanes of a warp)
 };
 
 inline int ilog2(int x) { int l = 0; while ((1 << l) < x) ++l; return l; }
@@ -44,24 +45,56 @@ inline int ep_for_bin(int bin, int lpr)
     return want[bin] < cap ? want[bin] : cap;
 }
 
-// Fills ranges for `lpr` lanes per row; returns the blocks of one column tile of one sweep.
-inline int64_t plan_ranges(const gnnfd_csr_t* csr, int lpr, Range* range, int32_t* n_ranges)
+// Warps of a block that share a row (or hub segment) of up to `entries` entries.  A warp walks its row in steps of
+// `per_step` entries whose loads are in flight together, one step after the other, so on a graph that
+// does not keep the chip busy for long the time of a launch is that of its longest walk, whatever the rest does.
+// A walk is therefore split until it is no longer than `limit` steps.
+inline int warps_log2_for(int entries, int per_step, int64_t limit)
+{
+    int w = 0;
+    while ((1 << w) < kBlock / 32 && (entries >> w) > per_step * limit) ++w;
+    return w;
+}
+
+// The longest walk to allow, in steps: twice what a warp slot of the chip has to do on average, and not under 16.  fp32 GCN
+// against unsplit rows (one warp up to 2048 entries): 4,000 rows of 10 entries and 304 columns 76 -> 18 us, 20,000 of 50 and
+// 128 columns 101 -> 40, 100,000 of 20 and 64 columns 75 -> 50; 200,000 of 16 and more stay unsplit.  With the
+// average itself or four times it as the limit: 38 and 58 us for the second, 52 and 75 for the third.
+inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t sweeps)
+{
+    constexpr int64_t kWarpSlots = 148 * 24;
+    const int64_t limit = 2 * (csr->nnz * sweeps / (per_step * kWarpSlots));
+    return limit > 16 ? limit : 16;
+}
+
+// Fills ranges for `lpr` lanes per row; returns the blocks of one column tile of one sweep.  `per_step`: entries a whole warp
+// has in flight; `limit`: steps of the longest walk (0: a row is never split).
+inline int64_t plan_ranges(const gnnfd_csr_t* csr, int lpr, int per_step, int64_t limit, Range* range, int32_t* n_ranges)
 {
     int nr = 0;
     int64_t blocks = 0;
-    if (csr->n_segments > 0) {
-        const int ep = ep_for_bin(4, lpr);
-        const int rows_per_block = kBlock / (lpr * ep);
-        range[nr++] = Range{(int32_t)blocks, 0, (int32_t)csr->n_segments, ilog2(ep), 1};
-        blocks += (csr->n_segments + rows_per_block - 1) / rows_per_block;
+    auto add = [&](int64_t begin, int64_t count, int ep, int entries, int hub) {
+        const int w = limit > 0 && lpr * ep == 32 ? warps_log2_for(entries, per_step, limit) : 0;
+        const int per_block = kBlock / (lpr * ep) >> w;
+        if (nr > 0 && !hub && !range[nr - 1].hub && range[nr - 1].warps_log2 == w && range[nr - 1].ep_log2 == ilog2(ep)) {
+            // the rows before those in the order, cut in the same way: one range
+            Range& r = range[nr - 1];
+            r.item_count += (int32_t)count;
+            blocks = r.first_block + (r.item_count + per_block - 1) / per_block;
+            return;
+        }
+        range[nr++] = Range{(int32_t)blocks, (int32_t)(begin + count - 1), (int32_t)count, ilog2(ep), hub, w};
+        blocks += (count + per_block - 1) / per_block;
+    };
+    if (csr->n_segments > 0) add(0, csr->n_segments, ep_for_bin(4, lpr), kHubSegment, 1);
+    int64_t end = csr->bin_start[3] + csr->bin_count[3];
+    for (int o = kOctaves - 1; o >= 0; --o) {
+        end -= csr->octave_count[o];
+        if (csr->octave_count[o] > 0) add(end, csr->octave_count[o], ep_for_bin(3, lpr), kBinDeg2 << (o + 1), 0);
     }
-    for (int bin = 3; bin >= 0; --bin) {
-        if (csr->bin_count[bin] == 0) continue;
-        const int ep = ep_for_bin(bin, lpr);
-        const int rows_per_block = kBlock / (lpr * ep);
-        range[nr++] = Range{(int32_t)blocks, (int32_t)csr->bin_start[bin], (int32_t)csr->bin_count[bin], ilog2(ep), 0};
-        blocks += (csr->bin_count[bin] + rows_per_block - 1) / rows_per_block;
-    }
+    const int longest[3] = {kBinDeg0, kBinDeg1, kBinDeg2};
+    for (int bin = 2; bin >= 0; --bin)
+        if (csr->bin_count[bin] > 0) add(csr->bin_start[bin], csr->bin_count[bin], ep_for_bin(bin, lpr), longest[bin], 0);
     *n_ranges = nr;
     return blocks;
 }

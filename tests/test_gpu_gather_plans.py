@@ -1,0 +1,113 @@
+"""Features whose rows or chunks do not start on 16-byte boundaries: the aligned copy that a larger scratch buffer allows, against the
+oracle and, bit for bit, against features laid out aligned; and long rows shared by several warps of a block."""
+import numpy as np
+import pytest
+
+import oracle as orc
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_2104_03058_b200 as lib
+    lib.lib()
+    return lib
+
+
+@pytest.fixture(scope="module")
+def graph(g):
+    rng = np.random.default_rng(5)
+    n, e = 1500, 1_200_000
+    dst = np.where(rng.random(e) < 0.2, 7, rng.integers(0, n - 1, e)).astype(np.int32)      # a hub row and an empty one
+    src = rng.integers(0, n, e).astype(np.int32)
+    row_ptr, col, _ = orc.build_csr(n, src, dst, 0)
+    return g.build_csr(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()), row_ptr, col
+
+
+def scratch(nbytes):
+    return torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("model", ["gcn", "sage"])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("f,ld,cw", [(57, 57, 57), (59, 64, 35), (66, 67, 64), (130, 130, 33), (301, 301, 64), (305, 306, 305)])
+def test_aligned_copy(g, graph, model, dtype, f, ld, cw):
+    csr, row_ptr, col = graph
+    fn = {"gcn": g.aggregate_gcn, "sage": g.aggregate_sage}[model]
+    gen = torch.Generator().manual_seed(f * 1000 + cw)
+    x = torch.full((csr.n, ld), float("nan"), dtype=dtype)                                  # padding never counts
+    x[:, :f] = torch.randn((csr.n, f), generator=gen).to(dtype)
+    x = x.cuda()
+    small, best = g.aggregate_workspace_bytes(csr, f), g.aggregate_best_workspace_bytes(csr, x, f, cw)
+    assert best > small > 0
+    plain = fn(csr, x, f=f, chunk_width=cw, scratch=scratch(small))
+    assert torch.equal(plain, fn(csr, x, f=f, chunk_width=cw, scratch=scratch(best - 256)))      # not enough for the copy
+    copied = fn(csr, x, f=f, chunk_width=cw)
+    assert torch.equal(copied, fn(csr, x, f=f, chunk_width=cw, scratch=scratch(best)))
+    if cw >= f or cw % 8 == 0:
+        wide = torch.zeros((csr.n, (f + 15) // 16 * 16), dtype=dtype, device="cuda")
+        wide[:, :f] = x[:, :f]
+        assert torch.equal(copied, fn(csr, wide, f=f, chunk_width=cw))
+    want, scale = orc.aggregate(model, row_ptr, col, np.ascontiguousarray(x[:, :f].float().cpu().numpy()), f)
+    for got in (plain, copied):
+        assert (np.abs(got.cpu().numpy() - want) <= 1e-5 * scale + 1e-6).all()
+    if model == "gcn":
+        out = torch.empty((csr.n, f), device="cuda")
+        assert torch.equal(plain, g.aggregate_gcn_static(csr, x, f=f, chunk_width=cw, out=out))
+
+
+def test_shifted_rows(g, graph):
+    csr, _, _ = graph
+    base = torch.randn((csr.n, 72), device="cuda")
+    for shift in (1, 2, 3, 5):
+        part = base[:, shift:shift + 64]
+        assert torch.equal(g.aggregate_gcn(csr, part), g.aggregate_gcn(csr, part.contiguous()))
+
+
+def test_where_no_copy_is_planned(g, graph):
+    n = 50_000
+    rng = np.random.default_rng(3)
+    csr = g.build_csr(n, *(torch.from_numpy(rng.integers(0, n, 3 * n).astype(np.int32)).cuda() for _ in range(2)))
+    x = torch.randn((n, 301), device="cuda")
+    assert g.aggregate_best_workspace_bytes(csr, x) == g.aggregate_workspace_bytes(csr, 301)         # few entries per row
+    x = torch.randn((graph[0].n, 31), device="cuda")
+    assert g.aggregate_best_workspace_bytes(graph[0], x) == g.aggregate_workspace_bytes(graph[0], 31)  # narrow fp32
+    x = torch.randn((graph[0].n, 64), device="cuda")
+    assert g.aggregate_best_workspace_bytes(graph[0], x) == g.aggregate_workspace_bytes(graph[0], 64)  # aligned
+
+
+# Rows of lengths around the octave bounds of the shared classes (a row of up to 256 / 512 / 1024 / 2048 entries is one, two, four or
+# eight warps' work when the graph is small), hub rows, and enough short rows beside them.
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("f", [4, 20, 40, 100, 264, 520])
+@pytest.mark.parametrize("model", ["gcn", "sage", "gat", "softmax"])
+def test_long_rows_of_small_graphs(g, model, f, dtype):
+    lengths = [0, 1, 8, 9, 32, 33, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2047, 2048, 2049, 3072, 5000] + [3] * 900
+    n = len(lengths)
+    rng = np.random.default_rng(f)
+    dst = np.repeat(np.arange(n), lengths).astype(np.int32)
+    src = rng.integers(0, n, len(dst)).astype(np.int32)
+    order = rng.permutation(len(dst))
+    src, dst = src[order], dst[order]
+    row_ptr, col, _ = orc.build_csr(n, src, dst, 0)
+    csr = g.build_csr(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda())
+    x = torch.randn((n, f), generator=torch.Generator().manual_seed(1)).to(dtype)
+    xs = np.ascontiguousarray(x.float().numpy())
+    if model in ("gcn", "sage"):
+        fn = {"gcn": g.aggregate_gcn, "sage": g.aggregate_sage}[model]
+        want, scale = orc.aggregate(model, row_ptr, col, xs, f)
+        run = lambda: fn(csr, x.cuda())
+    elif model == "gat":
+        heads, dim = (1, f) if f < 40 else (4, f // 4)
+        a = [torch.randn((heads, dim), generator=torch.Generator().manual_seed(k)) * 0.3 for k in (2, 3)]
+        want, scale = orc.aggregate_gat(row_ptr, col, xs, a[0].numpy(), a[1].numpy(), heads, dim, 0.2)
+        run = lambda: g.aggregate_gat(csr, x.cuda(), a[0].cuda(), a[1].cuda(), heads, dim, 0.2)
+    else:
+        s = [torch.randn((n, min(f // 4, 12)), generator=torch.Generator().manual_seed(k)) for k in (2, 3)]
+        want = scale = orc.edge_softmax(row_ptr, col, s[0].numpy(), s[1].numpy(), 0.2)
+        run = lambda: g.edge_softmax(csr, s[0].cuda(), s[1].cuda(), 0.2)
+    got = run()
+    assert (np.abs(got.cpu().numpy() - want) <= 1e-5 * scale + (1e-7 if model == "softmax" else 1e-6)).all()
+    assert torch.equal(got, run())
