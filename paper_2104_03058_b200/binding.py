@@ -47,8 +47,8 @@ def lib() -> ctypes.CDLL:
         pp = ctypes.POINTER
         L.gnnfd_csr_workspace_bytes.argtypes = [i64, i64, u32, pp(sz), pp(sz)]
         L.gnnfd_build_csr.argtypes = [i64, i64, vp, vp, i32, u32, vp, sz, vp, sz, vp, pp(vp)]
-        L.gnnfd_csr_info.argtypes = [vp, pp(i64), pp(i64), pp(vp), pp(vp), pp(vp), pp(vp), pp(vp), pp(vp), pp(i32)]
-        L.gnnfd_csr_schedule.argtypes = [vp, pp(i64 * 5), pp(vp), pp(i64), pp(vp), pp(vp), pp(vp), pp(vp), pp(vp)]
+        L.gnnfd_csr_info.argtypes = [vp] * 10             # all results are read out of one array: see Csr
+        L.gnnfd_csr_schedule.argtypes = [vp] * 9
         L.gnnfd_csr_destroy.argtypes = [vp]
         L.gnnfd_csr_destroy.restype = None
         L.gnnfd_aggregate_workspace_bytes.argtypes = [vp, i32, pp(sz)]
@@ -97,9 +97,13 @@ def _check(status: int, where: str):
         raise GnnfdError(status, where)
 
 
-def _stream_ptr(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+# The calls on small graphs take the GPU a few microseconds, so what Python does per call counts: raw stream handles
+# instead of Stream objects, plain integers for pointer arguments (the declared argtypes convert them), and no
+# overlap test against an output that the call itself has just allocated.
+def _stream_ptr(stream=None) -> int:
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -112,9 +116,11 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 def _matrix(t: torch.Tensor, cols: int, name: str):
     """(pointer, leading dimension) of a row-major device matrix with at least `cols` columns."""
-    if not t.is_cuda or t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1) or t.shape[1] < cols:
-        raise ValueError("%s must be a 2-D CUDA tensor with unit column stride and >= %d columns" % (name, cols))
-    return ctypes.c_void_p(t.data_ptr()), t.stride(0) if t.shape[0] > 1 else max(t.stride(0), t.shape[1])
+    if t.is_cuda and t.dim() == 2:
+        (rows, width), (pitch, step) = t.shape, t.stride()
+        if width >= cols and (width <= 1 or step == 1):
+            return t.data_ptr(), pitch if rows > 1 else max(pitch, width)
+    raise ValueError("%s must be a 2-D CUDA tensor with unit column stride and >= %d columns" % (name, cols))
 
 
 def _alloc_bytes(nbytes: int, device, stream=None) -> torch.Tensor:
@@ -130,7 +136,7 @@ def _alloc_bytes(nbytes: int, device, stream=None) -> torch.Tensor:
 def _same_device(csr_device, **tensors):
     """Every operand must live on the device the CSR was built on (the library never migrates data)."""
     for name, t in tensors.items():
-        if t is not None and torch.device(t.device) != torch.device(csr_device):
+        if t is not None and t.device != csr_device:
             raise ValueError("%s is on %s but the CSR is on %s" % (name, t.device, csr_device))
 
 
@@ -168,12 +174,24 @@ def _no_overlap(a, b, name_a: str, name_b: str):
     raise ValueError("%s and %s overlap in memory" % (name_a, name_b))
 
 
-def _check_aggregate_operands(csr, x, out, f: int, name_x: str = "x"):
-    """Shape, device and aliasing rules of the aggregation entry points, checked before any launch."""
-    _same_device(csr.device, **{name_x: x, "out": out})
+def _check_aggregate_operands(csr, x, out, f: int, name_x: str = "x", fresh: bool = False):
+    """Shape, device and aliasing rules of the aggregation entry points, checked before any launch; `fresh`: the call
+    itself allocated `out` beside x, with the right shape."""
+    if x.device != csr.device or out.device != csr.device:
+        _same_device(csr.device, **{name_x: x, "out": out})
     _need_rows(x, csr.n, name_x)
-    _need_rows(out, csr.n, "out")
-    _no_overlap(x, out, name_x, "out")
+    if not fresh:
+        _need_rows(out, csr.n, "out")
+        _no_overlap(x, out, name_x, "out")
+
+
+def _scratch_args(scratch, device):
+    """(pointer, bytes) of an optional scratch tensor."""
+    if scratch is None:
+        return None, 0
+    if scratch.device != device:
+        _same_device(device, scratch=scratch)
+    return scratch.data_ptr(), scratch.numel() * scratch.element_size()
 
 
 class Csr:
@@ -183,24 +201,16 @@ class Csr:
         self._h = handle
         self._persistent = persistent
         self.device = device
-        n, nnz, md = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int32()
-        ptrs = [ctypes.c_void_p() for _ in range(6)]
-        _check(lib().gnnfd_csr_info(self._h, ctypes.byref(n), ctypes.byref(nnz), *[ctypes.byref(p) for p in ptrs],
-                                    ctypes.byref(md)), "gnnfd_csr_info")
-        self.n, self.nnz, self.max_degree = n.value, nnz.value, md.value
-        self._ptrs = dict(zip(("row_ptr", "col_idx", "perm", "dinv_sqrt", "rdeg", "edge_weight"),
-                              [p.value for p in ptrs]))
-        bins = (ctypes.c_int64 * 5)()
-        nseg = ctypes.c_int64()
-        sp = [ctypes.c_void_p() for _ in range(6)]
-        _check(lib().gnnfd_csr_schedule(self._h, ctypes.byref(bins), ctypes.byref(sp[0]), ctypes.byref(nseg),
-                                        ctypes.byref(sp[1]), ctypes.byref(sp[2]), ctypes.byref(sp[3]), ctypes.byref(sp[4]),
-                                        ctypes.byref(sp[5])),
-               "gnnfd_csr_schedule")
-        self.bin_count = list(bins)
-        self.n_segments = nseg.value
-        self._ptrs.update(dict(zip(("row_order", "seg_row", "seg_begin", "seg_end", "seg_slot", "hub_seg_ptr"),
-                                   [p.value for p in sp])))
+        # one array of 64-bit words takes every result: n, nnz, max degree, segments, five bin counts, twelve pointers
+        r = (ctypes.c_int64 * 21)()
+        at = [ctypes.addressof(r) + 8 * i for i in range(21)]
+        _check(lib().gnnfd_csr_info(self._h, at[0], at[1], *at[9:15], at[2]), "gnnfd_csr_info")
+        _check(lib().gnnfd_csr_schedule(self._h, at[4], at[15], at[3], *at[16:21]), "gnnfd_csr_schedule")
+        self.n, self.nnz, self.n_segments = r[0], r[1], r[3]
+        self.max_degree = r[2]                     # an int32 in a zeroed little-endian word, never negative
+        self.bin_count = r[4:9]
+        self._ptrs = dict(zip(("row_ptr", "col_idx", "perm", "dinv_sqrt", "rdeg", "edge_weight", "row_order", "seg_row",
+                               "seg_begin", "seg_end", "seg_slot", "hub_seg_ptr"), r[9:21]))
 
     @property
     def handle(self):
@@ -260,11 +270,9 @@ def build_csr(n: int, src: torch.Tensor, dst: torch.Tensor, flags: int = 0, stre
     if scratch is None:
         scratch = _alloc_bytes(sb, src.device)
     handle = ctypes.c_void_p()
-    st = lib().gnnfd_build_csr(n, e, ctypes.c_void_p(src.data_ptr()), ctypes.c_void_p(dst.data_ptr()),
-                               I32 if src.dtype == torch.int32 else I64, flags,
-                               ctypes.c_void_p(persistent.data_ptr()), persistent.numel(),
-                               ctypes.c_void_p(scratch.data_ptr()), scratch.numel(), _stream_ptr(stream),
-                               ctypes.byref(handle))
+    st = lib().gnnfd_build_csr(n, e, src.data_ptr(), dst.data_ptr(), I32 if src.dtype == torch.int32 else I64, flags,
+                               persistent.data_ptr(), persistent.numel(), scratch.data_ptr(), scratch.numel(),
+                               _stream_ptr(stream), ctypes.byref(handle))
     _check(st, "gnnfd_build_csr")
     return Csr(handle, persistent, src.device)
 
@@ -288,20 +296,20 @@ def aggregate_best_workspace_bytes(csr: Csr, x: torch.Tensor, f: int | None = No
 def _aggregate(fn, name, csr: Csr, x, f, chunk_width, out, out_dtype, scratch, stream):
     f = x.shape[1] if f is None else f
     chunk_width = f if chunk_width is None else chunk_width
-    if out is None:
+    fresh = out is None
+    if fresh:
         out = torch.empty((csr.n, f), dtype=out_dtype or torch.float32, device=x.device)
     xp, ldx = _matrix(x, f, "x")
     op, ldo = _matrix(out, f, "out")
-    _check_aggregate_operands(csr, x, out, f)
+    _check_aggregate_operands(csr, x, out, f, fresh=fresh)
+    xdt = _dtype_code(x)
     if scratch is None:
-        need = aggregate_best_workspace_bytes(csr, x, f, chunk_width)
-        if need:
-            scratch = _alloc_bytes(need, x.device, stream)
-    _same_device(csr.device, scratch=scratch)
-    sp = ctypes.c_void_p(scratch.data_ptr()) if scratch is not None else None
-    sn = scratch.numel() * scratch.element_size() if scratch is not None else 0
-    _check(fn(csr.handle, xp, ldx, _dtype_code(x), op, ldo, _dtype_code(out), f, chunk_width, sp, sn,
-              _stream_ptr(stream)), name)
+        need = ctypes.c_size_t()
+        _check(lib().gnnfd_aggregate_best_workspace_bytes(csr.handle, xp, ldx, xdt, f, chunk_width, ctypes.byref(need)), name)
+        if need.value:
+            scratch = _alloc_bytes(need.value, x.device, stream)
+    sp, sn = _scratch_args(scratch, csr.device)
+    _check(fn(csr.handle, xp, ldx, xdt, op, ldo, _dtype_code(out), f, chunk_width, sp, sn, _stream_ptr(stream)), name)
     return out
 
 
@@ -345,9 +353,9 @@ def oneshot(model: str, n: int, src: torch.Tensor, dst: torch.Tensor, x: torch.T
         scratch = _alloc_bytes(oneshot_workspace_bytes(n, src.numel(), flags, f), x.device, stream)
     _same_device(src.device, scratch=scratch)
     fn = {"gcn": lib().gnnfd_oneshot_gcn, "sage": lib().gnnfd_oneshot_sage}[model]
-    _check(fn(n, src.numel(), ctypes.c_void_p(src.data_ptr()), ctypes.c_void_p(dst.data_ptr()),
+    _check(fn(n, src.numel(), src.data_ptr(), dst.data_ptr(),
               I32 if src.dtype == torch.int32 else I64, flags, xp, ldx, _dtype_code(x), op, ldo, _dtype_code(out), f,
-              chunk_width, ctypes.c_void_p(scratch.data_ptr()), scratch.numel() * scratch.element_size(),
+              chunk_width, scratch.data_ptr(), scratch.numel() * scratch.element_size(),
               _stream_ptr(stream)), "gnnfd_oneshot_" + model)
     return out
 
@@ -378,11 +386,11 @@ def oneshot_gat(n: int, src: torch.Tensor, dst: torch.Tensor, z: torch.Tensor, a
                "gnnfd_oneshot_gat_workspace_bytes")
         scratch = _alloc_bytes(need.value, z.device, stream)
     _same_device(src.device, scratch=scratch)
-    _check(lib().gnnfd_oneshot_gat(n, src.numel(), ctypes.c_void_p(src.data_ptr()), ctypes.c_void_p(dst.data_ptr()),
+    _check(lib().gnnfd_oneshot_gat(n, src.numel(), src.data_ptr(), dst.data_ptr(),
                                    I32 if src.dtype == torch.int32 else I64, flags, zp, ldz, _dtype_code(z),
-                                   ctypes.c_void_p(a_src.data_ptr()), ctypes.c_void_p(a_dst.data_ptr()), heads, dim,
+                                   a_src.data_ptr(), a_dst.data_ptr(), heads, dim,
                                    negative_slope, op, ldo, _dtype_code(out), chunk_width,
-                                   ctypes.c_void_p(scratch.data_ptr()), scratch.numel() * scratch.element_size(),
+                                   scratch.data_ptr(), scratch.numel() * scratch.element_size(),
                                    _stream_ptr(stream)), "gnnfd_oneshot_gat")
     return out
 
@@ -410,7 +418,7 @@ def tune_chunk_width(csr: Csr, x: torch.Tensor, model: str = "gcn", f: int | Non
         if need:
             scratch = _alloc_bytes(need, x.device, stream)
     _same_device(csr.device, scratch=scratch)
-    sp = ctypes.c_void_p(scratch.data_ptr()) if scratch is not None else None
+    sp = scratch.data_ptr() if scratch is not None else None
     sn = scratch.numel() * scratch.element_size() if scratch is not None else 0
     arr = (ctypes.c_int32 * len(candidates))(*candidates)
     best, ms = ctypes.c_int32(), ctypes.c_float()
@@ -444,8 +452,10 @@ def _attention_vectors(a_src, a_dst, heads: int, dim: int, device, stream):
     for name, a in (("a_src", a_src), ("a_dst", a_dst)):
         if a.numel() != heads * dim:
             raise ValueError("%s must hold heads*dim = %d values" % (name, heads * dim))
-        if torch.device(a.device) != torch.device(device):
+        if a.device != device:
             raise ValueError("%s is on %s, the features are on %s" % (name, a.device, device))
+    if a_src.dtype == a_dst.dtype == torch.float32 and a_src.is_contiguous() and a_dst.is_contiguous():
+        return a_src, a_dst
     if stream is None:
         return a_src.contiguous().float(), a_dst.contiguous().float()
     with torch.cuda.stream(stream):
@@ -458,9 +468,9 @@ def gat_scores(z: torch.Tensor, a_src: torch.Tensor, a_dst: torch.Tensor, heads:
     a_src, a_dst = _attention_vectors(a_src, a_dst, heads, dim, z.device, stream)
     s_src = torch.empty((n, heads), dtype=torch.float32, device=z.device)
     s_dst = torch.empty((n, heads), dtype=torch.float32, device=z.device)
-    _check(lib().gnnfd_gat_scores(n, zp, ldz, _dtype_code(z), ctypes.c_void_p(a_src.data_ptr()),
-                                  ctypes.c_void_p(a_dst.data_ptr()), heads, dim, ctypes.c_void_p(s_src.data_ptr()),
-                                  ctypes.c_void_p(s_dst.data_ptr()), _stream_ptr(stream)), "gnnfd_gat_scores")
+    _check(lib().gnnfd_gat_scores(n, zp, ldz, _dtype_code(z), a_src.data_ptr(),
+                                  a_dst.data_ptr(), heads, dim, s_src.data_ptr(),
+                                  s_dst.data_ptr(), _stream_ptr(stream)), "gnnfd_gat_scores")
     return s_src, s_dst
 
 
@@ -475,18 +485,19 @@ def aggregate_gat(csr: Csr, z: torch.Tensor, a_src: torch.Tensor, a_dst: torch.T
                   out_dtype=None, scratch=None, stream=None) -> torch.Tensor:
     f = heads * dim
     chunk_width = f if chunk_width is None else chunk_width
-    if out is None:
+    fresh = out is None
+    if fresh:
         out = torch.empty((csr.n, f), dtype=out_dtype or torch.float32, device=z.device)
     zp, ldz = _matrix(z, f, "z")
     op, ldo = _matrix(out, f, "out")
-    _check_aggregate_operands(csr, z, out, f, "z")
+    _check_aggregate_operands(csr, z, out, f, "z", fresh)
     a_src, a_dst = _attention_vectors(a_src, a_dst, heads, dim, z.device, stream)
     if scratch is None:
         scratch = _alloc_bytes(gat_workspace_bytes(csr, heads, dim), z.device, stream)
     _same_device(csr.device, scratch=scratch)
-    _check(lib().gnnfd_aggregate_gat(csr.handle, zp, ldz, _dtype_code(z), ctypes.c_void_p(a_src.data_ptr()),
-                                     ctypes.c_void_p(a_dst.data_ptr()), heads, dim, negative_slope, op, ldo,
-                                     _dtype_code(out), chunk_width, ctypes.c_void_p(scratch.data_ptr()),
+    _check(lib().gnnfd_aggregate_gat(csr.handle, zp, ldz, _dtype_code(z), a_src.data_ptr(),
+                                     a_dst.data_ptr(), heads, dim, negative_slope, op, ldo,
+                                     _dtype_code(out), chunk_width, scratch.data_ptr(),
                                      scratch.numel() * scratch.element_size(), _stream_ptr(stream)),
            "gnnfd_aggregate_gat")
     return out
@@ -508,20 +519,22 @@ def edge_softmax(csr: Csr, s_src: torch.Tensor, s_dst: torch.Tensor, negative_sl
         raise TypeError("scores must be float32 [n, heads]")
     if s_src.dim() != 2 or s_src.shape[0] != csr.n:
         raise ValueError("scores must be [n, heads] with n = %d rows, got %s" % (csr.n, tuple(s_src.shape)))
-    if out is None:
+    fresh = out is None
+    if fresh:
         out = torch.empty((csr.nnz, heads), dtype=torch.float32, device=s_src.device)
     if out.dtype != torch.float32 or out.dim() != 2 or not out.is_contiguous() or out.shape[1] != heads \
             or out.shape[0] < csr.nnz:
         raise ValueError("alpha must be a contiguous float32 [nnz >= %d, heads = %d] tensor" % (csr.nnz, heads))
     _same_device(csr.device, s_src=s_src, s_dst=s_dst, alpha=out)
-    _no_overlap(s_src, out, "s_src", "alpha")
-    _no_overlap(s_dst, out, "s_dst", "alpha")
+    if not fresh:
+        _no_overlap(s_src, out, "s_src", "alpha")
+        _no_overlap(s_dst, out, "s_dst", "alpha")
     if scratch is None:
         scratch = _alloc_bytes(edge_softmax_workspace_bytes(csr, heads), s_src.device, stream)
     _same_device(csr.device, scratch=scratch)
-    _check(lib().gnnfd_edge_softmax(csr.handle, ctypes.c_void_p(s_src.data_ptr()), ctypes.c_void_p(s_dst.data_ptr()),
-                                    heads, negative_slope, ctypes.c_void_p(out.data_ptr()),
-                                    ctypes.c_void_p(scratch.data_ptr()), scratch.numel() * scratch.element_size(),
+    _check(lib().gnnfd_edge_softmax(csr.handle, s_src.data_ptr(), s_dst.data_ptr(),
+                                    heads, negative_slope, out.data_ptr(),
+                                    scratch.data_ptr(), scratch.numel() * scratch.element_size(),
                                     _stream_ptr(stream)),
            "gnnfd_edge_softmax")
     return out
@@ -547,16 +560,18 @@ def combine(x: torch.Tensor, w_t: torch.Tensor, f_in: int | None = None, out: to
     f_out = w_t.shape[0]
     if x.dtype != w_t.dtype:
         raise TypeError("x and w_t must have the same dtype")
-    if out is None:
+    fresh = out is None
+    if fresh:
         out = torch.empty((x.shape[0], f_out), dtype=out_dtype or torch.float32, device=x.device)
     xp, ldx = _matrix(x, f_in, "x")
     wp, ldw = _matrix(w_t, f_in, "w_t")
     op, ldo = _matrix(out, f_out, "out")
     _same_device(x.device, w_t=w_t, out=out, status=status)
     _need_rows(out, x.shape[0], "out")
-    _no_overlap(x, out, "x", "out")
-    _no_overlap(w_t, out, "w_t", "out")
-    sp = ctypes.c_void_p(status.data_ptr()) if status is not None else None
+    if not fresh:
+        _no_overlap(x, out, "x", "out")
+        _no_overlap(w_t, out, "w_t", "out")
+    sp = status.data_ptr() if status is not None else None
     scores = a_src is not None or a_dst is not None
     s_src = s_dst = None
     asp = adp = ssp = sdp = None
@@ -564,8 +579,8 @@ def combine(x: torch.Tensor, w_t: torch.Tensor, f_in: int | None = None, out: to
         a_src, a_dst = _attention_vectors(a_src, a_dst, heads, dim, x.device, stream)
         s_src = torch.empty((x.shape[0], heads), dtype=torch.float32, device=x.device)
         s_dst = torch.empty((x.shape[0], heads), dtype=torch.float32, device=x.device)
-        asp, adp = ctypes.c_void_p(a_src.data_ptr()), ctypes.c_void_p(a_dst.data_ptr())
-        ssp, sdp = ctypes.c_void_p(s_src.data_ptr()), ctypes.c_void_p(s_dst.data_ptr())
+        asp, adp = a_src.data_ptr(), a_dst.data_ptr()
+        ssp, sdp = s_src.data_ptr(), s_dst.data_ptr()
     _check(lib().gnnfd_combine_ex(x.shape[0], xp, ldx, _dtype_code(x), f_in, wp, ldw, f_out, op, ldo, _dtype_code(out),
                                   _combine_mode(mode), asp, adp, heads, dim, ssp, sdp, sp, _stream_ptr(stream)),
            "gnnfd_combine_ex")
@@ -592,7 +607,8 @@ def layer(csr: Csr, model: str, x: torch.Tensor, w_t: torch.Tensor, f_in: int | 
     if model == "gat" and heads * dim != f_out:
         raise ValueError("heads * dim must equal the number of rows of w_t")
     chunk_width = f_out if chunk_width is None else chunk_width
-    if out is None:
+    fresh = out is None
+    if fresh:
         out = torch.empty((csr.n, f_out), dtype=out_dtype or torch.float32, device=x.device)
     xp, ldx = _matrix(x, f_in, "x")
     wp, ldw = _matrix(w_t, f_in, "w_t")
@@ -600,17 +616,18 @@ def layer(csr: Csr, model: str, x: torch.Tensor, w_t: torch.Tensor, f_in: int | 
     _same_device(csr.device, x=x, w_t=w_t, out=out, status=status)
     _need_rows(x, csr.n, "x")
     _need_rows(out, csr.n, "out")
-    _no_overlap(x, out, "x", "out")
-    _no_overlap(w_t, out, "w_t", "out")
+    if not fresh:
+        _no_overlap(x, out, "x", "out")
+        _no_overlap(w_t, out, "w_t", "out")
     if scratch is None:
         scratch = _alloc_bytes(layer_workspace_bytes(csr, model, f_out, heads, dim, x.dtype), x.device, stream)
     _same_device(csr.device, scratch=scratch)
-    sp = ctypes.c_void_p(status.data_ptr()) if status is not None else None
-    scr, scr_n = ctypes.c_void_p(scratch.data_ptr()), scratch.numel() * scratch.element_size()
+    sp = status.data_ptr() if status is not None else None
+    scr, scr_n = scratch.data_ptr(), scratch.numel() * scratch.element_size()
     if model == "gat":
         a_src, a_dst = _attention_vectors(a_src, a_dst, heads, dim, x.device, stream)
         _check(lib().gnnfd_layer_gat(csr.handle, xp, ldx, _dtype_code(x), f_in, wp, ldw, heads, dim,
-                                     ctypes.c_void_p(a_src.data_ptr()), ctypes.c_void_p(a_dst.data_ptr()), negative_slope,
+                                     a_src.data_ptr(), a_dst.data_ptr(), negative_slope,
                                      _combine_mode(mode), op, ldo, _dtype_code(out), chunk_width, scr, scr_n, sp,
                                      _stream_ptr(stream)), "gnnfd_layer_gat")
     else:
