@@ -36,10 +36,6 @@ struct GatArgs {
     Range range[kMaxRanges];
 };
 
-__device__ __forceinline__ float widen(float x) { return x; }
-__device__ __forceinline__ float widen(__nv_bfloat16 x) { return __bfloat162float(x); }
-
-
 constexpr float kLog2e = 1.4426950408889634f;
 
 // 2^x by the hardware approximation (2 ulp; results below 2^-126 become 0, 2^-inf = 0)
@@ -58,21 +54,29 @@ __device__ __forceinline__ float merge_scale(float m, float m_new)
 
 // ------------------------------------------------------------------ scores
 
-template <typename T>
+// One thread per vertex and head, elements in ascending order.  With VECN > 1 the head's elements come in 16-byte vectors
+// (a head is a whole number of them and starts on a 16-byte boundary): the element-wise form left half of every sector
+// it touched to a later instruction (25 us for [200,000, 8 x 8] fp32, 51 MB).
+template <typename T, int VECN>
 __global__ void __launch_bounds__(kBlock)
 gat_scores(const T* __restrict__ z, int64_t ldz, const float* __restrict__ a_src, const float* __restrict__ a_dst,
            int64_t n, int heads, int dim, float* __restrict__ s_src, float* __restrict__ s_dst)
 {
     const int64_t idx = (int64_t)blockIdx.x * kBlock + threadIdx.x;
     if (idx >= n * heads) return;
-    const int64_t v = idx / heads;
-    const int h = (int)(idx % heads);
+    const int64_t v = idx <= 0x7fffffffll ? (int64_t)((uint32_t)idx / (uint32_t)heads) : idx / heads;
+    const int h = (int)(idx - v * heads);
     const T* zr = z + v * ldz + (int64_t)h * dim;
+    const float *as = a_src + h * dim, *ad = a_dst + h * dim;
     float ss = 0.f, sd = 0.f;
-    for (int d = 0; d < dim; ++d) {
-        const float zv = widen(zr[d]);
-        ss = fmaf(__ldg(a_src + h * dim + d), zv, ss);
-        sd = fmaf(__ldg(a_dst + h * dim + d), zv, sd);
+    for (int d = 0; d < dim; d += VECN) {
+        Vec<T, VECN> zv;
+        zv.load(zr + d);
+#pragma unroll
+        for (int i = 0; i < VECN; ++i) {
+            ss = fmaf(__ldg(as + d + i), zv.get(i), ss);
+            sd = fmaf(__ldg(ad + d + i), zv.get(i), sd);
+        }
     }
     s_src[idx] = ss;
     s_dst[idx] = sd;
@@ -84,10 +88,16 @@ constexpr int kLoads = 8;      // 16-byte feature loads kept in flight per lane
 
 constexpr int kStageSlots = kLoads * 32;      // column indices a warp stages per batch, at most
 
+// Bound by instruction issue once the graph fills the chip (an entry costs a logit, an exponential and the unpacking of
+// its features on top of the gather), so products and rescalings go two to an instruction: on 200,000 rows of
+// 150 entries 8 heads of 16 bf16 columns 0.96 -> 0.89 ms, 8 x 8 bf16 0.54 -> 0.48, fp32 unchanged.  On smaller graphs the
+// longest row decided; shared by warps (see schedule.cuh) 4,000 rows of 10 entries, 8 x 16 fp32, take 23 us
+// instead of 71, 20,000 of 50 64 instead of 155, 100,000 of 20 146 instead of 221.
+//
 // One row (or hub segment) per S = LPR * EP lanes, same batching as the GCN / SAGE gather: the S lanes
 // fetch S column indices per round with one coalesced load and stage them in shared memory.  A lane
 // covers VPL adjacent vectors, all inside one head, so it needs one logit per entry.
-template <typename T, int VECN, int LPR, int VPL, int EP>
+template <typename T, int VECN, int LPR, int VPL, bool SHARED, int EP>
 __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int block_in_range, int col0, int chunk_end,
                                          int32_t (*stage_col)[kBlock / 32][kStageSlots], float (*tot_s)[kBlock])
 {
@@ -99,7 +109,9 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
     constexpr int EPB = R * S;
     constexpr unsigned kFull = 0xffffffffu;
     const int tid = threadIdx.x;
-    const int slot = block_in_range * ROWS + tid / S;
+    // a long row may be shared by several warps of the block, which take consecutive parts of it
+    const int warps_log2 = SHARED && S == 32 ? rg.warps_log2 : 0, sharer = tid / S & ((1 << warps_log2) - 1);
+    const int slot = block_in_range * (ROWS >> warps_log2) + (tid / S >> warps_log2);
     const int sl = tid % S;
     const int g = sl / LPR;
     const int c = sl % LPR;
@@ -129,6 +141,11 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
             b = a.row_ptr[row];
             e = a.row_ptr[row + 1];
         }
+    }
+    if (SHARED && S == 32 && warps_log2 > 0) {
+        const int32_t share = ((e - b) >> warps_log2) + 1;
+        b = min(b + sharer * share, e);
+        e = min(b + share, e);
     }
     // one 32-byte load per entry when both vectors of the lane exist and every row start allows it
     const bool wide = a.wide_ok && okq[VPL - 1];
@@ -235,7 +252,10 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
 #pragma unroll
                     for (int q = 0; q < VPL; ++q)
 #pragma unroll
-                        for (int i = 0; i < VECN; ++i) acc[q][i] *= rescale;
+                        for (int i = 0; i < VECN; i += VECN > 1 ? 2 : 1) {
+                            if constexpr (VECN > 1) mul_pair(acc[q][i], acc[q][i + 1], rescale);
+                            else acc[q][i] *= rescale;
+                        }
                 }
 #pragma unroll
                 for (int i = 0; i < UB; ++i) {
@@ -246,7 +266,10 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
 #pragma unroll
                     for (int q = 0; q < VPL; ++q)
 #pragma unroll
-                        for (int k = 0; k < VECN; ++k) acc[q][k] = fmaf(p, v[i][q].get(k), acc[q][k]);
+                        for (int k = 0; k < VECN; k += VECN > 1 ? 2 : 1) {
+                            if constexpr (VECN > 1) fma_pair(acc[q][k], acc[q][k + 1], p, v[i][q].get(k), v[i][q].get(k + 1));
+                            else acc[q][k] = fmaf(p, v[i][q].get(k), acc[q][k]);
+                        }
                 }
             }
         };
@@ -283,6 +306,27 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
         m = mn;
     }
 
+    if (SHARED && S == 32 && warps_log2 > 0) {      // the sharers' results, first to last; the whole block is on this side
+        constexpr int L = VPL * VECN, M = L + 1;
+        if (sharer > 0) {
+#pragma unroll
+            for (int k = 0; k < L; ++k) tot_s[k][tid] = acc[k / VECN][k % VECN];
+            tot_s[L][tid] = l;
+            tot_s[M][tid] = m;
+        }
+        __syncthreads();
+        if (sharer > 0) return;
+        for (int w = 1; w < 1 << warps_log2; ++w) {
+            const int other = tid + 32 * w;
+            const float m2 = tot_s[M][other], mn = fmaxf(m, m2);
+            const float sa = merge_scale(m, mn), sb = merge_scale(m2, mn);
+            l = l * sa + tot_s[L][other] * sb;
+#pragma unroll
+            for (int k = 0; k < L; ++k) acc[k / VECN][k % VECN] = acc[k / VECN][k % VECN] * sa + tot_s[k][other] * sb;
+            m = mn;
+        }
+    }
+
     if (!active || g != 0 || !lane_ok) return;
     // where a hub segment's partial results go (read here, at the end, so that it occupies no register during the walk)
     const int32_t part = rg.hub ? a.seg_slot[slot] : 0;
@@ -314,14 +358,15 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
     }
 }
 
-template <typename T, int VECN, int LPR, int VPL>
+template <typename T, int VECN, int LPR, int VPL, bool SHARED>
 // Register budget: left to itself the compiler gives the wide instantiations anything between 80 and 126
 // registers from one build to the next (two blocks per SM instead of three, 20 % slower); three blocks per SM for
 // the vector-pair forms and four for the others is what the measured-good builds had.
 __global__ void __launch_bounds__(kBlock, (VPL == 2 && VECN > 1) ? 3 : 4) gat_aggregate(const __grid_constant__ GatArgs a)
 {
     __shared__ int32_t stage_col[2][kBlock / 32][kStageSlots];
-    __shared__ float tot_s[VPL * VECN + 1][kBlock];        // second-level sums and denominator, one column per thread
+    // second-level sums and denominator (and a sharer's maximum), one column per thread
+    __shared__ float tot_s[VPL * VECN + 1 + SHARED][kBlock];
     // grid: x = (block of the sweep, column tile), y = chunk; blocks are issued x first, so the sweeps follow each
     // other chunk by chunk.  (The chunk used to be divided out of a linear 64-bit block number: two 64-bit
     // divisions per thread, more instructions than a short row's whole walk.)
@@ -335,17 +380,17 @@ __global__ void __launch_bounds__(kBlock, (VPL == 2 && VECN > 1) ? 3 : 4) gat_ag
     if (col0 >= chunk_end) return;
     int r = 0;
 #pragma unroll
-    for (int i = 1; i < kMaxRanges; ++i)
+    for (int i = 1; i < (SHARED ? kMaxRanges : kNumBins); ++i)      // unsplit, the fourth class is one range
         if (i < a.n_ranges && rb >= a.range[i].first_block) r = i;
     const Range rg = a.range[r];
     const int bir = rb - rg.first_block;
     switch (rg.ep_log2) {
-        case 0: gat_rows<T, VECN, LPR, VPL, 1>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
-        case 1: if constexpr (LPR * 2 <= 32) gat_rows<T, VECN, LPR, VPL, 2>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
-        case 2: if constexpr (LPR * 4 <= 32) gat_rows<T, VECN, LPR, VPL, 4>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
-        case 3: if constexpr (LPR * 8 <= 32) gat_rows<T, VECN, LPR, VPL, 8>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
-        case 4: if constexpr (LPR * 16 <= 32) gat_rows<T, VECN, LPR, VPL, 16>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
-        default: if constexpr (LPR == 1) gat_rows<T, VECN, LPR, VPL, 32>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
+        case 0: gat_rows<T, VECN, LPR, VPL, SHARED, 1>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
+        case 1: if constexpr (LPR * 2 <= 32) gat_rows<T, VECN, LPR, VPL, SHARED, 2>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
+        case 2: if constexpr (LPR * 4 <= 32) gat_rows<T, VECN, LPR, VPL, SHARED, 4>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
+        case 3: if constexpr (LPR * 8 <= 32) gat_rows<T, VECN, LPR, VPL, SHARED, 8>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
+        case 4: if constexpr (LPR * 16 <= 32) gat_rows<T, VECN, LPR, VPL, SHARED, 16>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
+        default: if constexpr (LPR == 1) gat_rows<T, VECN, LPR, VPL, SHARED, 32>(a, rg, bir, col0, chunk_end, stage_col, tot_s); break;
     }
 }
 
@@ -404,23 +449,24 @@ gat_hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict_
 
 typedef void (*GatKernel)(const GatArgs);
 
-template <typename T, int VECN, int VPL>
+template <typename T, int VECN, int VPL, bool SHARED>
 static GatKernel pick_lpr(int lpr)
 {
     switch (lpr) {
-        case 1: return gat_aggregate<T, VECN, 1, VPL>;
-        case 2: return gat_aggregate<T, VECN, 2, VPL>;
-        case 4: return gat_aggregate<T, VECN, 4, VPL>;
-        case 8: return gat_aggregate<T, VECN, 8, VPL>;
-        case 16: return gat_aggregate<T, VECN, 16, VPL>;
-        default: return gat_aggregate<T, VECN, 32, VPL>;
+        case 1: return gat_aggregate<T, VECN, 1, VPL, SHARED>;
+        case 2: return gat_aggregate<T, VECN, 2, VPL, SHARED>;
+        case 4: return gat_aggregate<T, VECN, 4, VPL, SHARED>;
+        case 8: return gat_aggregate<T, VECN, 8, VPL, SHARED>;
+        case 16: return gat_aggregate<T, VECN, 16, VPL, SHARED>;
+        default: return gat_aggregate<T, VECN, 32, VPL, SHARED>;
     }
 }
 
 template <typename T, int VECN>
-static GatKernel pick_vpl(int lpr, int vpl)
+static GatKernel pick_vpl(int lpr, int vpl, bool shared)
 {
-    return vpl == 2 ? pick_lpr<T, VECN, 2>(lpr) : pick_lpr<T, VECN, 1>(lpr);
+    if (shared) return vpl == 2 ? pick_lpr<T, VECN, 2, true>(lpr) : pick_lpr<T, VECN, 1, true>(lpr);
+    return vpl == 2 ? pick_lpr<T, VECN, 2, false>(lpr) : pick_lpr<T, VECN, 1, false>(lpr);
 }
 
 struct GatScratch {
@@ -441,12 +487,17 @@ static int launch_scores(int64_t n, const void* d_z, int64_t ldz, gnnfd_dtype_t 
 {
     const int64_t total = n * heads;
     const unsigned grid = (unsigned)((total + kBlock - 1) / kBlock);
-    if (zdt == GNNFD_F32)
-        GNNFD_LAUNCH("gat_scores", s, gat_scores<float>, grid, kBlock, 0, static_cast<const float*>(d_z), ldz, d_a_src,
-                     d_a_dst, n, heads, dim, d_s_src, d_s_dst);
-    else
-        GNNFD_LAUNCH("gat_scores", s, gat_scores<__nv_bfloat16>, grid, kBlock, 0, static_cast<const __nv_bfloat16*>(d_z),
-                     ldz, d_a_src, d_a_dst, n, heads, dim, d_s_src, d_s_dst);
+    const int zsize = zdt == GNNFD_F32 ? 4 : 2;
+    const bool vec = (uintptr_t)d_z % 16 == 0 && ldz * zsize % 16 == 0 && dim * zsize % 16 == 0;
+    if (zdt == GNNFD_F32) {
+        const float* z = static_cast<const float*>(d_z);
+        GNNFD_LAUNCH("gat_scores", s, (vec ? gat_scores<float, 4> : gat_scores<float, 1>), grid, kBlock, 0, z, ldz, d_a_src, d_a_dst,
+                     n, heads, dim, d_s_src, d_s_dst);
+    } else {
+        const __nv_bfloat16* z = static_cast<const __nv_bfloat16*>(d_z);
+        GNNFD_LAUNCH("gat_scores", s, (vec ? gat_scores<__nv_bfloat16, 8> : gat_scores<__nv_bfloat16, 1>), grid, kBlock, 0, z, ldz,
+                     d_a_src, d_a_dst, n, heads, dim, d_s_src, d_s_dst);
+    }
     GNNFD_CUDA_CHECK(cudaGetLastError());
     return GNNFD_OK;
 }
@@ -502,14 +553,18 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
     a.wide_ok = vec && vpl == 2 && ((uintptr_t)d_z % 32 == 0) && ((ldz * zsize) % 32 == 0) &&
                 (n_chunks == 1 || (cw * zsize) % 32 == 0);
 
-    const int64_t blocks = plan_ranges(csr, lpr, 1, 0, a.range, &a.n_ranges);
+    const int per_step = kLoads / vpl * (32 / lpr);
+    const int64_t limit = walk_limit(csr, per_step, (int64_t)n_chunks * a.n_ctiles);
+    const int64_t blocks = plan_ranges(csr, lpr, per_step, limit, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;
     if (grid_x > 0x7fffffffll) return GNNFD_TOO_LARGE;
     if (grid_x > 0) {
+        bool shared = false;
+        for (int i = 0; i < a.n_ranges; ++i) shared = shared || a.range[i].warps_log2 > 0;
         GatKernel kernel;
-        if (zdt == GNNFD_F32) kernel = vec ? pick_vpl<float, 4>(lpr, vpl) : pick_vpl<float, 1>(lpr, vpl);
-        else kernel = vec ? pick_vpl<__nv_bfloat16, 8>(lpr, vpl) : pick_vpl<__nv_bfloat16, 1>(lpr, vpl);
+        if (zdt == GNNFD_F32) kernel = vec ? pick_vpl<float, 4>(lpr, vpl, shared) : pick_vpl<float, 1>(lpr, vpl, shared);
+        else kernel = vec ? pick_vpl<__nv_bfloat16, 8>(lpr, vpl, shared) : pick_vpl<__nv_bfloat16, 1>(lpr, vpl, shared);
         for (int c0 = 0; c0 < n_chunks; c0 += kMaxGridY) {
             a.chunk_base = c0;
             const dim3 grid((unsigned)grid_x, (unsigned)(n_chunks - c0 < kMaxGridY ? n_chunks - c0 : kMaxGridY));
