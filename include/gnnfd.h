@@ -270,6 +270,11 @@ int gnnfd_gat_scores(int64_t n, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt,
  * Concat by writing each chunk into its own output columns. */
 int gnnfd_gat_workspace_bytes(const gnnfd_csr_t* csr, int32_t heads, int32_t dim, size_t* scratch_bytes);
 
+/* As gnnfd_aggregate_best_workspace_bytes: with this much scratch gnnfd_aggregate_gat can gather from a copy of z whose heads are
+ * padded to whole 16-byte vectors, where they are not and it is faster. */
+int gnnfd_gat_best_workspace_bytes(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads,
+                                   int32_t dim, int32_t chunk_width, size_t* scratch_bytes);
+
 int gnnfd_aggregate_gat(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt,
                         const float* d_a_src, const float* d_a_dst, int32_t heads, int32_t dim,
                         float negative_slope, void* d_out, int64_t ldo, gnnfd_dtype_t odt,

@@ -69,6 +69,7 @@ def lib() -> ctypes.CDLL:
                                              vp, sz, vp, pp(i32), pp(fl)]
         L.gnnfd_gat_scores.argtypes = [i64, vp, i64, i32, vp, vp, i32, i32, vp, vp, vp]
         L.gnnfd_gat_workspace_bytes.argtypes = [vp, i32, i32, pp(sz)]
+        L.gnnfd_gat_best_workspace_bytes.argtypes = [vp, vp, i64, i32, i32, i32, i32, pp(sz)]
         L.gnnfd_aggregate_gat.argtypes = [vp, vp, i64, i32, vp, vp, i32, i32, fl, vp, i64, i32, i32, vp, sz, vp]
         L.gnnfd_edge_softmax_workspace_bytes.argtypes = [vp, i32, pp(sz)]
         L.gnnfd_edge_softmax.argtypes = [vp, vp, vp, i32, fl, vp, vp, sz, vp]
@@ -493,7 +494,10 @@ def aggregate_gat(csr: Csr, z: torch.Tensor, a_src: torch.Tensor, a_dst: torch.T
     _check_aggregate_operands(csr, z, out, f, "z", fresh)
     a_src, a_dst = _attention_vectors(a_src, a_dst, heads, dim, z.device, stream)
     if scratch is None:
-        scratch = _alloc_bytes(gat_workspace_bytes(csr, heads, dim), z.device, stream)
+        need = ctypes.c_size_t()
+        _check(lib().gnnfd_gat_best_workspace_bytes(csr.handle, zp, ldz, _dtype_code(z), heads, dim, chunk_width,
+                                                    ctypes.byref(need)), "gnnfd_aggregate_gat")
+        scratch = _alloc_bytes(need.value, z.device, stream)
     _same_device(csr.device, scratch=scratch)
     _check(lib().gnnfd_aggregate_gat(csr.handle, zp, ldz, _dtype_code(z), a_src.data_ptr(),
                                      a_dst.data_ptr(), heads, dim, negative_slope, op, ldo,

@@ -407,7 +407,7 @@ align_features(const T* __restrict__ x, int64_t ldx, int64_t n, int32_t f, int32
     if (row >= n) return;
     const int32_t at = (int32_t)(idx - row * vectors) * VECN;
     const int32_t chunk = at / pitch, in_chunk = at - chunk * pitch, j = chunk * cw + in_chunk;
-    const int32_t count = min(f - j, cw - in_chunk);
+    const int32_t count = min(f - j, cw - in_chunk);       // none in the padding
     const T* p = x + row * ldx + j;
     union { T e[VECN]; uint4 v; } u;
     u.v = make_uint4(0u, 0u, 0u, 0u);
@@ -417,11 +417,35 @@ align_features(const T* __restrict__ x, int64_t ldx, int64_t n, int32_t f, int32
     out[idx] = u.v;
 }
 
-struct AlignedCopy {
-    int32_t pitch;       // columns from one chunk's start to the next one's
-    int64_t ld;          // row pitch
-    size_t bytes;        // 0: no copy
-};
+// Each row has to be gathered a few times, and the launch has to be won back.  fp32 GCN, element-wise loads -> copy and vector loads:
+// 100,000 rows of 4 entries and a loop, 41 columns 65 -> 37 us; 41 columns, 33 MB gathered, 17.8 -> 19.7 us; 100 columns, 56 MB,
+// 34 -> 29 us.
+bool copy_pays(const gnnfd_csr_t* csr, int64_t gathered_bytes)
+{
+    return csr->nnz >= 4 * csr->n && gathered_bytes >= (int64_t)40 << 20;
+}
+
+AlignedCopy layout_copy(int64_t n, gnnfd_dtype_t xdt, int32_t f, int32_t cw, int32_t unit_bytes)
+{
+    const int xsize = xdt == GNNFD_F32 ? 4 : 2, unit = unit_bytes / xsize, sector = 32 / xsize;
+    const int64_t pitch = ((int64_t)cw + unit - 1) / unit * unit;
+    const int64_t ld = ((f - 1) / cw * pitch + ((f - 1) % cw + unit) / unit * unit + sector - 1) / sector * sector;
+    if (ld > 0x7fffffffll || n * ld > 0x7fffffffll * kBlock) return AlignedCopy{cw, f, 0};
+    return AlignedCopy{(int32_t)pitch, ld, align_up((size_t)n * ld * xsize, 256)};
+}
+
+void launch_copy(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int64_t n, int32_t f, int32_t cw, const AlignedCopy& copy,
+                 void* d_aligned, cudaStream_t s)
+{
+    const int vecn = xdt == GNNFD_F32 ? 4 : 8;
+    const unsigned grid = (unsigned)((n * (copy.ld / vecn) + kBlock - 1) / kBlock);
+    if (xdt == GNNFD_F32)
+        GNNFD_LAUNCH("align_features", s, align_features<float>, grid, kBlock, 0, static_cast<const float*>(d_x), ldx, n, f, cw,
+                     copy.pitch, (uint32_t)copy.ld, static_cast<uint4*>(d_aligned));
+    else
+        GNNFD_LAUNCH("align_features", s, align_features<__nv_bfloat16>, grid, kBlock, 0, static_cast<const __nv_bfloat16*>(d_x),
+                     ldx, n, f, cw, copy.pitch, (uint32_t)copy.ld, static_cast<uint4*>(d_aligned));
+}
 
 static bool aligned_for_vectors(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f, int32_t cw)
 {
@@ -429,25 +453,15 @@ static bool aligned_for_vectors(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt,
     return ((uintptr_t)d_x % 16 == 0) && ((ldx * xsize) % 16 == 0) && (f <= cw || (cw * xsize) % 16 == 0);
 }
 
-// When the copy pays, element-wise loads against copy and vector loads.  bf16 always gains from vectors, fp32 from
-// where the scalar kernel needs a whole warp for 64 columns (33 up): 200,000 rows of 150 entries, 25 / 41 / 301 fp32
-// columns 0.45 / 0.67 / 4.69 -> 0.49 / 0.56 / 3.34 ms, 9 / 41 / 301 bf16 columns 0.40 / 0.73 / 3.91 -> 0.24 / 0.50 /
-// 1.95 ms.  Each row has to be gathered a few times (100,000 rows of 4 and a loop, 41 fp32 columns 65 -> 37 us), and the
-// launch has to be won back: 41 fp32 columns, 33 MB gathered, 17.8 -> 19.7 us; 100 columns, 56 MB, 34 -> 29 us.
+// bf16 always gains from vectors, fp32 from where the scalar kernel needs a whole warp for 64 columns (33 up): 200,000 rows of
+// 150 entries, 25 / 41 / 301 fp32 columns 0.45 / 0.67 / 4.69 -> 0.49 / 0.56 / 3.34 ms, 9 / 41 / 301 bf16 columns 0.40 / 0.73 /
+// 3.91 -> 0.24 / 0.50 / 1.95 ms.
 static AlignedCopy plan_copy(const gnnfd_csr_t* csr, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f, int32_t cw)
 {
-    const int xsize = xdt == GNNFD_F32 ? 4 : 2, unit = 32 / xsize;          // rows and chunks start on 32-byte sectors
-    AlignedCopy c{cw, ldx, 0};
-    if (aligned_for_vectors(d_x, ldx, xdt, f, cw)) return c;
-    if (xsize == 4 && cw <= 32) return c;
-    if (csr->nnz < 4 * csr->n || csr->nnz * f * xsize < (int64_t)40 << 20) return c;
-    const int64_t pitch = ((int64_t)cw + unit - 1) / unit * unit;
-    const int64_t ld = (f - 1) / cw * pitch + ((f - 1) % cw + unit) / unit * unit;
-    if (ld > 0x7fffffffll || csr->n * ld > 0x7fffffffll * kBlock) return c;
-    c.pitch = (int32_t)pitch;
-    c.ld = ld;
-    c.bytes = align_up((size_t)csr->n * ld * xsize, 256);
-    return c;
+    const int xsize = xdt == GNNFD_F32 ? 4 : 2;
+    if (aligned_for_vectors(d_x, ldx, xdt, f, cw) || (xsize == 4 && cw <= 32) || !copy_pays(csr, csr->nnz * f * xsize))
+        return AlignedCopy{cw, ldx, 0};
+    return layout_copy(csr->n, xdt, f, cw, 32);               // chunks start on 32-byte sectors
 }
 
 static size_t partial_bytes(const gnnfd_csr_t* csr, int32_t f)
@@ -477,14 +491,8 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     const bool copied = copy.bytes > 0 && d_scratch && ((uintptr_t)d_scratch & 15u) == 0 && scratch_bytes >= need + copy.bytes;
     int32_t x_gap = 0;
     if (copied) {
-        uint4* aligned = reinterpret_cast<uint4*>(static_cast<char*>(d_scratch) + need);
-        const unsigned grid = (unsigned)((csr->n * (copy.ld / vecn) + kBlock - 1) / kBlock);
-        if (xdt == GNNFD_F32)
-            GNNFD_LAUNCH("align_features", s, align_features<float>, grid, kBlock, 0, static_cast<const float*>(d_x), ldx, csr->n,
-                         f, cw, copy.pitch, (uint32_t)copy.ld, aligned);
-        else
-            GNNFD_LAUNCH("align_features", s, align_features<__nv_bfloat16>, grid, kBlock, 0,
-                         static_cast<const __nv_bfloat16*>(d_x), ldx, csr->n, f, cw, copy.pitch, (uint32_t)copy.ld, aligned);
+        void* aligned = static_cast<char*>(d_scratch) + need;
+        launch_copy(d_x, ldx, xdt, csr->n, f, cw, copy, aligned, s);
         d_x = aligned;
         ldx = copy.ld;
         x_gap = copy.pitch - cw;

@@ -86,6 +86,18 @@ struct Carver {
 size_t scan_temp_ints(size_t count);
 int exclusive_scan_i32(const int32_t* d_in, int32_t* d_out, size_t count, int32_t* d_temp, cudaStream_t s);
 
+// ---- aligned copies of features (aggregate.cu): chunks of cw columns placed `pitch` columns apart, rows ld apart
+
+struct AlignedCopy {
+    int32_t pitch;       // columns from one chunk's start to the next one's
+    int64_t ld;          // row pitch
+    size_t bytes;        // 0: no copy
+};
+bool copy_pays(const gnnfd_csr_t* csr, int64_t gathered_bytes);
+AlignedCopy layout_copy(int64_t n, gnnfd_dtype_t xdt, int32_t f, int32_t cw, int32_t unit_bytes);
+void launch_copy(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int64_t n, int32_t f, int32_t cw, const AlignedCopy& copy,
+                 void* d_aligned, cudaStream_t s);
+
 // ---- pieces of one translation unit that the layer entry points (layer.cu) put together
 
 int64_t segment_capacity(int64_t n, int64_t e, uint32_t flags);      // csr_build.cu; -1 for sizes the build rejects
@@ -98,6 +110,8 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
                        const float* d_a_dst, int32_t heads, int32_t dim, float negative_slope, void* d_out, int64_t ldo,
                        gnnfd_dtype_t odt, int32_t chunk_width, void* d_scratch, size_t scratch_bytes, bool scores_ready,
                        cudaStream_t s);
+size_t gat_copy_bytes(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads, int32_t dim,
+                      int32_t chunk_width);
 int gat_scratch_scores(const gnnfd_csr_t* csr, int32_t heads, int32_t dim, void* d_scratch, size_t scratch_bytes,
                        float** s_src, float** s_dst);
 

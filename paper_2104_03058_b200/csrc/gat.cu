@@ -30,7 +30,8 @@ struct GatArgs {
     float* partial_ml;   // [n_segments, heads, 2] running max and denominator of hub segments
     int64_t ldz, ldo;
     float slope;
-    int32_t f, heads, dim, chunk_width, n_ctiles, blocks_per_tile, fpad, out_bf16, wide_ok;
+    int32_t f, heads, dim, chunk_width, n_ctiles, blocks_per_tile, fpad, out_bf16, wide_ok;   // columns as z holds them
+    int32_t out_dim;         // columns of a head in the output (dim, or less where z is a copy with padded heads)
     int32_t chunk_base;      // first chunk of this launch (a launch covers at most 65,535 chunks)
     int32_t n_ranges;
     Range range[kMaxRanges];
@@ -350,10 +351,11 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
             for (int i = 0; i < VECN; ++i)
                 if (j + i < chunk_end) p[i] = acc[q][i];
         } else {
-            const int64_t o = (int64_t)row * a.ldo + j;
+            const int d = j - h * a.dim;                                     // column inside the head
+            const int64_t o = (int64_t)row * a.ldo + h * a.out_dim + d;
 #pragma unroll
             for (int i = 0; i < VECN; ++i)
-                if (j + i < chunk_end) store_elem(a.out, a.out_bf16, o + i, acc[q][i] * inv);
+                if (j + i < chunk_end && d + i < a.out_dim) store_elem(a.out, a.out_bf16, o + i, acc[q][i] * inv);
         }
     }
 }
@@ -403,7 +405,7 @@ constexpr int kReduceWays = kBlock / kReduceCols;
 __global__ void __launch_bounds__(kBlock)
 gat_hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict__ hub_seg_ptr,
                const float* __restrict__ partial, const float* __restrict__ partial_ml, int64_t hub_begin, int32_t n_hub,
-               int32_t f, int32_t fpad, int32_t heads, int32_t dim, void* __restrict__ out, int64_t ldo, int out_bf16)
+               int32_t f, int32_t fpad, int32_t heads, int32_t dim, int32_t out_dim, void* __restrict__ out, int64_t ldo, int out_bf16)
 {
     __shared__ float s_max[kReduceWays][kReduceCols], s_num[kReduceWays][kReduceCols], s_den[kReduceWays][kReduceCols];
     const int i = blockIdx.x;
@@ -442,7 +444,8 @@ gat_hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict_
     den = 0.f;
 #pragma unroll
     for (int w = 0; w < kReduceWays; ++w) { num += s_num[w][c]; den += s_den[w][c]; }
-    store_elem(out, out_bf16, (int64_t)row * ldo + j, den > 0.f ? num / den : 0.f);
+    const int d = j - h * dim;
+    if (d < out_dim) store_elem(out, out_bf16, (int64_t)row * ldo + h * out_dim + d, den > 0.f ? num / den : 0.f);
 }
 
 // ------------------------------------------------------------------ host side
@@ -502,6 +505,32 @@ static int launch_scores(int64_t n, const void* d_z, int64_t ldz, gnnfd_dtype_t 
     return GNNFD_OK;
 }
 
+// A copy of z whose heads are padded to whole 16-byte vectors, for heads that are not (7 fp32 or 4 bf16 columns): the vector
+// kernels need a vector to stay inside one head.  Heads are the copy's chunks, so the sweeps have to hold whole heads.  200,000
+// rows of 150 entries, 8 x 7 fp32 1.66 -> 0.66 ms, 8 x 7 bf16 1.71 -> 0.50, 6 x 4 bf16 0.65 -> 0.48; 100,000 rows of 4, 4 x 7
+// fp32 118 -> 38 us; a single head of 4 bf16 columns, one load as it is, 0.235 -> 0.243 ms, stays.
+static AlignedCopy plan_head_copy(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads, int32_t dim,
+                                  int32_t cw)
+{
+    const int zsize = zdt == GNNFD_F32 ? 4 : 2;
+    const int32_t f = heads * dim;
+    const bool aligned = (uintptr_t)d_z % 16 == 0 && ldz * zsize % 16 == 0 && dim * zsize % 16 == 0;
+    if (aligned || (cw < f && cw % dim != 0) || f * zsize <= 8 || !copy_pays(csr, csr->nnz * f * zsize)) return AlignedCopy{dim, ldz, 0};
+    return layout_copy(csr->n, zdt, f, dim, 16);
+}
+
+size_t gat_copy_bytes(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads, int32_t dim,
+                      int32_t chunk_width)
+{
+    const AlignedCopy copy = plan_head_copy(csr, d_z, ldz, zdt, heads, dim, chunk_width);
+    if (copy.bytes == 0) return 0;
+    Carver plain(nullptr, ~size_t(0)), padded(nullptr, ~size_t(0));        // the partial sums have the copy's columns
+    GatScratch g;
+    carve_gat(plain, csr, heads, dim, &g);
+    carve_gat(padded, csr, heads, copy.pitch, &g);
+    return padded.off - plain.off + copy.bytes;
+}
+
 // scores_ready: the two score arrays at the head of the scratch buffer (see gat_scratch_scores) already hold the
 // scores of d_z (the dense transform's epilogue wrote them), so the scores pass is left out.
 int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, const float* d_a_src,
@@ -515,7 +544,9 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
     if (f64 > 0x7fffffffll || ldz < f64 || ldo < f64 || ldz > 0x7fffffffll) return GNNFD_INVALID_ARG;
     if ((zdt != GNNFD_F32 && zdt != GNNFD_BF16) || (odt != GNNFD_F32 && odt != GNNFD_BF16)) return GNNFD_UNSUPPORTED;
     if (!d_scratch || ((uintptr_t)d_scratch & 255u)) return GNNFD_INVALID_ARG;
-    const int32_t f = (int32_t)f64;
+    const int32_t out_dim = dim;
+    int32_t f = (int32_t)f64;
+    int cw = chunk_width < f ? chunk_width : f;
     Carver c(d_scratch, scratch_bytes);
     GatScratch g;
     carve_gat(c, csr, heads, dim, &g);
@@ -524,8 +555,23 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
         int rc = launch_scores(csr->n, d_z, ldz, zdt, d_a_src, d_a_dst, heads, dim, g.s_src, g.s_dst, s);
         if (rc) return rc;
     }
+    const AlignedCopy copy = plan_head_copy(csr, d_z, ldz, zdt, heads, dim, cw);
+    if (copy.bytes > 0) {
+        Carver with_copy(d_scratch, scratch_bytes);          // the scores keep their place at the head of the buffer
+        GatScratch wider;
+        carve_gat(with_copy, csr, heads, copy.pitch, &wider);
+        void* aligned = with_copy.take<char>(copy.bytes);
+        if (with_copy.ok) {
+            launch_copy(d_z, ldz, zdt, csr->n, f, dim, copy, aligned, s);
+            g = wider;
+            cw = cw / dim * copy.pitch;
+            dim = copy.pitch;
+            f = heads * dim;
+            d_z = aligned;
+            ldz = copy.ld;
+        }
+    }
 
-    const int cw = chunk_width < f ? chunk_width : f;
     const int n_chunks = (f + cw - 1) / cw;
     const int zsize = zdt == GNNFD_F32 ? 4 : 2;
     const int vecn = 16 / zsize;
@@ -545,7 +591,7 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
     a.s_src = g.s_src; a.s_dst = g.s_dst; a.z = d_z; a.out = d_out;
     a.partial = g.partial; a.partial_ml = g.partial_ml;
     a.ldz = ldz; a.ldo = ldo; a.slope = negative_slope;
-    a.f = f; a.heads = heads; a.dim = dim; a.chunk_width = cw;
+    a.f = f; a.heads = heads; a.dim = dim; a.out_dim = out_dim; a.chunk_width = cw;
     a.n_ctiles = (cw + lpr * vpl * elems - 1) / (lpr * vpl * elems);
     a.fpad = (int32_t)align_up((size_t)f, 4);
     a.out_bf16 = odt == GNNFD_BF16;
@@ -575,7 +621,7 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
     if (n_hub > 0) {
         dim3 gr((unsigned)n_hub, (unsigned)((f + kReduceCols - 1) / kReduceCols));
         GNNFD_LAUNCH("gat_hub_reduce", s, gat_hub_reduce, gr, kBlock, 0, csr->row_order, csr->hub_seg_ptr, g.partial,
-                     g.partial_ml, csr->bin_start[4], (int32_t)n_hub, f, a.fpad, heads, dim, d_out, ldo, a.out_bf16);
+                     g.partial_ml, csr->bin_start[4], (int32_t)n_hub, f, a.fpad, heads, dim, out_dim, d_out, ldo, a.out_bf16);
     }
     GNNFD_CUDA_CHECK(cudaGetLastError());
     return GNNFD_OK;
@@ -618,6 +664,17 @@ int gnnfd_gat_workspace_bytes(const gnnfd_csr_t* csr, int32_t heads, int32_t dim
     gnnfd::GatScratch g;
     gnnfd::carve_gat(c, csr, heads, dim, &g);
     *scratch_bytes = c.off;
+    return GNNFD_OK;
+}
+
+int gnnfd_gat_best_workspace_bytes(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads,
+                                   int32_t dim, int32_t chunk_width, size_t* scratch_bytes)
+{
+    int rc = gnnfd_gat_workspace_bytes(csr, heads, dim, scratch_bytes);
+    if (rc) return rc;
+    if (chunk_width <= 0 || (int64_t)heads * dim > 0x7fffffffll || ldz < (int64_t)heads * dim) return GNNFD_INVALID_ARG;
+    if (zdt != GNNFD_F32 && zdt != GNNFD_BF16) return GNNFD_UNSUPPORTED;
+    *scratch_bytes += gnnfd::gat_copy_bytes(csr, d_z, ldz, zdt, heads, dim, chunk_width);
     return GNNFD_OK;
 }
 

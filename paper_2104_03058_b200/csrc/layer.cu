@@ -48,6 +48,7 @@ int gnnfd_layer_workspace_bytes(const gnnfd_csr_t* csr, int model, int32_t f_out
         if (heads <= 0 || dim <= 0 || (int64_t)heads * dim > 0x7fffffffll) return GNNFD_INVALID_ARG;
         f_out = heads * dim;
         rc = gnnfd_gat_workspace_bytes(csr, heads, dim, &rest);
+        if (!rc) rest += gat_copy_bytes(csr, nullptr, z_pitch(f_out), xdt, heads, dim, f_out);       // z is aligned, its heads may not be
     } else {
         if (f_out <= 0) return GNNFD_INVALID_ARG;
         rc = gnnfd_aggregate_workspace_bytes(csr, f_out, &rest);

@@ -96,7 +96,7 @@ int gnnfd_oneshot_gat(int64_t n, int64_t e, const void* d_src, const void* d_dst
                          L.build_scratch, stream, &csr);
     if (rc) return rc;
     rc = gnnfd_aggregate_gat(csr, d_z, ldz, zdt, d_a_src, d_a_dst, heads, dim, negative_slope, d_out, ldo, odt, chunk_width,
-                             base + L.persistent + L.build_scratch, L.aggregate, stream);
+                             base + L.persistent, L.build_scratch + L.aggregate, stream);
     gnnfd_csr_destroy(csr);
     return rc;
 }

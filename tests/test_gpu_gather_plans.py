@@ -78,6 +78,27 @@ def test_where_no_copy_is_planned(g, graph):
     assert g.aggregate_best_workspace_bytes(graph[0], x) == g.aggregate_workspace_bytes(graph[0], 64)  # aligned
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("heads,dim,ld,cw", [(4, 7, 28, 28), (4, 7, 32, 7), (5, 3, 15, 15), (3, 20, 61, 40), (6, 4, 24, 24), (2, 33, 66, 33),
+                                             (1, 41, 41, 41), (8, 7, 56, 14)])
+def test_padded_heads(g, graph, dtype, heads, dim, ld, cw):
+    csr, row_ptr, col = graph
+    f = heads * dim
+    gen = torch.Generator().manual_seed(f)
+    z = torch.full((csr.n, ld), float("nan"), dtype=dtype)
+    z[:, :f] = torch.randn((csr.n, f), generator=gen).to(dtype)
+    a = [torch.randn((heads, dim), generator=gen) * 0.3 for _ in range(2)]
+    dev = [t.cuda() for t in (z, *a)]
+    small = scratch(g.gat_workspace_bytes(csr, heads, dim))
+    plain = g.aggregate_gat(csr, *dev, heads, dim, 0.2, chunk_width=cw, scratch=small)
+    out = torch.full((csr.n, f + 3), 9.0, device="cuda")
+    got = g.aggregate_gat(csr, *dev, heads, dim, 0.2, chunk_width=cw, out=out)
+    assert (out[:, f:] == 9.0).all()
+    want, scale = orc.aggregate_gat(row_ptr, col, np.ascontiguousarray(z[:, :f].float().numpy()), a[0].numpy(), a[1].numpy(), heads, dim, 0.2)
+    for t in (plain, got[:, :f]):
+        assert (np.abs(t.cpu().numpy() - want) <= 1e-5 * scale + 1e-6).all()
+
+
 # Rows of lengths around the octave bounds of the shared classes (a row of up to 256 / 512 / 1024 / 2048 entries is one, two, four or
 # eight warps' work when the graph is small), hub rows, and enough short rows beside them.
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
