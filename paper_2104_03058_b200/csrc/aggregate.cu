@@ -529,7 +529,7 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
 
     const int per_step = kLoads / vpl * (32 / lpr);
     const int64_t limit = walk_limit(csr, per_step, (int64_t)n_chunks * a.n_ctiles);
-    const int64_t blocks = plan_ranges(csr, lpr, per_step, limit, a.range, &a.n_ranges);
+    const int64_t blocks = plan_ranges(csr, gather_groups(), lpr, per_step, limit, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;
     if (grid_x > 0x7fffffffll) return GNNFD_TOO_LARGE;

@@ -21,20 +21,15 @@
 #include <math_constants.h>
 
 #include "schedule.cuh"
+#include "vec.cuh"
 
 namespace gnnfd {
 
-#ifndef GNNFD_SOFTMAX_IN_FLIGHT
-#define GNNFD_SOFTMAX_IN_FLIGHT 4
-#endif
 #ifndef GNNFD_SOFTMAX_MIN_BLOCKS
 #define GNNFD_SOFTMAX_MIN_BLOCKS 4
 #endif
-// slots a lane has in flight when it holds HB heads of a slot: GNNFD_SOFTMAX_IN_FLIGHT 16-byte loads' worth, at most 16
-template <int HB> constexpr int slots_in_flight()
-{
-    return GNNFD_SOFTMAX_IN_FLIGHT * 4 / HB > 16 ? 16 : GNNFD_SOFTMAX_IN_FLIGHT * 4 / HB < 2 ? 2 : GNNFD_SOFTMAX_IN_FLIGHT * 4 / HB;
-}
+// slots a lane has in flight when it holds HB heads of a slot
+template <int HB> constexpr int slots_in_flight() { return HB == 4 ? 4 : 8; }
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct SoftmaxArgs {
@@ -105,15 +100,24 @@ __device__ __forceinline__ float rescale(float m, float mx) { return m == -CUDAR
 struct Leaky {
     float c1, c2;
     __device__ __forceinline__ explicit Leaky(float slope) : c1(0.5f * kLog2e * (1.f + slope)), c2(0.5f * kLog2e * (1.f - slope)) {}
-    __device__ __forceinline__ float operator()(float x) const { return fmaf(fabsf(x), c2, x * c1); }
+    __device__ __forceinline__ float operator()(float x) const { return fmaf(x, c1, fabsf(x) * c2); }     // |.| is free on a product
 };
 
-// column indices of slots k, k + SP, ... of one row (-1 past the end of the row)
-template <int SP, int NF>
-__device__ __forceinline__ void load_cols(const SoftmaxArgs& a, int32_t k, int32_t e, int32_t (&u)[NF])
+// Heads are worked on two to an instruction where a lane has an even number of them.
+template <int HB> constexpr int kPair = HB % 2 == 0 ? 2 : 1;
+template <int HB>
+__device__ __forceinline__ void add_heads(float* x, float a, float b)
+{
+    if constexpr (kPair<HB> == 2) add_pair(x[0], x[1], a, b);
+    else x[0] += a;
+}
+
+// column indices of slots k, k + step, ... of one row (-1 past the end of the row)
+template <int NF>
+__device__ __forceinline__ void load_cols(const SoftmaxArgs& a, int32_t k, int32_t e, int32_t step, int32_t (&u)[NF])
 {
 #pragma unroll
-    for (int i = 0; i < NF; ++i) u[i] = k + i * SP < e ? __ldg(a.col_idx + k + i * SP) : -1;
+    for (int i = 0; i < NF; ++i) u[i] = k + i * step < e ? __ldg(a.col_idx + k + i * step) : -1;
 }
 
 // base-2 logits of the slots whose column indices are u[].  FULL: all of them exist; otherwise the
@@ -134,9 +138,10 @@ __device__ __forceinline__ void load_logits(const SoftmaxArgs& a, const Leaky& l
 #pragma unroll
     for (int i = 0; i < NF; ++i)
 #pragma unroll
-        for (int h = 0; h < HB; ++h) {
-            const float y = leaky(t[i][h] + sd[h]);
-            t[i][h] = (FULL || u[i] >= 0) ? y : -CUDART_INF_F;
+        for (int h = 0; h < HB; h += kPair<HB>) {
+            add_heads<HB>(&t[i][h], sd[h], sd[h + kPair<HB> - 1]);
+#pragma unroll
+            for (int k = h; k < h + kPair<HB>; ++k) t[i][k] = (FULL || u[i] >= 0) ? leaky(t[i][k]) : -CUDART_INF_F;
         }
 }
 
@@ -145,32 +150,71 @@ template <int HB, int NF>
 __device__ __forceinline__ void online_update(const float (&t)[NF][HB], float (&m)[HB], float (&l)[HB])
 {
 #pragma unroll
-    for (int h = 0; h < HB; ++h) {
-        float mx = m[h];                                               // t[0] is a real slot, so mx ends finite
+    for (int h = 0; h < HB; h += kPair<HB>) {
+        constexpr int P = kPair<HB>;
+        float mx[P], sum[P];
 #pragma unroll
-        for (int i = 0; i < NF; ++i) mx = fmaxf(mx, t[i][h]);
-        float sum = 0.f;
+        for (int k = 0; k < P; ++k) {
+            mx[k] = m[h + k];                                          // t[0] is a real slot, so mx ends finite
 #pragma unroll
-        for (int i = 0; i < NF; ++i) sum += ex2(t[i][h] - mx);                  // 2^-inf = 0
-        l[h] = l[h] * ex2(m[h] - mx) + sum;
-        m[h] = mx;
+            for (int i = 0; i < NF; ++i) mx[k] = fmaxf(mx[k], t[i][h + k]);
+            sum[k] = 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            float p[P];
+#pragma unroll
+            for (int k = 0; k < P; ++k) p[k] = t[i][h + k];
+            add_heads<HB>(p, -mx[0], -mx[P - 1]);
+#pragma unroll
+            for (int k = 0; k < P; ++k) p[k] = ex2(p[k]);              // 2^-inf = 0
+            add_heads<HB>(sum, p[0], p[P - 1]);
+        }
+#pragma unroll
+        for (int k = 0; k < P; ++k) {
+            l[h + k] = l[h + k] * ex2(m[h + k] - mx[k]) + sum[k];
+            m[h + k] = mx[k];
+        }
+    }
+}
+
+// the alphas of one slot from its logits
+template <int HB>
+__device__ __forceinline__ void weights(const float (&t)[HB], const float (&m)[HB], const float (&inv)[HB], float (&w)[HB])
+{
+#pragma unroll
+    for (int h = 0; h < HB; h += kPair<HB>) {
+        constexpr int P = kPair<HB>;
+#pragma unroll
+        for (int k = h; k < h + P; ++k) w[k] = t[k];
+        add_heads<HB>(&w[h], -m[h], -m[h + P - 1]);
+#pragma unroll
+        for (int k = h; k < h + P; ++k) w[k] = ex2(w[k]);
+        if constexpr (P == 2) mul_pair(w[h], w[h + 1], inv[h], inv[h + 1]);
+        else w[h] *= inv[h];
     }
 }
 
 // One row (or hub segment) per S = LPS * SP lanes: SP slots are worked on side by side, and the heads
 // of a slot are spread over LPS lanes holding HB heads each (LPS * HB heads per round; more heads take
 // more rounds over the row).
-template <int HB, int LPS, int SP, int MODE>
-__device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range& rg, int block_in_range)
+//
+// A row of more slots than its lanes hold at once may be shared by up to all warps of the block (rg.warps_log2), which
+// take SP slots of a step each; their (max, sum) pairs are merged through shared memory, first warp to last.
+template <int HB, int LPS, int SP, bool SHARED, int MODE>
+__device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range& rg, int block_in_range, float2 (*shared_stats)[32])
 {
     constexpr int S = LPS * SP;
     constexpr int NF = slots_in_flight<HB>();
     constexpr unsigned kFull = 0xffffffffu;
     const int tid = threadIdx.x;
-    const int slot = block_in_range * (kBlock / S) + tid / S;
+    const int warps_log2 = SHARED && S == 32 ? rg.warps_log2 : 0;
+    const int warp = tid >> 5, sharer = warp & ((1 << warps_log2) - 1);
+    const int slot = block_in_range * (kBlock / S >> warps_log2) + (tid / S >> warps_log2);
     const int sl = tid % S;
-    const int hb = sl % LPS;             // which block of HB heads of a slot
-    const int sp = sl / LPS;             // which of the SP slots of a step
+    const int hb = sl % LPS;                       // which block of HB heads of a slot
+    const int sp = sl / LPS + sharer * SP;         // which slot of a step
+    const int step = SP << warps_log2;             // slots of a step, over all sharers
     const bool active = slot < rg.item_count;
     int32_t row = 0, b = 0, e = 0, part = 0;      // part: where a hub segment's (max, sum) lives
     if (active) {
@@ -186,7 +230,7 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
         }
     }
     // every row of the warp fits one batch: the write pass reuses the logits of the first pass
-    const bool fits = MODE == kModeRows && __all_sync(kFull, e - b <= SP * NF);
+    const bool fits = MODE == kModeRows && __all_sync(kFull, e - b <= step * NF);
     const Leaky leaky(a.slope);
 
     for (int hh = 0; hh < a.heads; hh += LPS * HB) {
@@ -206,11 +250,11 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
             for (int h = 0; h < HB; ++h) { m[h] = -CUDART_INF_F; l[h] = 0.f; }
             if (head_ok) {
                 int32_t u[NF], un[NF];
-                load_cols<SP, NF>(a, b + sp, e, u);
-                for (int32_t kb = b; kb < e; kb += SP * NF) {
+                load_cols<NF>(a, b + sp, e, step, u);
+                for (int32_t kb = b; kb < e; kb += step * NF) {
                     // the next batch's indices are on their way while this batch is gathered and reduced
-                    load_cols<SP, NF>(a, kb + SP * NF + sp, e, un);
-                    if (kb + SP * NF <= e) {               // the same for all lanes of the row
+                    load_cols<NF>(a, kb + step * NF + sp, e, step, un);
+                    if (kb + step * NF <= e) {               // the same for all lanes of the row
                         load_logits<HB, true, NF>(a, leaky, ssrc, sd, u, t);
                         online_update<HB, NF>(t, m, l);
                     } else if (u[0] >= 0) {
@@ -234,6 +278,23 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
                         m[h] = mx;
                     }
             }
+            if (SHARED && S == 32 && warps_log2 > 0) {   // the whole block is on this side, for every round of heads
+                __syncthreads();
+                if (sl / LPS == 0) {
+#pragma unroll
+                    for (int h = 0; h < HB; ++h) shared_stats[warp][hb * HB + h] = make_float2(m[h], l[h]);
+                }
+                __syncthreads();
+#pragma unroll
+                for (int h = 0; h < HB; ++h) {
+                    const float2* st = &shared_stats[warp - sharer][hb * HB + h];
+                    float mx = -CUDART_INF_F, sum = 0.f;
+                    for (int w = 0; w < 1 << warps_log2; ++w) mx = fmaxf(mx, st[w * 32].x);
+                    for (int w = 0; w < 1 << warps_log2; ++w) sum = fmaf(st[w * 32].y, rescale(st[w * 32].x, mx), sum);
+                    m[h] = mx;
+                    l[h] = sum;
+                }
+            }
             if constexpr (MODE == kModeHubStats) {
                 if (active && head_ok && sp == 0) {
 #pragma unroll
@@ -255,28 +316,26 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
         if (fits) {
 #pragma unroll
             for (int i = 0; i < NF; ++i) {
-                const int32_t k = b + sp + i * SP;
+                const int32_t k = b + sp + i * step;
                 if (k < e) {
                     float w[HB];
-#pragma unroll
-                    for (int h = 0; h < HB; ++h) w[h] = ex2(t[i][h] - m[h]) * inv[h];
+                    weights<HB>(t[i], m, inv, w);
                     store_heads<HB>(a.alpha + (int64_t)k * a.heads + h0, w);
                 }
             }
         } else {
             int32_t u[NF], un[NF];
-            load_cols<SP, NF>(a, b + sp, e, u);
-            for (int32_t kb = b; kb < e; kb += SP * NF) {
+            load_cols<NF>(a, b + sp, e, step, u);
+            for (int32_t kb = b; kb < e; kb += step * NF) {
                 const int32_t k = kb + sp;
-                load_cols<SP, NF>(a, k + SP * NF, e, un);
-                if (kb + SP * NF <= e) {
+                load_cols<NF>(a, k + step * NF, e, step, un);
+                if (kb + step * NF <= e) {
                     load_logits<HB, true, NF>(a, leaky, ssrc, sd, u, t);
 #pragma unroll
                     for (int i = 0; i < NF; ++i) {
                         float w[HB];
-#pragma unroll
-                        for (int h = 0; h < HB; ++h) w[h] = ex2(t[i][h] - m[h]) * inv[h];
-                        store_heads<HB>(a.alpha + (int64_t)(k + i * SP) * a.heads + h0, w);
+                        weights<HB>(t[i], m, inv, w);
+                        store_heads<HB>(a.alpha + (int64_t)(k + i * step) * a.heads + h0, w);
                     }
                 } else if (u[0] >= 0) {
                     load_logits<HB, false, NF>(a, leaky, ssrc, sd, u, t);
@@ -284,9 +343,8 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
                     for (int i = 0; i < NF; ++i) {
                         if (u[i] >= 0) {
                             float w[HB];
-#pragma unroll
-                            for (int h = 0; h < HB; ++h) w[h] = ex2(t[i][h] - m[h]) * inv[h];
-                            store_heads<HB>(a.alpha + (int64_t)(k + i * SP) * a.heads + h0, w);
+                            weights<HB>(t[i], m, inv, w);
+                            store_heads<HB>(a.alpha + (int64_t)(k + i * step) * a.heads + h0, w);
                         }
                     }
                 }
@@ -298,32 +356,34 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
 }
 
 // All ordinary rows (stats and write in one go) and, in the same grid, the write pass of the hub segments.
-template <int HB, int LPS>
+template <int HB, int LPS, bool SHARED>
 __global__ void __launch_bounds__(kBlock, GNNFD_SOFTMAX_MIN_BLOCKS) edge_softmax_rows(const __grid_constant__ SoftmaxArgs a)
 {
+    __shared__ float2 shared_stats[kBlock / 32][32];
     const int rb = blockIdx.x;
     int r = 0;
 #pragma unroll
-    for (int i = 1; i < kMaxRanges; ++i)
+    for (int i = 1; i < (SHARED ? kMaxRanges : kNumBins); ++i)      // unsplit, the fourth class is one range
         if (i < a.n_ranges && rb >= a.range[i].first_block) r = i;
     const Range rg = a.range[r];
     const int bir = rb - rg.first_block;
-    if (rg.hub) { softmax_items<HB, LPS, 32 / LPS, kModeHubWrite>(a, rg, bir); return; }
+    if (rg.hub) { softmax_items<HB, LPS, 32 / LPS, SHARED, kModeHubWrite>(a, rg, bir, shared_stats); return; }
     switch (rg.ep_log2) {
-        case 0: softmax_items<HB, LPS, 1, kModeRows>(a, rg, bir); break;
-        case 1: if constexpr (LPS * 2 <= 32) softmax_items<HB, LPS, 2, kModeRows>(a, rg, bir); break;
-        case 2: if constexpr (LPS * 4 <= 32) softmax_items<HB, LPS, 4, kModeRows>(a, rg, bir); break;
-        case 3: if constexpr (LPS * 8 <= 32) softmax_items<HB, LPS, 8, kModeRows>(a, rg, bir); break;
-        case 4: if constexpr (LPS * 16 <= 32) softmax_items<HB, LPS, 16, kModeRows>(a, rg, bir); break;
-        default: if constexpr (LPS == 1) softmax_items<HB, LPS, 32, kModeRows>(a, rg, bir); break;
+        case 0: softmax_items<HB, LPS, 1, SHARED, kModeRows>(a, rg, bir, shared_stats); break;
+        case 1: if constexpr (LPS * 2 <= 32) softmax_items<HB, LPS, 2, SHARED, kModeRows>(a, rg, bir, shared_stats); break;
+        case 2: if constexpr (LPS * 4 <= 32) softmax_items<HB, LPS, 4, SHARED, kModeRows>(a, rg, bir, shared_stats); break;
+        case 3: if constexpr (LPS * 8 <= 32) softmax_items<HB, LPS, 8, SHARED, kModeRows>(a, rg, bir, shared_stats); break;
+        case 4: if constexpr (LPS * 16 <= 32) softmax_items<HB, LPS, 16, SHARED, kModeRows>(a, rg, bir, shared_stats); break;
+        default: if constexpr (LPS == 1) softmax_items<HB, LPS, 32, SHARED, kModeRows>(a, rg, bir, shared_stats); break;
     }
 }
 
 // (max, sum) of every hub segment; range 0 of the plan is the hub range
-template <int HB, int LPS>
+template <int HB, int LPS, bool SHARED>
 __global__ void __launch_bounds__(kBlock, GNNFD_SOFTMAX_MIN_BLOCKS) edge_softmax_hub_stats(const __grid_constant__ SoftmaxArgs a)
 {
-    softmax_items<HB, LPS, 32 / LPS, kModeHubStats>(a, a.range[0], blockIdx.x);
+    __shared__ float2 shared_stats[kBlock / 32][32];
+    softmax_items<HB, LPS, 32 / LPS, SHARED, kModeHubStats>(a, a.range[0], blockIdx.x, shared_stats);
 }
 
 // One thread per (hub row, head): merges the segment results in ascending segment order and leaves the
@@ -352,22 +412,61 @@ static size_t softmax_scratch_bytes(const gnnfd_csr_t* csr, int32_t heads)
     return align_up((size_t)csr->n_segments * (size_t)heads * sizeof(float2), 256);
 }
 
-template <int HB, int LPS>
-static int launch_softmax(const gnnfd_csr_t* csr, SoftmaxArgs& a, cudaStream_t s)
+// Small graphs (the longest rows shared by warps, see schedule.cuh; here a step is a whole batch, so the limit may go down to
+// one): lanes enough for every row of a class to fit one batch of NF slots per lane.  8 heads, 20,000 rows of 6 entries
+// 50 -> 21 us, of 50 60 -> 33, 100,000 of 20 68 -> 53; 200,000 of 16 with one / four heads 51 -> 37 / 66 -> 53, but with
+// eight 67 us with the gathers' narrower groups and 80 with these, hence the second condition where they are used.  Splitting
+// rows on large graphs too, so that all fit, made 115 M slots of 8 heads 1.41 -> 2.55 ms: the block waits for its slowest gather
+// twice per row.  There the bound is the rate at which the L1 looks up scattered 32-byte pieces, one per slot and pass
+// (about 0.8 of the 1.4 ms); paired additions and products bring nothing at 8 heads, 6 heads 1.71 -> 1.48 ms.
+static Groups softmax_groups(int nf)
 {
-    const int64_t blocks = plan_ranges(csr, LPS, 1, 0, a.range, &a.n_ranges);
-    if (blocks > 0x7fffffffll) return GNNFD_TOO_LARGE;
-    if (blocks == 0) return GNNFD_OK;
+    const int longest[3] = {kBinDeg0, kBinDeg1, kBinDeg2};
+    Groups g{{1, 1, 1, 32, 32}};
+    for (int bin = 0; bin < 3; ++bin)
+        while (g.want[bin] < 32 && g.want[bin] * nf < longest[bin]) g.want[bin] *= 2;
+    return g;
+}
+
+template <int HB, int LPS, bool SHARED>
+static int launch_planned(const gnnfd_csr_t* csr, SoftmaxArgs& a, int64_t blocks, cudaStream_t s)
+{
     if (csr->n_segments > 0) {
-        const unsigned hub_blocks = (unsigned)((csr->n_segments + kBlock / 32 - 1) / (kBlock / 32));
-        GNNFD_LAUNCH("edge_softmax_hub_stats", s, (edge_softmax_hub_stats<HB, LPS>), hub_blocks, kBlock, 0, a);
+        const int per_block = kBlock / 32 >> a.range[0].warps_log2;
+        const unsigned hub_blocks = (unsigned)((csr->n_segments + per_block - 1) / per_block);
+        GNNFD_LAUNCH("edge_softmax_hub_stats", s, (edge_softmax_hub_stats<HB, LPS, SHARED>), hub_blocks, kBlock, 0, a);
         const int64_t pairs = (int64_t)a.n_hub * a.heads;
         GNNFD_LAUNCH("edge_softmax_hub_merge", s, edge_softmax_hub_merge, (unsigned)((pairs + kBlock - 1) / kBlock), kBlock,
                      0, a);
     }
-    GNNFD_LAUNCH("edge_softmax_rows", s, (edge_softmax_rows<HB, LPS>), (unsigned)blocks, kBlock, 0, a);
+    GNNFD_LAUNCH("edge_softmax_rows", s, (edge_softmax_rows<HB, LPS, SHARED>), (unsigned)blocks, kBlock, 0, a);
     GNNFD_CUDA_CHECK(cudaGetLastError());
     return GNNFD_OK;
+}
+
+template <int HB, int LPS>
+static int launch_softmax(const gnnfd_csr_t* csr, SoftmaxArgs& a, cudaStream_t s)
+{
+    constexpr int NF = slots_in_flight<HB>();
+    const int per_step = 32 / LPS * NF;
+    const int64_t limit = walk_limit(csr, per_step, 1, 1);
+    const bool shared = limit * per_step < kBinDeg3;
+    const bool wide = shared && (LPS == 1 || limit * per_step * 4 < kBinDeg3);
+    const int64_t blocks = plan_ranges(csr, wide ? softmax_groups(NF) : gather_groups(), LPS, per_step, limit, a.range, &a.n_ranges);
+    if (blocks > 0x7fffffffll) return GNNFD_TOO_LARGE;
+    if (blocks == 0) return GNNFD_OK;
+    return shared ? launch_planned<HB, LPS, true>(csr, a, blocks, s) : launch_planned<HB, LPS, false>(csr, a, blocks, s);
+}
+
+// Lanes of a slot: enough for all its heads in one round, up to 8.  3 of 4 or 5 of 8 lanes in use beat three or five rounds over
+// the row: 115 M slots of 3 / 6 / 12 heads 2.61 / 3.32 / 5.11 -> 1.12 / 1.48 / 2.2 ms.
+template <int HB>
+static int launch_lanes(const gnnfd_csr_t* csr, SoftmaxArgs& a, cudaStream_t s)
+{
+    const int lanes = (a.heads + HB - 1) / HB;
+    if (lanes > 4) return launch_softmax<HB, 8>(csr, a, s);
+    if (lanes > 2) return launch_softmax<HB, 4>(csr, a, s);
+    return lanes > 1 ? launch_softmax<HB, 2>(csr, a, s) : launch_softmax<HB, 1>(csr, a, s);
 }
 
 }  // namespace gnnfd
@@ -399,19 +498,10 @@ int gnnfd_edge_softmax(const gnnfd_csr_t* csr, const float* d_s_src, const float
     a.s_src = d_s_src; a.s_dst = d_s_dst; a.alpha = d_alpha; a.seg_stats = static_cast<float2*>(d_scratch);
     a.slope = negative_slope; a.heads = heads; a.n_hub = (int32_t)csr->bin_count[4];
 
-    // heads per lane (HB) and lanes per slot (LPS): 16-byte accesses when heads is a multiple of 4 and the
-    // pointers allow it, with the heads of a slot spread over up to 8 lanes so that a warp's accesses to
-    // alpha are contiguous; otherwise one lane per slot with 8- or 4-byte accesses
+    // heads per lane (HB): 16-byte accesses when heads is a multiple of 4 and the pointers allow it, otherwise 8- or 4-byte ones
     const uintptr_t ptrs = (uintptr_t)d_s_src | (uintptr_t)d_s_dst | (uintptr_t)d_alpha;
-    if (heads % 4 == 0 && ptrs % 16 == 0) {
-        const int blocks4 = heads / 4;
-        if (blocks4 % 8 == 0) return launch_softmax<4, 8>(csr, a, s);
-        if (blocks4 % 4 == 0) return launch_softmax<4, 4>(csr, a, s);
-        if (blocks4 % 2 == 0) return launch_softmax<4, 2>(csr, a, s);
-        return launch_softmax<4, 1>(csr, a, s);
-    }
-    if (heads % 2 == 0 && ptrs % 8 == 0) return launch_softmax<2, 1>(csr, a, s);
-    return launch_softmax<1, 1>(csr, a, s);
+    if (heads % 4 == 0 && ptrs % 16 == 0) return launch_lanes<4>(csr, a, s);
+    return heads % 2 == 0 && ptrs % 8 == 0 ? launch_lanes<2>(csr, a, s) : launch_lanes<1>(csr, a, s);
 }
 
 }  // extern "C"

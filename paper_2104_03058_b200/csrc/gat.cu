@@ -254,7 +254,7 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
                     for (int q = 0; q < VPL; ++q)
 #pragma unroll
                         for (int i = 0; i < VECN; i += VECN > 1 ? 2 : 1) {
-                            if constexpr (VECN > 1) mul_pair(acc[q][i], acc[q][i + 1], rescale);
+                            if constexpr (VECN > 1) mul_pair(acc[q][i], acc[q][i + 1], rescale, rescale);
                             else acc[q][i] *= rescale;
                         }
                 }
@@ -601,7 +601,7 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
 
     const int per_step = kLoads / vpl * (32 / lpr);
     const int64_t limit = walk_limit(csr, per_step, (int64_t)n_chunks * a.n_ctiles);
-    const int64_t blocks = plan_ranges(csr, lpr, per_step, limit, a.range, &a.n_ranges);
+    const int64_t blocks = plan_ranges(csr, gather_groups(), lpr, per_step, limit, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;
     if (grid_x > 0x7fffffffll) return GNNFD_TOO_LARGE;

@@ -24,12 +24,14 @@ struct Range {
 
 inline int ilog2(int x) { int l = 0; while ((1 << l) < x) ++l; return l; }
 
-// Edge-parallel groups per row for a degree class, limited by the lanes a row may use.  Rows of up to 32
+// Edge-parallel groups per row for a degree class, at most (the lanes a row may use limit them further).  The gathers: rows of up to 32
 // entries get one group, rows of up to 128 four: a short row is bound by its chain of dependent loads
 // (row number -> row pointer -> indices -> features), so more rows in flight per block beat more lanes per
 // row (config 2 at 64 columns 0.128 -> 0.115 ms, GAT on config 3 0.189 -> 0.167 ms, config 5 at 64 columns
 // 1.81 -> 1.62 ms against 4 and 8 groups).
-inline int ep_for_bin(int bin, int lpr)
+struct Groups { int want[kNumBins]; };
+
+inline Groups gather_groups()
 {
 #ifndef GNNFD_EP_BIN1
 #define GNNFD_EP_BIN1 1
@@ -40,9 +42,7 @@ inline int ep_for_bin(int bin, int lpr)
 #ifndef GNNFD_EP_BIN3
 #define GNNFD_EP_BIN3 32
 #endif
-    const int want[kNumBins] = {1, GNNFD_EP_BIN1, GNNFD_EP_BIN2, GNNFD_EP_BIN3, 32};
-    const int cap = 32 / lpr;
-    return want[bin] < cap ? want[bin] : cap;
+    return Groups{{1, GNNFD_EP_BIN1, GNNFD_EP_BIN2, GNNFD_EP_BIN3, 32}};
 }
 
 // Warps of a block that share a row (or hub segment) of up to `entries` entries.  A warp walks its row in steps of
@@ -56,21 +56,23 @@ inline int warps_log2_for(int entries, int per_step, int64_t limit)
     return w;
 }
 
-// The longest walk to allow, in steps: twice what a warp slot of the chip has to do on average, and not under 16.  fp32 GCN
+// The longest walk to allow, in steps: twice what a warp slot of the chip has to do on average, and not under 16 (of the gathers' steps).  fp32 GCN
 // against unsplit rows (one warp up to 2048 entries): 4,000 rows of 10 entries and 304 columns 76 -> 18 us, 20,000 of 50 and
 // 128 columns 101 -> 40, 100,000 of 20 and 64 columns 75 -> 50; 200,000 of 16 and more stay unsplit.  With the
 // average itself or four times it as the limit: 38 and 58 us for the second, 52 and 75 for the third.
-inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t sweeps)
+inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t sweeps, int64_t at_least = 16)
 {
     constexpr int64_t kWarpSlots = 148 * 24;
     const int64_t limit = 2 * (csr->nnz * sweeps / (per_step * kWarpSlots));
-    return limit > 16 ? limit : 16;
+    return limit > at_least ? limit : at_least;
 }
 
 // Fills ranges for `lpr` lanes per row; returns the blocks of one column tile of one sweep.  `per_step`: entries a whole warp
 // has in flight; `limit`: steps of the longest walk (0: a row is never split).
-inline int64_t plan_ranges(const gnnfd_csr_t* csr, int lpr, int per_step, int64_t limit, Range* range, int32_t* n_ranges)
+inline int64_t plan_ranges(const gnnfd_csr_t* csr, const Groups& groups, int lpr, int per_step, int64_t limit, Range* range,
+                           int32_t* n_ranges)
 {
+    auto ep_for_bin = [&](int bin) { return groups.want[bin] < 32 / lpr ? groups.want[bin] : 32 / lpr; };
     int nr = 0;
     int64_t blocks = 0;
     auto add = [&](int64_t begin, int64_t count, int ep, int entries, int hub) {
@@ -86,15 +88,15 @@ inline int64_t plan_ranges(const gnnfd_csr_t* csr, int lpr, int per_step, int64_
         range[nr++] = Range{(int32_t)blocks, (int32_t)(begin + count - 1), (int32_t)count, ilog2(ep), hub, w};
         blocks += (count + per_block - 1) / per_block;
     };
-    if (csr->n_segments > 0) add(0, csr->n_segments, ep_for_bin(4, lpr), kHubSegment, 1);
+    if (csr->n_segments > 0) add(0, csr->n_segments, ep_for_bin(4), kHubSegment, 1);
     int64_t end = csr->bin_start[3] + csr->bin_count[3];
     for (int o = kOctaves - 1; o >= 0; --o) {
         end -= csr->octave_count[o];
-        if (csr->octave_count[o] > 0) add(end, csr->octave_count[o], ep_for_bin(3, lpr), kBinDeg2 << (o + 1), 0);
+        if (csr->octave_count[o] > 0) add(end, csr->octave_count[o], ep_for_bin(3), kBinDeg2 << (o + 1), 0);
     }
     const int longest[3] = {kBinDeg0, kBinDeg1, kBinDeg2};
     for (int bin = 2; bin >= 0; --bin)
-        if (csr->bin_count[bin] > 0) add(csr->bin_start[bin], csr->bin_count[bin], ep_for_bin(bin, lpr), longest[bin], 0);
+        if (csr->bin_count[bin] > 0) add(csr->bin_start[bin], csr->bin_count[bin], ep_for_bin(bin), longest[bin], 0);
     *n_ranges = nr;
     return blocks;
 }

@@ -62,17 +62,22 @@ __device__ __forceinline__ void load_pair(Vec<__nv_bfloat16, 8>& a, Vec<__nv_bfl
 template <typename T>
 __device__ __forceinline__ void load_pair(Vec<T, 1>& a, Vec<T, 1>& b, const T* p) { a.load(p); b.load(p + 1); }
 
-// (x, y) += w * (a, b) and (x, y) *= w, each in one instruction: the same roundings as two scalar ones for half the issue
-// slots, which is what the attention kernel runs short of.
+// (x, y) += w * (a, b), (x, y) += (a, b) and (x, y) *= (a, b), each in one instruction: the same roundings as two scalar ones
+// for half the issue slots, which is what the attention kernels run short of.
 __device__ __forceinline__ void fma_pair(float& x, float& y, float w, float a, float b)
 {
     asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %2};\n\tmov.b64 q, {%3, %4};\n\tmov.b64 r, {%0, %1};\n\t"
         "fma.rn.f32x2 r, p, q, r;\n\tmov.b64 {%0, %1}, r;\n\t}" : "+f"(x), "+f"(y) : "f"(w), "f"(a), "f"(b));
 }
-__device__ __forceinline__ void mul_pair(float& x, float& y, float w)
+__device__ __forceinline__ void add_pair(float& x, float& y, float a, float b)
 {
-    asm("{\n\t.reg .b64 p, r;\n\tmov.b64 p, {%2, %2};\n\tmov.b64 r, {%0, %1};\n\t"
-        "mul.rn.f32x2 r, p, r;\n\tmov.b64 {%0, %1}, r;\n\t}" : "+f"(x), "+f"(y) : "f"(w));
+    asm("{\n\t.reg .b64 q, r;\n\tmov.b64 q, {%2, %3};\n\tmov.b64 r, {%0, %1};\n\t"
+        "add.rn.f32x2 r, q, r;\n\tmov.b64 {%0, %1}, r;\n\t}" : "+f"(x), "+f"(y) : "f"(a), "f"(b));
+}
+__device__ __forceinline__ void mul_pair(float& x, float& y, float a, float b)
+{
+    asm("{\n\t.reg .b64 q, r;\n\tmov.b64 q, {%2, %3};\n\tmov.b64 r, {%0, %1};\n\t"
+        "mul.rn.f32x2 r, q, r;\n\tmov.b64 {%0, %1}, r;\n\t}" : "+f"(x), "+f"(y) : "f"(a), "f"(b));
 }
 
 __device__ __forceinline__ void store_elem(void* out, int out_bf16, int64_t idx, float val)
