@@ -30,6 +30,7 @@ struct GatherArgs {
     float* partial;
     int64_t ldx, ldo;
     int32_t f, chunk_width, n_ctiles, blocks_per_tile, fpad, out_bf16, out_vec_ok, wide_ok;
+    int32_t part_filled;     // some lanes' vectors lie past the end of the chunk
     int32_t x_gap;           // columns between the end of a chunk and the start of the next one in x (the aligned copy may have some)
     int32_t chunk_base;      // first chunk of this launch (a launch covers at most 65,535 chunks)
     int32_t n_ranges;
@@ -44,7 +45,9 @@ struct GatherArgs {
 #endif
 constexpr int kLoads = GNNFD_GATHER_LOADS;      // 16-byte feature loads kept in flight per lane
 
-constexpr int kStageSlots = kLoads * 32;      // column indices (and weights) a warp stages per batch, at most
+// index registers per lane and batch, and the column indices (and weights) a warp stages per batch
+constexpr int index_regs(int lpr, int vpl) { return kLoads / vpl > lpr ? kLoads / vpl / lpr : 1; }
+constexpr int stage_slots(int lpr, int vpl) { return 32 * index_regs(lpr, vpl); }
 
 // One row (or hub segment) per S = LPR * EP lanes.  The S lanes fetch the row's indices and weights
 // S at a time with one coalesced streaming load each (R rounds per batch) and stage them in the
@@ -90,13 +93,13 @@ __device__ __forceinline__ void second_level(float (*tot_s)[kBlock], int tid, fl
 
 template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE, int EP>
 __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg, int block_in_range, int col0,
-                                            int chunk_end, int x_shift, int32_t (*stage_col)[kBlock / 32][kStageSlots],
-                                            float (*stage_w)[kBlock / 32][kStageSlots], float (*tot_s)[kBlock])
+                                            int chunk_end, int x_shift, int32_t (*stage_col)[kBlock / 32][stage_slots(LPR, VPL)],
+                                            float (*stage_w)[kBlock / 32][stage_slots(LPR, VPL)], float (*tot_s)[kBlock])
 {
     constexpr int S = LPR * EP;
     constexpr int ROWS = kBlock / S;
     constexpr int UB = kLoads / VPL;                      // steps whose loads are issued together
-    constexpr int R = UB > LPR ? UB / LPR : 1;            // index registers per lane and batch
+    constexpr int R = index_regs(LPR, VPL);
     constexpr int SPB = R * LPR;                          // steps per batch
     constexpr int EPB = R * S;                            // entries per batch
     constexpr unsigned kFull = 0xffffffffu;
@@ -118,7 +121,12 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
         okq[q] = jq[q] < chunk_end;
         xq[q] = static_cast<const T*>(a.x) + x_shift + (okq[q] ? jq[q] : col0);   // out-of-chunk lanes re-read a valid column
     }
-    const bool wide = WIDE && okq[VPL - 1];            // both vectors of the lane exist: one 32-byte load per entry
+    // Pair loads are for all lanes or none: a lane whose second vector, or both, lie past the chunk's end loads a pair all the
+    // same (padding of its own row, or the row's first pair) and drops it.  With a branch per lane, rows of 5 and 7 vectors took
+    // both sides of it: 116 M entries of 20 / 25 fp32 columns 1.58 / 1.59 -> 0.90 / 0.93 ms, of 48 bf16 columns 1.56 -> 1.19.
+    // For bf16 the test stays in the code (full chunks: no lane fails it): without it the loads are scheduled differently and
+    // 64 columns on 2 M RMAT rows take 1.61 instead of 1.49 ms.
+    const bool pairs = sizeof(T) == 4 || okq[VPL - 1] || a.part_filled;
     const uint32_t ld = (uint32_t)a.ldx;
 
     // a long row may be shared by several warps of the block, which take consecutive parts of it
@@ -214,7 +222,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
                     const int32_t u = LPR > 1 ? stage_col[buf][warp][r * 32 + seg + tt * EP + g] : ucur[r];
                     if (WEIGHTED) wv[i] = LPR > 1 ? stage_w[buf][warp][r * 32 + seg + tt * EP + g] : wcur[r];
                     const size_t off = (size_t)(uint32_t)u * ld;
-                    if (WIDE && wide) {
+                    if (WIDE && pairs) {
                         load_pair(v[i][0], v[i][VPL - 1], xq[0] + off);
                     } else {
 #pragma unroll
@@ -239,7 +247,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
                     const int32_t u = LPR > 1 ? stage_col[buf][warp][r * 32 + seg + tt * EP + g] : ucur[r];
                     if (WEIGHTED) wv[i] = LPR > 1 ? stage_w[buf][warp][r * 32 + seg + tt * EP + g] : wcur[r];
                     const size_t off = (size_t)(uint32_t)max(u, 0) * ld;
-                    if (WIDE && wide) {
+                    if (WIDE && pairs) {
                         if (u >= 0) load_pair(v[i][0], v[i][VPL - 1], xq[0] + off);
                         else { v[i][0].zero(); v[i][VPL - 1].zero(); }
                     } else {
@@ -305,8 +313,8 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
 template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE = false>
 __global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggregate(const __grid_constant__ GatherArgs a)
 {
-    __shared__ int32_t stage_col[2][kBlock / 32][kStageSlots];
-    __shared__ float stage_w[2][kBlock / 32][kStageSlots];
+    __shared__ int32_t stage_col[2][kBlock / 32][stage_slots(LPR, VPL)];
+    __shared__ float stage_w[2][kBlock / 32][stage_slots(LPR, VPL)];
     __shared__ __align__(16) float tot_s[VPL * VECN][kBlock];   // second-level sums of every thread
     // grid: x = (block of the sweep, column tile), y = chunk; blocks are issued x first, so the sweeps follow each
     // other chunk by chunk.  (The chunk used to be divided out of a linear 64-bit block number: two 64-bit
@@ -375,6 +383,9 @@ static GatherKernel pick_lpr(int lpr, int vpl, bool wide)
             }
         }
     }
+    if constexpr (VECN > 1) {
+        if (vpl == 3) return lpr == 8 ? gather_aggregate<T, VECN, 8, 3, WEIGHTED, SHARED> : gather_aggregate<T, VECN, 16, 3, WEIGHTED, SHARED>;
+    }
     switch (lpr) {
         case 1: return gather_aggregate<T, VECN, 1, 2, WEIGHTED, SHARED>;
         case 2: return gather_aggregate<T, VECN, 2, 2, WEIGHTED, SHARED>;
@@ -425,11 +436,11 @@ bool copy_pays(const gnnfd_csr_t* csr, int64_t gathered_bytes)
     return csr->nnz >= 4 * csr->n && gathered_bytes >= (int64_t)40 << 20;
 }
 
-AlignedCopy layout_copy(int64_t n, gnnfd_dtype_t xdt, int32_t f, int32_t cw, int32_t unit_bytes)
+AlignedCopy layout_copy(int64_t n, gnnfd_dtype_t xdt, int32_t f, int32_t cw, int32_t unit_bytes, int32_t row_bytes)
 {
-    const int xsize = xdt == GNNFD_F32 ? 4 : 2, unit = unit_bytes / xsize, sector = 32 / xsize;
+    const int xsize = xdt == GNNFD_F32 ? 4 : 2, unit = unit_bytes / xsize, row_unit = row_bytes / xsize;
     const int64_t pitch = ((int64_t)cw + unit - 1) / unit * unit;
-    const int64_t ld = ((f - 1) / cw * pitch + ((f - 1) % cw + unit) / unit * unit + sector - 1) / sector * sector;
+    const int64_t ld = ((f - 1) / cw * pitch + ((f - 1) % cw + unit) / unit * unit + row_unit - 1) / row_unit * row_unit;
     if (ld > 0x7fffffffll || n * ld > 0x7fffffffll * kBlock) return AlignedCopy{cw, f, 0};
     return AlignedCopy{(int32_t)pitch, ld, align_up((size_t)n * ld * xsize, 256)};
 }
@@ -461,7 +472,10 @@ static AlignedCopy plan_copy(const gnnfd_csr_t* csr, const void* d_x, int64_t ld
     const int xsize = xdt == GNNFD_F32 ? 4 : 2;
     if (aligned_for_vectors(d_x, ldx, xdt, f, cw) || (xsize == 4 && cw <= 32) || !copy_pays(csr, csr->nnz * f * xsize))
         return AlignedCopy{cw, ldx, 0};
-    return layout_copy(csr->n, xdt, f, cw, 32);               // chunks start on 32-byte sectors
+    // Chunks start on 32-byte sectors.  Rows of more than a line start on one where they are gathered often enough to make up for
+    // the larger copy (41 fp32 columns on 116 M entries: pitch 48 1.78 ms, 64 1.69; on 200,000 rows of 16 entries 93 and 97 us).
+    const bool lines = csr->nnz >= 64 * csr->n && (int64_t)f * xsize > 128;
+    return layout_copy(csr->n, xdt, f, cw, 32, lines ? 128 : 32);
 }
 
 static size_t partial_bytes(const gnnfd_csr_t* csr, int32_t f)
@@ -501,9 +515,16 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     const int elems = vec ? vecn : 1;
     // a lane covers two vectors of the chunk unless the chunk is a single vector wide
     const int vectors = (cw + elems - 1) / elems;
-    const int vpl = vectors > 1 ? 2 : 1;
+    int vpl = vectors > 1 ? 2 : 1;
     int lpr = 1;
     while (lpr * vpl < vectors && lpr < 32) lpr <<= 1;
+    // 17 - 24 and 33 - 48 vectors fit three per lane on half the lanes instead of leaving up to half of them idle: 192 fp32 columns on
+    // 200,000 rows of 16 entries 300 -> 230 us, 96 columns on 116 M entries 3.02 -> 2.64 ms.  Not 9 - 12: four lanes' vectors make
+    // 64-byte pieces, which split more cache lines than the idle lanes cost (44 columns there 1.88 -> 2.01 ms).
+    if (vec && lpr >= 16 && vectors <= lpr / 2 * 3) {
+        vpl = 3;
+        lpr /= 2;
+    }
     // Wider chunks go out in tiles of 64 vectors, or of 32 where the last tile of 64 would be mostly empty: 76 vectors (304
     // fp32 columns) on 200,000 rows of 16 entries 0.60 -> 0.52 ms; with full tiles the narrower one is 0 - 8 % slower.
     if (vec && vectors > 64 && (vectors + 31) / 32 * 32 * 1.04 < (vectors + 63) / 64 * 64) lpr = 16;
@@ -516,6 +537,7 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     a.ldx = ldx; a.ldo = ldo; a.f = f; a.chunk_width = cw;
     a.n_ctiles = (cw + lpr * vpl * elems - 1) / (lpr * vpl * elems);
     a.x_gap = x_gap;
+    a.part_filled = vectors != lpr * vpl;
     a.fpad = (int32_t)align_up((size_t)f, 4);
     a.out_bf16 = odt == GNNFD_BF16;
     // 32-byte loads of a lane's vector pair: every pair must start on a 32-byte boundary, and the chunk must

@@ -87,7 +87,9 @@ gat_scores(const T* __restrict__ z, int64_t ldz, const float* __restrict__ a_src
 
 constexpr int kLoads = 8;      // 16-byte feature loads kept in flight per lane
 
-constexpr int kStageSlots = kLoads * 32;      // column indices a warp stages per batch, at most
+// index registers per lane and batch, and the column indices a warp stages per batch
+constexpr int index_regs(int lpr, int vpl) { return kLoads / vpl > lpr ? kLoads / vpl / lpr : 1; }
+constexpr int stage_slots(int lpr, int vpl) { return 32 * index_regs(lpr, vpl); }
 
 // Bound by instruction issue once the graph fills the chip (an entry costs a logit, an exponential and the unpacking of
 // its features on top of the gather), so products and rescalings go two to an instruction: on 200,000 rows of
@@ -100,12 +102,12 @@ constexpr int kStageSlots = kLoads * 32;      // column indices a warp stages pe
 // covers VPL adjacent vectors, all inside one head, so it needs one logit per entry.
 template <typename T, int VECN, int LPR, int VPL, bool SHARED, int EP>
 __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int block_in_range, int col0, int chunk_end,
-                                         int32_t (*stage_col)[kBlock / 32][kStageSlots], float (*tot_s)[kBlock])
+                                         int32_t (*stage_col)[kBlock / 32][stage_slots(LPR, VPL)], float (*tot_s)[kBlock])
 {
     constexpr int S = LPR * EP;
     constexpr int ROWS = kBlock / S;
     constexpr int UB = kLoads / VPL;
-    constexpr int R = UB > LPR ? UB / LPR : 1;
+    constexpr int R = index_regs(LPR, VPL);
     constexpr int SPB = R * LPR;
     constexpr int EPB = R * S;
     constexpr unsigned kFull = 0xffffffffu;
@@ -148,8 +150,8 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
         b = min(b + sharer * share, e);
         e = min(b + share, e);
     }
-    // one 32-byte load per entry when both vectors of the lane exist and every row start allows it
-    const bool wide = a.wide_ok && okq[VPL - 1];
+    // one 32-byte load per entry where every row start allows it (a lane past the chunk's end loads the row's first pair)
+    const bool wide = a.wide_ok;
     const float sd = active ? a.s_dst[(int64_t)row * a.heads + h] : 0.f;
     const float* ssrc = a.s_src + h;
     // logits are kept in base 2: LeakyReLU(x) * log2 e = c1 * x + c2 * |x|
@@ -366,7 +368,7 @@ template <typename T, int VECN, int LPR, int VPL, bool SHARED>
 // the vector-pair forms and four for the others is what the measured-good builds had.
 __global__ void __launch_bounds__(kBlock, (VPL == 2 && VECN > 1) ? 3 : 4) gat_aggregate(const __grid_constant__ GatArgs a)
 {
-    __shared__ int32_t stage_col[2][kBlock / 32][kStageSlots];
+    __shared__ int32_t stage_col[2][kBlock / 32][stage_slots(LPR, VPL)];
     // second-level sums and denominator (and a sharer's maximum), one column per thread
     __shared__ float tot_s[VPL * VECN + 1 + SHARED][kBlock];
     // grid: x = (block of the sweep, column tile), y = chunk; blocks are issued x first, so the sweeps follow each
@@ -516,7 +518,7 @@ static AlignedCopy plan_head_copy(const gnnfd_csr_t* csr, const void* d_z, int64
     const int32_t f = heads * dim;
     const bool aligned = (uintptr_t)d_z % 16 == 0 && ldz * zsize % 16 == 0 && dim * zsize % 16 == 0;
     if (aligned || (cw < f && cw % dim != 0) || f * zsize <= 8 || !copy_pays(csr, csr->nnz * f * zsize)) return AlignedCopy{dim, ldz, 0};
-    return layout_copy(csr->n, zdt, f, dim, 16);
+    return layout_copy(csr->n, zdt, f, dim, 16, 32);
 }
 
 size_t gat_copy_bytes(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads, int32_t dim,
