@@ -470,7 +470,7 @@ static bool aligned_for_vectors(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt,
 static AlignedCopy plan_copy(const gnnfd_csr_t* csr, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f, int32_t cw)
 {
     const int xsize = xdt == GNNFD_F32 ? 4 : 2;
-    if (aligned_for_vectors(d_x, ldx, xdt, f, cw) || (xsize == 4 && cw <= 32) || !copy_pays(csr, csr->nnz * f * xsize))
+    if (aligned_for_vectors(d_x, ldx, xdt, f, cw) || (xsize == 4 && cw <= 32) || !copy_pays(csr, csr->nnz * cw * xsize))
         return AlignedCopy{cw, ldx, 0};
     // Chunks start on 32-byte sectors.  Rows of more than a line start on one where they are gathered often enough to make up for
     // the larger copy (41 fp32 columns on 116 M entries: pitch 48 1.78 ms, 64 1.69; on 200,000 rows of 16 entries 93 and 97 us).
@@ -550,7 +550,7 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     a.out_vec_ok = odt == GNNFD_F32 && ((uintptr_t)d_out % 16 == 0) && (ldo % 4 == 0) && (n_chunks == 1 || cw % 4 == 0);
 
     const int per_step = kLoads / vpl * (32 / lpr);
-    const int64_t limit = walk_limit(csr, per_step, (int64_t)n_chunks * a.n_ctiles);
+    const int64_t limit = walk_limit(csr, per_step, a.n_ctiles);
     const int64_t blocks = plan_ranges(csr, gather_groups(), lpr, per_step, limit, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;

@@ -516,8 +516,9 @@ static AlignedCopy plan_head_copy(const gnnfd_csr_t* csr, const void* d_z, int64
 {
     const int zsize = zdt == GNNFD_F32 ? 4 : 2;
     const int32_t f = heads * dim;
+    cw = cw < f ? cw : f;
     const bool aligned = (uintptr_t)d_z % 16 == 0 && ldz * zsize % 16 == 0 && dim * zsize % 16 == 0;
-    if (aligned || (cw < f && cw % dim != 0) || f * zsize <= 8 || !copy_pays(csr, csr->nnz * f * zsize)) return AlignedCopy{dim, ldz, 0};
+    if (aligned || (cw < f && cw % dim != 0) || cw * zsize <= 8 || !copy_pays(csr, csr->nnz * cw * zsize)) return AlignedCopy{dim, ldz, 0};
     return layout_copy(csr->n, zdt, f, dim, 16, 32);
 }
 
@@ -602,7 +603,7 @@ int gat_aggregate_impl(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnn
                 (n_chunks == 1 || (cw * zsize) % 32 == 0);
 
     const int per_step = kLoads / vpl * (32 / lpr);
-    const int64_t limit = walk_limit(csr, per_step, (int64_t)n_chunks * a.n_ctiles);
+    const int64_t limit = walk_limit(csr, per_step, a.n_ctiles);
     const int64_t blocks = plan_ranges(csr, gather_groups(), lpr, per_step, limit, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;

@@ -56,14 +56,17 @@ inline int warps_log2_for(int entries, int per_step, int64_t limit)
     return w;
 }
 
-// The longest walk to allow, in steps: twice what a warp slot of the chip has to do on average, and not under 16 (of the gathers' steps).  fp32 GCN
+// The longest walk to allow, in steps: twice what a warp slot of the chip has to do on average in the sweep over one chunk, and
+// not under 16 (of the gathers' steps).  A chunk's column tiles run side by side and count; chunks run one after the other, so the
+// longest rows end every one of their sweeps, and a column slab of whole chunks is cut like the full width, with the same
+// bits.  In entries the limit is 2 * nnz * tiles / 3552: with one tile, rows are split on graphs of up to 3.6 M entries.  fp32 GCN
 // against unsplit rows (one warp up to 2048 entries): 4,000 rows of 10 entries and 304 columns 76 -> 18 us, 20,000 of 50 and
-// 128 columns 101 -> 40, 100,000 of 20 and 64 columns 75 -> 50; 200,000 of 16 and more stay unsplit.  With the
-// average itself or four times it as the limit: 38 and 58 us for the second, 52 and 75 for the third.
-inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t sweeps, int64_t at_least = 16)
+// 128 columns 101 -> 40, 100,000 of 20 and 64 columns 75 -> 50.  With the average itself or four times it as the limit: 38 and
+// 58 us for the second, 52 and 75 for the third.
+inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t tiles, int64_t at_least = 16)
 {
     constexpr int64_t kWarpSlots = 148 * 24;
-    const int64_t limit = 2 * (csr->nnz * sweeps / (per_step * kWarpSlots));
+    const int64_t limit = 2 * (csr->nnz * tiles / (per_step * kWarpSlots));
     return limit > at_least ? limit : at_least;
 }
 

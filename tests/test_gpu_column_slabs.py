@@ -74,6 +74,38 @@ def test_virtual_ranks_reassemble_gat_by_whole_heads(world):
                                 a_dst=a_dst, heads=w.heads, dim=w.dim)
 
 
+# Which rows warps share and whether an aligned copy is gathered goes by the entries and the chunk's width, so a rank's slab of whole
+# chunks has the bits of the full-width call: graphs on both sides of the points where rows of up to 2048 entries are split.
+@pytest.mark.parametrize("entries", [500_000, 2_000_000])
+@pytest.mark.parametrize("model,f,ld,cw", [("gcn", 150, 152, 32), ("gcn", 192, 192, 64), ("sage", 150, 152, 32), ("sage", 192, 200, 64),
+                                           ("gcn", 301, 301, 64), ("sage", 83, 83, 16), ("gat", 64, 64, 8), ("gat", 96, 96, 32),
+                                           ("gat", 63, 63, 21), ("gat", 63, 64, 7)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_slabs_have_the_bits_of_the_full_width(entries, model, f, ld, cw, dtype):
+    import paper_2104_03058_b200 as g
+    from paper_2104_03058_b200 import sharding
+    rng = np.random.default_rng(entries)
+    lengths = np.concatenate([[5000, 2048, 2047, 1500, 1025, 1024, 700, 513, 400, 257, 200, 129], np.full(400, 1100), np.full(400, 300)])
+    n = 20_000
+    lengths = np.concatenate([lengths, np.full(n - len(lengths), max(1, (entries - lengths.sum()) // (n - len(lengths))))]).astype(np.int64)
+    lengths = np.minimum(lengths, np.maximum(entries - np.concatenate([[0], lengths.cumsum()[:-1]]), 0))
+    dst = rng.permutation(np.repeat(np.arange(n), lengths)).astype(np.int32)
+    csr = g.build_csr(n, dev(rng.integers(0, n, len(dst)).astype(np.int32)), dev(dst))
+    x = torch.randn((n, ld), generator=torch.Generator().manual_seed(f)).to(dtype).cuda()
+    heads, dim = (f // 7, 7) if f == 63 else (f // 8, 8)
+    a = [torch.randn((heads, dim), generator=torch.Generator().manual_seed(k)).cuda() * 0.3 for k in (1, 2)]
+    kw = dict(a_src=a[0], a_dst=a[1], heads=heads, dim=dim) if model == "gat" else {}
+    full = torch.empty((n, f), device="cuda")
+    sharding.aggregate_slab(csr, x, model, f, cw, 1, 0, full, **kw)
+    n_chunks = -(-f // cw)
+    whole = f // cw * cw
+    for world in (2, n_chunks):
+        out = torch.full((n, f), SENTINEL, device="cuda")
+        for rank in range(world):
+            sharding.aggregate_slab(csr, x, model, f, cw, world, rank, out, **kw)
+        assert torch.equal(out[:, :whole], full[:, :whole])
+
+
 def test_more_ranks_than_chunks_leaves_idle_ranks_without_work():
     import paper_2104_03058_b200 as g
     from paper_2104_03058_b200 import sharding
