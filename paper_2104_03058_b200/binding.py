@@ -83,6 +83,7 @@ def lib() -> ctypes.CDLL:
         L.gnnfd_layer_gat.argtypes = [vp, vp, i64, i32, i32, vp, i64, i32, i32, vp, vp, fl, ctypes.c_int, vp, i64, i32, i32,
                                       vp, sz, vp, vp]
         L.gnnfd_debug_combine_fault.argtypes = [i64, i32]
+        L.gnnfd_debug_build_fault.argtypes = [i32, i32]
         L.gnnfd_status_string.argtypes = [ctypes.c_int]
         L.gnnfd_status_string.restype = ctypes.c_char_p
         L.gnnfd_last_cuda_error.restype = ctypes.c_int
@@ -644,6 +645,11 @@ def layer(csr: Csr, model: str, x: torch.Tensor, w_t: torch.Tensor, f_in: int | 
 def debug_combine_fault(wait_ns: int, skip_k_block: int):
     """gnnfd_debug_combine_fault: arms the give-up drill for this thread's next transform launch."""
     _check(lib().gnnfd_debug_combine_fault(wait_ns, skip_k_block), "gnnfd_debug_combine_fault")
+
+
+def debug_build_fault(max_polls: int, sweep: int):
+    """gnnfd_debug_build_fault: arms the give-up drill for this thread's next build."""
+    _check(lib().gnnfd_debug_build_fault(max_polls, sweep), "gnnfd_debug_build_fault")
 
 
 def launch_count() -> int:

@@ -143,7 +143,8 @@ edge_histograms(const __grid_constant__ Candidates c, int first_bit, int digit_b
 // counter by blocks that are already running: tile 0 never waits, and every tile publishes its own counts before it
 // waits, so some waiting block can always go on.  The wait is limited all the same: a block that polls one
 // word kMaxPolls times marks the build as failed and leaves, the others follow, and the host returns
-// GNNFD_CUDA_ERROR.
+// GNNFD_CUDA_ERROR.  The launches after it are queued already and would take partly unwritten keys, so every kernel that
+// works on the sort's results looks at the mark first and does nothing.
 
 // A published word: 0 nothing yet; count + 1: the tile's own count; kSumBit | sum: keys of this digit value in all tiles
 // up to and including this one, plus the keys of smaller digit values (so the sum is a position).
@@ -164,7 +165,7 @@ __device__ __forceinline__ void publish(uint32_t* p, uint32_t v)
 
 // position of the tile's first key of one digit value: `column` points at the digit's word of tile 0, words of
 // consecutive tiles are kRadix apart.  false: gave up.
-__device__ __forceinline__ bool look_back(const uint32_t* column, int64_t tile, const int32_t* failed, uint32_t* before)
+__device__ __forceinline__ bool look_back(const uint32_t* column, int64_t tile, int max_polls, const int32_t* failed, uint32_t* before)
 {
     uint32_t sum = 0;
     int polls = 0;
@@ -182,7 +183,7 @@ __device__ __forceinline__ bool look_back(const uint32_t* column, int64_t tile, 
             }
         }
         t -= used;
-        if (used == 0 && (++polls & 255) == 0 && (polls >= kMaxPolls || load_published(reinterpret_cast<const uint32_t*>(failed)) != 0u))
+        if (used == 0 && (++polls & 255) == 0 && (polls >= max_polls || load_published(reinterpret_cast<const uint32_t*>(failed)) != 0u))
             return false;
     }
     *before = sum;
@@ -224,6 +225,7 @@ struct SweepArgs {
     uint32_t* published;           // [tiles][kRadix], all 0
     uint32_t* published_next;      // set to 0 for the next sweep (may be null)
     BuildCounts* counts;
+    int max_polls;                 // of one word, before a block gives up
 };
 
 // Degree class of a row: exact degree up to 8, then quarter octaves of (deg - 1) up to the hub
@@ -346,7 +348,10 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
         for (int i = tid; i < kWarps * kRadix / 4; i += kBlock) reinterpret_cast<int4*>(&sm.warp_count[0][0])[i] = make_int4(0, 0, 0, 0);
     };
 
-    if (tid == 0) sm.tile[0] = atomicAdd(a.ticket, 1);
+    if (tid == 0) {
+        const int first = atomicAdd(a.ticket, 1);
+        sm.tile[0] = load_published(reinterpret_cast<const uint32_t*>(&a.counts->sort_failed)) ? a.n_tiles : first;
+    }
     clear_counts();
     __syncthreads();
     int tile = sm.tile[0];
@@ -471,7 +476,7 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
             for (int q = 0; q < kOwn; ++q) {
                 const int d = tid + q * kBlock;
                 uint32_t before = 0;
-                if (look_back(a.published + d, tile, &a.counts->sort_failed, &before))
+                if (look_back(a.published + d, tile, a.max_polls, &a.counts->sort_failed, &before))
                     publish(published + d, kSumBit | (before + (uint32_t)total[q]));
                 else
                     ok = false;
@@ -515,6 +520,8 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 // looks after kUniqueItems consecutive candidates, a block after kUniqueTile.
 constexpr int kUniqueItems = 8;
 constexpr int kUniqueTile = kThreads * kUniqueItems;
+
+__device__ __forceinline__ int64_t sorted_candidates(const BuildCounts* counts) { return counts->sort_failed ? 0 : counts->n_valid; }
 
 // bit j of the result: candidate first + j is the first of a run of equal keys among the n_valid kept ones
 __device__ __forceinline__ uint32_t first_of_run_mask(const u64* __restrict__ keys, int64_t first, int64_t n_valid, int val_bits,
@@ -574,7 +581,7 @@ unique_tile_counts(const u64* __restrict__ keys, int val_bits, const BuildCounts
     __shared__ int32_t smem[kThreads / 32];
     u64 word[kUniqueItems];
     const int64_t first = (int64_t)blockIdx.x * kUniqueTile + (int64_t)threadIdx.x * kUniqueItems;
-    const int32_t mine = __popc(first_of_run_mask(keys, first, counts->n_valid, val_bits, word));
+    const int32_t mine = __popc(first_of_run_mask(keys, first, sorted_candidates(counts), val_bits, word));
     int32_t total;
     block_prefix_256(mine, &total, smem);
     if (threadIdx.x == 0) tile_count[blockIdx.x] = total;
@@ -591,7 +598,7 @@ compact_unique(const u64* __restrict__ keys, const int32_t* __restrict__ vals, c
     __shared__ int32_t kept_val[kUniqueTile];
     u64 word[kUniqueItems];
     const int64_t first = (int64_t)blockIdx.x * kUniqueTile + (int64_t)threadIdx.x * kUniqueItems;
-    const uint32_t mask = first_of_run_mask(keys, first, counts->n_valid, val_bits, word);
+    const uint32_t mask = first_of_run_mask(keys, first, sorted_candidates(counts), val_bits, word);
     int32_t total;
     int32_t pos = block_prefix_256(__popc(mask), &total, smem);
     // the kept candidates of the tile are gathered in shared memory so that they leave as one contiguous piece
@@ -971,6 +978,10 @@ static int launch_sweep(const char* name, SweepArgs& a, cudaStream_t s)
                                : launch_sweep_shape<SmallTile, SOURCE, HAS_VALS>(name, a, s);
 }
 
+// One-shot settings of the drill (see gnnfd_debug_build_fault): consumed by the next build on this thread.
+struct BuildDrill { int max_polls, sweep; };
+static thread_local BuildDrill t_drill = {kMaxPolls, -1};
+
 }  // namespace gnnfd
 
 extern "C" {
@@ -1001,6 +1012,8 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
                     gnnfd_csr_t** out)
 {
     using namespace gnnfd;
+    const BuildDrill drill = t_drill;
+    t_drill = BuildDrill{kMaxPolls, -1};
     if (!out) return GNNFD_INVALID_ARG;
     *out = nullptr;
     BuildLayout L;
@@ -1017,6 +1030,9 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     carve_scratch(sc, L, &S);
     if (!pc.ok || !sc.ok) return GNNFD_WORKSPACE_TOO_SMALL;
 
+    // the drill leaves out a sweep's first tile: another one has to be there to miss it
+    if (drill.sweep >= 0 && (drill.sweep > L.passes || (drill.sweep < L.passes ? L.n_tiles : L.row_tiles) < 2)) return GNNFD_INVALID_ARG;
+
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t m = L.m;
     GNNFD_CUDA_CHECK(cudaMemsetAsync(P.counts, 0, sizeof(BuildCounts), s));
@@ -1032,11 +1048,13 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     const int vb = L.val_bits;
     const bool packed = vb > 0;                     // values ride in the low bits of the keys
     GNNFD_CUDA_CHECK(cudaMemsetAsync(S.digit_count, 0, S.zero_bytes, s));
+    if (drill.sweep >= 0) GNNFD_CUDA_CHECK(cudaMemsetAsync(S.ticket + drill.sweep, 1, 1, s));      // tile 0 is never drawn
     SweepArgs sw{};
     sw.cand = Candidates{d_src, d_dst, n, e, m, flags, L.src_bits};
     sw.m = m;
     sw.val_bits = vb;
     sw.counts = P.counts;
+    sw.max_polls = drill.max_polls;
     if (m > 0) {
         const unsigned walkers = blocks_for(m, kHistTile) < 6u * kSmCount ? blocks_for(m, kHistTile) : 6u * kSmCount;
         const size_t hist_bytes = (size_t)L.passes * kRadix * sizeof(int32_t);
@@ -1152,6 +1170,14 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     h->seg_slot = P.seg_slot;
     h->hub_seg_ptr = P.hub_seg_ptr;
     *out = h;
+    return GNNFD_OK;
+}
+
+int gnnfd_debug_build_fault(int32_t max_polls, int32_t sweep)
+{
+    using namespace gnnfd;
+    if (max_polls < 0 || max_polls > kMaxPolls || sweep < 0) return GNNFD_INVALID_ARG;
+    t_drill = BuildDrill{max_polls ? max_polls : kMaxPolls, sweep};
     return GNNFD_OK;
 }
 

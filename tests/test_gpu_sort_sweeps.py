@@ -88,3 +88,50 @@ def test_equal_and_ordered_digits(g, m, kind):
     src, dst = {"one pair": (np.full(m, 4999), np.full(m, 17)), "one destination": (rng.integers(0, n, m), np.full(m, 3)),
                 "pairs in turn": (i // 2 % n, i // 3 % n), "sorted": (i * n // m, i * n // m)}[kind]
     check(g, n, src.astype(np.int32), dst.astype(np.int32), 0)
+
+
+# ------------------------------------------------------------------ the give-up path, drilled without a fault
+
+GUARD = 1 << 20
+
+
+def guarded(nbytes):
+    """a buffer of ones (leftover words that look like published sums) with guard bytes on both sides"""
+    whole = torch.full((nbytes + 2 * GUARD,), 0xFF, dtype=torch.uint8, device="cuda")
+    whole[:GUARD] = whole[GUARD + nbytes:] = 0xAB
+    return whole, whole[GUARD:GUARD + nbytes]
+
+
+# (vertices, candidates, passes): key and value in one word and apart
+@pytest.mark.parametrize("n,m,passes", [(70_001, 200_000, 4), ((1 << 22) + 3, 300_000, 6)])
+@pytest.mark.parametrize("sweep", ["first", "second", "last", "rows"])
+@pytest.mark.parametrize("flags", [0, DD | SL])
+def test_a_tile_that_is_never_published_ends_the_build_with_an_error(g, n, m, passes, sweep, flags):
+    rng = np.random.default_rng(m)
+    src, dst = (rng.integers(0, n, m).astype(np.int32) for _ in range(2))
+    ds, dd = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()
+    pb, sb = g.csr_workspace_bytes(n, m, flags)
+    (p_all, persistent), (s_all, scratch) = guarded(pb), guarded(sb)
+    g.debug_build_fault(1024, {"first": 0, "second": 1, "last": passes - 1, "rows": passes}[sweep])
+    with pytest.raises(g.GnnfdError) as err:
+        g.build_csr(n, ds, dd, flags, persistent=persistent, scratch=scratch)
+    assert err.value.status == g.CUDA_ERROR
+    torch.cuda.synchronize()
+    for whole, nbytes in ((p_all, pb), (s_all, sb)):
+        assert bool((whole[:GUARD] == 0xAB).all()) and bool((whole[GUARD + nbytes:] == 0xAB).all())
+    # the drill is one-shot: the next build, from the same buffers, is an ordinary one
+    csr = g.build_csr(n, ds, dd, flags, persistent=persistent, scratch=scratch)
+    row_ptr, col, perm = reference(n, src, dst, flags)
+    np.testing.assert_array_equal(csr.row_ptr.cpu().numpy(), row_ptr)
+    np.testing.assert_array_equal(csr.col_idx.cpu().numpy(), col)
+    np.testing.assert_array_equal(csr.perm.cpu().numpy(), perm)
+
+
+def test_the_drill_refuses_sweeps_that_nobody_would_miss(g):
+    src = torch.arange(3000, dtype=torch.int32, device="cuda")
+    for sweep in (0, 9):                                             # one tile of edges only; no such sweep
+        g.debug_build_fault(1024, sweep)
+        with pytest.raises(g.GnnfdError) as err:
+            g.build_csr(3000, src[:2000], src[1000:], 0)
+        assert err.value.status == g.INVALID_ARG
+    assert g.build_csr(3000, src[:2000], src[1000:], 0).nnz == 2000
