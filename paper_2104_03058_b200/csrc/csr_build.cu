@@ -256,6 +256,14 @@ static int64_t sweep_tiles(int64_t m)
     const int keys = use_large_tile(m) ? tile_keys<LargeTile>() : tile_keys<SmallTile>();
     return m > 0 ? (m + keys - 1) / keys : 1;
 }
+// Tiles to reserve words for: at least those of the largest input in small tiles, where this one is in large tiles, so that
+// buffers sized for an input hold every smaller one.
+static int64_t reserved_tiles(int64_t m)
+{
+    constexpr int64_t kMostSmall = (int64_t)4 * kSmCount * tile_keys<LargeTile>() / tile_keys<SmallTile>();
+    const int64_t tiles = sweep_tiles(m);
+    return use_large_tile(m) && tiles < kMostSmall ? kMostSmall : tiles;
+}
 
 template <typename Shape>
 struct SweepSmem {
@@ -839,6 +847,7 @@ struct BuildLayout {
     int64_t m;             // candidate edges
     int64_t n_tiles;       // tiles of an edge sweep
     int64_t row_tiles;     // tiles of the row (degree class) sweep
+    int64_t tile_cap, row_tile_cap;      // tiles that words are reserved for
     int64_t hub_cap;       // upper bound on hub rows
     int64_t seg_cap;       // upper bound on hub segments
     int src_bits, key_bits, passes, digit_bits;
@@ -864,6 +873,8 @@ static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L)
     L->m = m;
     L->n_tiles = sweep_tiles(m);
     L->row_tiles = sweep_tiles(n);
+    L->tile_cap = reserved_tiles(m);
+    L->row_tile_cap = reserved_tiles(n);
     L->hub_cap = m / (GNNFD_HUB_DEGREE + 1) + 1;
     // source ranges of GNNFD_HUB_RANGE_ROWS vertices, at most 64 of them (narrower ranges would keep a band of x
     // resident in L2, but on the RMAT workload the extra, shorter segments cost more than the saved traffic: 32
@@ -950,10 +961,10 @@ static void carve_scratch(Carver& c, const BuildLayout& L, ScratchPtrs* p)
     const size_t zero_begin = c.off;
     p->digit_count = c.take<int32_t>((size_t)(L.passes + 1) * kRadix);
     p->ticket = c.take<int32_t>((size_t)L.passes + 1);
-    p->row_published = c.take<uint32_t>((size_t)kRadix * L.row_tiles);
-    p->published = c.take<uint32_t>((size_t)kRadix * L.n_tiles);
-    p->zero_bytes = c.off - zero_begin;
-    p->published_alt = c.take<uint32_t>((size_t)kRadix * L.n_tiles);
+    p->row_published = c.take<uint32_t>((size_t)kRadix * L.row_tile_cap);
+    p->zero_bytes = c.off - zero_begin + (size_t)kRadix * L.n_tiles * sizeof(uint32_t);
+    p->published = c.take<uint32_t>((size_t)kRadix * L.tile_cap);
+    p->published_alt = c.take<uint32_t>((size_t)kRadix * L.tile_cap);
     const size_t fl = flag_ints(L);
     p->flags = c.take<int32_t>(fl);
     p->scan_temp = c.take<int32_t>(scan_temp_ints(fl));
