@@ -482,6 +482,16 @@ def gat_workspace_bytes(csr: Csr, heads: int, dim: int) -> int:
     return s.value
 
 
+def gat_best_workspace_bytes(csr: Csr, z: torch.Tensor, heads: int, dim: int, chunk_width: int | None = None) -> int:
+    """Scratch with which the attention aggregation of these features is fastest (at least gat_workspace_bytes)."""
+    f = heads * dim
+    zp, ldz = _matrix(z, f, "z")
+    s = ctypes.c_size_t()
+    _check(lib().gnnfd_gat_best_workspace_bytes(csr.handle, zp, ldz, _dtype_code(z), heads, dim, f if chunk_width is None else chunk_width,
+                                                ctypes.byref(s)), "gnnfd_gat_best_workspace_bytes")
+    return s.value
+
+
 def aggregate_gat(csr: Csr, z: torch.Tensor, a_src: torch.Tensor, a_dst: torch.Tensor, heads: int, dim: int,
                   negative_slope: float = 0.2, chunk_width: int | None = None, out: torch.Tensor | None = None,
                   out_dtype=None, scratch=None, stream=None) -> torch.Tensor:

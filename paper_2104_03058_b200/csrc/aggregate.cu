@@ -428,12 +428,11 @@ align_features(const T* __restrict__ x, int64_t ldx, int64_t n, int32_t f, int32
     out[idx] = u.v;
 }
 
-// Each row has to be gathered a few times, and the launch has to be won back.  fp32 GCN, element-wise loads -> copy and vector loads:
-// 100,000 rows of 4 entries and a loop, 41 columns 65 -> 37 us; 41 columns, 33 MB gathered, 17.8 -> 19.7 us; 100 columns, 56 MB,
-// 34 -> 29 us.
-bool copy_pays(const gnnfd_csr_t* csr, int64_t gathered_bytes)
+// Each row has to be gathered a few times, and the launch has to be won back within one chunk.  `per_entry` is what an entry of
+// the chunk costs without the copy.
+bool copy_pays(const gnnfd_csr_t* csr, int64_t per_entry, int64_t least)
 {
-    return csr->nnz >= 4 * csr->n && gathered_bytes >= (int64_t)40 << 20;
+    return csr->nnz >= 4 * csr->n && csr->nnz * per_entry >= least;
 }
 
 AlignedCopy layout_copy(int64_t n, gnnfd_dtype_t xdt, int32_t f, int32_t cw, int32_t unit_bytes, int32_t row_bytes)
@@ -464,18 +463,26 @@ static bool aligned_for_vectors(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt,
     return ((uintptr_t)d_x % 16 == 0) && ((ldx * xsize) % 16 == 0) && (f <= cw || (cw * xsize) % 16 == 0);
 }
 
-// bf16 always gains from vectors, fp32 from where the scalar kernel needs a whole warp for 64 columns (33 up): 200,000 rows of
-// 150 entries, 25 / 41 / 301 fp32 columns 0.45 / 0.67 / 4.69 -> 0.49 / 0.56 / 3.34 ms, 9 / 41 / 301 bf16 columns 0.40 / 0.73 /
-// 3.91 -> 0.24 / 0.50 / 1.95 ms.
+// Where the copy is faster than element-wise loads: fp32 from where those need a whole warp for 64 columns (33 up), bf16 from 3
+// columns, below which the padding to 16 bytes outweighs the loads.  132,534 rows of 300 entries, loads -> copy: bf16 1 / 2 / 3 / 5 / 9 /
+// 41 columns 113 / 170 / 221 / 281 / 387 / 866 -> 182 / 182 / 183 / 184 / 240 / 443 us, 301 in chunks of 4 17.7 -> 15.7 ms, fp32
+// 33 / 41 / 301 columns 803 / 806 / 5410 -> 636 / 644 / 3704 us; 200,000 rows of 150, 25 fp32 columns 0.45 -> 0.49 ms.
 static AlignedCopy plan_copy(const gnnfd_csr_t* csr, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f, int32_t cw)
 {
     const int xsize = xdt == GNNFD_F32 ? 4 : 2;
-    if (aligned_for_vectors(d_x, ldx, xdt, f, cw) || (xsize == 4 && cw <= 32) || !copy_pays(csr, csr->nnz * cw * xsize))
-        return AlignedCopy{cw, ldx, 0};
-    // Chunks start on 32-byte sectors.  Rows of more than a line start on one where they are gathered often enough to make up for
-    // the larger copy (41 fp32 columns on 116 M entries: pitch 48 1.78 ms, 64 1.69; on 200,000 rows of 16 entries 93 and 97 us).
+    if (aligned_for_vectors(d_x, ldx, xdt, f, cw) || cw <= (xsize == 4 ? 32 : 2)) return AlignedCopy{cw, ldx, 0};
+    // In lanes that the element-wise kernel puts on an entry (two columns each).  Loads -> copy: 50,000 rows of 9 entries, 41 bf16
+    // columns (14 M) 41 -> 29 us; 200,000 of 17, 7 columns (14 M) 41 -> 38, 4 columns (7 M) 33 -> 35; 5,000 of 51, 41 fp32 columns (8 M)
+    // 15 -> 18.
+    int64_t lanes = 1;
+    while (lanes < 32 && 2 * lanes < cw) lanes <<= 1;
+    if (!copy_pays(csr, lanes * ((cw + 63) / 64), 10000000)) return AlignedCopy{cw, ldx, 0};
+    // Chunks of one vector start on 16 bytes, wider ones on 32-byte sectors, so the copy is at most 2.7 times the features.  Rows
+    // of more than a line start on one where they are gathered often enough to make up for the larger copy (41 fp32 columns
+    // on 116 M entries: pitch 48 1.78 ms, 64 1.69; on 200,000 rows of 16 entries 93 and 97 us).
+    const int unit = cw * xsize <= 16 ? 16 : 32;
     const bool lines = csr->nnz >= 64 * csr->n && (int64_t)f * xsize > 128;
-    return layout_copy(csr->n, xdt, f, cw, 32, lines ? 128 : 32);
+    return layout_copy(csr->n, xdt, f, cw, unit, lines ? 128 : unit);
 }
 
 static size_t partial_bytes(const gnnfd_csr_t* csr, int32_t f)

@@ -93,7 +93,7 @@ struct AlignedCopy {
     int64_t ld;          // row pitch
     size_t bytes;        // 0: no copy
 };
-bool copy_pays(const gnnfd_csr_t* csr, int64_t gathered_bytes);
+bool copy_pays(const gnnfd_csr_t* csr, int64_t per_entry, int64_t least);
 AlignedCopy layout_copy(int64_t n, gnnfd_dtype_t xdt, int32_t f, int32_t cw, int32_t unit_bytes, int32_t row_bytes);
 void launch_copy(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int64_t n, int32_t f, int32_t cw, const AlignedCopy& copy,
                  void* d_aligned, cudaStream_t s);

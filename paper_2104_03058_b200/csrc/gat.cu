@@ -508,18 +508,23 @@ static int launch_scores(int64_t n, const void* d_z, int64_t ldz, gnnfd_dtype_t 
 }
 
 // A copy of z whose heads are padded to whole 16-byte vectors, for heads that are not (7 fp32 or 4 bf16 columns): the vector
-// kernels need a vector to stay inside one head.  Heads are the copy's chunks, so the sweeps have to hold whole heads.  200,000
-// rows of 150 entries, 8 x 7 fp32 1.66 -> 0.66 ms, 8 x 7 bf16 1.71 -> 0.50, 6 x 4 bf16 0.65 -> 0.48; 100,000 rows of 4, 4 x 7
-// fp32 118 -> 38 us; a single head of 4 bf16 columns, one load as it is, 0.235 -> 0.243 ms, stays.
+// kernels need a vector to stay inside one head.  Heads are the copy's chunks, so the sweeps have to hold whole heads.  132,534
+// rows of 300 entries, 8 x 3 / 5 / 7 fp32 1.03 / 2.02 / 2.02 -> 0.43 / 0.71 / 0.72 ms, bf16 1.06 / 2.09 / 2.09 -> 0.54 / 0.55 / 0.55;
+// 100,000 rows of 4, 4 x 7 fp32 118 -> 38 us.  Not for heads of one or two columns (8 x 1 fp32 367 -> 428 us, 8 x 2 bf16 474 -> 542;
+// on 200,000 rows of 17 8 x 2 fp32 81 -> 90, 32 x 2 286 -> 344), so z grows by 8/3 at most, nor for chunks of up to four
+// columns (1 x 3 fp32 273 -> 281; 1 x 5 363 -> 307).
 static AlignedCopy plan_head_copy(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads, int32_t dim,
                                   int32_t cw)
 {
     const int zsize = zdt == GNNFD_F32 ? 4 : 2;
     const int32_t f = heads * dim;
     cw = cw < f ? cw : f;
+    const int32_t vecn = 16 / zsize;
     const bool aligned = (uintptr_t)d_z % 16 == 0 && ldz * zsize % 16 == 0 && dim * zsize % 16 == 0;
-    if (aligned || (cw < f && cw % dim != 0) || cw * zsize <= 8 || !copy_pays(csr, csr->nnz * cw * zsize)) return AlignedCopy{dim, ldz, 0};
-    return layout_copy(csr->n, zdt, f, dim, 16, 32);
+    // In elements, each of which costs a load, a logit and an exponential.  Loads -> copy: 50,000 rows of 9 entries, 4 x 5 fp32 (9 M)
+    // 49 -> 29 us; 200,000 of 6, 1 x 7 bf16 (8 M) 49 -> 39; 20,000 of 51, 1 x 7 bf16 (7 M) 25 -> 29.
+    if (aligned || (cw < f && cw % dim != 0) || cw <= 4 || dim <= 2 || !copy_pays(csr, cw, 8000000)) return AlignedCopy{dim, ldz, 0};
+    return layout_copy(csr->n, zdt, f, dim, 16, f <= vecn ? 16 : 32);
 }
 
 size_t gat_copy_bytes(const gnnfd_csr_t* csr, const void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int32_t heads, int32_t dim,

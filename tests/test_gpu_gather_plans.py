@@ -99,6 +99,69 @@ def test_padded_heads(g, graph, dtype, heads, dim, ld, cw):
         assert (np.abs(t.cpu().numpy() - want) <= 1e-5 * scale + 1e-6).all()
 
 
+@pytest.fixture(scope="module")
+def long_graph(g):
+    rng = np.random.default_rng(6)
+    n, e = 5000, 7_100_000                                  # 4 columns put 14 M lanes on a chunk: copies start at 10 M
+    dst = np.where(rng.random(e) < 0.001, 7, rng.integers(0, n - 1, e)).astype(np.int32)
+    src = rng.integers(0, n, e).astype(np.int32)
+    row_ptr, col, _ = orc.build_csr(n, src, dst, 0)
+    return g.build_csr(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda()), row_ptr, col
+
+
+# Which features get an aligned copy, and how large it may be: from 3 bf16 / 33 fp32 columns and at most 8/3 of the features; heads
+# of three columns or more in chunks of more than four.
+@pytest.mark.parametrize("dtype,f,ld,cw,copied", [
+    (torch.bfloat16, 17, 17, 1, False), (torch.bfloat16, 17, 17, 2, False), (torch.bfloat16, 19, 21, 3, True), (torch.bfloat16, 5, 5, 5, True),
+    (torch.bfloat16, 23, 23, 7, True), (torch.bfloat16, 23, 23, 8, True), (torch.bfloat16, 26, 27, 9, True), (torch.bfloat16, 41, 41, 41, True),
+    (torch.float32, 65, 65, 32, False), (torch.float32, 66, 67, 33, True), (torch.float32, 40, 41, 40, True)])
+@pytest.mark.parametrize("model", ["gcn", "sage"])
+def test_what_is_copied(g, long_graph, model, dtype, f, ld, cw, copied):
+    csr, row_ptr, col = long_graph
+    fn = {"gcn": g.aggregate_gcn, "sage": g.aggregate_sage}[model]
+    x = torch.full((csr.n, ld), float("nan"), dtype=dtype)
+    x[:, :f] = torch.randn((csr.n, f), generator=torch.Generator().manual_seed(f)).to(dtype)
+    x = x.cuda()
+    small, best = g.aggregate_workspace_bytes(csr, f), g.aggregate_best_workspace_bytes(csr, x, f, cw)
+    size = csr.n * f * x.element_size()
+    assert (best > small) == copied and best - small <= 8 / 3 * size + csr.n * 128 + 256
+    plain, got = fn(csr, x, f=f, chunk_width=cw, scratch=scratch(max(small, 256))), fn(csr, x, f=f, chunk_width=cw)
+    if copied:
+        assert torch.equal(plain, fn(csr, x, f=f, chunk_width=cw, scratch=scratch(best - 256)))
+    else:
+        assert torch.equal(plain, got)
+    want, scale = orc.aggregate(model, row_ptr, col, np.ascontiguousarray(x[:, :f].float().cpu().numpy()), f)
+    for t in (plain, got):
+        assert (np.abs(t.cpu().numpy() - want) <= 1e-5 * scale + 1e-6).all()
+
+
+@pytest.mark.parametrize("dtype,heads,dim,ld,cw,copied", [
+    (torch.float32, 8, 1, 8, 8, False), (torch.float32, 64, 1, 64, 64, False), (torch.bfloat16, 8, 1, 8, 8, False),
+    (torch.bfloat16, 8, 2, 16, 16, False), (torch.float32, 1, 3, 3, 3, False), (torch.bfloat16, 1, 4, 4, 4, False),
+    (torch.float32, 8, 2, 16, 18, False), (torch.float32, 32, 2, 65, 64, False), (torch.float32, 5, 3, 15, 15, True), (torch.bfloat16, 5, 3, 15, 15, True),
+    (torch.bfloat16, 1, 5, 5, 5, True), (torch.bfloat16, 6, 4, 24, 24, True), (torch.float32, 4, 7, 32, 7, True),
+    (torch.bfloat16, 4, 7, 28, 14, True), (torch.float32, 4, 7, 28, 10, False), (torch.float32, 6, 4, 24, 24, False)])
+def test_which_heads_are_padded(g, long_graph, dtype, heads, dim, ld, cw, copied):
+    csr, row_ptr, col = long_graph
+    f = heads * dim
+    gen = torch.Generator().manual_seed(f)
+    z = torch.full((csr.n, ld), float("nan"), dtype=dtype)
+    z[:, :f] = torch.randn((csr.n, f), generator=gen).to(dtype)
+    a = [torch.randn((heads, dim), generator=gen) * 0.3 for _ in range(2)]
+    dev = [t.cuda() for t in (z, *a)]
+    small, best = g.gat_workspace_bytes(csr, heads, dim), g.gat_best_workspace_bytes(csr, dev[0], heads, dim, cw)
+    assert (best > small) == copied
+    plain = g.aggregate_gat(csr, *dev, heads, dim, 0.2, chunk_width=cw, scratch=scratch(small))
+    got = g.aggregate_gat(csr, *dev, heads, dim, 0.2, chunk_width=cw)
+    if copied:
+        assert torch.equal(plain, g.aggregate_gat(csr, *dev, heads, dim, 0.2, chunk_width=cw, scratch=scratch(best - 256)))
+    else:
+        assert torch.equal(plain, got)
+    want, scale = orc.aggregate_gat(row_ptr, col, np.ascontiguousarray(z[:, :f].float().numpy()), a[0].numpy(), a[1].numpy(), heads, dim, 0.2)
+    for t in (plain, got):
+        assert (np.abs(t.cpu().numpy() - want) <= 1e-5 * scale + 1e-6).all()
+
+
 # Rows of lengths around the octave bounds of the shared classes (a row of up to 256 / 512 / 1024 / 2048 entries is one, two, four or
 # eight warps' work when the graph is small), hub rows, and enough short rows beside them.
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
