@@ -350,6 +350,10 @@ int gnnfd_combine_ex(int64_t n, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt,
 int gnnfd_layer_workspace_bytes(const gnnfd_csr_t* csr, int model, int32_t f_out, int32_t heads, int32_t dim,
                                 gnnfd_dtype_t xdt, size_t* scratch_bytes);
 
+/* As gnnfd_gat_best_workspace_bytes: room for a copy of z with padded heads, where gnnfd_layer_gat is faster with one. */
+int gnnfd_layer_best_workspace_bytes(const gnnfd_csr_t* csr, int model, int32_t f_out, int32_t heads, int32_t dim,
+                                     gnnfd_dtype_t xdt, int32_t chunk_width, size_t* scratch_bytes);
+
 int gnnfd_layer_gcn(const gnnfd_csr_t* csr, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f_in,
                     const void* d_w_t, int64_t ldw, int32_t f_out, int mode, void* d_out, int64_t ldo, gnnfd_dtype_t odt,
                     int32_t chunk_width, void* d_scratch, size_t scratch_bytes, int32_t* d_status, void* stream);

@@ -77,6 +77,7 @@ def lib() -> ctypes.CDLL:
         L.gnnfd_combine_ex.argtypes = [i64, vp, i64, i32, i32, vp, i64, i32, vp, i64, i32, ctypes.c_int, vp, vp, i32, i32,
                                        vp, vp, vp, vp]
         L.gnnfd_layer_workspace_bytes.argtypes = [vp, ctypes.c_int, i32, i32, i32, i32, pp(sz)]
+        L.gnnfd_layer_best_workspace_bytes.argtypes = [vp, ctypes.c_int, i32, i32, i32, i32, i32, pp(sz)]
         layer = [vp, vp, i64, i32, i32, vp, i64, i32, ctypes.c_int, vp, i64, i32, i32, vp, sz, vp, vp]
         L.gnnfd_layer_gcn.argtypes = layer
         L.gnnfd_layer_sage.argtypes = layer
@@ -133,6 +134,20 @@ def _alloc_bytes(nbytes: int, device, stream=None) -> torch.Tensor:
         return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
     with torch.cuda.stream(stream):
         return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
+
+
+def _alloc_best(best: int, least, device, stream=None):
+    """`best` bytes of scratch or, where the device has no room for them, the `least()` bytes that the call needs (the library then
+    does without its aligned copy).  None for no bytes at all."""
+    if best == 0:
+        return None
+    try:
+        return _alloc_bytes(best, device, stream)
+    except torch.OutOfMemoryError:
+        need = least()
+        if need >= best:
+            raise
+    return _alloc_bytes(need, device, stream) if need else None
 
 
 def _same_device(csr_device, **tensors):
@@ -308,8 +323,7 @@ def _aggregate(fn, name, csr: Csr, x, f, chunk_width, out, out_dtype, scratch, s
     if scratch is None:
         need = ctypes.c_size_t()
         _check(lib().gnnfd_aggregate_best_workspace_bytes(csr.handle, xp, ldx, xdt, f, chunk_width, ctypes.byref(need)), name)
-        if need.value:
-            scratch = _alloc_bytes(need.value, x.device, stream)
+        scratch = _alloc_best(need.value, lambda: aggregate_workspace_bytes(csr, f), x.device, stream)
     sp, sn = _scratch_args(scratch, csr.device)
     _check(fn(csr.handle, xp, ldx, xdt, op, ldo, _dtype_code(out), f, chunk_width, sp, sn, _stream_ptr(stream)), name)
     return out
@@ -417,8 +431,7 @@ def tune_chunk_width(csr: Csr, x: torch.Tensor, model: str = "gcn", f: int | Non
     _check_aggregate_operands(csr, x, out, f)
     if scratch is None:
         need = max([aggregate_best_workspace_bytes(csr, x, f, w) for w in candidates if w > 0], default=0)
-        if need:
-            scratch = _alloc_bytes(need, x.device, stream)
+        scratch = _alloc_best(need, lambda: aggregate_workspace_bytes(csr, f), x.device, stream)
     _same_device(csr.device, scratch=scratch)
     sp = scratch.data_ptr() if scratch is not None else None
     sn = scratch.numel() * scratch.element_size() if scratch is not None else 0
@@ -508,7 +521,7 @@ def aggregate_gat(csr: Csr, z: torch.Tensor, a_src: torch.Tensor, a_dst: torch.T
         need = ctypes.c_size_t()
         _check(lib().gnnfd_gat_best_workspace_bytes(csr.handle, zp, ldz, _dtype_code(z), heads, dim, chunk_width,
                                                     ctypes.byref(need)), "gnnfd_aggregate_gat")
-        scratch = _alloc_bytes(need.value, z.device, stream)
+        scratch = _alloc_best(need.value, lambda: gat_workspace_bytes(csr, heads, dim), z.device, stream)
     _same_device(csr.device, scratch=scratch)
     _check(lib().gnnfd_aggregate_gat(csr.handle, zp, ldz, _dtype_code(z), a_src.data_ptr(),
                                      a_dst.data_ptr(), heads, dim, negative_slope, op, ldo,
@@ -610,6 +623,16 @@ def layer_workspace_bytes(csr: Csr, model: str, f_out: int, heads: int = 0, dim:
     return s.value
 
 
+def layer_best_workspace_bytes(csr: Csr, model: str, f_out: int, heads: int = 0, dim: int = 0, dtype=torch.float32,
+                               chunk_width: int | None = None) -> int:
+    """Scratch with which a layer is fastest (at least layer_workspace_bytes)."""
+    s = ctypes.c_size_t()
+    _check(lib().gnnfd_layer_best_workspace_bytes(csr.handle, {"gcn": 0, "sage": 1, "gat": 2}[model], f_out, heads, dim,
+                                                  F32 if dtype == torch.float32 else BF16, f_out if chunk_width is None else chunk_width,
+                                                  ctypes.byref(s)), "gnnfd_layer_best_workspace_bytes")
+    return s.value
+
+
 def layer(csr: Csr, model: str, x: torch.Tensor, w_t: torch.Tensor, f_in: int | None = None, mode="tf32",
           chunk_width: int | None = None, out: torch.Tensor | None = None, out_dtype=None, a_src=None, a_dst=None,
           heads: int = 0, dim: int = 0, negative_slope: float = 0.2, scratch=None, status=None, stream=None):
@@ -635,7 +658,8 @@ def layer(csr: Csr, model: str, x: torch.Tensor, w_t: torch.Tensor, f_in: int | 
         _no_overlap(x, out, "x", "out")
         _no_overlap(w_t, out, "w_t", "out")
     if scratch is None:
-        scratch = _alloc_bytes(layer_workspace_bytes(csr, model, f_out, heads, dim, x.dtype), x.device, stream)
+        scratch = _alloc_best(layer_best_workspace_bytes(csr, model, f_out, heads, dim, x.dtype, chunk_width),
+                              lambda: layer_workspace_bytes(csr, model, f_out, heads, dim, x.dtype), x.device, stream)
     _same_device(csr.device, scratch=scratch)
     sp = status.data_ptr() if status is not None else None
     scr, scr_n = scratch.data_ptr(), scratch.numel() * scratch.element_size()

@@ -36,6 +36,18 @@ static int layer_sum(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
 
 extern "C" {
 
+int gnnfd_layer_best_workspace_bytes(const gnnfd_csr_t* csr, int model, int32_t f_out, int32_t heads, int32_t dim,
+                                     gnnfd_dtype_t xdt, int32_t chunk_width, size_t* scratch_bytes)
+{
+    using namespace gnnfd;
+    int rc = gnnfd_layer_workspace_bytes(csr, model, f_out, heads, dim, xdt, scratch_bytes);
+    if (rc) return rc;
+    if (chunk_width <= 0) return GNNFD_INVALID_ARG;
+    // z is aligned, its heads may not be
+    if (model == 2) *scratch_bytes += gat_copy_bytes(csr, nullptr, z_pitch(heads * dim), xdt, heads, dim, chunk_width);
+    return GNNFD_OK;
+}
+
 int gnnfd_layer_workspace_bytes(const gnnfd_csr_t* csr, int model, int32_t f_out, int32_t heads, int32_t dim,
                                 gnnfd_dtype_t xdt, size_t* scratch_bytes)
 {
@@ -48,7 +60,6 @@ int gnnfd_layer_workspace_bytes(const gnnfd_csr_t* csr, int model, int32_t f_out
         if (heads <= 0 || dim <= 0 || (int64_t)heads * dim > 0x7fffffffll) return GNNFD_INVALID_ARG;
         f_out = heads * dim;
         rc = gnnfd_gat_workspace_bytes(csr, heads, dim, &rest);
-        if (!rc) rest += gat_copy_bytes(csr, nullptr, z_pitch(f_out), xdt, heads, dim, f_out);       // z is aligned, its heads may not be
     } else {
         if (f_out <= 0) return GNNFD_INVALID_ARG;
         rc = gnnfd_aggregate_workspace_bytes(csr, f_out, &rest);

@@ -64,3 +64,20 @@ def test_attention_vector_shape_is_checked():
         b._attention_vectors(torch.zeros(2, 2), torch.zeros(2, 3), 2, 3, torch.device("cpu"), None)
     a, c = b._attention_vectors(torch.zeros(2, 3, dtype=torch.float64), torch.ones(2, 3), 2, 3, torch.device("cpu"), None)
     assert a.dtype == torch.float32 and c.dtype == torch.float32
+
+
+def test_scratch_falls_back_to_what_the_call_needs(monkeypatch):
+    sizes = []
+
+    def alloc(nbytes, device, stream=None):
+        sizes.append(nbytes)
+        if nbytes > 1000:
+            raise torch.OutOfMemoryError("no room")
+        return nbytes
+    monkeypatch.setattr(b, "_alloc_bytes", alloc)
+    assert b._alloc_best(900, lambda: 1 / 0, "cpu") == 900                       # the second size is not even asked for
+    assert b._alloc_best(5000, lambda: 600, "cpu") == 600 and b._alloc_best(5000, lambda: 0, "cpu") is None
+    assert b._alloc_best(0, lambda: 1 / 0, "cpu") is None
+    with pytest.raises(torch.OutOfMemoryError):
+        b._alloc_best(5000, lambda: 5000, "cpu")                                 # nothing smaller would do
+    assert sizes == [900, 5000, 600, 5000, 5000]

@@ -162,6 +162,33 @@ def test_which_heads_are_padded(g, long_graph, dtype, heads, dim, ld, cw, copied
         assert (np.abs(t.cpu().numpy() - want) <= 1e-5 * scale + 1e-6).all()
 
 
+def test_calls_do_without_the_copy_where_there_is_no_room(g, long_graph, monkeypatch):
+    csr, _, _ = long_graph
+    gen = torch.Generator().manual_seed(1)
+    x = torch.randn((csr.n, 41), generator=gen).cuda()
+    z, a = torch.randn((csr.n, 28), generator=gen).cuda(), [torch.randn((4, 7), generator=gen).cuda() * 0.3 for _ in range(2)]
+    feats, w_t = torch.randn((csr.n, 32), generator=gen).cuda(), torch.randn((28, 32), generator=gen).cuda()
+    layer = dict(a_src=a[0], a_dst=a[1], heads=4, dim=7, mode="fp32")
+    sizes = {"gcn": (g.aggregate_workspace_bytes(csr, 41), g.aggregate_best_workspace_bytes(csr, x)),
+             "gat": (g.gat_workspace_bytes(csr, 4, 7), g.gat_best_workspace_bytes(csr, z, 4, 7)),
+             "layer": (g.layer_workspace_bytes(csr, "gat", 28, 4, 7), g.layer_best_workspace_bytes(csr, "gat", 28, 4, 7))}
+    assert all(best > least for least, best in sizes.values())
+    plain = [g.aggregate_gcn(csr, x, scratch=scratch(sizes["gcn"][0])), g.aggregate_gat(csr, z, *a, 4, 7, scratch=scratch(sizes["gat"][0])),
+             g.layer(csr, "gat", feats, w_t, scratch=scratch(sizes["layer"][0]), **layer)]
+    copied = [g.aggregate_gcn(csr, x), g.aggregate_gat(csr, z, *a, 4, 7), g.layer(csr, "gat", feats, w_t, **layer)]
+    alloc, largest = g.binding._alloc_bytes, {least for least, _ in sizes.values()}
+
+    def no_room(nbytes, device, stream=None):
+        if nbytes not in largest:
+            raise torch.OutOfMemoryError("no room")
+        return alloc(nbytes, device, stream)
+    monkeypatch.setattr(g.binding, "_alloc_bytes", no_room)
+    got = [g.aggregate_gcn(csr, x), g.aggregate_gat(csr, z, *a, 4, 7), g.layer(csr, "gat", feats, w_t, **layer)]
+    assert g.tune_chunk_width(csr, x, candidates=[41, 20])[0] in (41, 20)
+    for p, c, t in zip(plain, copied, got):
+        assert torch.equal(p, t) and not torch.equal(p, c) and torch.allclose(p, c, rtol=1e-3, atol=1e-4)
+
+
 # Rows of lengths around the octave bounds of the shared classes (a row of up to 256 / 512 / 1024 / 2048 entries is one, two, four or
 # eight warps' work when the graph is small), hub rows, and enough short rows beside them.
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
