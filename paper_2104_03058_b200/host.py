@@ -56,6 +56,22 @@ class HostPipeline:
             self.ev_in[slot].record(self.s_in)
         return slot, e
 
+    def _job_scratch(self, x):
+        """Workspace of the current job's aggregation.  It depends on the graph's hub rows, so it is asked for per job, and the buffer
+        behind it grows when needed (torch frees the old one in stream order: the previous job's kernels may still use it).  The
+        job gets exactly its own size: whether unaligned features are copied, and with it the last bits of the sums, goes by
+        the size, which must not depend on the jobs before."""
+        if self.model == "gat":
+            best = g.gat_best_workspace_bytes(self.csr, x, self.heads, self.dim, self.chunk_width)
+            least = g.gat_workspace_bytes(self.csr, self.heads, self.dim)
+        else:
+            best = g.aggregate_best_workspace_bytes(self.csr, x, self.f, self.chunk_width)
+            least = g.aggregate_workspace_bytes(self.csr, self.f)
+        best, least = max(best, 256), max(least, 256)
+        if self.agg_scratch is None or self.agg_scratch.numel() < best:
+            self.agg_scratch = g._alloc_best(best, lambda: least, self.device)
+        return self.agg_scratch[:best if self.agg_scratch.numel() >= best else least]
+
     def submit(self, h_src, h_dst, h_x, h_out, next_job=None):
         """Runs one job.  ``next_job`` = (h_src, h_dst, h_x) of the following job, if known: its copies
         are enqueued before this job's kernels so that they overlap them."""
@@ -71,23 +87,15 @@ class HostPipeline:
             self.csr.destroy()
         self.csr = g.build_csr(self.n, self.d_src[slot][:e], self.d_dst[slot][:e], self.flags,
                                persistent=self.persistent, scratch=self.scratch)
-        # the workspace depends on this graph's hub rows, so it is asked for per job and grown when needed
-        # (the old buffer may still be in use by the previous job's kernels on this stream: torch frees it
-        # in stream order)
-        need = (g.gat_workspace_bytes(self.csr, self.heads, self.dim) if self.model == "gat"
-                else g.aggregate_workspace_bytes(self.csr, self.f))
-        if self.agg_scratch is None or self.agg_scratch.numel() < need:
-            self.agg_scratch = torch.empty(max(need, 256), dtype=torch.uint8, device=self.device)
+        scratch = self._job_scratch(self.d_x[slot])
         out = self.d_out[slot][:, :self.f]
         if self.model == "gat":
             g.aggregate_gat(self.csr, self.d_x[slot], self.a_src, self.a_dst, self.heads, self.dim,
-                            self.negative_slope, chunk_width=self.chunk_width, out=out, scratch=self.agg_scratch)
+                            self.negative_slope, chunk_width=self.chunk_width, out=out, scratch=scratch)
         elif self.model == "sage":
-            g.aggregate_sage(self.csr, self.d_x[slot], f=self.f, chunk_width=self.chunk_width, out=out,
-                             scratch=self.agg_scratch)
+            g.aggregate_sage(self.csr, self.d_x[slot], f=self.f, chunk_width=self.chunk_width, out=out, scratch=scratch)
         else:
-            g.aggregate_gcn(self.csr, self.d_x[slot], f=self.f, chunk_width=self.chunk_width, out=out,
-                            scratch=self.agg_scratch)
+            g.aggregate_gcn(self.csr, self.d_x[slot], f=self.f, chunk_width=self.chunk_width, out=out, scratch=scratch)
         self.ev_done[slot].record(cur)
         with torch.cuda.stream(self.s_out):
             self.s_out.wait_event(self.ev_done[slot])

@@ -429,6 +429,24 @@ def test_host_pipeline_grows_its_workspace_for_a_graph_with_more_hub_rows(g):
         assert torch.equal(out, g.aggregate_gcn(csr, h_x.cuda(), f=f, chunk_width=4).cpu())
 
 
+def test_host_pipeline_results_do_not_depend_on_earlier_jobs(g):
+    """Features without padding are gathered from an aligned copy; a job between with many hub rows grows the pipeline's workspace."""
+    from paper_2104_03058_b200.host import HostPipeline
+    n, f, most = 5000, 41, 6_500_000
+    rng = np.random.default_rng(2)
+    x = torch.randn((n, f), generator=torch.Generator().manual_seed(2)).pin_memory()
+    small, large = ([torch.from_numpy(rng.integers(0, k, e).astype(np.int32)).pin_memory() for k in (n, rows)]
+                    for e, rows in ((400_000, n), (most, 500)))
+    pipe = HostPipeline(n, most, f, f, 0, f)
+    outs = [torch.empty((n, f)).pin_memory() for _ in range(3)]
+    for job, out in zip((small, large, small), outs):
+        csr = pipe.submit(*job, x, out)
+    pipe.finish()
+    torch.cuda.synchronize()
+    assert g.aggregate_best_workspace_bytes(csr, x.cuda()) > g.aggregate_workspace_bytes(csr, f)
+    assert torch.equal(outs[0], outs[2]) and torch.equal(outs[0], g.aggregate_gcn(csr, x.cuda()).cpu())
+
+
 def test_binding_refuses_bad_operands_before_any_launch(g):
     n, f = 500, 8
     src, dst = gg.uniform_graph(n, 4000, seed=3)
