@@ -31,7 +31,6 @@ struct GatherArgs {
     int64_t ldx, ldo;
     int32_t f, chunk_width, n_ctiles, blocks_per_tile, fpad, out_bf16, out_vec_ok, wide_ok;
     int32_t part_filled;     // some lanes' vectors lie past the end of the chunk
-    int32_t x_gap;           // columns between the end of a chunk and the start of the next one in x (the aligned copy may have some)
     int32_t chunk_base;      // first chunk of this launch (a launch covers at most 65,535 chunks)
     int32_t n_ranges;
     Range range[kMaxRanges];
@@ -47,7 +46,16 @@ constexpr int kLoads = GNNFD_GATHER_LOADS;      // 16-byte feature loads kept in
 
 // index registers per lane and batch, and the column indices (and weights) a warp stages per batch
 constexpr int index_regs(int lpr, int vpl) { return kLoads / vpl > lpr ? kLoads / vpl / lpr : 1; }
-constexpr int stage_slots(int lpr, int vpl) { return 32 * index_regs(lpr, vpl); }
+constexpr int stage_slots(int lpr, int vpl, bool roomy) { return roomy ? 256 : 32 * index_regs(lpr, vpl); }
+
+// fp32 chunks of 9 - 16 vectors on graphs that fill the chip take rows from the shortest of a class up and, oddly, gain from a
+// smaller L1 beside 40 instead of 12 KB of shared memory per block.  132,534 rows of 300 entries, 64 columns: longest first
+// 583 us, shortest first 567, with both 564; 304 columns in chunks of 64 3.15 / 3.03 / 3.04 ms; 60,000 of 200, 128 in chunks of 64 378 / 373 / 366 us.
+// All other widths are the same or up to 5 % faster longest first, bf16 ones too.
+constexpr bool shortest_first(int elem_bytes, int vecn, int lpr, int vpl, bool shared)
+{
+    return elem_bytes == 4 && vecn == 4 && lpr == 8 && vpl == 2 && !shared;
+}
 
 // One row (or hub segment) per S = LPR * EP lanes.  The S lanes fetch the row's indices and weights
 // S at a time with one coalesced streaming load each (R rounds per batch) and stage them in the
@@ -91,10 +99,10 @@ __device__ __forceinline__ void second_level(float (*tot_s)[kBlock], int tid, fl
     }
 }
 
-template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE, int EP>
+template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE, int EP, int SLOTS>
 __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg, int block_in_range, int col0,
-                                            int chunk_end, int x_shift, int32_t (*stage_col)[kBlock / 32][stage_slots(LPR, VPL)],
-                                            float (*stage_w)[kBlock / 32][stage_slots(LPR, VPL)], float (*tot_s)[kBlock])
+                                            int chunk_end, int32_t (*stage_col)[kBlock / 32][SLOTS], float (*stage_w)[kBlock / 32][SLOTS],
+                                            float (*tot_s)[kBlock])
 {
     constexpr int S = LPR * EP;
     constexpr int ROWS = kBlock / S;
@@ -119,7 +127,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
         // with 32-byte loads a lane's two vectors are neighbours, otherwise they lie LPR vectors apart
         jq[q] = col0 + (WIDE ? c * VPL + q : c + q * LPR) * VECN;
         okq[q] = jq[q] < chunk_end;
-        xq[q] = static_cast<const T*>(a.x) + x_shift + (okq[q] ? jq[q] : col0);   // out-of-chunk lanes re-read a valid column
+        xq[q] = static_cast<const T*>(a.x) + (okq[q] ? jq[q] : col0);   // out-of-chunk lanes re-read a valid column
     }
     // Pair loads are for all lanes or none: a lane whose second vector, or both, lie past the chunk's end loads a pair all the
     // same (padding of its own row, or the row's first pair) and drops it.  With a branch per lane, rows of 5 and 7 vectors took
@@ -141,7 +149,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
             e = a.seg_end[slot];
             part = a.seg_slot[slot];
         } else {
-            row = a.row_order[rg.item_last - slot];
+            row = a.row_order[rg.item_first + rg.item_step * slot];
             b = a.row_ptr[row];
             e = a.row_ptr[row + 1];
         }
@@ -313,8 +321,9 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
 template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE = false>
 __global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggregate(const __grid_constant__ GatherArgs a)
 {
-    __shared__ int32_t stage_col[2][kBlock / 32][stage_slots(LPR, VPL)];
-    __shared__ float stage_w[2][kBlock / 32][stage_slots(LPR, VPL)];
+    constexpr int SLOTS = stage_slots(LPR, VPL, shortest_first(sizeof(T), VECN, LPR, VPL, SHARED));
+    __shared__ int32_t stage_col[2][kBlock / 32][SLOTS];
+    __shared__ float stage_w[2][kBlock / 32][SLOTS];
     __shared__ __align__(16) float tot_s[VPL * VECN][kBlock];   // second-level sums of every thread
     // grid: x = (block of the sweep, column tile), y = chunk; blocks are issued x first, so the sweeps follow each
     // other chunk by chunk.  (The chunk used to be divided out of a linear 64-bit block number: two 64-bit
@@ -327,7 +336,6 @@ __global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggreg
     const int chunk_end = min(a.f, chunk_begin + a.chunk_width);
     const int col0 = chunk_begin + ctile * (LPR * VPL * VECN);
     if (col0 >= chunk_end) return;
-    const int x_shift = chunk * a.x_gap;
     int r = 0;
 #pragma unroll
     for (int i = 1; i < (SHARED ? kMaxRanges : kNumBins); ++i)      // unsplit, the fourth class is one range
@@ -335,12 +343,12 @@ __global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggreg
     const Range rg = a.range[r];
     const int bir = rb - rg.first_block;
     switch (rg.ep_log2) {
-        case 0: gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 1>(a, rg, bir, col0, chunk_end, x_shift, stage_col, stage_w, tot_s); break;
-        case 1: if constexpr (LPR * 2 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 2>(a, rg, bir, col0, chunk_end, x_shift, stage_col, stage_w, tot_s); break;
-        case 2: if constexpr (LPR * 4 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 4>(a, rg, bir, col0, chunk_end, x_shift, stage_col, stage_w, tot_s); break;
-        case 3: if constexpr (LPR * 8 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 8>(a, rg, bir, col0, chunk_end, x_shift, stage_col, stage_w, tot_s); break;
-        case 4: if constexpr (LPR * 16 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 16>(a, rg, bir, col0, chunk_end, x_shift, stage_col, stage_w, tot_s); break;
-        default: if constexpr (LPR == 1) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 32>(a, rg, bir, col0, chunk_end, x_shift, stage_col, stage_w, tot_s); break;
+        case 0: gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 1, SLOTS>(a, rg, bir, col0, chunk_end, stage_col, stage_w, tot_s); break;
+        case 1: if constexpr (LPR * 2 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 2, SLOTS>(a, rg, bir, col0, chunk_end, stage_col, stage_w, tot_s); break;
+        case 2: if constexpr (LPR * 4 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 4, SLOTS>(a, rg, bir, col0, chunk_end, stage_col, stage_w, tot_s); break;
+        case 3: if constexpr (LPR * 8 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 8, SLOTS>(a, rg, bir, col0, chunk_end, stage_col, stage_w, tot_s); break;
+        case 4: if constexpr (LPR * 16 <= 32) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 16, SLOTS>(a, rg, bir, col0, chunk_end, stage_col, stage_w, tot_s); break;
+        default: if constexpr (LPR == 1) gather_rows<T, VECN, LPR, VPL, WEIGHTED, SHARED, WIDE, 32, SLOTS>(a, rg, bir, col0, chunk_end, stage_col, stage_w, tot_s); break;
     }
 }
 
@@ -543,7 +551,6 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     a.x = d_x; a.out = d_out; a.partial = static_cast<float*>(d_scratch);
     a.ldx = ldx; a.ldo = ldo; a.f = f; a.chunk_width = cw;
     a.n_ctiles = (cw + lpr * vpl * elems - 1) / (lpr * vpl * elems);
-    a.x_gap = x_gap;
     a.part_filled = vectors != lpr * vpl;
     a.fpad = (int32_t)align_up((size_t)f, 4);
     a.out_bf16 = odt == GNNFD_BF16;
@@ -566,12 +573,21 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     if (grid_x > 0) {
         bool shared = false;
         for (int i = 0; i < a.n_ranges; ++i) shared = shared || a.range[i].warps_log2 > 0;
+        if (shortest_first(xsize, elems, lpr, vpl, shared))
+            for (int i = 0; i < a.n_ranges; ++i) {
+                a.range[i].item_first -= a.range[i].item_count - 1;
+                a.range[i].item_step = 1;
+            }
         const bool wide = a.wide_ok != 0;
         GatherKernel kernel = weighted ? (shared ? pick_kernel<true, true>(xdt, vec, lpr, vpl, wide) : pick_kernel<true, false>(xdt, vec, lpr, vpl, wide))
                                        : (shared ? pick_kernel<false, true>(xdt, vec, lpr, vpl, wide) : pick_kernel<false, false>(xdt, vec, lpr, vpl, wide));
-        for (int c0 = 0; c0 < n_chunks; c0 += kMaxGridY) {
+        // A copy with columns between its chunks is gathered chunk by chunk: with the offset computed in the kernel every other call pays
+        // for it too (GCN, 48 fp32 columns on 60,000 rows of 200 entries 209 -> 214 us).
+        const int per_launch = x_gap > 0 ? 1 : kMaxGridY;
+        for (int c0 = 0; c0 < n_chunks; c0 += per_launch) {
             a.chunk_base = c0;
-            const dim3 grid((unsigned)grid_x, (unsigned)(n_chunks - c0 < kMaxGridY ? n_chunks - c0 : kMaxGridY));
+            a.x = static_cast<const char*>(d_x) + (int64_t)c0 * x_gap * xsize;
+            const dim3 grid((unsigned)grid_x, (unsigned)(n_chunks - c0 < per_launch ? n_chunks - c0 : per_launch));
             GNNFD_LAUNCH(weighted ? "gather_aggregate_gcn" : "gather_aggregate_sage", s, kernel, grid, kBlock, 0, a);
         }
     }

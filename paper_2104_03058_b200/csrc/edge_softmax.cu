@@ -224,7 +224,7 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
             e = a.seg_end[slot];
             part = a.seg_slot[slot];
         } else {
-            row = a.row_order[rg.item_last - slot];
+            row = a.row_order[rg.item_first + rg.item_step * slot];
             b = a.row_ptr[row];
             e = a.row_ptr[row + 1];
         }

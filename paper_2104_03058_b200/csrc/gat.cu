@@ -140,7 +140,7 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
             b = a.seg_begin[slot];
             e = a.seg_end[slot];
         } else {
-            row = a.row_order[rg.item_last - slot];
+            row = a.row_order[rg.item_first + rg.item_step * slot];
             b = a.row_ptr[row];
             e = a.row_ptr[row + 1];
         }

@@ -15,7 +15,8 @@ constexpr int kMaxGridY = 65535;               // chunks one launch of a gather 
 
 struct Range {
     int32_t first_block;   // first block (within one column tile of one sweep) of this range
-    int32_t item_last;     // rows: place of the last one in row_order, from where the range goes down (longest first)
+    int32_t item_first;    // rows: place of the first one to take in row_order
+    int32_t item_step;     // rows: -1 from the longest row down, 1 from the shortest up
     int32_t item_count;
     int32_t ep_log2;       // log2 of the edge-parallel groups per row
     int32_t hub;           // 1: items are hub segments writing partial results
@@ -71,31 +72,31 @@ inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t tiles, i
 }
 
 // Fills ranges for `lpr` lanes per row; returns the blocks of one column tile of one sweep.  `per_step`: entries a whole warp
-// has in flight; `limit`: steps of the longest walk (0: a row is never split).
+// has in flight; `limit`: steps of the longest walk.
 inline int64_t plan_ranges(const gnnfd_csr_t* csr, const Groups& groups, int lpr, int per_step, int64_t limit, Range* range,
                            int32_t* n_ranges)
 {
     auto ep_for_bin = [&](int bin) { return groups.want[bin] < 32 / lpr ? groups.want[bin] : 32 / lpr; };
     int nr = 0;
     int64_t blocks = 0;
-    auto add = [&](int64_t begin, int64_t count, int ep, int entries, int hub) {
-        const int w = limit > 0 && lpr * ep == 32 ? warps_log2_for(entries, per_step, limit) : 0;
+    auto add = [&](int64_t begin, int64_t count, int ep, int entries, int hub, bool octave = false) {
+        const int w = lpr * ep == 32 ? warps_log2_for(entries, per_step, limit) : 0;
         const int per_block = kBlock / (lpr * ep) >> w;
-        if (nr > 0 && !hub && !range[nr - 1].hub && range[nr - 1].warps_log2 == w && range[nr - 1].ep_log2 == ilog2(ep)) {
-            // the rows before those in the order, cut in the same way: one range
+        if (octave && nr > 0 && !range[nr - 1].hub && range[nr - 1].warps_log2 == w) {
+            // the octave before the last one in the order, cut in the same way: one range
             Range& r = range[nr - 1];
             r.item_count += (int32_t)count;
             blocks = r.first_block + (r.item_count + per_block - 1) / per_block;
             return;
         }
-        range[nr++] = Range{(int32_t)blocks, (int32_t)(begin + count - 1), (int32_t)count, ilog2(ep), hub, w};
+        range[nr++] = Range{(int32_t)blocks, (int32_t)(begin + count - 1), -1, (int32_t)count, ilog2(ep), hub, w};
         blocks += (count + per_block - 1) / per_block;
     };
     if (csr->n_segments > 0) add(0, csr->n_segments, ep_for_bin(4), kHubSegment, 1);
     int64_t end = csr->bin_start[3] + csr->bin_count[3];
     for (int o = kOctaves - 1; o >= 0; --o) {
         end -= csr->octave_count[o];
-        if (csr->octave_count[o] > 0) add(end, csr->octave_count[o], ep_for_bin(3), kBinDeg2 << (o + 1), 0);
+        if (csr->octave_count[o] > 0) add(end, csr->octave_count[o], ep_for_bin(3), kBinDeg2 << (o + 1), 0, true);
     }
     const int longest[3] = {kBinDeg0, kBinDeg1, kBinDeg2};
     for (int bin = 2; bin >= 0; --bin)
