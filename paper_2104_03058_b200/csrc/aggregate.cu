@@ -132,9 +132,10 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
     // Pair loads are for all lanes or none: a lane whose second vector, or both, lie past the chunk's end loads a pair all the
     // same (padding of its own row, or the row's first pair) and drops it.  With a branch per lane, rows of 5 and 7 vectors took
     // both sides of it: 116 M entries of 20 / 25 fp32 columns 1.58 / 1.59 -> 0.90 / 0.93 ms, of 48 bf16 columns 1.56 -> 1.19.
-    // For bf16 the test stays in the code (full chunks: no lane fails it): without it the loads are scheduled differently and
-    // 64 columns on 2 M RMAT rows take 1.61 instead of 1.49 ms.
-    const bool pairs = sizeof(T) == 4 || okq[VPL - 1] || a.part_filled;
+    // For weighted bf16 sums the test stays in the code (full chunks: no lane fails it): without it the loads are scheduled differently
+    // and 64 columns on 2 M RMAT rows take 1.61 instead of 1.50 ms.  Unweighted ones are faster without it: 32 / 48 / 64 columns
+    // there 1003 / 1471 / 1452 -> 883 / 1419 / 1396 us.
+    const bool pairs = sizeof(T) == 4 || !WEIGHTED || okq[VPL - 1] || a.part_filled;
     const uint32_t ld = (uint32_t)a.ldx;
 
     // a long row may be shared by several warps of the block, which take consecutive parts of it
