@@ -144,9 +144,13 @@ def _alloc_best(best: int, least, device, stream=None):
     try:
         return _alloc_bytes(best, device, stream)
     except torch.OutOfMemoryError:
-        need = least()
-        if need >= best:
-            raise
+        return _alloc_less(best, least(), device, stream)
+
+
+def _alloc_less(best: int, need: int, device, stream=None):
+    """The rest of _alloc_best, called while its allocation error is handled."""
+    if need >= best:
+        raise
     return _alloc_bytes(need, device, stream) if need else None
 
 
@@ -323,7 +327,11 @@ def _aggregate(fn, name, csr: Csr, x, f, chunk_width, out, out_dtype, scratch, s
     if scratch is None:
         need = ctypes.c_size_t()
         _check(lib().gnnfd_aggregate_best_workspace_bytes(csr.handle, xp, ldx, xdt, f, chunk_width, ctypes.byref(need)), name)
-        scratch = _alloc_best(need.value, lambda: aggregate_workspace_bytes(csr, f), x.device, stream)
+        if need.value:
+            try:
+                scratch = _alloc_bytes(need.value, x.device, stream)
+            except torch.OutOfMemoryError:
+                scratch = _alloc_less(need.value, aggregate_workspace_bytes(csr, f), x.device, stream)
     sp, sn = _scratch_args(scratch, csr.device)
     _check(fn(csr.handle, xp, ldx, xdt, op, ldo, _dtype_code(out), f, chunk_width, sp, sn, _stream_ptr(stream)), name)
     return out
@@ -521,7 +529,10 @@ def aggregate_gat(csr: Csr, z: torch.Tensor, a_src: torch.Tensor, a_dst: torch.T
         need = ctypes.c_size_t()
         _check(lib().gnnfd_gat_best_workspace_bytes(csr.handle, zp, ldz, _dtype_code(z), heads, dim, chunk_width,
                                                     ctypes.byref(need)), "gnnfd_aggregate_gat")
-        scratch = _alloc_best(need.value, lambda: gat_workspace_bytes(csr, heads, dim), z.device, stream)
+        try:
+            scratch = _alloc_bytes(need.value, z.device, stream)
+        except torch.OutOfMemoryError:
+            scratch = _alloc_less(need.value, gat_workspace_bytes(csr, heads, dim), z.device, stream)
     _same_device(csr.device, scratch=scratch)
     _check(lib().gnnfd_aggregate_gat(csr.handle, zp, ldz, _dtype_code(z), a_src.data_ptr(),
                                      a_dst.data_ptr(), heads, dim, negative_slope, op, ldo,
