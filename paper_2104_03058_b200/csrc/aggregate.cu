@@ -6,10 +6,11 @@
 // chunk-major), so at any time the blocks in flight gather from one chunk's n x chunk_width slice of
 // x, which is what keeps the gathered working set small enough for L2.  Inside a sweep the rows come
 // grouped by degree class.  A row is owned by S = LPR * EP lanes: LPR lanes cover the chunk's columns
-// with one or two 16-byte vectors each, and EP groups of LPR lanes walk interleaved entries of the
-// row, each keeping 8 loads in flight; column indices and edge weights are staged per warp in shared memory.  The EP partial sums are combined by a fixed shuffle tree, hub rows
-// (degree > GNNFD_HUB_DEGREE) by per-segment partial sums that a second kernel adds in ascending
-// segment order: no atomics, bit-identical from run to run.
+// with one to three 16-byte vectors each, and EP groups of LPR lanes walk interleaved entries of the
+// row, each keeping 8 loads in flight (6 with three vectors); column indices and edge weights are staged per warp in shared
+// memory.  The EP partial sums are combined by a fixed shuffle tree, the parts of a long row that several warps share by shared
+// memory, first warp to last, hub rows (degree > GNNFD_HUB_DEGREE) by per-segment partial sums that a second kernel adds in
+// ascending segment order: no atomics, bit-identical from run to run.
 #include "schedule.cuh"
 #include "vec.cuh"
 
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggreg
     __shared__ float stage_w[2][kBlock / 32][SLOTS];
     __shared__ __align__(16) float tot_s[VPL * VECN][kBlock];   // second-level sums of every thread
     // grid: x = (block of the sweep, column tile), y = chunk; blocks are issued x first, so the sweeps follow each
-    // other chunk by chunk.  (The chunk used to be divided out of a linear 64-bit block number: two 64-bit
+    // other chunk by chunk.  (Dividing the chunk out of a linear 64-bit block number would take two 64-bit
     // divisions per thread, more instructions than a short row's whole walk.)
     const int chunk = a.chunk_base + (int)blockIdx.y;
     const unsigned n_ct = (unsigned)a.n_ctiles;

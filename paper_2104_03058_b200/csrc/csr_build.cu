@@ -136,8 +136,8 @@ edge_histograms(const __grid_constant__ Candidates c, int first_bit, int digit_b
 // A sweep reads every key once and writes it once to its place in the order of the digit.  A block takes a tile
 // of keys, ranks them, publishes how many keys of each digit value it holds, and finds out how many the tiles
 // before it hold by walking back over their published counts until it meets one that already knows its own sum
-// (a chained scan with look-back).  Against the former histogram + three-kernel scan + scatter per digit
-// this drops one read of the keys and four launches.
+// (a chained scan with look-back, after Merrill and Garland's single-pass scan).  A histogram, a scan and a scatter per digit
+// would read the keys once more and take four more launches.
 //
 // The walk waits for other blocks, but only for tiles with a smaller number, and tile numbers are drawn from a
 // counter by blocks that are already running: tile 0 never waits, and every tile publishes its own counts before it
@@ -290,9 +290,7 @@ struct SweepSmem {
 // Blocks stay and draw one tile after the other; the next tile's keys are requested as soon as this tile's have
 // moved to shared memory, so that they arrive while the block walks back and writes out.
 //
-// Bound by the shared-memory pipe and by latency, not by HBM: 116 M words of 8 bytes on 233 k vertices take 0.74 ms per
-// sweep (2.5 TB/s; the former histogram, scans and scatter took 0.96), of which the counters (at 20 M words) give
-// the pipe for shared and global accesses 55 % and the issue slots 45 %.  Measured per four sweeps: of every four
+// Not bound by HBM: 116 M words of 8 bytes on 233 k vertices take 0.74 ms per sweep (2.5 TB/s).  Measured per four sweeps: of every four
 // rounds 0 / 1 / 2 / 3 / 4 with the match instruction 3.02 / 3.03 / 3.28 / 3.70 / 4.18 ms (with values of their own,
 // 122 M keys, five sweeps: 6.63 / 6.24 / 6.36 / 6.65 / 7.60); 2 / 4 / 8 / 16 earlier tiles read together in the walk 3.11 /
 // 2.97 / 3.03 / 3.49 ms; 512 x 8 keys with three blocks per SM 3.69, 256 x 16 with four 3.79 ms.

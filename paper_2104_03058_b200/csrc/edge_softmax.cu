@@ -417,8 +417,7 @@ static size_t softmax_scratch_bytes(const gnnfd_csr_t* csr, int32_t heads)
 // 50 -> 21 us, of 50 60 -> 33, 100,000 of 20 68 -> 53; 200,000 of 16 with one / four heads 51 -> 37 / 66 -> 53, but with
 // eight 67 us with the gathers' narrower groups and 80 with these, hence the second condition where they are used.  Splitting
 // rows on large graphs too, so that all fit, made 115 M slots of 8 heads 1.41 -> 2.55 ms: the block waits for its slowest gather
-// twice per row.  There the bound is the rate at which the L1 looks up scattered 32-byte pieces, one per slot and pass
-// (about 0.8 of the 1.4 ms); paired additions and products bring nothing at 8 heads, 6 heads 1.71 -> 1.48 ms.
+// twice per row.  Paired additions and products bring nothing there at 8 heads, 6 heads 1.71 -> 1.48 ms.
 static Groups softmax_groups(int nf)
 {
     const int longest[3] = {kBinDeg0, kBinDeg1, kBinDeg2};

@@ -91,8 +91,8 @@ constexpr int kLoads = 8;      // 16-byte feature loads kept in flight per lane
 constexpr int index_regs(int lpr, int vpl) { return kLoads / vpl > lpr ? kLoads / vpl / lpr : 1; }
 constexpr int stage_slots(int lpr, int vpl) { return 32 * index_regs(lpr, vpl); }
 
-// Bound by instruction issue once the graph fills the chip (an entry costs a logit, an exponential and the unpacking of
-// its features on top of the gather), so products and rescalings go two to an instruction: on 200,000 rows of
+// On graphs that fill the chip an entry costs a logit, an exponential and the unpacking of its features on top of the
+// gather, so products and rescalings go two to an instruction: on 200,000 rows of
 // 150 entries 8 heads of 16 bf16 columns 0.96 -> 0.89 ms, 8 x 8 bf16 0.54 -> 0.48, fp32 unchanged.  On smaller graphs the
 // longest row decided; shared by warps (see schedule.cuh) 4,000 rows of 10 entries, 8 x 16 fp32, take 23 us
 // instead of 71, 20,000 of 50 64 instead of 155, 100,000 of 20 146 instead of 221.
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kBlock, (VPL == 2 && VECN > 1) ? 3 : 4) gat_ag
     // second-level sums and denominator (and a sharer's maximum), one column per thread
     __shared__ float tot_s[VPL * VECN + 1 + SHARED][kBlock];
     // grid: x = (block of the sweep, column tile), y = chunk; blocks are issued x first, so the sweeps follow each
-    // other chunk by chunk.  (The chunk used to be divided out of a linear 64-bit block number: two 64-bit
+    // other chunk by chunk.  (Dividing the chunk out of a linear 64-bit block number would take two 64-bit
     // divisions per thread, more instructions than a short row's whole walk.)
     const int chunk = a.chunk_base + (int)blockIdx.y;
     const unsigned n_ct = (unsigned)a.n_ctiles;

@@ -63,7 +63,7 @@ template <typename T>
 __device__ __forceinline__ void load_pair(Vec<T, 1>& a, Vec<T, 1>& b, const T* p) { a.load(p); b.load(p + 1); }
 
 // (x, y) += w * (a, b), (x, y) += (a, b) and (x, y) *= (a, b), each in one instruction: the same roundings as two scalar ones
-// for half the issue slots, which is what the attention kernels run short of.
+// for half the issue slots.
 __device__ __forceinline__ void fma_pair(float& x, float& y, float w, float a, float b)
 {
     asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %2};\n\tmov.b64 q, {%3, %4};\n\tmov.b64 r, {%0, %1};\n\t"
