@@ -1032,6 +1032,8 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     if ((e > 0 && (!d_src || !d_dst)) || !d_persistent || !d_scratch) return GNNFD_INVALID_ARG;
     if (((uintptr_t)d_persistent | (uintptr_t)d_scratch) & 255u) return GNNFD_INVALID_ARG;
 
+    L.tile_cap = L.n_tiles;                // the query reserves more; what this input needs is enough
+    L.row_tile_cap = L.row_tiles;
     Carver pc(d_persistent, persistent_bytes), sc(d_scratch, scratch_bytes);
     PersistentPtrs P;
     ScratchPtrs S;
