@@ -123,15 +123,19 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
     int jq[VPL];
     bool okq[VPL];
     const T* xq[VPL];
+    // A vector past the end of the chunk re-reads the chunk's last vector (or pair of them), which a neighbour reads in the same
+    // instruction.  The L1's lookups bound rows that end inside a line (88 % busy): with the chunk's first column in its place, 41 columns (11 of
+    // 16 vectors) on 132,534 rows of 300 entries looked up two lines where one was needed, 622 -> 542 us; 48 on 60,000 rows 295 -> 260.
+    const int last = col0 + (chunk_end - 1 - col0) / (WIDE ? VPL * VECN : VECN) * (WIDE ? VPL * VECN : VECN);
 #pragma unroll
     for (int q = 0; q < VPL; ++q) {
         // with 32-byte loads a lane's two vectors are neighbours, otherwise they lie LPR vectors apart
         jq[q] = col0 + (WIDE ? c * VPL + q : c + q * LPR) * VECN;
         okq[q] = jq[q] < chunk_end;
-        xq[q] = static_cast<const T*>(a.x) + (okq[q] ? jq[q] : col0);   // out-of-chunk lanes re-read a valid column
+        xq[q] = static_cast<const T*>(a.x) + (okq[q] ? jq[q] : last);
     }
     // Pair loads are for all lanes or none: a lane whose second vector, or both, lie past the chunk's end loads a pair all the
-    // same (padding of its own row, or the row's first pair) and drops it.  With a branch per lane, rows of 5 and 7 vectors took
+    // same (padding of its own row, or the chunk's last pair) and drops it.  With a branch per lane, rows of 5 and 7 vectors took
     // both sides of it: 116 M entries of 20 / 25 fp32 columns 1.58 / 1.59 -> 0.90 / 0.93 ms, of 48 bf16 columns 1.56 -> 1.19.
     // For weighted bf16 sums the test stays in the code (full chunks: no lane fails it): without it the loads are scheduled differently
     // and 64 columns on 2 M RMAT rows take 1.61 instead of 1.50 ms.  Unweighted ones are faster without it: 32 / 48 / 64 columns
