@@ -102,6 +102,9 @@ void launch_copy(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int64_t n, int
 
 int64_t segment_capacity(int64_t n, int64_t e, uint32_t flags);      // csr_build.cu; -1 for sizes the build rejects
 
+int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, gnnfd_itype_t itype, uint32_t flags, bool need_perm,
+                   bool need_weights, void* d_persistent, size_t persistent_bytes, void* d_scratch, size_t scratch_bytes, cudaStream_t s,
+                   gnnfd_csr_t** out);                                // csr_build.cu
 int combine_impl(int64_t n, const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int32_t f_in, const void* d_w_t, int64_t ldw,
                  int32_t f_out, void* d_z, int64_t ldz, gnnfd_dtype_t zdt, int mode, const float* d_a_src,
                  const float* d_a_dst, int32_t heads, int32_t dim, float* d_s_src, float* d_s_dst, int32_t* d_status,

@@ -40,11 +40,13 @@ struct Candidates {
     int src_bits;
 };
 
-__device__ __forceinline__ u64 edge_key(const Candidates& c, int64_t s64, int64_t d64, bool reverse, bool* kept, bool* bad)
+template <typename IdT>
+__device__ __forceinline__ u64 edge_key(const Candidates& c, IdT s, IdT d, bool reverse, bool* kept, bool* bad)
 {
-    *bad = s64 < 0 || s64 >= c.n || d64 < 0 || d64 >= c.n;
-    *kept = !*bad && !((reverse || (c.flags & GNNFD_CSR_ADD_SELF_LOOPS)) && s64 == d64);
-    return *kept ? ((u64)d64 << c.src_bits) | (u64)s64 : (u64)c.n << c.src_bits;
+    using U = typename std::make_unsigned<IdT>::type;              // negative ids are above n too
+    *bad = (U)s >= (U)c.n || (U)d >= (U)c.n;
+    *kept = !*bad && !((reverse || (c.flags & GNNFD_CSR_ADD_SELF_LOOPS)) && s == d);
+    return *kept ? ((u64)d << c.src_bits) | (u64)s : (u64)c.n << c.src_bits;
 }
 
 // key and value of candidate i < m
@@ -54,10 +56,10 @@ __device__ __forceinline__ u64 candidate_key(const Candidates& c, int64_t i, int
     const IdT* src = static_cast<const IdT*>(c.src);
     const IdT* dst = static_cast<const IdT*>(c.dst);
     *val = (int32_t)i;
-    if (i < c.e) return edge_key(c, (int64_t)__ldcs(src + i), (int64_t)__ldcs(dst + i), false, kept, bad);
+    if (i < c.e) return edge_key<IdT>(c, __ldcs(src + i), __ldcs(dst + i), false, kept, bad);
     const int64_t n_rev = (c.flags & GNNFD_CSR_SYMMETRIZE) ? c.e : 0;
     if (i < c.e + n_rev) {
-        const u64 key = edge_key(c, (int64_t)__ldcs(dst + i - c.e), (int64_t)__ldcs(src + i - c.e), true, kept, bad);
+        const u64 key = edge_key<IdT>(c, __ldcs(dst + i - c.e), __ldcs(src + i - c.e), true, kept, bad);
         *bad = false;                                  // counted once, by the edge itself
         return key;
     }
@@ -101,7 +103,7 @@ edge_histograms(const __grid_constant__ Candidates c, int first_bit, int digit_b
 #pragma unroll
             for (int j = 0; j < kHistItems; ++j) {
                 bool kept, bad;
-                const u64 key = edge_key(c, (int64_t)sv[j], (int64_t)dv[j], false, &kept, &bad);
+                const u64 key = edge_key<IdT>(c, sv[j], dv[j], false, &kept, &bad);
                 n_kept += kept;
                 n_bad += bad;
                 count(key);
@@ -150,7 +152,6 @@ edge_histograms(const __grid_constant__ Candidates c, int first_bit, int digit_b
 // up to and including this one, plus the keys of smaller digit values (so the sum is a position).
 constexpr uint32_t kSumBit = 0x80000000u;
 constexpr int kMaxPolls = 1 << 20;                   // at up to 1 us a poll
-constexpr int kWalk = 4;                             // earlier tiles read together
 
 __device__ __forceinline__ uint32_t load_published(const uint32_t* p)
 {
@@ -164,7 +165,8 @@ __device__ __forceinline__ void publish(uint32_t* p, uint32_t v)
 }
 
 // position of the tile's first key of one digit value: `column` points at the digit's word of tile 0, words of
-// consecutive tiles are kRadix apart.  false: gave up.
+// consecutive tiles are kRadix apart; kWalk of them are read together.  false: gave up.
+template <int kWalk>
 __device__ __forceinline__ bool look_back(const uint32_t* column, int64_t tile, int max_polls, const int32_t* failed, uint32_t* before)
 {
     uint32_t sum = 0;
@@ -210,6 +212,19 @@ __device__ __forceinline__ int32_t block_scan(int32_t v, int32_t* total, int32_t
 
 enum Source { kWords, kEdges32, kEdges64, kRows };    // where a sweep takes its keys from
 
+// The degrees of a sorted list's rows: lanes hold consecutive entries, the first of each run of one destination adds the run's length.
+// All lanes take part; `ok`: the lane holds an entry.
+__device__ __forceinline__ void count_runs(uint32_t dst, bool ok, int32_t* __restrict__ degree)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t before = __shfl_up_sync(0xffffffffu, dst, 1);
+    const unsigned present = __ballot_sync(0xffffffffu, ok);                     // the first so many lanes
+    const bool first = ok && (lane == 0 || dst != before);
+    const unsigned later = __ballot_sync(0xffffffffu, first) & ~((2u << lane) - 1u);
+    const int end = later ? __ffs(later) - 1 : __popc(present);
+    if (first) atomicAdd(degree + dst, end - lane);
+}
+
 struct SweepArgs {
     Candidates cand;               // kEdges*: the edge list (first sweep)
     const u64* keys_in;            // kWords
@@ -217,6 +232,8 @@ struct SweepArgs {
     const int32_t* row_ptr;        // kRows: the keys are the rows' degree classes
     u64* keys_out;
     int32_t* vals_out;             // values apart from the keys; kRows: the row ids
+    int32_t* col_out;              // ENTRIES: the finished entries and the rows' degrees (zeroed)
+    int32_t* degree;
     int64_t m;
     int n_tiles;
     int shift, mask, val_bits;
@@ -232,6 +249,7 @@ struct SweepArgs {
 // threshold, then one class for hub rows.  Classes are monotone in the degree, so each of the five
 // launch bins (<= 8, <= 32, <= 128, <= hub threshold, hub) is a contiguous range of classes.
 constexpr int kHubClass = 41;
+constexpr int kClassMask = 63;                       // digit values of the row sweep
 __device__ __forceinline__ int degree_class(int32_t deg)
 {
     if (deg <= kBinDeg0) return deg;
@@ -249,6 +267,9 @@ __device__ __forceinline__ int degree_bin(int32_t deg)
 // per SM: 256 threads x 8 keys, so that more SMs take part.
 struct LargeTile { static constexpr int kThreads = 512, kItems = 16, kMinBlocks = 2; };
 struct SmallTile { static constexpr int kThreads = 256, kItems = 8, kMinBlocks = 4; };
+// Where all tiles run at once none knows its sum yet, and the walks go back over most of them: more words are read together.  220,000
+// candidates, 8 / 16 / 32 words: 143 / 145 / 150 us a build.
+constexpr int kWalk = 4, kLongWalk = 8;
 template <typename Shape> constexpr int tile_keys() { return Shape::kThreads * Shape::kItems; }
 static bool use_large_tile(int64_t m) { return m >= (int64_t)4 * kSmCount * tile_keys<LargeTile>(); }
 static int64_t sweep_tiles(int64_t m)
@@ -297,7 +318,7 @@ struct SweepSmem {
 constexpr int kRankRounds = 4;      // rounds whose counts are in flight together
 constexpr int kMatchRounds = 1;     // how many of them use the match instruction
 
-template <typename Shape, int SOURCE, bool HAS_VALS>
+template <typename Shape, int SOURCE, bool HAS_VALS, bool ENTRIES>
 __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_sweep(const __grid_constant__ SweepArgs a)
 {
     constexpr int kBlock = Shape::kThreads, kItems = Shape::kItems, kWarps = kBlock / 32, kTile = kBlock * kItems;
@@ -328,14 +349,14 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
             }
         } else {
             using IdT = typename std::conditional<SOURCE == kEdges32, int32_t, long long>::type;
-            auto word = [&](u64 k, int32_t val) { return HAS_VALS ? k : (k << a.val_bits) | (u64)(uint32_t)(val + 1); };
+            auto word = [&](u64 k, int32_t val) { return HAS_VALS || a.val_bits == 0 ? k : (k << a.val_bits) | (u64)(uint32_t)(val + 1); };
             bool kept, bad;
             if (base + kTile <= a.cand.e) {          // inside the plain input edges: straight-line loads
 #pragma unroll
                 for (int r = 0; r < kItems; ++r) {
-                    const int64_t sv = (int64_t)__ldcs(static_cast<const IdT*>(a.cand.src) + first + r * 32);
-                    const int64_t dv = (int64_t)__ldcs(static_cast<const IdT*>(a.cand.dst) + first + r * 32);
-                    key[r] = word(edge_key(a.cand, sv, dv, false, &kept, &bad), (int32_t)(first + r * 32));
+                    const IdT sv = __ldcs(static_cast<const IdT*>(a.cand.src) + first + r * 32);
+                    const IdT dv = __ldcs(static_cast<const IdT*>(a.cand.dst) + first + r * 32);
+                    key[r] = word(edge_key<IdT>(a.cand, sv, dv, false, &kept, &bad), (int32_t)(first + r * 32));
                 }
             } else {
 #pragma unroll
@@ -422,6 +443,7 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 #pragma unroll
         for (int q = 0; q < kOwn; ++q) {
             total[q] = 0;
+            if (q * kBlock > a.mask) continue;       // no such digit in this sweep
 #pragma unroll
             for (int w = 0; w < kWarps; ++w) total[q] += sm.warp_count[w][tid + q * kBlock];
             if (tile > 0) publish(published + tid + q * kBlock, (uint32_t)total[q] + 1u);
@@ -429,6 +451,7 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 #pragma unroll
         for (int q = 0; q < kOwn; ++q) {
             int32_t sum;
+            if (q * kBlock > a.mask) continue;
             if (q) __syncthreads();
             base[q] = block_scan(total[q], &sum, sm.scan) + carry;
             carry += sum;
@@ -445,6 +468,7 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 #pragma unroll
             for (int q = 0; q < kOwn; ++q) {
                 int32_t sum;
+                if (q * kBlock > a.mask) continue;
                 __syncthreads();
                 const int32_t start = block_scan(a.digit_count[tid + q * kBlock], &sum, sm.scan) + smaller;
                 smaller += sum;
@@ -481,8 +505,11 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 #pragma unroll
             for (int q = 0; q < kOwn; ++q) {
                 const int d = tid + q * kBlock;
+                if (d > a.mask) continue;
                 uint32_t before = 0;
-                if (look_back(a.published + d, tile, a.max_polls, &a.counts->sort_failed, &before))
+                const bool together = Shape::kMinBlocks > 2 && a.n_tiles <= Shape::kMinBlocks * kSmCount;
+                if (together ? look_back<kLongWalk>(a.published + d, tile, a.max_polls, &a.counts->sort_failed, &before)
+                             : look_back<kWalk>(a.published + d, tile, a.max_polls, &a.counts->sort_failed, &before))
                     publish(published + d, kSumBit | (before + (uint32_t)total[q]));
                 else
                     ok = false;
@@ -500,6 +527,22 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
             if (next < a.n_tiles) load_keys((int64_t)next * kTile);
             __syncthreads();
         }
+        if constexpr (ENTRIES) {                     // the words are keys alone, and these are their final places
+            // the order inside a digit's run is the final one, so a destination's entries are neighbours
+            const uint32_t src_mask = (uint32_t)((1ull << a.cand.src_bits) - 1ull);
+#pragma unroll 4
+            for (int i0 = tid - lane; i0 < count; i0 += kBlock) {
+                const int i = i0 + lane;
+                const u64 k = i < count ? sm.keys[i] : ~0ull;
+                const uint32_t d = (uint32_t)(k >> a.cand.src_bits);
+                const bool ok = i < count && d < (uint32_t)a.cand.n;             // dropped candidates come last
+                if (ok) {
+                    const int64_t pos = (int64_t)sm.to_global[(int)(k >> a.shift) & a.mask] + i;
+                    __stcs(a.col_out + pos, (int32_t)((uint32_t)k & src_mask));
+                }
+                count_runs(d, ok, a.degree);
+            }
+        } else
 #pragma unroll 4
         for (int i = tid; i < count; i += kBlock) {
             const u64 k = sm.keys[i];
@@ -523,7 +566,8 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 
 // Duplicate removal after the sort, in two sweeps with a scan of one count per tile between them: a
 // sorted candidate is kept when it is valid and its key differs from its predecessor's.  A thread
-// looks after kUniqueItems consecutive candidates, a block after kUniqueTile.
+// looks after kUniqueItems consecutive candidates, a block after kUniqueTile.  (One sweep that chains the tiles' sums, like
+// rows_from_degrees, is slower: 122 M candidates in 1.10 ms against 0.77.)
 constexpr int kUniqueItems = 8;
 constexpr int kUniqueTile = kThreads * kUniqueItems;
 
@@ -631,6 +675,7 @@ compact_unique(const u64* __restrict__ keys, const int32_t* __restrict__ vals, c
 // is an entry, which thread 0 records.
 constexpr int kRowsPerBlock = kThreads - 1;
 constexpr int kClasses = kHubClass + 1;
+static_assert(kClasses <= kClassMask + 1 && kClassMask < kRadix, "digit of the row sweep");
 
 __global__ void __launch_bounds__(kThreads)
 rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts, int64_t n, int src_bits, int val_bits,
@@ -648,6 +693,19 @@ rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts,
     if (v == 0 && !dedup) counts->nnz = nnz;
     int32_t lo = 0, hi = v <= n ? nnz : 0;
     const u64 target = (u64)v << src_bits;
+    // three words a step while there are as many: half as many steps, each of which waits for memory
+    while (hi - lo >= 4) {
+        const int32_t q = (hi - lo) >> 2;
+        bool below[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) below[j] = (keys[lo + (j + 1) * q] >> val_bits) < target;
+        const int32_t lo0 = lo;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (below[j]) lo = lo0 + (j + 1) * q + 1;
+            else hi = min(hi, lo0 + (j + 1) * q);
+        }
+    }
     while (lo < hi) {
         const int32_t mid = lo + ((hi - lo) >> 1);
         if ((keys[mid] >> val_bits) < target) lo = mid + 1; else hi = mid;
@@ -703,6 +761,182 @@ finalize_entries(const u64* __restrict__ keys, const int32_t* __restrict__ vals,
         __stcs(col_idx + k, (int32_t)(key & ((1ull << src_bits) - 1ull)));
         __stcs(edge_w + k, ws[j] * wd[j]);
         if (write_perm) __stcs(perm + k, vals ? __ldcs(vals + k) : (int32_t)(word[j] & ((1ull << val_bits) - 1ull)) - 1);
+    }
+}
+
+// ---- entries written by the last sweep itself (ENTRIES), where no words are left to search.  39.6 M edges without ids: the last sweep 310
+// instead of 277 us, and 14 us for the rows instead of 28 and 200 for finalize_entries.
+
+// A chain of sums over tiles that are drawn in order (like look_back, one value per tile, 64-bit words): 0 nothing yet, kOwn64 |
+// count: the tile's own count, kSum64 | sum: of all tiles up to and including this one.
+constexpr u64 kOwn64 = 1ull << 61, kSum64 = 1ull << 62;
+
+// By one whole warp: the sum of all tiles before `tile`, which holds `total` itself; publishes both.  Every lane gets the result,
+// or -1: gave up (and the build is marked as failed).
+__device__ __forceinline__ int64_t chain_sums(u64* __restrict__ words, int64_t tile, int32_t total, int32_t* failed)
+{
+    const int lane = threadIdx.x & 31;
+    auto store = [&](u64 v) { asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(words + tile), "l"(v) : "memory"); };
+    if (lane == 0) store((tile == 0 ? kSum64 : kOwn64) | (u64)(uint32_t)total);
+    int64_t before = 0;
+    for (int64_t t = tile - 1; t >= 0; t -= 32) {
+        u64 w = kSum64;                                // before the first tile: a sum of nothing
+        unsigned sums;
+        for (int polls = 0;; ++polls) {
+            if (t - lane >= 0) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(words + t - lane) : "memory");
+            const unsigned missing = __ballot_sync(0xffffffffu, w == 0ull);
+            sums = __ballot_sync(0xffffffffu, (w & kSum64) != 0ull);
+            // everything up to the nearest sum is there
+            if (missing == 0u || (sums != 0u && (missing & ((sums & (0u - sums)) - 1u)) == 0u)) break;
+            if ((polls & 255) == 255 && (polls >= kMaxPolls || load_published(reinterpret_cast<const uint32_t*>(failed)) != 0u)) {
+                if (lane == 0) atomicExch(failed, 1);
+                return -1;
+            }
+        }
+        const int nearest = sums ? __ffs(sums) - 1 : 31;
+        int64_t part = lane <= nearest ? (int64_t)(w & (kOwn64 - 1ull)) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        before += part;
+        if (sums) break;
+    }
+    if (lane == 0 && tile > 0) store(kSum64 | (u64)(before + total));
+    return before;
+}
+
+// What rows_and_degrees does, from the degrees: row_ptr is their sums, chained over tiles of rows.  Also, for every piece of kSlotTile
+// entries, the row that its first one belongs to.
+constexpr int kRowItems = 8;
+constexpr int kRowTile = kThreads * kRowItems;
+constexpr int kSlotItems = 8;                        // entries per thread of slot_weights
+constexpr int kSlotTile = kThreads * kSlotItems;
+
+__global__ void __launch_bounds__(kThreads)
+rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ counts, int64_t n, int32_t* __restrict__ ticket,
+                  u64* __restrict__ words, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
+                  int32_t* __restrict__ class_count, int32_t* __restrict__ slot_tile_row)
+{
+    __shared__ int32_t smem[kThreads / 32], class_smem[kClasses], bin_smem[kNumBins], octave_smem[kOctaves], max_smem, drawn;
+    __shared__ int64_t before;
+    if (threadIdx.x == 0) {
+        drawn = counts->sort_failed ? -1 : atomicAdd(ticket, 1);
+        max_smem = 0;
+    }
+    if (threadIdx.x < kClasses) class_smem[threadIdx.x] = 0;
+    if (threadIdx.x < kNumBins) bin_smem[threadIdx.x] = 0;
+    if (threadIdx.x < kOctaves) octave_smem[threadIdx.x] = 0;
+    __syncthreads();
+    const int tile = drawn;
+    if (tile < 0) return;
+    if (tile == 0 && threadIdx.x == 0) counts->nnz = counts->n_valid;
+    const int64_t first = (int64_t)tile * kRowTile + threadIdx.x * kRowItems;
+    int32_t deg[kRowItems], sum = 0, total;
+#pragma unroll
+    for (int j = 0; j < kRowItems; ++j) {
+        deg[j] = first + j < n ? degree[first + j] : 0;
+        sum += deg[j];
+    }
+    const int32_t in_tile = block_prefix_256(sum, &total, smem);
+    if (threadIdx.x < 32) {
+        const int64_t start = chain_sums(words, tile, total, &counts->sort_failed);
+        if (threadIdx.x == 0) before = start;
+    }
+    int32_t most = 0;
+#pragma unroll
+    for (int j = 0; j < kRowItems; ++j) {
+        const int64_t v = first + j;
+        if (v >= n) break;
+        dinv[v] = deg[j] > 0 ? (float)(1.0 / sqrt((double)deg[j])) : 0.f;
+        rdeg[v] = deg[j] > 0 ? (float)(1.0 / (double)deg[j]) : 0.f;
+        atomicAdd(&class_smem[degree_class(deg[j])], 1);
+        atomicAdd(&bin_smem[degree_bin(deg[j])], 1);
+        if (degree_bin(deg[j]) == 3) atomicAdd(&octave_smem[31 - __clz((deg[j] - 1) / kBinDeg2)], 1);
+        most = max(most, deg[j]);
+    }
+    if (most) atomicMax(&max_smem, most);
+    __syncthreads();
+    if (before < 0) return;
+    int32_t ptr = (int32_t)before + in_tile;
+#pragma unroll
+    for (int j = 0; j < kRowItems; ++j) {
+        const int64_t v = first + j;
+        if (v >= n) break;
+        row_ptr[v] = ptr;
+        for (int64_t t = ((int64_t)ptr + kSlotTile - 1) / kSlotTile; t * kSlotTile < (int64_t)ptr + deg[j]; ++t) slot_tile_row[t] = (int32_t)v;
+        ptr += deg[j];
+        if (v == n - 1) row_ptr[n] = ptr;
+    }
+    // few global atomics: all blocks add to the same words
+    if (threadIdx.x < kClasses && class_smem[threadIdx.x]) atomicAdd(class_count + threadIdx.x, class_smem[threadIdx.x]);
+    if (threadIdx.x < kNumBins && bin_smem[threadIdx.x]) atomicAdd(&counts->bin_count[threadIdx.x], bin_smem[threadIdx.x]);
+    if (threadIdx.x < kOctaves && octave_smem[threadIdx.x]) atomicAdd(&counts->octave_count[threadIdx.x], octave_smem[threadIdx.x]);
+    if (threadIdx.x == 0 && max_smem) atomicMax(&counts->max_degree, max_smem);
+}
+
+// The GCN weight of every entry.  A block takes a piece of kSlotTile consecutive entries: the row starts that fall into it are marked in
+// shared memory, and a running maximum gives every entry its row.  Bound by the L1's lookups (one line
+// per gathered dinv[source]), like finalize_entries.
+__global__ void __launch_bounds__(kThreads)
+slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ slot_tile_row,
+             const float* __restrict__ dinv, int64_t n, const BuildCounts* __restrict__ counts, float* __restrict__ edge_w)
+{
+    __shared__ __align__(16) int32_t row_of[kSlotTile];
+    __shared__ int32_t warp_last[kThreads / 32];
+    const int64_t nnz = counts->sort_failed ? 0 : counts->nnz, base = (int64_t)blockIdx.x * kSlotTile;
+    if (base >= nnz) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t first = base + tid * kSlotItems;
+    int32_t u[kSlotItems];
+    const bool whole = first + kSlotItems <= nnz;
+    if (whole) {
+#pragma unroll
+        for (int j = 0; j < kSlotItems; j += 4) {
+            const int4 v = __ldcs(reinterpret_cast<const int4*>(col_idx + first + j));
+            u[j] = v.x; u[j + 1] = v.y; u[j + 2] = v.z; u[j + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kSlotItems; ++j) u[j] = first + j < nnz ? __ldcs(col_idx + first + j) : 0;
+    }
+    const int64_t row0 = slot_tile_row[blockIdx.x], row1 = base + kSlotTile < nnz ? slot_tile_row[blockIdx.x + 1] : n - 1;
+#pragma unroll
+    for (int j = 0; j < kSlotItems; j += 4) reinterpret_cast<int4*>(row_of)[tid + j / 4 * kThreads] = make_int4(0, 0, 0, 0);
+    float ws[kSlotItems];
+#pragma unroll
+    for (int j = 0; j < kSlotItems; ++j) ws[j] = __ldg(dinv + u[j]);
+    __syncthreads();
+    for (int64_t r = row0 + 1 + tid; r <= row1; r += kThreads) {         // empty rows share their start with a later one, which counts
+        const int64_t at = row_ptr[r] - base;
+        if (at < kSlotTile) atomicMax(&row_of[at], (int32_t)(r - row0));
+    }
+    __syncthreads();
+    int32_t row[kSlotItems];
+#pragma unroll
+    for (int j = 0; j < kSlotItems; j += 4) {
+        const int4 v = reinterpret_cast<const int4*>(row_of)[(tid * kSlotItems + j) / 4];
+        row[j] = v.x; row[j + 1] = v.y; row[j + 2] = v.z; row[j + 3] = v.w;
+    }
+#pragma unroll
+    for (int j = 1; j < kSlotItems; ++j) row[j] = max(row[j], row[j - 1]);
+    int32_t upto = row[kSlotItems - 1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) upto = max(upto, __shfl_up_sync(0xffffffffu, upto, o));
+    if (lane == 31) warp_last[warp] = upto;
+    int32_t earlier = __shfl_up_sync(0xffffffffu, upto, 1);
+    if (lane == 0) earlier = 0;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) earlier = max(earlier, warp_last[w]);
+    float w[kSlotItems];
+#pragma unroll
+    for (int j = 0; j < kSlotItems; ++j) w[j] = ws[j] * __ldg(dinv + row0 + max(row[j], earlier));
+    if (whole) {
+#pragma unroll
+        for (int j = 0; j < kSlotItems; j += 4)
+            __stcs(reinterpret_cast<float4*>(edge_w + first + j), make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]));
+    } else {
+#pragma unroll
+        for (int j = 0; j < kSlotItems; ++j)
+            if (first + j < nnz) __stcs(edge_w + first + j, w[j]);
     }
 }
 
@@ -853,9 +1087,11 @@ struct BuildLayout {
     int n_ranges;          // source ranges the hub rows are cut at (1: no cut)
     int64_t range_rows;    // vertex ids per source range
     int val_bits;          // > 0: keys and values share one 64-bit word (key << val_bits | value + 1)
+    int64_t row_words;     // tiles of rows_from_degrees
+    bool with_vals;        // edge ids travel through the sort
 };
 
-static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L)
+static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L, bool with_vals = true)
 {
     if (n <= 0 || e < 0) return GNNFD_INVALID_ARG;
     if (flags & ~(uint32_t)(GNNFD_CSR_ADD_SELF_LOOPS | GNNFD_CSR_DEDUP | GNNFD_CSR_SYMMETRIZE | GNNFD_CSR_INPUT_ORDER))
@@ -873,6 +1109,7 @@ static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L)
     L->row_tiles = sweep_tiles(n);
     L->tile_cap = reserved_tiles(m);
     L->row_tile_cap = reserved_tiles(n);
+    L->row_words = (n + kRowTile - 1) / kRowTile;
     L->hub_cap = m / (GNNFD_HUB_DEGREE + 1) + 1;
     // source ranges of GNNFD_HUB_RANGE_ROWS vertices, at most 64 of them (narrower ranges would keep a band of x
     // resident in L2, but on the RMAT workload the extra, shorter segments cost more than the saved traffic: 32
@@ -897,6 +1134,7 @@ static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L)
     int vb = 1;
     while ((int64_t(1) << vb) < m + 2) ++vb;                  // values -1 .. m-1 stored as 0 .. m
     L->val_bits = L->key_bits + vb <= 64 ? vb : 0;
+    L->with_vals = with_vals;
     return GNNFD_OK;
 }
 
@@ -922,28 +1160,30 @@ static void carve_persistent(Carver& c, int64_t n, const BuildLayout& L, Persist
     p->edge_w = c.take<float>(cap);
     p->dinv = c.take<float>((size_t)n);
     p->rdeg = c.take<float>((size_t)n);
-    p->row_order = c.take<int32_t>((size_t)n);
+    p->row_order = c.take<int32_t>((size_t)n);            // may hold the degrees until the rows are sorted by them
+    p->counts = c.take<BuildCounts>(1);
     p->seg_row = c.take<int32_t>((size_t)L.seg_cap);
     p->seg_begin = c.take<int32_t>((size_t)L.seg_cap);
     p->seg_end = c.take<int32_t>((size_t)L.seg_cap);
     p->seg_slot = c.take<int32_t>((size_t)L.seg_cap);
     p->hub_seg_ptr = c.take<int32_t>((size_t)L.hub_cap + 1);
-    p->counts = c.take<BuildCounts>(1);
 }
 
 struct ScratchPtrs {
     u64 *keys_a, *keys_b;
     int32_t *vals_a, *vals_b, *flags, *scan_temp;
     // zeroed together before the first kernel: digit counts (a row per edge sweep, then the degree classes), tile
-    // counters (likewise), the words the row sweep's and the first edge sweep's tiles publish
+    // counters (likewise, then of rows_from_degrees), the words that the tiles of the latter, of the row sweep and of the first edge sweep publish
     int32_t *digit_count, *ticket;
+    u64* row_words;
     uint32_t *row_published, *published, *published_alt;
     size_t zero_bytes;
 };
 
 static size_t flag_ints(const BuildLayout& L)
 {
-    // one count per tile of the duplicate removal; hub segment counts (per source range and hub row, then per hub row)
+    // one count per tile of the duplicate removal, or a row per piece of the entries; hub segment counts (per source range and hub row, then per hub row)
+    static_assert(kUniqueTile == kSlotTile, "one count or one row for as many candidates");
     size_t a = (size_t)L.m / kUniqueTile + 2, c = (size_t)L.hub_cap * (L.n_ranges + 1) + 4;
     return (a > c ? a : c) + 1;
 }
@@ -953,12 +1193,13 @@ static void carve_scratch(Carver& c, const BuildLayout& L, ScratchPtrs* p)
     const size_t cap = (size_t)(L.m > 0 ? L.m : 1);
     p->keys_a = c.take<u64>(cap);
     p->keys_b = c.take<u64>(cap);
-    const size_t val_cap = L.val_bits > 0 ? 1 : cap;      // no value buffers when the values travel inside the key words
+    const size_t val_cap = L.val_bits > 0 || !L.with_vals ? 1 : cap;      // no value buffers when the values travel inside the key words
     p->vals_a = c.take<int32_t>(val_cap);
     p->vals_b = c.take<int32_t>(val_cap);
     const size_t zero_begin = c.off;
     p->digit_count = c.take<int32_t>((size_t)(L.passes + 1) * kRadix);
-    p->ticket = c.take<int32_t>((size_t)L.passes + 1);
+    p->ticket = c.take<int32_t>((size_t)L.passes + 2);
+    p->row_words = c.take<u64>((size_t)L.row_words);
     p->row_published = c.take<uint32_t>((size_t)kRadix * L.row_tile_cap);
     p->zero_bytes = c.off - zero_begin + (size_t)kRadix * L.n_tiles * sizeof(uint32_t);
     p->published = c.take<uint32_t>((size_t)kRadix * L.tile_cap);
@@ -968,10 +1209,10 @@ static void carve_scratch(Carver& c, const BuildLayout& L, ScratchPtrs* p)
     p->scan_temp = c.take<int32_t>(scan_temp_ints(fl));
 }
 
-template <typename Shape, int SOURCE, bool HAS_VALS>
+template <typename Shape, int SOURCE, bool HAS_VALS, bool ENTRIES>
 static int launch_sweep_shape(const char* name, const SweepArgs& a, cudaStream_t s)
 {
-    const auto kernel = radix_sweep<Shape, SOURCE, HAS_VALS>;
+    const auto kernel = radix_sweep<Shape, SOURCE, HAS_VALS, ENTRIES>;
     const int blocks = a.n_tiles < Shape::kMinBlocks * kSmCount ? a.n_tiles : Shape::kMinBlocks * kSmCount;
     const int smem = (int)sizeof(SweepSmem<Shape>);
     GNNFD_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -979,54 +1220,37 @@ static int launch_sweep_shape(const char* name, const SweepArgs& a, cudaStream_t
     return GNNFD_OK;
 }
 
-template <int SOURCE, bool HAS_VALS>
+template <int SOURCE, bool HAS_VALS, bool ENTRIES>
 static int launch_sweep(const char* name, SweepArgs& a, cudaStream_t s)
 {
     a.n_tiles = (int)sweep_tiles(a.m);
-    return use_large_tile(a.m) ? launch_sweep_shape<LargeTile, SOURCE, HAS_VALS>(name, a, s)
-                               : launch_sweep_shape<SmallTile, SOURCE, HAS_VALS>(name, a, s);
+    return use_large_tile(a.m) ? launch_sweep_shape<LargeTile, SOURCE, HAS_VALS, ENTRIES>(name, a, s)
+                               : launch_sweep_shape<SmallTile, SOURCE, HAS_VALS, ENTRIES>(name, a, s);
+}
+
+template <int SOURCE>
+static int launch_edge_sweep(bool has_vals, bool entries, SweepArgs& a, cudaStream_t s)
+{
+    if (has_vals) return launch_sweep<SOURCE, true, false>("radix_sweep", a, s);
+    return entries ? launch_sweep<SOURCE, false, true>("radix_sweep", a, s) : launch_sweep<SOURCE, false, false>("radix_sweep", a, s);
 }
 
 // One-shot settings of the drill (see gnnfd_debug_build_fault): consumed by the next build on this thread.
 struct BuildDrill { int max_polls, sweep; };
 static thread_local BuildDrill t_drill = {kMaxPolls, -1};
 
-}  // namespace gnnfd
-
-extern "C" {
-
-int gnnfd_csr_workspace_bytes(int64_t n, int64_t e, uint32_t flags, size_t* persistent_bytes, size_t* scratch_bytes)
+// need_perm, need_weights: whether the caller looks at perm and edge_w (their places are left as they are where not).  Edge ids that nobody
+// needs do not travel through the sort, unless duplicates are removed, where the order among them decides.
+int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, gnnfd_itype_t itype, uint32_t flags, bool need_perm,
+                   bool need_weights, void* d_persistent, size_t persistent_bytes, void* d_scratch, size_t scratch_bytes, cudaStream_t s,
+                   gnnfd_csr_t** out)
 {
-    using namespace gnnfd;
-    BuildLayout L;
-    int rc = make_layout(n, e, flags, &L);
-    if (rc) return rc;
-    if (persistent_bytes) {
-        Carver c(nullptr, ~size_t(0));
-        PersistentPtrs p;
-        carve_persistent(c, n, L, &p);
-        *persistent_bytes = c.off;
-    }
-    if (scratch_bytes) {
-        Carver c(nullptr, ~size_t(0));
-        ScratchPtrs s;
-        carve_scratch(c, L, &s);
-        *scratch_bytes = c.off;
-    }
-    return GNNFD_OK;
-}
-
-int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, gnnfd_itype_t itype, uint32_t flags,
-                    void* d_persistent, size_t persistent_bytes, void* d_scratch, size_t scratch_bytes, void* stream,
-                    gnnfd_csr_t** out)
-{
-    using namespace gnnfd;
     const BuildDrill drill = t_drill;
     t_drill = BuildDrill{kMaxPolls, -1};
     if (!out) return GNNFD_INVALID_ARG;
     *out = nullptr;
     BuildLayout L;
-    int rc = make_layout(n, e, flags, &L);
+    int rc = make_layout(n, e, flags, &L, need_perm || (flags & GNNFD_CSR_DEDUP));
     if (rc) return rc;
     if (itype != GNNFD_I32 && itype != GNNFD_I64) return GNNFD_UNSUPPORTED;
     if ((e > 0 && (!d_src || !d_dst)) || !d_persistent || !d_scratch) return GNNFD_INVALID_ARG;
@@ -1044,9 +1268,12 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     // the drill leaves out a sweep's first tile: another one has to be there to miss it
     if (drill.sweep >= 0 && (drill.sweep > L.passes || (drill.sweep < L.passes ? L.n_tiles : L.row_tiles) < 2)) return GNNFD_INVALID_ARG;
 
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t m = L.m;
-    GNNFD_CUDA_CHECK(cudaMemsetAsync(P.counts, 0, sizeof(BuildCounts), s));
+    // Without ids the last sweep writes the entries and counts the degrees.  With them it is better to write words once more: 80 M
+    // entries 2.86 ms with words, 2.92 without.
+    const bool entries = !L.with_vals;
+    char* const zero_from = entries ? reinterpret_cast<char*>(P.row_order) : reinterpret_cast<char*>(P.counts);      // the degrees lie before the counts
+    GNNFD_CUDA_CHECK(cudaMemsetAsync(zero_from, 0, (size_t)(reinterpret_cast<char*>(P.counts + 1) - zero_from), s));
 
     BuildCounts host_counts;
     std::memset(&host_counts, 0, sizeof(host_counts));
@@ -1056,8 +1283,9 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     int32_t* vals_alt = S.vals_b;
 
     const bool dedup = (flags & GNNFD_CSR_DEDUP) != 0;
-    const int vb = L.val_bits;
-    const bool packed = vb > 0;                     // values ride in the low bits of the keys
+    const int vb = L.with_vals ? L.val_bits : 0;
+    const bool apart = L.with_vals && vb == 0;      // values in arrays of their own, else in the low bits of the keys
+    int32_t* const degree = P.row_order;
     GNNFD_CUDA_CHECK(cudaMemsetAsync(S.digit_count, 0, S.zero_bytes, s));
     if (drill.sweep >= 0) GNNFD_CUDA_CHECK(cudaMemsetAsync(S.ticket + drill.sweep, 1, 1, s));      // tile 0 is never drawn
     SweepArgs sw{};
@@ -1065,6 +1293,8 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     sw.m = m;
     sw.val_bits = vb;
     sw.counts = P.counts;
+    sw.col_out = P.col_idx;
+    sw.degree = degree;
     sw.max_polls = drill.max_polls;
     if (m > 0) {
         const unsigned walkers = blocks_for(m, kHistTile) < 6u * kSmCount ? blocks_for(m, kHistTile) : 6u * kSmCount;
@@ -1086,12 +1316,10 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
             sw.published_next = pass + 1 < L.passes ? published_alt : nullptr;
             sw.keys_in = keys; sw.keys_out = keys_alt;
             sw.vals_in = vals; sw.vals_out = vals_alt;
-            if (pass > 0)
-                rc = packed ? launch_sweep<kWords, false>("radix_sweep", sw, s) : launch_sweep<kWords, true>("radix_sweep", sw, s);
-            else if (itype == GNNFD_I32)
-                rc = packed ? launch_sweep<kEdges32, false>("radix_sweep", sw, s) : launch_sweep<kEdges32, true>("radix_sweep", sw, s);
-            else
-                rc = packed ? launch_sweep<kEdges64, false>("radix_sweep", sw, s) : launch_sweep<kEdges64, true>("radix_sweep", sw, s);
+            const bool last = entries && pass + 1 == L.passes;
+            if (pass > 0) rc = launch_edge_sweep<kWords>(apart, last, sw, s);
+            else if (itype == GNNFD_I32) rc = launch_edge_sweep<kEdges32>(apart, last, sw, s);
+            else rc = launch_edge_sweep<kEdges64>(apart, last, sw, s);
             if (rc) return rc;
             u64* tk = keys; keys = keys_alt; keys_alt = tk;
             int32_t* tv = vals; vals = vals_alt; vals_alt = tv;
@@ -1104,29 +1332,38 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
             rc = exclusive_scan_i32(tile_first, tile_first, (size_t)unique_tiles, S.scan_temp, s);
             if (rc) return rc;
             GNNFD_LAUNCH("compact_unique", s, compact_unique, unique_tiles, kThreads, 0, keys,
-                         packed ? (const int32_t*)nullptr : (const int32_t*)vals, (const int32_t*)tile_first, m, vb, keys_alt,
+                         apart ? (const int32_t*)vals : (const int32_t*)nullptr, (const int32_t*)tile_first, m, vb, keys_alt,
                          P.perm, P.counts);
             u64* tk = keys; keys = keys_alt; keys_alt = tk;
         }
     }
     int32_t* class_count = S.digit_count + (size_t)L.passes * kRadix;
-    GNNFD_LAUNCH("rows_and_degrees", s, rows_and_degrees, blocks_for((size_t)n + 1, kRowsPerBlock), kThreads, 0, keys, P.counts, n,
-                 L.src_bits, vb, dedup ? 1 : 0, P.row_ptr, P.dinv, P.rdeg, class_count);
-    if (m > 0)
-        GNNFD_LAUNCH("finalize_entries", s, finalize_entries, blocks_for(m, kThreads * kKeyItems), kThreads, 0, keys,
-                     packed ? (const int32_t*)nullptr : (const int32_t*)vals, dedup ? 0 : 1, P.counts, L.src_bits, vb,
-                     P.dinv, P.col_idx, P.edge_w, P.perm, m);
+    if (entries) {
+        int32_t* slot_tile_row = S.flags;
+        GNNFD_LAUNCH("rows_from_degrees", s, rows_from_degrees, (unsigned)L.row_words, kThreads, 0, degree, P.counts, n,
+                     S.ticket + L.passes + 1, S.row_words, P.row_ptr, P.dinv, P.rdeg, class_count, slot_tile_row);
+        if (m > 0 && need_weights)
+            GNNFD_LAUNCH("slot_weights", s, slot_weights, blocks_for(m, kSlotTile), kThreads, 0, P.row_ptr, P.col_idx, slot_tile_row,
+                         P.dinv, n, P.counts, P.edge_w);
+    } else {
+        GNNFD_LAUNCH("rows_and_degrees", s, rows_and_degrees, blocks_for((size_t)n + 1, kRowsPerBlock), kThreads, 0, keys, P.counts, n,
+                     L.src_bits, vb, dedup ? 1 : 0, P.row_ptr, P.dinv, P.rdeg, class_count);
+        if (m > 0)
+            GNNFD_LAUNCH("finalize_entries", s, finalize_entries, blocks_for(m, kThreads * kKeyItems), kThreads, 0, keys,
+                         apart ? (const int32_t*)vals : (const int32_t*)nullptr, dedup ? 0 : 1, P.counts, L.src_bits, vb,
+                         P.dinv, P.col_idx, P.edge_w, P.perm, m);
+    }
     // row_order = rows sorted by degree class, ascending row id inside a class: one sweep over the rows
     sw.row_ptr = P.row_ptr;
     sw.vals_out = P.row_order;
     sw.m = n;
     sw.shift = 32;
-    sw.mask = kRadix - 1;
+    sw.mask = kClassMask;
     sw.digit_count = class_count;
     sw.ticket = S.ticket + L.passes;
     sw.published = S.row_published;
     sw.published_next = nullptr;
-    rc = launch_sweep<kRows, false>("radix_sweep_rows", sw, s);
+    rc = launch_sweep<kRows, false, false>("radix_sweep_rows", sw, s);
     if (rc) return rc;
     // segment counts per (source range, hub row), then per hub row
     int32_t* range_count = S.flags;
@@ -1182,6 +1419,39 @@ int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, 
     h->hub_seg_ptr = P.hub_seg_ptr;
     *out = h;
     return GNNFD_OK;
+}
+
+}  // namespace gnnfd
+
+extern "C" {
+
+int gnnfd_csr_workspace_bytes(int64_t n, int64_t e, uint32_t flags, size_t* persistent_bytes, size_t* scratch_bytes)
+{
+    using namespace gnnfd;
+    BuildLayout L;
+    int rc = make_layout(n, e, flags, &L);
+    if (rc) return rc;
+    if (persistent_bytes) {
+        Carver c(nullptr, ~size_t(0));
+        PersistentPtrs p;
+        carve_persistent(c, n, L, &p);
+        *persistent_bytes = c.off;
+    }
+    if (scratch_bytes) {
+        Carver c(nullptr, ~size_t(0));
+        ScratchPtrs s;
+        carve_scratch(c, L, &s);
+        *scratch_bytes = c.off;
+    }
+    return GNNFD_OK;
+}
+
+int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, gnnfd_itype_t itype, uint32_t flags,
+                    void* d_persistent, size_t persistent_bytes, void* d_scratch, size_t scratch_bytes, void* stream,
+                    gnnfd_csr_t** out)
+{
+    return gnnfd::build_csr_impl(n, e, d_src, d_dst, itype, flags, true, true, d_persistent, persistent_bytes, d_scratch, scratch_bytes,
+                                 static_cast<cudaStream_t>(stream), out);
 }
 
 int gnnfd_debug_build_fault(int32_t max_polls, int32_t sweep)

@@ -42,8 +42,8 @@ static int oneshot(bool weighted, int64_t n, int64_t e, const void* d_src, const
     if (scratch_bytes < L.persistent + L.build_scratch + L.aggregate) return GNNFD_WORKSPACE_TOO_SMALL;
     char* base = static_cast<char*>(d_scratch);
     gnnfd_csr_t* csr = nullptr;
-    rc = gnnfd_build_csr(n, e, d_src, d_dst, itype, oneshot_flags(flags), base, L.persistent, base + L.persistent,
-                         L.build_scratch, stream, &csr);
+    rc = build_csr_impl(n, e, d_src, d_dst, itype, oneshot_flags(flags), false, weighted, base, L.persistent, base + L.persistent,
+                        L.build_scratch, static_cast<cudaStream_t>(stream), &csr);
     if (rc) return rc;
     // the build is done with its scratch (same stream), so the aggregation gets that as well: room for an aligned copy of x
     void* agg = base + L.persistent;
@@ -92,8 +92,8 @@ int gnnfd_oneshot_gat(int64_t n, int64_t e, const void* d_src, const void* d_dst
     if (scratch_bytes < L.persistent + L.build_scratch + L.aggregate) return GNNFD_WORKSPACE_TOO_SMALL;
     char* base = static_cast<char*>(d_scratch);
     gnnfd_csr_t* csr = nullptr;
-    rc = gnnfd_build_csr(n, e, d_src, d_dst, itype, oneshot_flags(flags), base, L.persistent, base + L.persistent,
-                         L.build_scratch, stream, &csr);
+    rc = build_csr_impl(n, e, d_src, d_dst, itype, oneshot_flags(flags), false, false, base, L.persistent, base + L.persistent,
+                        L.build_scratch, static_cast<cudaStream_t>(stream), &csr);
     if (rc) return rc;
     rc = gnnfd_aggregate_gat(csr, d_z, ldz, zdt, d_a_src, d_a_dst, heads, dim, negative_slope, d_out, ldo, odt, chunk_width,
                              base + L.persistent, L.build_scratch + L.aggregate, stream);

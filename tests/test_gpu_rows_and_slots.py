@@ -1,0 +1,64 @@
+"""Row pointers, entry weights and duplicate removal at the edges of their tiles (2048 rows, 2048 entries, 2048 candidates), with empty rows
+before, between and behind the others."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def destinations(kind, n, m, rng):
+    if kind == "one row":
+        return np.full(m, n // 2)
+    if kind == "last row":
+        return np.full(m, n - 1)
+    if kind == "first rows":
+        return rng.integers(0, min(n, 3), m)
+    if kind == "far apart":
+        return rng.choice(np.array([0, n // 3, n - 1]), m)
+    return rng.integers(0, n, m)
+
+
+@pytest.mark.parametrize("n,m", [(1, 1), (1, 5000), (2047, 2048), (2048, 2047), (2049, 6145), (40_000, 2048), (300_001, 10), (300_001, 40_961),
+                                 (5000, 0)])
+@pytest.mark.parametrize("kind", ["one row", "last row", "first rows", "far apart", "any"])
+@pytest.mark.parametrize("flags", [0, 2])                     # without and with duplicate removal
+def test_rows_and_weights(n, m, kind, flags):
+    import paper_2104_03058_b200 as g
+    rng = np.random.default_rng(n + m)
+    src, dst = rng.integers(0, max(1, n // 2), m).astype(np.int32), destinations(kind, n, m, rng).astype(np.int32)
+    order = np.lexsort((src, dst))
+    s, d, p = src[order], dst[order], order
+    if flags and m:
+        first = np.r_[True, (s[1:] != s[:-1]) | (d[1:] != d[:-1])]
+        s, d, p = s[first], d[first], p[first]
+    row_ptr = np.searchsorted(d, np.arange(n + 1))
+    deg = np.diff(row_ptr)
+    dinv = np.where(deg > 0, 1 / np.sqrt(np.maximum(deg, 1).astype(np.float64)), 0).astype(np.float32)
+    csr = g.build_csr(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), flags)
+    assert csr.nnz == len(s) and csr.max_degree == deg.max()
+    for name, want in (("row_ptr", row_ptr), ("col_idx", s), ("perm", p), ("dinv_sqrt", dinv), ("edge_weight", dinv[s] * dinv[d])):
+        np.testing.assert_array_equal(getattr(csr, name).cpu().numpy(), want, err_msg=name)
+    assert np.array_equal(np.sort(csr.row_order.cpu().numpy()), np.arange(n))
+
+
+@pytest.mark.parametrize("n,m", [(1, 1), (1, 5000), (2047, 2048), (2048, 2047), (2049, 6145), (40_000, 2048), (300_001, 10), (300_001, 40_961),
+                                 (5000, 0), (70_001, 148 * 4 * 8192 + 1)])
+@pytest.mark.parametrize("kind", ["one row", "last row", "first rows", "far apart", "any"])
+def test_light_build(n, m, kind):
+    """The same edges through the one-shot path, whose last sweep writes the entries and counts the degrees; sums of whole numbers."""
+    import paper_2104_03058_b200 as g
+    rng = np.random.default_rng(n + m)
+    src, dst = rng.integers(0, n, m).astype(np.int32), destinations(kind, n, m, rng).astype(np.int32)
+    x = rng.integers(-8, 9, (n, 4)).astype(np.float32)
+    ds, dd, dx = (torch.from_numpy(a).cuda() for a in (src, dst, x))
+    deg = np.bincount(dst, minlength=n)
+    sums = np.stack([np.bincount(dst, weights=x[src, j], minlength=n) for j in range(4)], axis=1)
+    rdeg = np.where(deg > 0, 1 / np.maximum(deg, 1).astype(np.float64), 0).astype(np.float32)
+    got = g.oneshot("sage", n, ds, dd, dx).cpu().numpy()
+    np.testing.assert_array_equal(got, sums.astype(np.float32) * rdeg[:, None])
+    dinv = np.where(deg > 0, 1 / np.sqrt(np.maximum(deg, 1).astype(np.float64)), 0)
+    want, scale = (np.stack([np.bincount(dst, weights=dinv[src] * dinv[dst] * v[src, j], minlength=n) for j in range(4)], axis=1)
+                   for v in (x.astype(np.float64), np.abs(x).astype(np.float64)))
+    got = g.oneshot("gcn", n, ds, dd, dx).cpu().numpy()
+    assert (np.abs(got - want) <= 1e-5 * scale + 1e-6).all()
