@@ -327,6 +327,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
 template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE = false>
 __global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggregate(const __grid_constant__ GatherArgs a)
 {
+    grid_dependency<true>();
     constexpr int SLOTS = stage_slots(LPR, VPL, shortest_first(sizeof(T), VECN, LPR, VPL, SHARED));
     __shared__ int32_t stage_col[2][kBlock / 32][SLOTS];
     __shared__ float stage_w[2][kBlock / 32][SLOTS];
@@ -364,6 +365,7 @@ hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict__ hu
            const float* __restrict__ partial, int64_t hub_begin, int32_t n_hub, int32_t f, int32_t fpad, int use_rdeg,
            void* __restrict__ out, int64_t ldo, int out_bf16)
 {
+    grid_dependency<true>();
     const int i = blockIdx.x;
     const int j = blockIdx.y * kBlock + threadIdx.x;
     if (i >= n_hub || j >= f) return;
@@ -425,6 +427,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock)
 align_features(const T* __restrict__ x, int64_t ldx, int64_t n, int32_t f, int32_t cw, int32_t pitch, uint32_t ld, uint4* __restrict__ out)
 {
+    grid_dependency<true>();
     constexpr int VECN = 16 / sizeof(T);
     const uint32_t vectors = ld / VECN;
     const int64_t idx = (int64_t)blockIdx.x * kBlock + threadIdx.x;

@@ -252,6 +252,7 @@ template <bool BF16, bool SPLIT, bool XT = false>
 __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kCombineThreads)
 combine_mma(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const CombineArgs a)
 {
+    grid_dependency<false>();
     static_assert(!(BF16 && SPLIT), "bf16 operands are used as they are");
     static_assert(!XT || SPLIT, "x_lo in tensor memory belongs to the fp32-faithful mode");
     extern __shared__ __align__(1024) unsigned char smem_raw[];

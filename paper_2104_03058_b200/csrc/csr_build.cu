@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(kThreads)
 edge_histograms(const __grid_constant__ Candidates c, int first_bit, int digit_bits, int passes, int32_t* __restrict__ hist,
                 BuildCounts* __restrict__ counts)
 {
+    grid_dependency<true>();
     extern __shared__ int32_t hist_smem[];           // [passes][kRadix]
     for (int i = threadIdx.x; i < passes * kRadix; i += kThreads) hist_smem[i] = 0;
     __syncthreads();
@@ -321,6 +322,7 @@ constexpr int kMatchRounds = 1;     // how many of them use the match instructio
 template <typename Shape, int SOURCE, bool HAS_VALS, bool ENTRIES>
 __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_sweep(const __grid_constant__ SweepArgs a)
 {
+    grid_dependency<(Shape::kMinBlocks > 2)>();
     constexpr int kBlock = Shape::kThreads, kItems = Shape::kItems, kWarps = kBlock / 32, kTile = kBlock * kItems;
     constexpr int kOwn = kRadix / kBlock;            // digit values a thread looks after
     static_assert(kRadix % kBlock == 0 && kTile <= kWarps * kRadix, "digit values per thread; values fit the counts' place");
@@ -628,6 +630,7 @@ __global__ void __launch_bounds__(kThreads)
 unique_tile_counts(const u64* __restrict__ keys, int val_bits, const BuildCounts* __restrict__ counts,
                    int32_t* __restrict__ tile_count)
 {
+    grid_dependency<true>();
     __shared__ int32_t smem[kThreads / 32];
     u64 word[kUniqueItems];
     const int64_t first = (int64_t)blockIdx.x * kUniqueTile + (int64_t)threadIdx.x * kUniqueItems;
@@ -643,6 +646,7 @@ compact_unique(const u64* __restrict__ keys, const int32_t* __restrict__ vals, c
                int64_t m, int val_bits, u64* __restrict__ keys_out, int32_t* __restrict__ perm,
                BuildCounts* __restrict__ counts)
 {
+    grid_dependency<false>();
     __shared__ int32_t smem[kThreads / 32];
     __shared__ u64 kept_key[kUniqueTile];
     __shared__ int32_t kept_val[kUniqueTile];
@@ -682,6 +686,7 @@ rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts,
                  int dedup, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
                  int32_t* __restrict__ class_count)
 {
+    grid_dependency<true>();
     __shared__ int32_t ptr[kThreads], class_smem[kClasses], bin_smem[kNumBins], octave_smem[kOctaves], max_smem;
     if (counts->sort_failed) return;
     if (threadIdx.x < kClasses) class_smem[threadIdx.x] = 0;
@@ -738,6 +743,7 @@ finalize_entries(const u64* __restrict__ keys, const int32_t* __restrict__ vals,
                  const BuildCounts* __restrict__ counts, int src_bits, int val_bits, const float* __restrict__ dinv,
                  int32_t* __restrict__ col_idx, float* __restrict__ edge_w, int32_t* __restrict__ perm, int64_t m)
 {
+    grid_dependency<true>();
     const int64_t base = (int64_t)blockIdx.x * (kThreads * kKeyItems) + threadIdx.x;
     const int64_t nnz = counts->sort_failed ? 0 : counts->nnz;
     u64 word[kKeyItems];
@@ -816,6 +822,7 @@ rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ 
                   u64* __restrict__ words, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
                   int32_t* __restrict__ class_count, int32_t* __restrict__ slot_tile_row)
 {
+    grid_dependency<true>();
     __shared__ int32_t smem[kThreads / 32], class_smem[kClasses], bin_smem[kNumBins], octave_smem[kOctaves], max_smem, drawn;
     __shared__ int64_t before;
     if (threadIdx.x == 0) {
@@ -880,6 +887,7 @@ __global__ void __launch_bounds__(kThreads)
 slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ slot_tile_row,
              const float* __restrict__ dinv, int64_t n, const BuildCounts* __restrict__ counts, float* __restrict__ edge_w)
 {
+    grid_dependency<true>();
     __shared__ __align__(16) int32_t row_of[kSlotTile];
     __shared__ int32_t warp_last[kThreads / 32];
     const int64_t nnz = counts->sort_failed ? 0 : counts->nnz, base = (int64_t)blockIdx.x * kSlotTile;
@@ -1003,6 +1011,7 @@ hub_segment_counts(const int32_t* __restrict__ row_ptr, const int32_t* __restric
                    const int32_t* __restrict__ row_order, int64_t n, const BuildCounts* __restrict__ counts, int64_t hub_cap,
                    int32_t n_ranges, int64_t range_rows, int32_t* __restrict__ range_count, int32_t* __restrict__ seg_count)
 {
+    grid_dependency<true>();
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i > hub_cap) return;
     const int32_t n_hub = counts->sort_failed ? 0 : counts->bin_count[4];
@@ -1025,6 +1034,7 @@ fill_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ c
               int32_t* __restrict__ seg_row, int32_t* __restrict__ seg_begin, int32_t* __restrict__ seg_end,
               int32_t* __restrict__ seg_slot)
 {
+    grid_dependency<true>();
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int32_t n_hub = counts->sort_failed ? 0 : counts->bin_count[4];
     if (i == 0) counts->n_segments = hub_seg_ptr[n_hub];
@@ -1044,6 +1054,7 @@ hub_segments_few(const int32_t* __restrict__ row_ptr, const int32_t* __restrict_
                  int32_t* hub_seg_ptr, int32_t* __restrict__ seg_row, int32_t* __restrict__ seg_begin,
                  int32_t* __restrict__ seg_end, int32_t* __restrict__ seg_slot)
 {
+    grid_dependency<true>();
     __shared__ int32_t smem[32];
     const int32_t n_hub = counts->sort_failed ? 0 : counts->bin_count[4];
     for (int32_t i = threadIdx.x; i < n_hub; i += kHubThreads)

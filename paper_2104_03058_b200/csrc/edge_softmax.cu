@@ -359,6 +359,7 @@ __device__ __forceinline__ void softmax_items(const SoftmaxArgs& a, const Range&
 template <int HB, int LPS, bool SHARED>
 __global__ void __launch_bounds__(kBlock, GNNFD_SOFTMAX_MIN_BLOCKS) edge_softmax_rows(const __grid_constant__ SoftmaxArgs a)
 {
+    grid_dependency<false>();
     __shared__ float2 shared_stats[kBlock / 32][32];
     const int rb = blockIdx.x;
     int r = 0;
@@ -382,6 +383,7 @@ __global__ void __launch_bounds__(kBlock, GNNFD_SOFTMAX_MIN_BLOCKS) edge_softmax
 template <int HB, int LPS, bool SHARED>
 __global__ void __launch_bounds__(kBlock, GNNFD_SOFTMAX_MIN_BLOCKS) edge_softmax_hub_stats(const __grid_constant__ SoftmaxArgs a)
 {
+    grid_dependency<false>();
     __shared__ float2 shared_stats[kBlock / 32][32];
     softmax_items<HB, LPS, 32 / LPS, SHARED, kModeHubStats>(a, a.range[0], blockIdx.x, shared_stats);
 }
@@ -390,6 +392,7 @@ __global__ void __launch_bounds__(kBlock, GNNFD_SOFTMAX_MIN_BLOCKS) edge_softmax
 // row's (max, 1 / sum) in every segment's entry.
 __global__ void __launch_bounds__(kBlock) edge_softmax_hub_merge(const __grid_constant__ SoftmaxArgs a)
 {
+    grid_dependency<false>();
     const int64_t idx = (int64_t)blockIdx.x * kBlock + threadIdx.x;
     if (idx >= (int64_t)a.n_hub * a.heads) return;
     const int i = (int)(idx / a.heads), h = (int)(idx % a.heads);

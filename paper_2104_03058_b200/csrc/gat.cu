@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kBlock)
 gat_scores(const T* __restrict__ z, int64_t ldz, const float* __restrict__ a_src, const float* __restrict__ a_dst,
            int64_t n, int heads, int dim, float* __restrict__ s_src, float* __restrict__ s_dst)
 {
+    grid_dependency<true>();
     const int64_t idx = (int64_t)blockIdx.x * kBlock + threadIdx.x;
     if (idx >= n * heads) return;
     const int64_t v = idx <= 0x7fffffffll ? (int64_t)((uint32_t)idx / (uint32_t)heads) : idx / heads;
@@ -378,6 +379,7 @@ template <typename T, int VECN, int LPR, int VPL, bool SHARED>
 // the vector-pair forms and four for the others is what the measured-good builds had.
 __global__ void __launch_bounds__(kBlock, (VPL == 2 && VECN > 1) ? 3 : 4) gat_aggregate(const __grid_constant__ GatArgs a)
 {
+    grid_dependency<true>();
     __shared__ int32_t stage_col[2][kBlock / 32][stage_slots(LPR, VPL)];
     // second-level sums and denominator (and a sharer's maximum), one column per thread
     __shared__ float tot_s[VPL * VECN + 1 + SHARED][kBlock];
@@ -419,6 +421,7 @@ gat_hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict_
                const float* __restrict__ partial, const float* __restrict__ partial_ml, int64_t hub_begin, int32_t n_hub,
                int32_t f, int32_t fpad, int32_t heads, int32_t dim, int32_t out_dim, void* __restrict__ out, int64_t ldo, int out_bf16)
 {
+    grid_dependency<true>();
     __shared__ float s_max[kReduceWays][kReduceCols], s_num[kReduceWays][kReduceCols], s_den[kReduceWays][kReduceCols];
     const int i = blockIdx.x;
     const int c = threadIdx.x % kReduceCols, q = threadIdx.x / kReduceCols;

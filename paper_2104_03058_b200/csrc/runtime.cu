@@ -93,6 +93,7 @@ __device__ __forceinline__ void load_scan_items(const int32_t* in, size_t base, 
 __global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __restrict__ in, size_t count,
                                                              int32_t* __restrict__ sums)
 {
+    grid_dependency<true>();
     __shared__ int32_t smem[8];
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
     const bool vec = (reinterpret_cast<uintptr_t>(in) & 15u) == 0;
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __
 __global__ void __launch_bounds__(kScanThreads) scan_tiles(const int32_t* in, int32_t* out, size_t count,
                                                          const int32_t* offsets)
 {
+    grid_dependency<true>();
     __shared__ int32_t smem[8];
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
     const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15u) == 0;
