@@ -40,9 +40,6 @@ struct GatherArgs {
 #ifndef GNNFD_GATHER_LOADS
 #define GNNFD_GATHER_LOADS 8
 #endif
-#ifndef GNNFD_GATHER_MIN_BLOCKS
-#define GNNFD_GATHER_MIN_BLOCKS 3
-#endif
 constexpr int kLoads = GNNFD_GATHER_LOADS;      // 16-byte feature loads kept in flight per lane
 
 // index registers per lane and batch, and the column indices (and weights) a warp stages per batch
@@ -56,6 +53,17 @@ constexpr int stage_slots(int lpr, int vpl, bool roomy) { return roomy ? 256 : 3
 constexpr bool shortest_first(int elem_bytes, int vecn, int lpr, int vpl, bool shared)
 {
     return elem_bytes == 4 && vecn == 4 && lpr == 8 && vpl == 2 && !shared;
+}
+
+// Blocks per SM that the registers are shared out for.  Four where the loop fits 64 registers without giving up loads in flight: rows are
+// bound by waiting for the loads of their own chain, and more of them wait side by side.  Three / four blocks: SAGE fp32, 100,000 rows of
+// 20 entries, 128 columns in chunks of 64 96 -> 86 us, 200,000 of 16, 64 columns 90 -> 76, 32 39 -> 32, RMAT 2^19, 64 columns 368 -> 315; GCN fp32
+// without split rows, 41 columns on 132,534 rows of 300 542 -> 515, 304 in chunks of 64 371 -> 348, 32 on 233,000 of 86 211 -> 190.  But wider
+// rows lose: GCN of 144 / 256 columns 214 -> 228 / 240 -> 277, SAGE of 256 on 20,000 rows of 50 59 -> 65; so do split rows of GCN (64 columns 28 -> 31)
+// and bf16 (SAGE of 64 / 256 columns 35 -> 41 / 130 -> 151, GCN of 64 on RMAT 2^21 1487 -> 1832).
+constexpr int min_blocks(int elem_bytes, bool weighted, bool shared, int lpr)
+{
+    return elem_bytes == 4 && lpr <= 8 && !(weighted && shared) ? 4 : 3;
 }
 
 // One row (or hub segment) per S = LPR * EP lanes.  The S lanes fetch the row's indices and weights
@@ -325,7 +333,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
 }
 
 template <typename T, int VECN, int LPR, int VPL, bool WEIGHTED, bool SHARED, bool WIDE = false>
-__global__ void __launch_bounds__(kBlock, GNNFD_GATHER_MIN_BLOCKS) gather_aggregate(const __grid_constant__ GatherArgs a)
+__global__ void __launch_bounds__(kBlock, min_blocks(sizeof(T), WEIGHTED, SHARED, LPR)) gather_aggregate(const __grid_constant__ GatherArgs a)
 {
     grid_dependency<true>();
     constexpr int SLOTS = stage_slots(LPR, VPL, shortest_first(sizeof(T), VECN, LPR, VPL, SHARED));
