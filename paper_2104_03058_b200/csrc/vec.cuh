@@ -27,12 +27,21 @@ template <> struct Vec<__nv_bfloat16, 8> {
     uint4 v;
     __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const uint4*>(p)); }
     __device__ __forceinline__ void zero() { v = make_uint4(0u, 0u, 0u, 0u); }
+    __device__ __forceinline__ uint32_t word(int i) const { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
     __device__ __forceinline__ float get(int i) const
     {
-        const uint32_t w = (i >> 1) == 0 ? v.x : (i >> 1) == 1 ? v.y : (i >> 1) == 2 ? v.z : v.w;
+        const uint32_t w = word(i >> 1);
         return __uint_as_float((i & 1) ? (w & 0xffff0000u) : (w << 16));   // bf16 -> fp32 is exact
     }
 };
+// (x, y) += the two bf16 values of a word, widened in the addition: the same rounding as widening first, in half the instructions.
+// SAGE, 64 columns on 40 M entries 412 -> 379 us, 100 on 18 M 279 -> 259, 301 on 6 M 308 -> 265 (but 256 on 4 M, 16 lanes with two vectors
+// each, 126 -> 129, so not there).
+__device__ __forceinline__ void add_widened(float& x, float& y, uint32_t w)
+{
+    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
+        : "+f"(x), "+f"(y) : "r"(w));
+}
 template <> struct Vec<__nv_bfloat16, 1> {
     unsigned short v;
     __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const unsigned short*>(p)); }
