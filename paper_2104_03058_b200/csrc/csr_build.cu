@@ -940,8 +940,8 @@ __device__ __forceinline__ int64_t chain_sums(u64* __restrict__ words, int64_t t
     return before;
 }
 
-// What rows_and_degrees does, from the degrees: row_ptr is their sums, chained over tiles of rows.  Also, for every piece of kSlotTile
-// entries, the row that its first one belongs to.
+// What rows_and_degrees does, from the degrees: row_ptr is their sums, chained over tiles of rows.  Also (slot_tile_row, unless null), for
+// every piece of kSlotTile entries, the row that its first one belongs to, and behind the last piece the row of the last entry.
 constexpr int kRowItems = 8;
 constexpr int kRowTile = kThreads * kRowItems;
 constexpr int kSlotItems = 8;                        // entries per thread of slot_weights
@@ -993,13 +993,26 @@ rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ 
     if (most) atomicMax(&max_smem, most);
     __syncthreads();
     if (before < 0) return;
+    const int32_t n_entries = counts->n_valid;
     int32_t ptr = (int32_t)before + in_tile;
 #pragma unroll
     for (int j = 0; j < kRowItems; ++j) {
         const int64_t v = first + j;
-        if (v >= n) break;
-        row_ptr[v] = ptr;
-        for (int64_t t = ((int64_t)ptr + kSlotTile - 1) / kSlotTile; t * kSlotTile < (int64_t)ptr + deg[j]; ++t) slot_tile_row[t] = (int32_t)v;
+        if (v < n) row_ptr[v] = ptr;
+        if (slot_tile_row) {
+            int32_t t = (int32_t)(((int64_t)ptr + kSlotTile - 1) / kSlotTile);
+            const int32_t t_end = (int32_t)(((int64_t)ptr + deg[j] + kSlotTile - 1) / kSlotTile);      // t where the row starts no piece
+            // the pieces of a long row are written by the whole warp: by one thread, those of a row of 40 M entries took 90 us
+            unsigned many = __ballot_sync(0xffffffffu, t_end - t > 4);
+            if (t_end - t <= 4)
+                for (; t < t_end; ++t) slot_tile_row[t] = (int32_t)v;
+            for (; many; many &= many - 1u) {
+                const int from = __ffs(many) - 1;
+                const int32_t row = __shfl_sync(0xffffffffu, (int32_t)v, from), end = __shfl_sync(0xffffffffu, t_end, from);
+                for (int32_t i = __shfl_sync(0xffffffffu, t, from) + (int)(threadIdx.x & 31); i < end; i += 32) slot_tile_row[i] = row;
+            }
+            if (deg[j] > 0 && ptr + deg[j] == n_entries) slot_tile_row[t_end] = (int32_t)v;
+        }
         ptr += deg[j];
         if (v == n - 1) row_ptr[n] = ptr;
     }
@@ -1012,10 +1025,14 @@ rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ 
 
 // The GCN weight of every entry.  A block takes a piece of kSlotTile consecutive entries: the row starts that fall into it are marked in
 // shared memory, and a running maximum gives every entry its row.  Bound by the L1's lookups (one line
-// per gathered dinv[source]), like finalize_entries.
+// per gathered dinv[source]), like finalize_entries.  Where a piece spans more than kMarkedRows rows, most of them without entries, each
+// entry's row is searched instead: marking takes the block 0.3 us per 256 rows while the chip is idle.  2 M vertices, marked / searched:
+// 4,000 entries 1150 / 23 us, 200,000 35 / 17, 500,000 20.7 / 18.7, 1 M 18.6 / 20.8, 4 M 31 / 39.
+constexpr int kMarkedRows = 3 * kSlotTile;
+
 __global__ void __launch_bounds__(kThreads)
 slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ slot_tile_row,
-             const float* __restrict__ dinv, int64_t n, const BuildCounts* __restrict__ counts, float* __restrict__ edge_w)
+             const float* __restrict__ dinv, const BuildCounts* __restrict__ counts, float* __restrict__ edge_w)
 {
     grid_dependency<true>();
     __shared__ __align__(16) int32_t row_of[kSlotTile];
@@ -1036,34 +1053,50 @@ slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ co
 #pragma unroll
         for (int j = 0; j < kSlotItems; ++j) u[j] = first + j < nnz ? __ldcs(col_idx + first + j) : 0;
     }
-    const int64_t row0 = slot_tile_row[blockIdx.x], row1 = base + kSlotTile < nnz ? slot_tile_row[blockIdx.x + 1] : n - 1;
-#pragma unroll
-    for (int j = 0; j < kSlotItems; j += 4) reinterpret_cast<int4*>(row_of)[tid + j / 4 * kThreads] = make_int4(0, 0, 0, 0);
+    const int32_t row0 = slot_tile_row[blockIdx.x], row1 = slot_tile_row[blockIdx.x + 1];
     float ws[kSlotItems];
+    int32_t row[kSlotItems], earlier = 0;                // counted from row0
+    if (row1 - row0 <= kMarkedRows) {
 #pragma unroll
-    for (int j = 0; j < kSlotItems; ++j) ws[j] = __ldg(dinv + u[j]);
-    __syncthreads();
-    for (int64_t r = row0 + 1 + tid; r <= row1; r += kThreads) {         // empty rows share their start with a later one, which counts
-        const int64_t at = row_ptr[r] - base;
-        if (at < kSlotTile) atomicMax(&row_of[at], (int32_t)(r - row0));
+        for (int j = 0; j < kSlotItems; j += 4) reinterpret_cast<int4*>(row_of)[tid + j / 4 * kThreads] = make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int j = 0; j < kSlotItems; ++j) ws[j] = __ldg(dinv + u[j]);
+        __syncthreads();
+        for (int32_t r = row0 + 1 + tid; r <= row1; r += kThreads) {     // empty rows share their start with a later one, which counts
+            const int64_t at = row_ptr[r] - base;
+            if (at < kSlotTile) atomicMax(&row_of[at], r - row0);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kSlotItems; j += 4) {
+            const int4 v = reinterpret_cast<const int4*>(row_of)[(tid * kSlotItems + j) / 4];
+            row[j] = v.x; row[j + 1] = v.y; row[j + 2] = v.z; row[j + 3] = v.w;
+        }
+#pragma unroll
+        for (int j = 1; j < kSlotItems; ++j) row[j] = max(row[j], row[j - 1]);
+        int32_t upto = row[kSlotItems - 1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) upto = max(upto, __shfl_up_sync(0xffffffffu, upto, o));
+        if (lane == 31) warp_last[warp] = upto;
+        earlier = __shfl_up_sync(0xffffffffu, upto, 1);
+        if (lane == 0) earlier = 0;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) earlier = max(earlier, warp_last[w]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < kSlotItems; ++j) {
+            ws[j] = __ldg(dinv + u[j]);
+            row[j] = 0;
+        }
+        // the last row that starts at the entry or before it: the searches of a thread's entries take the same steps side by side
+        for (int32_t left = row1 - row0 + 1; left > 1;) {
+            const int32_t half = left / 2;
+#pragma unroll
+            for (int j = 0; j < kSlotItems; ++j)
+                if (row_ptr[row0 + row[j] + half] <= first + j) row[j] += half;
+            left -= half;
+        }
     }
-    __syncthreads();
-    int32_t row[kSlotItems];
-#pragma unroll
-    for (int j = 0; j < kSlotItems; j += 4) {
-        const int4 v = reinterpret_cast<const int4*>(row_of)[(tid * kSlotItems + j) / 4];
-        row[j] = v.x; row[j + 1] = v.y; row[j + 2] = v.z; row[j + 3] = v.w;
-    }
-#pragma unroll
-    for (int j = 1; j < kSlotItems; ++j) row[j] = max(row[j], row[j - 1]);
-    int32_t upto = row[kSlotItems - 1];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) upto = max(upto, __shfl_up_sync(0xffffffffu, upto, o));
-    if (lane == 31) warp_last[warp] = upto;
-    int32_t earlier = __shfl_up_sync(0xffffffffu, upto, 1);
-    if (lane == 0) earlier = 0;
-    __syncthreads();
-    for (int w = 0; w < warp; ++w) earlier = max(earlier, warp_last[w]);
     float w[kSlotItems];
 #pragma unroll
     for (int j = 0; j < kSlotItems; ++j) w[j] = ws[j] * __ldg(dinv + row0 + max(row[j], earlier));
@@ -1532,12 +1565,12 @@ int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, g
     }
     int32_t* class_count = S.digit_count + (size_t)L.sweeps() * kRadix;
     if (entries) {
-        int32_t* slot_tile_row = S.flags;
+        int32_t* slot_tile_row = need_weights ? S.flags : nullptr;
         GNNFD_LAUNCH("rows_from_degrees", s, rows_from_degrees, (unsigned)L.row_words, kThreads, 0, degree, P.counts, n,
                      S.ticket + L.sweeps() + 1, S.row_words, P.row_ptr, P.dinv, P.rdeg, class_count, slot_tile_row);
         if (m > 0 && need_weights)
             GNNFD_LAUNCH("slot_weights", s, slot_weights, blocks_for(m, kSlotTile), kThreads, 0, P.row_ptr, P.col_idx, slot_tile_row,
-                         P.dinv, n, P.counts, P.edge_w);
+                         P.dinv, P.counts, P.edge_w);
     } else {
         GNNFD_LAUNCH("rows_and_degrees", s, rows_and_degrees, blocks_for((size_t)n + 1, kRowsPerBlock), kThreads, 0, keys, P.counts, n,
                      L.src_bits, vb, dedup ? 1 : 0, P.row_ptr, P.dinv, P.rdeg, class_count);

@@ -62,3 +62,42 @@ def test_light_build(n, m, kind):
                    for v in (x.astype(np.float64), np.abs(x).astype(np.float64)))
     got = g.oneshot("gcn", n, ds, dd, dx).cpu().numpy()
     assert (np.abs(got - want) <= 1e-5 * scale + 1e-6).all()
+
+
+def kernel_ms(g, call, kernel, rounds=5):
+    """least time of one launch of `kernel` over a few calls"""
+    call()
+    least = float("inf")
+    for _ in range(rounds):
+        g.kernel_timing_enable(True)
+        call()
+        torch.cuda.synchronize()
+        least = min(least, g.kernel_timing_read()[kernel][0])
+        g.kernel_timing_enable(False)
+    return least
+
+
+@pytest.mark.parametrize("rows", ["first", "both ends", "any"])
+def test_entry_weights_do_not_wait_for_rows_without_entries(rows):
+    """A few thousand entries on 2 M vertices: a handful of blocks must not walk millions of row pointers (which took 2 ms; the same
+    entries on 1000 vertices about 6 us)."""
+    import paper_2104_03058_b200 as g
+    n, m, x = 2_000_000, 4000, torch.ones((2_000_000, 4), device="cuda")
+    rng = np.random.default_rng(5)
+    src, dst = rng.integers(0, 1000, m), rng.integers(0, 1000, m)
+    few = [torch.from_numpy(a.astype(np.int32)).cuda() for a in (src, dst)]
+    dst = {"first": dst, "both ends": np.where(dst % 2, dst, n - 1 - dst), "any": rng.integers(0, n, m)}[rows]
+    many = [torch.from_numpy(a.astype(np.int32)).cuda() for a in (src, dst)]
+    short = kernel_ms(g, lambda: g.oneshot("gcn", 1000, *few, x[:1000]), "slot_weights")
+    assert kernel_ms(g, lambda: g.oneshot("gcn", n, *many, x), "slot_weights") < 10 * short + 0.02
+    assert (g.oneshot("sage", n, *many, x).sum(1) > 0).sum() == len(np.unique(dst))
+
+
+def test_row_pointers_of_one_long_row():
+    """The rows of the pieces of one row of 8 M entries are not written by a single thread (which took 20 us)."""
+    import paper_2104_03058_b200 as g
+    n, m, x = 5000, 8_000_000, torch.ones((5000, 4), device="cuda")
+    src = torch.randint(n, (m,), dtype=torch.int32, device="cuda")
+    one, every = torch.full_like(src, 7), torch.randint(n, (m,), dtype=torch.int32, device="cuda")
+    spread = kernel_ms(g, lambda: g.oneshot("gcn", n, src, every, x), "rows_from_degrees")
+    assert kernel_ms(g, lambda: g.oneshot("gcn", n, src, one, x), "rows_from_degrees") < spread + 0.008
