@@ -328,6 +328,7 @@ struct SweepSmem {
     int32_t to_global[kRadix];      // global position of tile slot i holding digit value d: to_global[d] + i
     int32_t scan[32];
     int32_t tile[2];
+    int32_t long_run;               // kToEntries: a quarter of the tile's keys have one digit value
 };
 
 // The tile a block is at: its keys, the first tile of the chain it belongs to, its bucket (kBucketWords).
@@ -445,7 +446,10 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
     load_keys(place.base, place.count);
 
     for (int turn = 1;; turn ^= 1) {
-        if (tid == 0) sm.tile[turn] = atomicAdd(a.ticket, 1);
+        if (tid == 0) {
+            sm.tile[turn] = atomicAdd(a.ticket, 1);
+            sm.long_run = 0;
+        }
         const int64_t tile_base = place.base;
         const int count = place.count, first_tile = place.first_tile, bucket = place.bucket;
         uint32_t* const published = a.published + (int64_t)tile * kRadix;
@@ -509,6 +513,7 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 #pragma unroll
             for (int w = 0; w < kWarps; ++w) total[q] += sm.warp_count[w][tid + q * kBlock];
             if (tile > first_tile) publish(published + tid + q * kBlock, (uint32_t)total[q] + 1u);
+            if (OUT == kToEntries && total[q] >= kTile / 4) sm.long_run = 1;
         }
 #pragma unroll
         for (int q = 0; q < kOwn; ++q) {
@@ -598,19 +603,41 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
             __syncthreads();
         }
         if constexpr (OUT == kToEntries) {                     // the words are keys alone, and these are their final places
-            // the order inside a digit's run is the final one, so a destination's entries are neighbours
+            // the order inside a digit's run is the final one, so the tile's destinations ascend
             const uint32_t src_mask = (uint32_t)((1ull << a.cand.src_bits) - 1ull);
+            auto dst_at = [&](int i) { return i < count ? (uint32_t)(sm.keys[i] >> a.cand.src_bits) : 0xffffffffu; };
+            auto write = [&](int i, u64 k) {
+                const int64_t pos = (int64_t)sm.to_global[(int)(k >> a.shift) & a.mask] + i;
+                __stcs(a.col_out + pos, (int32_t)((uint32_t)k & src_mask));
+            };
+            const uint32_t n = (uint32_t)a.cand.n;                               // dropped candidates have it for a destination and come last
+            // An atomic for every 32 entries of a row, all on a few words, made the two sweeps of 40 M entries of 1 / 10 / 1000 rows
+            // 1225 / 1310 / 775 us instead of 584 / 665 / 539.  So in a tile with many keys of one digit value, kBlock entries of one row are added
+            // together (asked of every tile, 132,534 rows would take 1.5 % longer).
+            if (!sm.long_run) {
 #pragma unroll 4
-            for (int i0 = tid - lane; i0 < count; i0 += kBlock) {
-                const int i = i0 + lane;
-                const u64 k = i < count ? sm.keys[i] : ~0ull;
-                const uint32_t d = (uint32_t)(k >> a.cand.src_bits);
-                const bool ok = i < count && d < (uint32_t)a.cand.n;             // dropped candidates come last
-                if (ok) {
-                    const int64_t pos = (int64_t)sm.to_global[(int)(k >> a.shift) & a.mask] + i;
-                    __stcs(a.col_out + pos, (int32_t)((uint32_t)k & src_mask));
+                for (int i0 = tid - lane; i0 < count; i0 += kBlock) {
+                    const int i = i0 + lane;
+                    const u64 k = i < count ? sm.keys[i] : ~0ull;
+                    const uint32_t d = (uint32_t)(k >> a.cand.src_bits);
+                    const bool ok = i < count && d < n;
+                    if (ok) write(i, k);
+                    count_runs(d, ok, a.degree);
                 }
-                count_runs(d, ok, a.degree);
+            } else {
+                static_assert(kTile / kBlock <= 32, "a lane for kBlock entries");
+                const unsigned whole = __ballot_sync(0xffffffffu, lane < kTile / kBlock && (lane + 1) * kBlock <= count &&
+                                                                  dst_at(lane * kBlock) == dst_at((lane + 1) * kBlock - 1));
+#pragma unroll 1
+                for (int i = tid; i < count; i += kBlock) {
+                    const u64 k = sm.keys[i];
+                    if ((uint32_t)(k >> a.cand.src_bits) < n) write(i, k);
+                }
+                if (tid < kTile / kBlock && (whole >> tid & 1u) && dst_at(tid * kBlock) < n) atomicAdd(a.degree + dst_at(tid * kBlock), kBlock);
+                for (unsigned rest = ~whole & ((1u << (count + kBlock - 1) / kBlock) - 1u); rest; rest &= rest - 1u) {
+                    const uint32_t d = dst_at((__ffs(rest) - 1) * kBlock + tid);
+                    count_runs(d, d < n, a.degree);
+                }
             }
         } else
 #pragma unroll 4
@@ -1002,9 +1029,10 @@ rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ 
         if (slot_tile_row) {
             int32_t t = (int32_t)(((int64_t)ptr + kSlotTile - 1) / kSlotTile);
             const int32_t t_end = (int32_t)(((int64_t)ptr + deg[j] + kSlotTile - 1) / kSlotTile);      // t where the row starts no piece
-            // the pieces of a long row are written by the whole warp: by one thread, those of a row of 40 M entries took 90 us
-            unsigned many = __ballot_sync(0xffffffffu, t_end - t > 4);
-            if (t_end - t <= 4)
+            // many pieces of one row are written by the whole warp: by one thread, those of a row of 40 M entries took 90 us (but 20 pieces each
+            // of 1000 neighbouring rows by whole warps 56 instead of 21)
+            unsigned many = __ballot_sync(0xffffffffu, t_end - t > 64);
+            if (t_end - t <= 64)
                 for (; t < t_end; ++t) slot_tile_row[t] = (int32_t)v;
             for (; many; many &= many - 1u) {
                 const int from = __ffs(many) - 1;

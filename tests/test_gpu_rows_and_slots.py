@@ -101,3 +101,30 @@ def test_row_pointers_of_one_long_row():
     one, every = torch.full_like(src, 7), torch.randint(n, (m,), dtype=torch.int32, device="cuda")
     spread = kernel_ms(g, lambda: g.oneshot("gcn", n, src, every, x), "rows_from_degrees")
     assert kernel_ms(g, lambda: g.oneshot("gcn", n, src, one, x), "rows_from_degrees") < spread + 0.008
+
+
+@pytest.mark.parametrize("rows", [1, 10, 3000])
+def test_long_rows_are_counted_as_fast_as_short_ones(rows):
+    """The last sweep of the one-shot path adds a run of equal destinations once, not once per 32 entries (which took twice as long for
+    rows of millions of entries)."""
+    import paper_2104_03058_b200 as g
+    n, m = 130_000, 20_000_000
+    src, dst = (torch.randint(n, (m,), dtype=torch.int32, device="cuda") for _ in range(2))
+    x, few = torch.ones((n, 4), device="cuda"), dst % rows * (n // rows)
+    spread = kernel_ms(g, lambda: g.oneshot("sage", n, src, dst, x), "radix_sweep")
+    assert kernel_ms(g, lambda: g.oneshot("sage", n, src, few, x), "radix_sweep") < 1.4 * spread
+
+
+@pytest.mark.parametrize("m", [31, 32, 33, 2047, 2048, 6200, 148 * 4 * 8192 + 77])
+def test_degrees_of_runs(m):
+    """Runs of lengths around the 32 entries that a warp looks at together, in tiles of both sizes."""
+    import paper_2104_03058_b200 as g
+    rng = np.random.default_rng(m)
+    for lengths in (rng.integers(1, 100, m), rng.choice([31, 32, 33, 63, 64, 65, 96], m), rng.choice([1, 2000, 2100], m), np.full(m, 32)):
+        dst = np.repeat(np.arange(m), lengths)[:m].astype(np.int32)
+        n = int(dst[-1]) + 2
+        src, dst = rng.integers(0, n, m).astype(np.int32), dst[rng.permutation(m)]
+        got = g.oneshot("sage", n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), torch.from_numpy(np.arange(n, dtype=np.float32)[:, None] % 64).cuda())
+        deg = np.bincount(dst, minlength=n)
+        want = (np.bincount(dst, weights=src % 64, minlength=n).astype(np.float32) * np.where(deg > 0, 1 / np.maximum(deg, 1), 0).astype(np.float32))
+        np.testing.assert_array_equal(got.cpu().numpy()[:, 0], want)
