@@ -128,3 +128,16 @@ def test_degrees_of_runs(m):
         deg = np.bincount(dst, minlength=n)
         want = (np.bincount(dst, weights=src % 64, minlength=n).astype(np.float32) * np.where(deg > 0, 1 / np.maximum(deg, 1), 0).astype(np.float32))
         np.testing.assert_array_equal(got.cpu().numpy()[:, 0], want)
+
+
+@pytest.mark.parametrize("rows", [1000, 8_000_000])
+def test_row_pointers_of_many_vertices(rows):
+    """Blocks of vertices without entries find their row pointers without searching all keys thread by thread (which took twice the time
+    of the sweep over the rows)."""
+    import paper_2104_03058_b200 as g
+    n, m = 8_000_000, 1_000_000
+    src, dst = (torch.randint(k, (m,), dtype=torch.int32, device="cuda") for k in (n, rows))
+    times = [kernel_ms(g, lambda: g.build_csr(n, src, dst, 0), k) for k in ("rows_and_degrees", "radix_sweep_rows")]
+    assert times[0] < (1.6 if rows == 1000 else 2.0) * times[1]
+    csr, deg = g.build_csr(n, src, dst, 0), torch.bincount(dst, minlength=n)
+    assert torch.equal(csr.row_ptr.long(), torch.cat([deg.new_zeros(1), deg.cumsum(0)]))
