@@ -371,8 +371,8 @@ __global__ void __launch_bounds__(kBlock, min_blocks(sizeof(T), WEIGHTED, SHARED
 
 // out[row, j] = scale * sum over the row's segments, ascending, of partial[segment, j]
 __global__ void __launch_bounds__(kBlock)
-hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict__ hub_seg_ptr, const float* __restrict__ rdeg,
-           const float* __restrict__ partial, int64_t hub_begin, int32_t n_hub, int32_t f, int32_t fpad, int use_rdeg,
+hub_reduce(const int32_t* row_order, const int32_t* hub_seg_ptr, const float* rdeg,
+           const float* partial, int64_t hub_begin, int32_t n_hub, int32_t f, int32_t fpad, int use_rdeg,
            void* __restrict__ out, int64_t ldo, int out_bf16)
 {
     grid_dependency<true>();
@@ -435,7 +435,7 @@ static GatherKernel pick_kernel(gnnfd_dtype_t xdt, bool vec, int lpr, int vpl, b
 // One 16-byte vector of the copy per thread: chunks of cw columns placed `pitch` columns apart, rows ld apart, zeros between.
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-align_features(const T* __restrict__ x, int64_t ldx, int64_t n, int32_t f, int32_t cw, int32_t pitch, uint32_t ld, uint4* __restrict__ out)
+align_features(const T* x, int64_t ldx, int64_t n, int32_t f, int32_t cw, int32_t pitch, uint32_t ld, uint4* __restrict__ out)
 {
     grid_dependency<true>();
     constexpr int VECN = 16 / sizeof(T);

@@ -68,10 +68,16 @@ struct LaunchScope {
 // A call is a chain of launches, on small graphs of a few microseconds each.  Every kernel of the library is launched with
 // programmatic stream serialisation: where the kernel before it lets it (grid_dependency<true>), its blocks take their places as soon as all
 // blocks of that one have started.  They wait there (grid_dependency, the first statement of every kernel) until that launch has
-// ended and its writes can be seen; as every kernel waits before it reads or writes memory, what happens in memory is what plain
-// launches do.  Build and aggregation of 20,000 vertices and 89,000 edges 134 -> 118 us, GAT 8 x 8 on 200,000 rows 121 -> 115.  Kernels that
-// leave an SM with little L1 (tensor tiles, large sort tiles, compaction) do not let the next one start early: it would keep
-// that share for as long as it runs (GCN layer 602 -> 64 on 116 M entries 1.78 -> 2.28 ms, build of 80 M edges 2.85 -> 3.14); nor do the edge
+// ended and its writes can be seen.  Every kernel waits before it reads or writes memory, and reads what launches before it may have written
+// by plain loads: the non-coherent path is for memory that nobody writes while the kernel exists, and it exists already while the one before it
+// writes (plain loads cost nothing: GAT 8 x 16 bf16 on 39.6 M entries 906 -> 889 us, all else the same).
+// Build and aggregation of 20,000 vertices and 89,000 edges 134 -> 118 us, GAT 8 x 8 on 200,000 rows 121 -> 115.
+// A kernel lets the next one start when it has waited itself, not before: with several launches lined up, the longest rows of one, which come
+// first, took the places that the last blocks of another left, a few SMs for most of them.  20,000 rows of 50 entries, GCN, 256 bf16
+// columns one at a time 46, lined up 53, now 44 us; GAT 1 x 64 40, 42, 35; 5000 rows of 100, GAT 4 x 32 fp32 37, 45, 34.  The
+// GAT aggregation, whose scores come in between, does not let it start at all (20,000 rows of 50, 4 x 32 64 -> 56 us).
+// Nor do kernels that leave an SM with little L1 (tensor tiles, large sort tiles, compaction): the next one would keep
+// that share for as long as it runs (GCN layer 602 -> 64 on 116 M entries 1.78 -> 2.28 ms, build of 80 M edges 2.85 -> 3.14); nor the edge
 // softmax kernels (20,000 rows of 50 entries 37 -> 41 us).
 template <typename... Params, typename... Args>
 inline void launch_early(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args)
@@ -92,8 +98,8 @@ inline void launch_early(void (*kernel)(Params...), dim3 grid, dim3 block, size_
 template <bool LET_NEXT_START>
 __device__ __forceinline__ void grid_dependency()
 {
-    if (LET_NEXT_START) asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (LET_NEXT_START) asm volatile("griddepcontrol.launch_dependents;");
 }
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) radix_swee
 
 // The buckets' first words and tiles from the counts of the highest digit; one block.
 __global__ void __launch_bounds__(kBuckets)
-bucket_tables(const int32_t* __restrict__ count, int tile_keys, BucketTables* __restrict__ tables)
+bucket_tables(const int32_t* count, int tile_keys, BucketTables* __restrict__ tables)
 {
     grid_dependency<true>();
     __shared__ int32_t smem[32];
@@ -680,7 +680,7 @@ bucket_tables(const int32_t* __restrict__ count, int tile_keys, BucketTables* __
 // Digit counts of every further pass, for every bucket: blocks take runs of consecutive tiles and add to the global counts when they
 // come to another bucket.
 __global__ void __launch_bounds__(kThreads)
-bucket_histograms(const u64* __restrict__ keys, const BucketTables* __restrict__ tables, const BuildCounts* __restrict__ counts, int tile_keys,
+bucket_histograms(const u64* keys, const BucketTables* tables, const BuildCounts* counts, int tile_keys,
                   int first_bit, int digit_bits, int passes, int32_t* __restrict__ hist)
 {
     grid_dependency<true>();
@@ -703,7 +703,7 @@ bucket_histograms(const u64* __restrict__ keys, const BucketTables* __restrict__
         for (int64_t at = begin + threadIdx.x; at < end; at += kThreads * kHistItems) {
             u64 word[kHistItems];
 #pragma unroll
-            for (int j = 0; j < kHistItems; ++j) word[j] = at + j * kThreads < end ? __ldg(keys + at + j * kThreads) : 0ull;
+            for (int j = 0; j < kHistItems; ++j) word[j] = at + j * kThreads < end ? keys[at + j * kThreads] : 0ull;
 #pragma unroll
             for (int j = 0; j < kHistItems; ++j) {
                 u64 k = word[j] >> first_bit;
@@ -733,10 +733,10 @@ constexpr int kUniqueTile = kThreads * kUniqueItems;
 __device__ __forceinline__ int64_t sorted_candidates(const BuildCounts* counts) { return counts->sort_failed ? 0 : counts->n_valid; }
 
 // bit j of the result: candidate first + j is the first of a run of equal keys among the n_valid kept ones
-__device__ __forceinline__ uint32_t first_of_run_mask(const u64* __restrict__ keys, int64_t first, int64_t n_valid, int val_bits,
+__device__ __forceinline__ uint32_t first_of_run_mask(const u64* keys, int64_t first, int64_t n_valid, int val_bits,
                                                       u64 (&word)[kUniqueItems])
 {
-    u64 prev = first > 0 && first <= n_valid ? (__ldg(keys + first - 1) >> val_bits) : 0ull;
+    u64 prev = first > 0 && first <= n_valid ? (keys[first - 1] >> val_bits) : 0ull;
     if (first + kUniqueItems <= n_valid) {            // whole group present: 16-byte loads (first is a multiple of 8)
         const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(keys + first);
 #pragma unroll
@@ -784,7 +784,7 @@ __device__ __forceinline__ int32_t block_prefix_256(int32_t v, int32_t* total, i
 }
 
 __global__ void __launch_bounds__(kThreads)
-unique_tile_counts(const u64* __restrict__ keys, int val_bits, const BuildCounts* __restrict__ counts,
+unique_tile_counts(const u64* keys, int val_bits, const BuildCounts* counts,
                    int32_t* __restrict__ tile_count)
 {
     grid_dependency<true>();
@@ -799,7 +799,7 @@ unique_tile_counts(const u64* __restrict__ keys, int val_bits, const BuildCounts
 
 // tile_first[t] = kept candidates in earlier tiles; the kept ones move to keys_out / perm in order
 __global__ void __launch_bounds__(kThreads)
-compact_unique(const u64* __restrict__ keys, const int32_t* __restrict__ vals, const int32_t* __restrict__ tile_first,
+compact_unique(const u64* keys, const int32_t* vals, const int32_t* tile_first,
                int64_t m, int val_bits, u64* __restrict__ keys_out, int32_t* __restrict__ perm,
                BuildCounts* __restrict__ counts)
 {
@@ -840,7 +840,7 @@ constexpr int kClasses = kHubClass + 1;
 static_assert(kClasses <= kClassMask + 1 && kClassMask < kRadix, "digit of the row sweep");
 
 __global__ void __launch_bounds__(kThreads)
-rows_and_degrees(const u64* __restrict__ keys, BuildCounts* __restrict__ counts, int64_t n, int src_bits, int val_bits,
+rows_and_degrees(const u64* keys, BuildCounts* __restrict__ counts, int64_t n, int src_bits, int val_bits,
                  int dedup, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
                  int32_t* __restrict__ class_count)
 {
@@ -918,8 +918,8 @@ constexpr int kKeyItems = 4;                          // entries per thread of f
 
 // col_idx, the GCN weight and (unless the duplicate removal already wrote it) perm of every slot
 __global__ void __launch_bounds__(kThreads)
-finalize_entries(const u64* __restrict__ keys, const int32_t* __restrict__ vals, int write_perm,
-                 const BuildCounts* __restrict__ counts, int src_bits, int val_bits, const float* __restrict__ dinv,
+finalize_entries(const u64* keys, const int32_t* vals, int write_perm,
+                 const BuildCounts* counts, int src_bits, int val_bits, const float* dinv,
                  int32_t* __restrict__ col_idx, float* __restrict__ edge_w, int32_t* __restrict__ perm, int64_t m)
 {
     grid_dependency<true>();
@@ -935,8 +935,8 @@ finalize_entries(const u64* __restrict__ keys, const int32_t* __restrict__ vals,
 #pragma unroll
     for (int j = 0; j < kKeyItems; ++j) {
         const u64 key = word[j] >> val_bits;
-        ws[j] = __ldg(dinv + (int32_t)(key & ((1ull << src_bits) - 1ull)));       // 0 for the padding words: in range
-        wd[j] = __ldg(dinv + (int32_t)(key >> src_bits));
+        ws[j] = dinv[(int32_t)(key & ((1ull << src_bits) - 1ull))];       // 0 for the padding words: in range
+        wd[j] = dinv[(int32_t)(key >> src_bits)];
     }
 #pragma unroll
     for (int j = 0; j < kKeyItems; ++j) {
@@ -997,7 +997,7 @@ constexpr int kSlotItems = 8;                        // entries per thread of sl
 constexpr int kSlotTile = kThreads * kSlotItems;
 
 __global__ void __launch_bounds__(kThreads)
-rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ counts, int64_t n, int32_t* __restrict__ ticket,
+rows_from_degrees(const int32_t* degree, BuildCounts* __restrict__ counts, int64_t n, int32_t* __restrict__ ticket,
                   u64* __restrict__ words, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
                   int32_t* __restrict__ class_count, int32_t* __restrict__ slot_tile_row)
 {
@@ -1081,8 +1081,8 @@ rows_from_degrees(const int32_t* __restrict__ degree, BuildCounts* __restrict__ 
 constexpr int kMarkedRows = 3 * kSlotTile;
 
 __global__ void __launch_bounds__(kThreads)
-slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ slot_tile_row,
-             const float* __restrict__ dinv, const BuildCounts* __restrict__ counts, float* __restrict__ edge_w)
+slot_weights(const int32_t* row_ptr, const int32_t* col_idx, const int32_t* slot_tile_row,
+             const float* dinv, const BuildCounts* counts, float* __restrict__ edge_w)
 {
     grid_dependency<true>();
     __shared__ __align__(16) int32_t row_of[kSlotTile];
@@ -1110,7 +1110,7 @@ slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ co
 #pragma unroll
         for (int j = 0; j < kSlotItems; j += 4) reinterpret_cast<int4*>(row_of)[tid + j / 4 * kThreads] = make_int4(0, 0, 0, 0);
 #pragma unroll
-        for (int j = 0; j < kSlotItems; ++j) ws[j] = __ldg(dinv + u[j]);
+        for (int j = 0; j < kSlotItems; ++j) ws[j] = dinv[u[j]];
         __syncthreads();
         for (int32_t r = row0 + 1 + tid; r <= row1; r += kThreads) {     // empty rows share their start with a later one, which counts
             const int64_t at = row_ptr[r] - base;
@@ -1135,7 +1135,7 @@ slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ co
     } else {
 #pragma unroll
         for (int j = 0; j < kSlotItems; ++j) {
-            ws[j] = __ldg(dinv + u[j]);
+            ws[j] = dinv[u[j]];
             row[j] = 0;
         }
         // the last row that starts at the entry or before it: the searches of a thread's entries take the same steps side by side
@@ -1149,7 +1149,7 @@ slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ co
     }
     float w[kSlotItems];
 #pragma unroll
-    for (int j = 0; j < kSlotItems; ++j) w[j] = ws[j] * __ldg(dinv + row0 + max(row[j], earlier));
+    for (int j = 0; j < kSlotItems; ++j) w[j] = ws[j] * dinv[row0 + max(row[j], earlier)];
     if (whole) {
 #pragma unroll
         for (int j = 0; j < kSlotItems; j += 4)
@@ -1169,7 +1169,7 @@ slot_weights(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ co
 // its slot: slots count a row's segments in ascending source order, row after row, and index the partial
 // results, so that the per-row reductions run over a contiguous, ordered slot range.
 
-__device__ __forceinline__ int32_t lower_bound_col(const int32_t* __restrict__ col, int32_t lo, int32_t hi, int64_t bound)
+__device__ __forceinline__ int32_t lower_bound_col(const int32_t* col, int32_t lo, int32_t hi, int64_t bound)
 {
     while (lo < hi) {
         const int32_t mid = lo + ((hi - lo) >> 1);
@@ -1179,7 +1179,7 @@ __device__ __forceinline__ int32_t lower_bound_col(const int32_t* __restrict__ c
 }
 
 // segments of hub row v per source range (stored `pitch` apart) and altogether
-__device__ __forceinline__ int32_t count_row_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+__device__ __forceinline__ int32_t count_row_segments(const int32_t* row_ptr, const int32_t* col_idx,
                                                       int32_t v, int32_t* range_count, int64_t pitch, int32_t n_ranges,
                                                       int64_t range_rows)
 {
@@ -1196,7 +1196,7 @@ __device__ __forceinline__ int32_t count_row_segments(const int32_t* __restrict_
 }
 
 // the segments themselves: `slot` is the row's first slot, range_first (`pitch` apart) its first schedule position per range
-__device__ __forceinline__ void fill_row_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+__device__ __forceinline__ void fill_row_segments(const int32_t* row_ptr, const int32_t* col_idx,
                                                   int32_t v, int32_t slot, const int32_t* range_first, int64_t pitch,
                                                   int32_t n_ranges, int64_t range_rows, int32_t* __restrict__ seg_row,
                                                   int32_t* __restrict__ seg_begin, int32_t* __restrict__ seg_end,
@@ -1220,8 +1220,8 @@ __device__ __forceinline__ void fill_row_segments(const int32_t* __restrict__ ro
 // per hub row and source range: the number of segments (range-major: count[r * hub_cap + i]) and per hub row
 // the total; entries past the last hub row are 0 so that the scans yield the totals
 __global__ void __launch_bounds__(kThreads)
-hub_segment_counts(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                   const int32_t* __restrict__ row_order, int64_t n, const BuildCounts* __restrict__ counts, int64_t hub_cap,
+hub_segment_counts(const int32_t* row_ptr, const int32_t* col_idx,
+                   const int32_t* row_order, int64_t n, const BuildCounts* counts, int64_t hub_cap,
                    int32_t n_ranges, int64_t range_rows, int32_t* __restrict__ range_count, int32_t* __restrict__ seg_count)
 {
     grid_dependency<true>();
@@ -1241,9 +1241,9 @@ hub_segment_counts(const int32_t* __restrict__ row_ptr, const int32_t* __restric
 // range_first: exclusive scan of range_count (the schedule position of a row's first segment in a range);
 // hub_seg_ptr: exclusive scan of seg_count (the row's first slot)
 __global__ void __launch_bounds__(kThreads)
-fill_segments(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ row_order,
-              int64_t n, BuildCounts* __restrict__ counts, const int32_t* __restrict__ hub_seg_ptr,
-              const int32_t* __restrict__ range_first, int64_t hub_cap, int32_t n_ranges, int64_t range_rows,
+fill_segments(const int32_t* row_ptr, const int32_t* col_idx, const int32_t* row_order,
+              int64_t n, BuildCounts* __restrict__ counts, const int32_t* hub_seg_ptr,
+              const int32_t* range_first, int64_t hub_cap, int32_t n_ranges, int64_t range_rows,
               int32_t* __restrict__ seg_row, int32_t* __restrict__ seg_begin, int32_t* __restrict__ seg_end,
               int32_t* __restrict__ seg_slot)
 {
@@ -1262,7 +1262,7 @@ constexpr int kFewHubPieces = 8192;
 constexpr int kHubThreads = 1024;
 
 __global__ void __launch_bounds__(kHubThreads)
-hub_segments_few(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const int32_t* __restrict__ row_order,
+hub_segments_few(const int32_t* row_ptr, const int32_t* col_idx, const int32_t* row_order,
                  int64_t n, BuildCounts* __restrict__ counts, int32_t n_ranges, int64_t range_rows, int32_t* range_count,
                  int32_t* hub_seg_ptr, int32_t* __restrict__ seg_row, int32_t* __restrict__ seg_begin,
                  int32_t* __restrict__ seg_end, int32_t* __restrict__ seg_slot)

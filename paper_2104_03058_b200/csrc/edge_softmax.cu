@@ -60,14 +60,14 @@ __device__ __forceinline__ void load_heads(const float* p, float (&v)[HB])
     if constexpr (HB % 4 == 0) {
 #pragma unroll
         for (int i = 0; i < HB; i += 4) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(p + i));
+            const float4 q = *reinterpret_cast<const float4*>(p + i);
             v[i] = q.x; v[i + 1] = q.y; v[i + 2] = q.z; v[i + 3] = q.w;
         }
     } else if constexpr (HB == 2) {
-        const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 q = *reinterpret_cast<const float2*>(p);
         v[0] = q.x; v[1] = q.y;
     } else {
-        v[0] = __ldg(p);
+        v[0] = *p;
     }
 }
 
@@ -117,7 +117,7 @@ template <int NF>
 __device__ __forceinline__ void load_cols(const SoftmaxArgs& a, int32_t k, int32_t e, int32_t step, int32_t (&u)[NF])
 {
 #pragma unroll
-    for (int i = 0; i < NF; ++i) u[i] = k + i * step < e ? __ldg(a.col_idx + k + i * step) : -1;
+    for (int i = 0; i < NF; ++i) u[i] = k + i * step < e ? a.col_idx[k + i * step] : -1;
 }
 
 // base-2 logits of the slots whose column indices are u[].  FULL: all of them exist; otherwise the

@@ -60,7 +60,7 @@ __device__ __forceinline__ float merge_scale(float m, float m_new)
 // it touched to a later instruction (25 us for [200,000, 8 x 8] fp32, 51 MB).
 template <typename T, int VECN>
 __global__ void __launch_bounds__(kBlock)
-gat_scores(const T* __restrict__ z, int64_t ldz, const float* __restrict__ a_src, const float* __restrict__ a_dst,
+gat_scores(const T* z, int64_t ldz, const float* a_src, const float* a_dst,
            int64_t n, int heads, int dim, float* __restrict__ s_src, float* __restrict__ s_dst)
 {
     grid_dependency<true>();
@@ -76,8 +76,8 @@ gat_scores(const T* __restrict__ z, int64_t ldz, const float* __restrict__ a_src
         zv.load(zr + d);
 #pragma unroll
         for (int i = 0; i < VECN; ++i) {
-            ss = fmaf(__ldg(as + d + i), zv.get(i), ss);
-            sd = fmaf(__ldg(ad + d + i), zv.get(i), sd);
+            ss = fmaf(load4(as + d + i), zv.get(i), ss);
+            sd = fmaf(load4(ad + d + i), zv.get(i), sd);
         }
     }
     s_src[idx] = ss;
@@ -153,7 +153,7 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
         b = min(b + sharer * share, e);
         e = min(b + share, e);
     }
-    // one 32-byte load per entry where every row start allows it (a lane past the chunk's end loads the row's first pair)
+    // one 32-byte load per entry where every row start allows it (a lane past the chunk's end loads the chunk's last pair)
     const bool wide = a.wide_ok;
     const float sd = active ? a.s_dst[(int64_t)row * a.heads + h] : 0.f;
     const float* ssrc = a.s_src + h;
@@ -232,7 +232,7 @@ __device__ __forceinline__ void gat_rows(const GatArgs& a, const Range& rg, int 
                     const int32_t u = stage_col[buf][warp][r * 32 + seg + t * EP + g];
                     valid[i] = FULL || u >= 0;
                     const uint32_t uu = FULL ? (uint32_t)u : (uint32_t)max(u, 0);
-                    lg[i] = valid[i] ? __ldg(ssrc + (size_t)uu * heads) : 0.f;
+                    lg[i] = valid[i] ? load4(ssrc + (size_t)uu * heads) : 0.f;
                     const size_t off = (size_t)uu * ld;
                     if (VPL == 2 && VECN * sizeof(T) == 16 && wide) {
                         if (valid[i]) load_pair(v[i][0], v[i][VPL - 1], zq[0] + off);     // the lane's two vectors are adjacent
@@ -379,7 +379,7 @@ template <typename T, int VECN, int LPR, int VPL, bool SHARED>
 // the vector-pair forms and four for the others is what the measured-good builds had.
 __global__ void __launch_bounds__(kBlock, (VPL == 2 && VECN > 1) ? 3 : 4) gat_aggregate(const __grid_constant__ GatArgs a)
 {
-    grid_dependency<true>();
+    grid_dependency<false>();
     __shared__ int32_t stage_col[2][kBlock / 32][stage_slots(LPR, VPL)];
     // second-level sums and denominator (and a sharer's maximum), one column per thread
     __shared__ float tot_s[VPL * VECN + 1 + SHARED][kBlock];
@@ -417,8 +417,8 @@ constexpr int kReduceCols = 64;
 constexpr int kReduceWays = kBlock / kReduceCols;
 
 __global__ void __launch_bounds__(kBlock)
-gat_hub_reduce(const int32_t* __restrict__ row_order, const int32_t* __restrict__ hub_seg_ptr,
-               const float* __restrict__ partial, const float* __restrict__ partial_ml, int64_t hub_begin, int32_t n_hub,
+gat_hub_reduce(const int32_t* row_order, const int32_t* hub_seg_ptr,
+               const float* partial, const float* partial_ml, int64_t hub_begin, int32_t n_hub,
                int32_t f, int32_t fpad, int32_t heads, int32_t dim, int32_t out_dim, void* __restrict__ out, int64_t ldo, int out_bf16)
 {
     grid_dependency<true>();

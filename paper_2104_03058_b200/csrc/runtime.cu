@@ -90,7 +90,7 @@ __device__ __forceinline__ void load_scan_items(const int32_t* in, size_t base, 
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* __restrict__ in, size_t count,
+__global__ void __launch_bounds__(kScanThreads) scan_tile_sums(const int32_t* in, size_t count,
                                                              int32_t* __restrict__ sums)
 {
     grid_dependency<true>();

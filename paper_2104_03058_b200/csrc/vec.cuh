@@ -9,23 +9,41 @@ namespace gnnfd {
 
 // ---- per-lane vectors: VECN elements of T, widened to fp32
 
+// plain loads from global memory: what they read may have been written by the launch before (see grid_dependency)
+__device__ __forceinline__ uint4 load16(const void* p)
+{
+    uint4 v;
+    asm("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float load4(const float* p)
+{
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 template <typename T, int VECN> struct Vec;
 
 template <> struct Vec<float, 4> {
     float4 v;
-    __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float4*>(p)); }
+    __device__ __forceinline__ void load(const float* p)
+    {
+        const uint4 w = load16(p);
+        v = make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+    }
     __device__ __forceinline__ void zero() { v = make_float4(0.f, 0.f, 0.f, 0.f); }
     __device__ __forceinline__ float get(int i) const { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 };
 template <> struct Vec<float, 1> {
     float v;
-    __device__ __forceinline__ void load(const float* p) { v = __ldg(p); }
+    __device__ __forceinline__ void load(const float* p) { v = load4(p); }
     __device__ __forceinline__ void zero() { v = 0.f; }
     __device__ __forceinline__ float get(int) const { return v; }
 };
 template <> struct Vec<__nv_bfloat16, 8> {
     uint4 v;
-    __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const uint4*>(p)); }
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = load16(p); }
     __device__ __forceinline__ void zero() { v = make_uint4(0u, 0u, 0u, 0u); }
     __device__ __forceinline__ uint32_t word(int i) const { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
     __device__ __forceinline__ float get(int i) const
@@ -44,7 +62,7 @@ __device__ __forceinline__ void add_widened(float& x, float& y, uint32_t w)
 }
 template <> struct Vec<__nv_bfloat16, 1> {
     unsigned short v;
-    __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const unsigned short*>(p)); }
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { asm("ld.global.b16 %0, [%1];" : "=h"(v) : "l"(p)); }
     __device__ __forceinline__ void zero() { v = 0; }
     __device__ __forceinline__ float get(int) const { return __uint_as_float((uint32_t)v << 16); }
 };
@@ -55,7 +73,7 @@ template <> struct Vec<__nv_bfloat16, 1> {
 __device__ __forceinline__ void load_pair(Vec<float, 4>& a, Vec<float, 4>& b, const float* p)
 {
     uint32_t r[8];
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "l"(p));
     a.v = make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3]));
@@ -63,7 +81,7 @@ __device__ __forceinline__ void load_pair(Vec<float, 4>& a, Vec<float, 4>& b, co
 }
 __device__ __forceinline__ void load_pair(Vec<__nv_bfloat16, 8>& a, Vec<__nv_bfloat16, 8>& b, const __nv_bfloat16* p)
 {
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(a.v.x), "=r"(a.v.y), "=r"(a.v.z), "=r"(a.v.w), "=r"(b.v.x), "=r"(b.v.y), "=r"(b.v.z), "=r"(b.v.w)
                  : "l"(p));
 }
