@@ -583,7 +583,7 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     a.out_vec_ok = odt == GNNFD_F32 && ((uintptr_t)d_out % 16 == 0) && (ldo % 4 == 0) && (n_chunks == 1 || cw % 4 == 0);
 
     const int per_step = kLoads / vpl * (32 / lpr);
-    const int64_t limit = walk_limit(csr, per_step, a.n_ctiles);
+    const int64_t limit = walk_limit(csr, per_step, a.n_ctiles, 16, min_blocks(xsize, weighted, true, lpr));
     const int64_t blocks = plan_ranges(csr, gather_groups(), lpr, per_step, limit, a.range, &a.n_ranges);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;

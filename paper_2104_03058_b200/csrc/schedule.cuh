@@ -63,11 +63,13 @@ inline int warps_log2_for(int entries, int per_step, int64_t limit)
 // bits.  In entries the limit is 2 * nnz * tiles / 3552: with one tile, rows are split on graphs of up to 3.6 M entries.  fp32 GCN
 // against unsplit rows (one warp up to 2048 entries): 4,000 rows of 10 entries and 304 columns 76 -> 18 us, 20,000 of 50 and
 // 128 columns 101 -> 40, 100,000 of 20 and 64 columns 75 -> 50.  With the average itself or four times it as the limit: 38 and
-// 58 us for the second, 52 and 75 for the third.
-inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t tiles, int64_t at_least = 16)
+// 58 us for the second, 52 and 75 for the third.  `blocks_per_sm`: blocks of the kernel that an SM holds.  Kernels with four are slower per warp and have
+// more slots: counted as three, SAGE of 72 / 96 fp32 columns on 20,000 rows of 50 took 32 us instead of 26.5, on 100,000 of 20 61 / 62 instead
+// of 48 / 49, of 64 columns on 20,000 rows of 50 23 instead of 20.
+inline int64_t walk_limit(const gnnfd_csr_t* csr, int per_step, int64_t tiles, int64_t at_least = 16, int blocks_per_sm = 3)
 {
-    constexpr int64_t kWarpSlots = 148 * 24;
-    const int64_t limit = 2 * (csr->nnz * tiles / (per_step * kWarpSlots));
+    const int64_t warp_slots = (int64_t)148 * blocks_per_sm * (kBlock / 32);
+    const int64_t limit = 2 * (csr->nnz * tiles / (per_step * warp_slots));
     return limit > at_least ? limit : at_least;
 }
 
