@@ -139,8 +139,8 @@ void launch_copy(const void* d_x, int64_t ldx, gnnfd_dtype_t xdt, int64_t n, int
 
 // ---- pieces of one translation unit that the layer entry points (layer.cu) put together
 
-int64_t segment_capacity(int64_t n, int64_t e, uint32_t flags);      // csr_build.cu; -1 for sizes the build rejects
-
+int csr_sizes(int64_t n, int64_t e, uint32_t flags, bool for_smaller, size_t* persistent_bytes, size_t* scratch_bytes,
+              int64_t* segments);                                     // csr_build.cu
 int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, gnnfd_itype_t itype, uint32_t flags, bool need_perm,
                    bool need_weights, void* d_persistent, size_t persistent_bytes, void* d_scratch, size_t scratch_bytes, cudaStream_t s,
                    gnnfd_csr_t** out);                                // csr_build.cu

@@ -1306,6 +1306,7 @@ struct BuildLayout {
     int64_t tile_cap, row_tile_cap;      // tiles that words are reserved for
     int64_t hub_cap;       // upper bound on hub rows
     int64_t seg_cap;       // upper bound on hub segments
+    int range_cap;         // source ranges that words are reserved for
     int src_bits, key_bits, passes, digit_bits;     // passes: sweeps over the edges but the one that makes buckets
     int first_bit;         // lowest key bit the sort looks at (0; src_bits when rows keep their input order)
     int n_ranges;          // source ranges the hub rows are cut at (1: no cut)
@@ -1316,6 +1317,12 @@ struct BuildLayout {
     int top_bits;          // > 0: the first sweep takes this many highest bits of the destination and makes buckets of them
     int sweeps() const { return passes + (top_bits > 0); }
 };
+
+static void reserve_ranges(BuildLayout* L, int ranges)
+{
+    L->range_cap = ranges;
+    L->seg_cap = L->m / kHubSegment + L->hub_cap * ranges + 1;
+}
 
 static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L, bool with_vals = true)
 {
@@ -1343,7 +1350,9 @@ static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L, boo
     L->range_rows = GNNFD_HUB_RANGE_ROWS;
     while ((n + L->range_rows - 1) / L->range_rows > 64) L->range_rows <<= 1;
     L->n_ranges = (flags & GNNFD_CSR_INPUT_ORDER) ? 1 : (int)((n + L->range_rows - 1) / L->range_rows);
-    L->seg_cap = m / kHubSegment + L->hub_cap * L->n_ranges + 1;
+    // (beyond 2^25 vertices wider ranges are fewer: as many are reserved for as smaller graphs have)
+    const int64_t narrow = (n + GNNFD_HUB_RANGE_ROWS - 1) / GNNFD_HUB_RANGE_ROWS;
+    reserve_ranges(L, (flags & GNNFD_CSR_INPUT_ORDER) ? 1 : narrow < 64 ? (int)narrow : 64);
     int bits = 1;
     while ((int64_t(1) << bits) < n) ++bits;
     int dst_bits = 1;
@@ -1367,13 +1376,6 @@ static int make_layout(int64_t n, int64_t e, uint32_t flags, BuildLayout* L, boo
     L->tile_cap = reserved_tiles(m) + (buckets ? kBuckets : 0);
     L->with_vals = with_vals;
     return GNNFD_OK;
-}
-
-// upper bound on the hub segments of any graph with these sizes (what the persistent buffer reserves)
-int64_t segment_capacity(int64_t n, int64_t e, uint32_t flags)
-{
-    BuildLayout L;
-    return make_layout(n, e, flags, &L) == GNNFD_OK ? L.seg_cap : -1;
 }
 
 struct PersistentPtrs {
@@ -1416,7 +1418,7 @@ static size_t flag_ints(const BuildLayout& L)
 {
     // one count per tile of the duplicate removal, or a row per piece of the entries; hub segment counts (per source range and hub row, then per hub row)
     static_assert(kUniqueTile == kSlotTile, "one count or one row for as many candidates");
-    size_t a = (size_t)L.m / kUniqueTile + 2, c = (size_t)L.hub_cap * (L.n_ranges + 1) + 4;
+    size_t a = (size_t)L.m / kUniqueTile + 2, c = (size_t)L.hub_cap * (L.range_cap + 1) + 4;
     return (a > c ? a : c) + 1;
 }
 
@@ -1426,7 +1428,7 @@ static void carve_scratch(Carver& c, const BuildLayout& L, ScratchPtrs* p)
     p->keys_a = c.take<u64>(cap);
     p->keys_b = c.take<u64>(cap);
     // No value buffers when the values travel inside the key words.  With buckets one is enough, but the other is as large as the largest
-    // input without buckets needs: buffers sized for an input hold every smaller one.
+    // input without buckets needs that has fewer candidates.
     const size_t val_cap = !L.with_vals || (L.val_bits > 0 && L.top_bits == 0) ? 1 : cap;
     p->vals_a = c.take<int32_t>(val_cap);
     p->vals_b = c.take<int32_t>(L.top_bits > 0 && (size_t)kSmallInput < val_cap ? (size_t)kSmallInput : val_cap);
@@ -1508,6 +1510,7 @@ int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, g
 
     L.tile_cap = L.n_tiles + (L.top_bits ? kBuckets : 0);      // the query reserves more; what this input needs is enough
     L.row_tile_cap = L.row_tiles;
+    reserve_ranges(&L, L.n_ranges);
     Carver pc(d_persistent, persistent_bytes), sc(d_scratch, scratch_bytes);
     PersistentPtrs P;
     ScratchPtrs S;
@@ -1697,29 +1700,52 @@ int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, g
     return GNNFD_OK;
 }
 
-}  // namespace gnnfd
-
-extern "C" {
-
-int gnnfd_csr_workspace_bytes(int64_t n, int64_t e, uint32_t flags, size_t* persistent_bytes, size_t* scratch_bytes)
+static size_t scratch_size(const BuildLayout& L)
 {
-    using namespace gnnfd;
+    Carver c(nullptr, ~size_t(0));
+    ScratchPtrs s;
+    carve_scratch(c, L, &s);
+    return c.off;
+}
+
+// Sizes of a build's buffers and the most hub segments of such a graph (each may be null).  for_smaller: buffers that hold every graph with
+// fewer vertices or edges too, which is what the queries return.  Larger inputs need more in nearly every place.  Where one more vertex ends the buckets
+// (their keys no longer share a word with the values), the buckets' words are kept: 33,554,432 vertices with 4.9 M edges
+// need 136 MB, one vertex less 144.
+int csr_sizes(int64_t n, int64_t e, uint32_t flags, bool for_smaller, size_t* persistent_bytes, size_t* scratch_bytes, int64_t* segments)
+{
     BuildLayout L;
-    int rc = make_layout(n, e, flags, &L);
+    const int rc = make_layout(n, e, flags, &L);
     if (rc) return rc;
+    if (!for_smaller) reserve_ranges(&L, L.n_ranges);
     if (persistent_bytes) {
         Carver c(nullptr, ~size_t(0));
         PersistentPtrs p;
         carve_persistent(c, n, L, &p);
         *persistent_bytes = c.off;
     }
-    if (scratch_bytes) {
-        Carver c(nullptr, ~size_t(0));
-        ScratchPtrs s;
-        carve_scratch(c, L, &s);
-        *scratch_bytes = c.off;
-    }
+    if (segments) *segments = L.seg_cap;
+    if (!scratch_bytes) return GNNFD_OK;
+    *scratch_bytes = scratch_size(L);
+    if (!for_smaller || L.top_bits > 0 || !use_large_tile(L.m)) return GNNFD_OK;
+    for (int bits = 31; bits > 0; --bits)                   // the largest graph with buckets: key bits grow at 2^bits and behind it
+        for (int64_t less = int64_t(1) << bits; less >= (int64_t(1) << bits) - 1; --less) {
+            BuildLayout with;
+            if (less >= n || make_layout(less, e, flags, &with) || with.top_bits == 0) continue;
+            const size_t bytes = scratch_size(with);
+            if (bytes > *scratch_bytes) *scratch_bytes = bytes;
+            return GNNFD_OK;
+        }
     return GNNFD_OK;
+}
+
+}  // namespace gnnfd
+
+extern "C" {
+
+int gnnfd_csr_workspace_bytes(int64_t n, int64_t e, uint32_t flags, size_t* persistent_bytes, size_t* scratch_bytes)
+{
+    return gnnfd::csr_sizes(n, e, flags, true, persistent_bytes, scratch_bytes, nullptr);
 }
 
 int gnnfd_build_csr(int64_t n, int64_t e, const void* d_src, const void* d_dst, gnnfd_itype_t itype, uint32_t flags,

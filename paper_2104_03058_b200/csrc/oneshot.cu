@@ -16,14 +16,14 @@ static uint32_t oneshot_flags(uint32_t flags)
     return (flags & GNNFD_CSR_DEDUP) ? flags : (flags | GNNFD_CSR_INPUT_ORDER);
 }
 
-// heads > 0: the GAT aggregation's workspace (two [n, heads] score arrays, per-segment sums, maxima and denominators)
-static int oneshot_layout(int64_t n, int64_t e, uint32_t flags, int32_t f, int32_t heads, OneshotLayout* L)
+// heads > 0: the GAT aggregation's workspace (two [n, heads] score arrays, per-segment sums, maxima and denominators).  query: with room for
+// every smaller graph
+static int oneshot_layout(int64_t n, int64_t e, uint32_t flags, int32_t f, int32_t heads, bool query, OneshotLayout* L)
 {
     if (f <= 0 || heads < 0) return GNNFD_INVALID_ARG;
-    int rc = gnnfd_csr_workspace_bytes(n, e, oneshot_flags(flags), &L->persistent, &L->build_scratch);
+    int64_t segs = 0;
+    int rc = csr_sizes(n, e, oneshot_flags(flags), query, &L->persistent, &L->build_scratch, &segs);
     if (rc) return rc;
-    const int64_t segs = segment_capacity(n, e, oneshot_flags(flags));
-    if (segs < 0) return GNNFD_INVALID_ARG;
     L->aggregate = align_up((size_t)segs * align_up((size_t)f, 4) * sizeof(float), 256);
     if (heads > 0)
         L->aggregate += 2 * align_up((size_t)n * heads * sizeof(float), 256) +
@@ -37,7 +37,7 @@ static int oneshot(bool weighted, int64_t n, int64_t e, const void* d_src, const
 {
     if (!d_scratch || ((uintptr_t)d_scratch & 255u)) return GNNFD_INVALID_ARG;
     OneshotLayout L;
-    int rc = oneshot_layout(n, e, flags, f, 0, &L);
+    int rc = oneshot_layout(n, e, flags, f, 0, false, &L);
     if (rc) return rc;
     if (scratch_bytes < L.persistent + L.build_scratch + L.aggregate) return GNNFD_WORKSPACE_TOO_SMALL;
     char* base = static_cast<char*>(d_scratch);
@@ -62,7 +62,7 @@ int gnnfd_oneshot_workspace_bytes(int64_t n, int64_t e, uint32_t flags, int32_t 
 {
     if (!scratch_bytes) return GNNFD_INVALID_ARG;
     gnnfd::OneshotLayout L;
-    int rc = gnnfd::oneshot_layout(n, e, flags, f, 0, &L);
+    int rc = gnnfd::oneshot_layout(n, e, flags, f, 0, true, &L);
     if (rc) return rc;
     *scratch_bytes = L.persistent + L.build_scratch + L.aggregate;
     return GNNFD_OK;
@@ -72,7 +72,7 @@ int gnnfd_oneshot_gat_workspace_bytes(int64_t n, int64_t e, uint32_t flags, int3
 {
     if (!scratch_bytes || heads <= 0 || dim <= 0 || (int64_t)heads * dim > 0x7fffffffll) return GNNFD_INVALID_ARG;
     gnnfd::OneshotLayout L;
-    int rc = gnnfd::oneshot_layout(n, e, flags, heads * dim, heads, &L);
+    int rc = gnnfd::oneshot_layout(n, e, flags, heads * dim, heads, true, &L);
     if (rc) return rc;
     *scratch_bytes = L.persistent + L.build_scratch + L.aggregate;
     return GNNFD_OK;
@@ -87,7 +87,7 @@ int gnnfd_oneshot_gat(int64_t n, int64_t e, const void* d_src, const void* d_dst
     if (!d_scratch || ((uintptr_t)d_scratch & 255u) || heads <= 0 || dim <= 0 || (int64_t)heads * dim > 0x7fffffffll)
         return GNNFD_INVALID_ARG;
     OneshotLayout L;
-    int rc = oneshot_layout(n, e, flags, heads * dim, heads, &L);
+    int rc = oneshot_layout(n, e, flags, heads * dim, heads, false, &L);
     if (rc) return rc;
     if (scratch_bytes < L.persistent + L.build_scratch + L.aggregate) return GNNFD_WORKSPACE_TOO_SMALL;
     char* base = static_cast<char*>(d_scratch);
