@@ -396,7 +396,7 @@ int gnnfd_debug_combine_fault(int64_t wait_ns, int32_t skip_k_block);
 /* Drill of the CSR build's give-up path, for tests.  It arms the NEXT gnnfd_build_csr or gnnfd_oneshot_* call made by this host
  * thread, and only that one: a block of the sort gives up after max_polls reads (rounded up to 256; 0 keeps the usual million)
  * of a word that another block has not written yet, and in sweep `sweep` (0 ..: the digits; one past the last digit: the row
- * order) nobody takes the first tile, so all others wait for it and give up.  The kernels that follow do nothing, the
+ * order; two past it, in gnnfd_oneshot_* calls without duplicate removal: the row pointers' sums) nobody takes the first tile, so all others wait for it and give up.  The kernels that follow do nothing, the
  * call returns GNNFD_CUDA_ERROR and no handle, nothing outside the call's buffers is touched and the device stays usable.
  * Where the sweep does not exist, has a single tile, or sorts buckets that need not hold a second one (all but the first of a large
  * graph's, where ids and edge numbers together need more than 64 bits), the armed call returns GNNFD_INVALID_ARG and launches nothing. */

@@ -958,7 +958,7 @@ constexpr u64 kOwn64 = 1ull << 61, kSum64 = 1ull << 62;
 
 // By one whole warp: the sum of all tiles before `tile`, which holds `total` itself; publishes both.  Every lane gets the result,
 // or -1: gave up (and the build is marked as failed).
-__device__ __forceinline__ int64_t chain_sums(u64* __restrict__ words, int64_t tile, int32_t total, int32_t* failed)
+__device__ __forceinline__ int64_t chain_sums(u64* __restrict__ words, int64_t tile, int32_t total, int max_polls, int32_t* failed)
 {
     const int lane = threadIdx.x & 31;
     auto store = [&](u64 v) { asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(words + tile), "l"(v) : "memory"); };
@@ -973,7 +973,7 @@ __device__ __forceinline__ int64_t chain_sums(u64* __restrict__ words, int64_t t
             sums = __ballot_sync(0xffffffffu, (w & kSum64) != 0ull);
             // everything up to the nearest sum is there
             if (missing == 0u || (sums != 0u && (missing & ((sums & (0u - sums)) - 1u)) == 0u)) break;
-            if ((polls & 255) == 255 && (polls >= kMaxPolls || load_published(reinterpret_cast<const uint32_t*>(failed)) != 0u)) {
+            if ((polls & 255) == 255 && (polls >= max_polls - 1 || load_published(reinterpret_cast<const uint32_t*>(failed)) != 0u)) {
                 if (lane == 0) atomicExch(failed, 1);
                 return -1;
             }
@@ -999,7 +999,7 @@ constexpr int kSlotTile = kThreads * kSlotItems;
 __global__ void __launch_bounds__(kThreads)
 rows_from_degrees(const int32_t* degree, BuildCounts* __restrict__ counts, int64_t n, int32_t* __restrict__ ticket,
                   u64* __restrict__ words, int32_t* __restrict__ row_ptr, float* __restrict__ dinv, float* __restrict__ rdeg,
-                  int32_t* __restrict__ class_count, int32_t* __restrict__ slot_tile_row)
+                  int32_t* __restrict__ class_count, int32_t* __restrict__ slot_tile_row, int max_polls)
 {
     grid_dependency<true>();
     __shared__ int32_t smem[kThreads / 32], class_smem[kClasses], bin_smem[kNumBins], octave_smem[kOctaves], max_smem, drawn;
@@ -1013,7 +1013,7 @@ rows_from_degrees(const int32_t* degree, BuildCounts* __restrict__ counts, int64
     if (threadIdx.x < kOctaves) octave_smem[threadIdx.x] = 0;
     __syncthreads();
     const int tile = drawn;
-    if (tile < 0) return;
+    if (tile < 0 || (int64_t)tile * kRowTile >= n) return;             // (a drawn number is past the last tile only where the drill left out the first)
     if (tile == 0 && threadIdx.x == 0) counts->nnz = counts->n_valid;
     const int64_t first = (int64_t)tile * kRowTile + threadIdx.x * kRowItems;
     int32_t deg[kRowItems], sum = 0, total;
@@ -1024,7 +1024,7 @@ rows_from_degrees(const int32_t* degree, BuildCounts* __restrict__ counts, int64
     }
     const int32_t in_tile = block_prefix_256(sum, &total, smem);
     if (threadIdx.x < 32) {
-        const int64_t start = chain_sums(words, tile, total, &counts->sort_failed);
+        const int64_t start = chain_sums(words, tile, total, max_polls, &counts->sort_failed);
         if (threadIdx.x == 0) before = start;
     }
     int32_t most = 0;
@@ -1520,7 +1520,11 @@ int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, g
 
     // the drill leaves out a sweep's first tile: another one has to be there to miss it, of the same bucket where there are buckets
     if (drill.sweep > 0 && drill.sweep < L.sweeps() && L.top_bits > 0) return GNNFD_INVALID_ARG;
-    if (drill.sweep >= 0 && (drill.sweep > L.sweeps() || (drill.sweep < L.sweeps() ? L.n_tiles : L.row_tiles) < 2)) return GNNFD_INVALID_ARG;
+    if (drill.sweep >= 0) {
+        const int64_t tiles = drill.sweep < L.sweeps() ? L.n_tiles : drill.sweep == L.sweeps() ? L.row_tiles :
+                              drill.sweep == L.sweeps() + 1 && !L.with_vals ? L.row_words : 0;
+        if (tiles < 2) return GNNFD_INVALID_ARG;
+    }
 
     const int64_t m = L.m;
     // Without ids the last sweep writes the entries and counts the degrees.  With them it is better to write words once more: 80 M
@@ -1620,7 +1624,8 @@ int build_csr_impl(int64_t n, int64_t e, const void* d_src, const void* d_dst, g
     if (entries) {
         int32_t* slot_tile_row = need_weights ? S.flags : nullptr;
         GNNFD_LAUNCH("rows_from_degrees", s, rows_from_degrees, (unsigned)L.row_words, kThreads, 0, degree, P.counts, n,
-                     S.ticket + L.sweeps() + 1, S.row_words, P.row_ptr, P.dinv, P.rdeg, class_count, slot_tile_row);
+                     S.ticket + L.sweeps() + 1, S.row_words, P.row_ptr, P.dinv, P.rdeg, class_count, slot_tile_row,
+                     drill.max_polls);
         if (m > 0 && need_weights)
             GNNFD_LAUNCH("slot_weights", s, slot_weights, blocks_for(m, kSlotTile), kThreads, 0, P.row_ptr, P.col_idx, slot_tile_row,
                          P.dinv, P.counts, P.edge_w);

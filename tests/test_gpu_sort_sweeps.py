@@ -127,6 +127,41 @@ def test_a_tile_that_is_never_published_ends_the_build_with_an_error(g, n, m, pa
     np.testing.assert_array_equal(csr.perm.cpu().numpy(), perm)
 
 
+# the one-shot path, whose words are keys alone (17 destination bits, two digits of 9; 23 bits, three): each sweep over the edges, the last of which writes the
+# entries, the rows' order, and the chain of the row pointers' sums
+@pytest.mark.parametrize("n,passes", [(70_001, 2), ((1 << 22) + 3, 3)])
+@pytest.mark.parametrize("sweep", ["first", "last", "rows", "sums"])
+@pytest.mark.parametrize("model", ["gcn", "sage"])
+def test_a_light_build_that_gives_up_ends_the_call_with_an_error(g, n, passes, sweep, model):
+    m = 200_000
+    rng = np.random.default_rng(m)
+    src, dst = (rng.integers(0, n, m).astype(np.int32) for _ in range(2))
+    ds, dd, x = torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), torch.randint(-8, 9, (n, 4), device="cuda").float()
+    need = g.oneshot_workspace_bytes(n, m, 0, 4)
+    s_all, scratch = guarded(need)
+    out = torch.full((n, 4), 7.0, device="cuda")
+    g.debug_build_fault(1024, {"first": 0, "last": passes - 1, "rows": passes, "sums": passes + 1}[sweep])
+    with pytest.raises(g.GnnfdError) as err:
+        g.oneshot(model, n, ds, dd, x, out=out, scratch=scratch)
+    assert err.value.status == g.CUDA_ERROR
+    torch.cuda.synchronize()
+    assert bool((s_all[:GUARD] == 0xAB).all()) and bool((s_all[GUARD + need:] == 0xAB).all()) and bool((out == 7.0).all())
+    got = g.oneshot(model, n, ds, dd, x, out=out, scratch=scratch)
+    csr = g.build_csr(n, ds, dd, LIGHT)
+    assert torch.equal(got, (g.aggregate_gcn if model == "gcn" else g.aggregate_sage)(csr, x))
+
+
+def test_the_drill_refuses_row_sums_where_there_are_none(g):
+    ids = torch.zeros(200_000, dtype=torch.int32, device="cuda")
+    x = torch.zeros((70_001, 4), device="cuda")
+    for sweep, call in ((5, lambda: g.build_csr(70_001, ids, ids, 0)), (5, lambda: g.oneshot("gcn", 70_001, ids, ids, x, flags=DD)),
+                        (3, lambda: g.oneshot("gcn", 2000, ids, ids, x[:2000]))):       # edge ids, duplicate removal; a single tile of rows
+        g.debug_build_fault(1024, sweep)
+        with pytest.raises(g.GnnfdError) as err:
+            call()
+        assert err.value.status == g.INVALID_ARG
+
+
 def test_the_drill_refuses_sweeps_that_nobody_would_miss(g):
     src = torch.arange(3000, dtype=torch.int32, device="cuda")
     for sweep in (0, 9):                                             # one tile of edges only; no such sweep
