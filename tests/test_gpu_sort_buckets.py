@@ -64,3 +64,20 @@ def test_the_drill_refuses_sweeps_inside_buckets(g):
         with pytest.raises(g.GnnfdError) as err:
             g.build_csr(N, ids, ids, 0)
         assert err.value.status == g.INVALID_ARG
+
+
+@pytest.mark.parametrize("flags", [0, DD, LIGHT])
+def test_words_that_fill_64_bits(g, flags):
+    """2^25 - 1 vertices and 4.85 to 8.4 M candidates: 41 key bits and 23 value bits.  Out of buffers sized for one more vertex, with which
+    there are no buckets."""
+    n, m = (1 << 25) - 1, LARGE + 12_345
+    rng = np.random.default_rng(flags)
+    src = rng.integers(0, n, m).astype(np.int32)
+    dst = np.where(np.arange(m) % 3 == 0, n - 1, rng.integers(n // 2, n, m)).astype(np.int32)
+    src[:9], src[9:18], dst[:18] = n - 1, 0, n - 1
+    pb, sb = g.csr_workspace_bytes(n + 1, m, flags)
+    persistent, scratch = (torch.empty(b, dtype=torch.uint8, device="cuda") for b in (pb, sb))
+    csr = g.build_csr(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), flags, persistent=persistent, scratch=scratch)
+    row_ptr, col, perm = reference(n, src, dst, flags)
+    for name, want in (("row_ptr", row_ptr), ("col_idx", col), ("perm", perm)):
+        np.testing.assert_array_equal(getattr(csr, name).cpu().numpy(), want, err_msg=name)
