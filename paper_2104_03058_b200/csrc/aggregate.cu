@@ -60,7 +60,9 @@ constexpr bool shortest_first(int elem_bytes, int vecn, int lpr, int vpl, bool s
 // 20 entries, 128 columns in chunks of 64 96 -> 86 us, 200,000 of 16, 64 columns 90 -> 76, 32 39 -> 32, RMAT 2^19, 64 columns 368 -> 315; GCN fp32
 // without split rows, 41 columns on 132,534 rows of 300 542 -> 515, 304 in chunks of 64 371 -> 348, 32 on 233,000 of 86 211 -> 190.  But wider
 // rows lose: GCN of 144 / 256 columns 214 -> 228 / 240 -> 277, SAGE of 256 on 20,000 rows of 50 59 -> 65; so do split rows of GCN (64 columns 28 -> 31)
-// and bf16 (SAGE of 64 / 256 columns 35 -> 41 / 130 -> 151, GCN of 64 on RMAT 2^21 1487 -> 1832).
+// and bf16 (SAGE of 64 / 256 columns 35 -> 41 / 130 -> 151, GCN of 64 on RMAT 2^21 1487 -> 1832).  Chunks of 65 - 96 fp32 columns, three vectors
+// per lane, too: 72 / 96 columns SAGE on 200,000 rows of 16 105 -> 91 / 113 -> 98, on 132,534 of 300 728 -> 692 / 768 -> 726, GCN there 770 -> 760 / 788 -> 785.
+// Spilled at 64 registers, outside the loop over entries: 4 - 32 bytes of <4, 8, 3> and <4, 2, 2> SAGE, 24 - 56 of <4, 8, 2>, <4, 2, 2> and <4, 8, 3> GCN.
 constexpr int min_blocks(int elem_bytes, bool weighted, bool shared, int lpr)
 {
     return elem_bytes == 4 && lpr <= 8 && !(weighted && shared) ? 4 : 3;
@@ -583,15 +585,23 @@ static int aggregate(bool weighted, const gnnfd_csr_t* csr, const void* d_x, int
     a.out_vec_ok = odt == GNNFD_F32 && ((uintptr_t)d_out % 16 == 0) && (ldo % 4 == 0) && (n_chunks == 1 || cw % 4 == 0);
 
     const int per_step = kLoads / vpl * (32 / lpr);
-    const int64_t limit = walk_limit(csr, per_step, a.n_ctiles, 16, min_blocks(xsize, weighted, true, lpr));
-    const int64_t blocks = plan_ranges(csr, gather_groups(), lpr, per_step, limit, a.range, &a.n_ranges);
+    bool shared = false;
+    int64_t blocks = 0;
+    auto plan = [&](int blocks_per_sm) {
+        blocks = plan_ranges(csr, gather_groups(), lpr, per_step, walk_limit(csr, per_step, a.n_ctiles, 16, blocks_per_sm), a.range, &a.n_ranges);
+        for (int i = 0; i < a.n_ranges; ++i) shared = shared || a.range[i].warps_log2 > 0;
+    };
+    const int unsplit = min_blocks(xsize, weighted, false, lpr), split = min_blocks(xsize, weighted, true, lpr);
+    // GCN's kernel for unsplit rows has four blocks per SM, that for split ones three.  From where four would call for splitting to where three do
+    // (3.6 to 4.8 M entries), the longest rows decide and three are faster unsplit: 100,000 rows of 40, 16 / 64 / 96 columns 44 / 99 / 125 us
+    // with four, 36 / 79 / 104 with three; above, 200,000 of 30, 50 / 113 / 165 with four, 52 / 121 / 170 with three.
+    plan(unsplit);
+    if (shared && split != unsplit) plan(split);
     a.blocks_per_tile = (int32_t)blocks;
     const int64_t grid_x = blocks * a.n_ctiles;
     if (grid_x > 0x7fffffffll) return GNNFD_TOO_LARGE;
 
     if (grid_x > 0) {
-        bool shared = false;
-        for (int i = 0; i < a.n_ranges; ++i) shared = shared || a.range[i].warps_log2 > 0;
         if (shortest_first(xsize, elems, lpr, vpl, shared))
             for (int i = 0; i < a.n_ranges; ++i) {
                 a.range[i].item_first -= a.range[i].item_count - 1;

@@ -116,3 +116,25 @@ def test_long_rows_of_sage_are_split_as_finely_as_its_blocks_need(f):
         return least
 
     assert us(g.aggregate_sage) < 1.05 * us(g.aggregate_gcn)
+
+
+def test_gcn_just_above_the_size_that_splits_rows():
+    """Between the sizes at which rows are split for three and for four blocks on an SM, GCN keeps three: with four, a quarter more entries
+    took half as long again, for the longest rows' sake."""
+    import paper_2104_03058_b200 as g
+    n, f, times = 100_000, 96, []
+    for e in (3_300_000, 4_200_000):
+        csr = g.build_csr(n, *graph(n, e, 1), g.CSR_ADD_SELF_LOOPS)
+        x, out = torch.randn((n, f), device="cuda"), torch.empty((n, f), device="cuda")
+        begin, end, least = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True), float("inf")
+        for _ in range(6):
+            begin.record()
+            for _ in range(50):
+                g.aggregate_gcn(csr, x, out=out)
+            end.record()
+            end.synchronize()
+            least = min(least, begin.elapsed_time(end) * 20)
+        times.append((least, csr.nnz))
+    (small, few), (large, many) = times
+    assert few < 3_640_000 < many < 4_700_000
+    assert large / small < 1.15 * many / few, times
