@@ -230,7 +230,7 @@ __device__ __forceinline__ void gather_rows(const GatherArgs& a, const Range& rg
                 for (int q = 0; q < VPL; ++q)
 #pragma unroll
                     for (int k = 0; k < VECN; ++k) {
-                        if constexpr (!WEIGHTED && sizeof(T) == 2 && VECN > 1 && !(LPR >= 16 && VPL == 2)) {
+                        if constexpr (!WEIGHTED && sizeof(T) == 2 && VECN > 1) {
                             if (k % 2 == 0) add_widened(acc[q][k], acc[q][k + 1], v[i][q].word(k / 2));
                         } else if (WEIGHTED) acc[q][k] = fmaf(wv[i], v[i][q].get(k), acc[q][k]);
                         else acc[q][k] += v[i][q].get(k);
