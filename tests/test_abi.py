@@ -40,14 +40,37 @@ def test_host_only_entry_points_work_without_a_device():
 
 def test_workspaces_never_shrink_as_a_graph_grows():
     """A buffer sized for the largest graph has to hold every smaller one: sizes around the points where the build changes its tiles
-    (4,849,664 candidates or rows), parts keys and values, makes buckets or no longer (at 2^25 vertices with 4.85 to 8.4 M candidates, at 2^24
-    with twice as many), or widens its source ranges (behind 2^25), and between."""
+    (4,849,664 candidates or rows) or parts keys and values, and between."""
     import paper_2104_03058_b200 as g
     switch = 4 * 148 * 8192
     around = [switch + d for d in (-500_000, -200_000, -2049, -2048, -1, 0, 1, 8192, 200_000, 500_000, 2_000_000, 14_000_000, 15_000_000)]
     edges = sorted([0, 1, 2047, 2048, 2049, 1 << 16, 1 << 20, 1 << 22, 30_000_000, 60_000_000, 115_000_000, 1_000_000_000] + around +
                    [a - 100_000 for a in around] + [a // 2 for a in around])
-    for n in (1, 100_000, 1 << 20, (1 << 22) + 3, 1 << 24, (1 << 25) - 1, 1 << 25, (1 << 25) + 1):
+    for n in (1, 100_000, 1 << 20, (1 << 22) + 3, 1 << 24):
+        for flags in (0, 1, 2, 7, 8, 13):
+            sizes = [g.csr_workspace_bytes(n, e, flags) for e in edges if (2 if flags & 4 else 1) * e + n < 1 << 31]
+            for small, large in zip(sizes, sizes[1:]):
+                assert small[0] <= large[0] and small[1] <= large[1]
+            if not flags & 8:
+                one = [g.oneshot_workspace_bytes(n, e, flags, 32) for e in edges if (2 if flags & 4 else 1) * e + n < 1 << 31]
+                assert one == sorted(one)
+    rows = sorted([1, 1000, 1 << 17, 1 << 20, 1 << 22, 20_000_000] + around)
+    for e in (0, 100_000, 4_000_000, 40_000_000):
+        for flags in (0, 1, 8):
+            sizes = [g.csr_workspace_bytes(n, e, flags) for n in rows]
+            for small, large in zip(sizes, sizes[1:]):
+                assert small[0] <= large[0] and small[1] <= large[1]
+
+
+def test_workspaces_never_shrink_around_the_end_of_the_bucket_sort():
+    """The same at the sizes where the build makes buckets or no longer (at 2^25 vertices with 4.85 to 8.4 M candidates, at 2^24 with twice
+    as many) or widens its source ranges (behind 2^25)."""
+    import paper_2104_03058_b200 as g
+    switch = 4 * 148 * 8192
+    around = [switch + d for d in (-500_000, -200_000, -2049, -2048, -1, 0, 1, 8192, 200_000, 500_000, 2_000_000, 14_000_000, 15_000_000)]
+    edges = sorted([0, 1, 2047, 2048, 2049, 1 << 16, 1 << 20, 1 << 22, 30_000_000, 60_000_000, 115_000_000, 1_000_000_000] + around +
+                   [a - 100_000 for a in around] + [a // 2 for a in around])
+    for n in ((1 << 25) - 1, 1 << 25, (1 << 25) + 1):
         for flags in (0, 1, 2, 7, 8, 13):
             sizes = [g.csr_workspace_bytes(n, e, flags) for e in edges if (2 if flags & 4 else 1) * e + n < 1 << 31]
             for small, large in zip(sizes, sizes[1:]):
